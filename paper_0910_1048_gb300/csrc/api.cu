@@ -134,6 +134,7 @@ ovl_status ovl_destroy_lattice(ovl_lattice* lat) {
   free_multi_ws(lat->mws);
   if (lat->owns_links) {
     cudaFree(lat->u64);
+    cudaFree(lat->ufx);
     cudaFree(lat->u32);
     cudaFree(lat->u16);
     cudaFree(lat->defl.R);
@@ -161,6 +162,10 @@ ovl_status ovl_set_links(ovl_lattice* lat, const void* U, int32_t U_on_device, u
   if (lat->u32) formats |= OVL_F32;
   if (lat->u16) formats |= OVL_F16R12;
   if (!lat->u64) OVL_CHECK_CUDA(cudaMalloc(&lat->u64, nl * 16));
+  if (!lat->ufx) {
+    OVL_CHECK_CUDA(cudaMalloc(&lat->ufx, nl * 16 + fx_field_bytes()));
+    lat->fxf = (FxField*)((char*)lat->ufx + nl * 16);
+  }
   if ((formats & OVL_F32) && !lat->u32) OVL_CHECK_CUDA(cudaMalloc(&lat->u32, nl * 8));
   if ((formats & OVL_F16R12) && !lat->u16) OVL_CHECK_CUDA(cudaMalloc(&lat->u16, (size_t)24 * lat->g.vol * 4));
   const double* src = (const double*)U;
@@ -171,7 +176,7 @@ ovl_status ovl_set_links(ovl_lattice* lat, const void* U, int32_t U_on_device, u
     OVL_CHECK_CUDA(cudaMemcpyAsync(tmp, U, nl * 16, cudaMemcpyHostToDevice, st));
     src = tmp;
   }
-  cudaError_t e = launch_ingest_links(lat->g, src, lat->u64, (formats & OVL_F32) ? lat->u32 : nullptr,
+  cudaError_t e = launch_ingest_links(lat->g, src, lat->u64, lat->ufx, lat->fxf, (formats & OVL_F32) ? lat->u32 : nullptr,
                                       (formats & OVL_F16R12) ? lat->u16 : nullptr, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (tmp) cudaFree(tmp);
@@ -281,7 +286,7 @@ ovl_status ovl_apply_DW(ovl_lattice* lat, double m_W, double mu, uint32_t flags,
   }
   const bool dag = flags & OVL_DAGGER, g5 = flags & OVL_GAMMA5, nat = flags & OVL_NATIVE;
   // D^H = g5 D(-mu) g5; output gamma5 count = dag xor g5
-  OVL_CHECK_CUDA(launch_dslash(lat->g, lat->src()->links(), lf, f64, m_W, dag ? -mu : mu, dag, dag != g5, nat, nat, nrhs, in,
+  OVL_CHECK_CUDA(launch_dslash(lat->g, lat->src()->links(), lf, f64, m_W, dag ? -mu : mu, dag, dag != g5, nat, nrhs, in,
                                out, (cudaStream_t)stream));
   return OVL_OK;
 }

@@ -110,8 +110,12 @@ struct Geom {
 // Device-resident links in the formats the caller asked for. Layout [dir][comp][V]
 // (component-major, site fastest) so that a warp's 32 consecutive sites read one
 // contiguous segment per component.
+struct FxC;
+struct FxField;
 struct Links {
   const double2* f64 = nullptr;   // [4][9][V]
+  const FxC* fx = nullptr;        // [4][9][V] fixed-point copy of the FP64 links (fixedpt.cuh)
+  const FxField* fxf = nullptr;   // its scale, and whether it can be used
   const float2* f32 = nullptr;    // [4][9][V]
   const uint32_t* f16 = nullptr;  // [4][6][V] half2 bits, rows 0 and 1
 };
@@ -154,6 +158,8 @@ struct ovl_lattice {
   ovl::Geom g{};
   uint32_t formats = 0;
   double2* u64 = nullptr;
+  ovl::FxC* ufx = nullptr;        // fixed-point copy of u64 and its scale (one allocation)
+  ovl::FxField* fxf = nullptr;
   float2* u32 = nullptr;
   uint32_t* u16 = nullptr;
   ovl_deflation defl;
@@ -162,6 +168,8 @@ struct ovl_lattice {
   ovl::Links links() const {
     ovl::Links l;
     l.f64 = u64;
+    l.fx = ufx;
+    l.fxf = fxf;
     l.f32 = u32;
     l.f16 = u16;
     return l;

@@ -1,6 +1,7 @@
 // Device helpers shared by the kernel translation units.
 #pragma once
 
+#include "fixedpt.cuh"
 #include "wilson.cuh"
 
 namespace ovl {
@@ -314,6 +315,96 @@ __device__ __forceinline__ void store_spin(typename V2<R>::T* p, int vol, int s,
 }
 
 
+// ------------------------------------------------------------------ hops of a site
+// Hop coefficients by precision: the FP64 stencil runs in fixed point (fixedpt.cuh).
+template <class R> struct HopsOf { using T = HopCoef<R>; };
+template <> struct HopsOf<double> { using T = FxCoef; };
+template <class R>
+inline typename HopsOf<R>::T hops_of(double m_w, double mu) {
+  if constexpr (sizeof(R) == 8) return fx_coef(m_w, mu);
+  else return hop_coef<R>(m_w, mu);
+}
+
+// Spinor loads with the layout as run-time strides: component c of site s at s * ss + c * cs.
+struct StrideLoader {
+  const double2* p;
+  int ss, cs;
+  __device__ __forceinline__ void operator()(int s, Spin<double>& o) const {
+#pragma unroll
+    for (int c = 0; c < 12; ++c) o.c[c / 3][c % 3] = ldc<double>(p, (size_t)s * ss + (size_t)c * cs);
+  }
+};
+struct StrideLoaderG5 : StrideLoader {
+  __device__ __forceinline__ void operator()(int s, Spin<double>& o) const {
+    StrideLoader::operator()(s, o);
+    gamma5_inplace(o);
+  }
+};
+
+// The FP64 hops k0 .. k1-1 (k0, k1 even) at site s, added to `out`: where fixed point cannot be used
+// (see fixedpt.cuh). A call, not inlined: it is rare, and inlined it would add its registers to every
+// stencil kernel.
+template <class Load>
+__device__ __forceinline__ void hops_f64_ld(const Geom& g, const Links& U, int s, const HopCoef<double>& c, int k0, int k1,
+                                            Load ld, Spin<double>& out) {
+  Nbr n;
+  neighbours(g, s, n);
+  if (k0 <= 0 && k1 > 0) hop_dir<0, LINK_F64>(g, U, s, n, c.ks, c.ks, ld, out);
+  if (k0 <= 2 && k1 > 2) hop_dir<1, LINK_F64>(g, U, s, n, c.ks, c.ks, ld, out);
+  if (k0 <= 4 && k1 > 4) hop_dir<2, LINK_F64>(g, U, s, n, c.ks, c.ks, ld, out);
+  if (k0 <= 6 && k1 > 6) {
+    const double ktf = (n.t == g.lt - 1) ? g.t_bc * c.ktf : c.ktf;
+    const double ktb = (n.t == 0) ? g.t_bc * c.ktb : c.ktb;
+    hop_dir<3, LINK_F64>(g, U, s, n, ktf, ktb, ld, out);
+  }
+}
+// (static: one copy per translation unit)
+static __device__ __noinline__ void hops_f64(const Geom& g, const double2* u64, int s, const HopCoef<double>& c, int k0,
+                                             int k1, StrideLoader ld, bool g5in, Spin<double>& out) {
+  Links U;
+  U.f64 = u64;
+  if (g5in)
+    hops_f64_ld(g, U, s, c, k0, k1, StrideLoaderG5{ld}, out);
+  else
+    hops_f64_ld(g, U, s, c, k0, k1, ld, out);
+}
+
+// out += the hops k0 .. k1-1 of psi = in (or gamma5 in).
+__device__ __forceinline__ void add_hops(const Geom& g, const Links& U, int s, int k0, int k1, const FxCoef& c,
+                                         StrideLoader ld, bool g5in, bool self, Spin<double>& out) {
+  FxAcc acc;
+  fx_clear(acc);
+  const bool fx = c.ok && U.fxf->ok;
+  if (fx) fx_hops(g, U.fx, s, k0, k1, c, ld, g5in, acc);
+  if (self) {
+    ld(s, out);
+    if (g5in) gamma5_inplace(out);
+  }
+  if (fx && fx_usable(acc)) {
+    const double f = fx_unit(acc, c, U.fxf->uexp);
+#pragma unroll
+    for (int i = 0; i < 12; ++i) {
+      cplx<double>& o = out.c[i / 3][i % 3];
+      o.re = fma(f, (double)acc.re[i / 3][i % 3], o.re);
+      o.im = fma(f, (double)acc.im[i / 3][i % 3], o.im);
+    }
+  } else {
+    Spin<double> t = out;
+    hops_f64(g, U.f64, s, c.k, k0, k1, ld, g5in, t);
+    out = t;
+  }
+}
+
+// out = D_W psi at site s, psi native.
+template <int LF, class R>
+__device__ __forceinline__ void stencil_site(const Geom& g, const Links& U, int s, const typename HopsOf<R>::T& c,
+                                             const typename V2<R>::T* in, Spin<R>& out) {
+  if constexpr (sizeof(R) == 8)
+    add_hops(g, U, s, 0, 8, c, StrideLoader{in, 1, g.vol}, false, true, out);
+  else
+    dslash_site<LF, R>(g, U, s, c, Loader<R, true>{in, g.vol, false}, out);
+}
+
 // ------------------------------------------------------------------ split-site pair stencil
 // For small lattices (too few sites to fill 152 SMs with one thread per site) every site is
 // shared by 8 threads: threadIdx.y = which * 4 + dir, `which` selecting input 0 (coefficients
@@ -332,13 +423,14 @@ struct SplitSmem {
 };
 
 template <class R, int LF, int SITES = kSplitSites, class Emit>
-__device__ __forceinline__ void pair_split(const Geom& g, const Links& U, const HopCoef<R>& c0, const HopCoef<R>& c1,
+__device__ __forceinline__ void pair_split(const Geom& g, const Links& U, const typename HopsOf<R>::T& c0,
+                                           const typename HopsOf<R>::T& c1,
                                            const typename V2<R>::T* in0, const typename V2<R>::T* in1,
                                            SplitSmem<R, SITES>& sm, Emit emit) {
   const int tx = threadIdx.x, which = threadIdx.y >> 2, dir = threadIdx.y & 3;
   const int s = blockIdx.x * SITES + tx;
   const typename V2<R>::T* in = which ? in1 : in0;
-  const HopCoef<R>& c = which ? c1 : c0;
+  const typename HopsOf<R>::T& c = which ? c1 : c0;
   Loader<R, true> ld{in, g.vol, false};
   Spin<R> acc;
 #pragma unroll
@@ -346,7 +438,9 @@ __device__ __forceinline__ void pair_split(const Geom& g, const Links& U, const 
   if (s < g.vol) {
     Nbr n;
     neighbours(g, s, n);
-    if (dir == 0) {
+    if constexpr (sizeof(R) == 8) {
+      add_hops(g, U, s, 2 * dir, 2 * dir + 2, c, StrideLoader{in, 1, g.vol}, false, false, acc);
+    } else if (dir == 0) {
       hop_dir<0, LF>(g, U, s, n, c.ks, c.ks, ld, acc);
     } else if (dir == 1) {
       hop_dir<1, LF>(g, U, s, n, c.ks, c.ks, ld, acc);

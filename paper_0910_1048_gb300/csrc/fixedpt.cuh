@@ -1,0 +1,423 @@
+// The FP64 stencil's hop sums in fixed point on the integer pipe.
+//
+// GB300 issues two FP64 operations per SM and clock (a DFMA chain probe: 1.7 lanes) but 64 32 x 32 + 64
+// bit integer multiply-adds (mad.wide.s32: 63 lanes measured), so a product of two 59-bit fixed-point
+// numbers from three of them costs 1/12 of a DFMA. A hop's link product is a sum of six real products with
+// a common scale, which fixed point holds exactly, so the stencil's FP64 work is left only where
+// values leave a site: one conversion and one fused multiply-add per output component.
+//
+// A number is x = (h 2^30 + l) 2^-59 S: h a signed, l a 30-bit limb, S a power of two.
+//  - Spinors: S is 2^(e+1) for e the exponent of the site's largest component (block floating point:
+//    one S for the 24 reals of a neighbour), |h| <= 2^29, 0 <= l < 2^30. A component is cut at
+//    2^-59 S; FP64 arithmetic on the same site rounds every partial sum at about 2^-54 S.
+//  - Links: S is one power of two for the field, at least its largest component and its largest row or
+//    column sum of moduli of components over sqrt(6) (1 for SU(3)), l balanced in [-2^29, 2^29), so
+//    that the dropped l l products have mean zero.
+//  - Projected half spinors are limb-wise sums: |h| <= 2^30, l in (-2^30, 2^31).
+//  - Products: H = sum h_u h, X = sum (h_u l + l_u h) over a row's six components, |H| < 2^60.4 and
+//    |X| < 2^62.5; the l_u l terms, below 2^-59 of full scale, are dropped.
+//  - A hop's 12 reals T = H + (X >> 30) are rounded once, to the common unit 2^-56 2^(E-1022) of
+//    the site's accumulators, E the largest exponent among its neighbours met so far (+1); eight
+//    hops stay below 2^61.4.
+// The error of a hop sum is about 2^-56 of the largest neighbouring component (the rounding of eight
+// hops and the dropped products), against about 2^-52 for the FP64 chains it replaces.
+//
+// Integer sums do not depend on their order, so every shape of the stencil gives the same hop sums
+// up to that rounding. Sites next to an infinity, a NaN or only components below 2^-959 (E < 64), and
+// fields whose links do not share a scale (FxField::ok = 0: a non-finite field, a link whose largest
+// component is below a quarter of the field's scale, or a scale far from 1) take the FP64 hops.
+#pragma once
+
+#include "wilson.cuh"
+
+namespace ovl {
+
+typedef long long fx64;
+
+struct alignas(16) FxC {  // a complex link entry: limbs of its real and imaginary part
+  int rh, rl, ih, il;
+};
+
+// Hop coefficients of the fixed-point stencil: the time hops' factors e^{+-mu} as 59-bit fractions of 2^e.
+struct FxCoef {
+  HopCoef<double> k;
+  int fh, fl, fe;  // forward: (fh 2^30 + fl) 2^-59 2^fe
+  int bh, bl, be;  // backward
+  int unit;        // 1: both factors are 1 (mu = 0)
+  int ok;          // 0: a factor is outside the fixed-point range (FP64 path)
+};
+
+inline FxCoef fx_coef(double m_w, double mu) {
+  FxCoef c;
+  c.k = hop_coef<double>(m_w, mu);
+  c.unit = mu == 0.0;
+  c.ok = std::fabs(mu) <= 16.0;
+  auto split = [&](double f, int& h, int& l, int& e) {
+    const double m = std::frexp(c.ok ? f : 1.0, &e);
+    const fx64 q = std::llrint(std::ldexp(m, 59));
+    h = (int)(q >> 30);
+    l = (int)(q & ((1 << 30) - 1));
+  };
+  split(std::exp(mu), c.fh, c.fl, c.fe);
+  split(std::exp(-mu), c.bh, c.bl, c.be);
+  if (c.unit) c.fe = c.be = 0;  // not applied
+  return c;
+}
+
+// Shifts with the amount clamped to the word (PTX semantics).
+OVL_HD unsigned long long fx_shr(unsigned long long v, int n) {
+#if defined(__CUDA_ARCH__)
+  unsigned long long r;
+  asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(n));
+  return r;
+#else
+  return n > 63 ? 0ull : v >> n;
+#endif
+}
+OVL_HD fx64 fx_sar(fx64 v, int n) {
+#if defined(__CUDA_ARCH__)
+  fx64 r;
+  asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(n));
+  return r;
+#else
+  return v >> (n > 63 ? 63 : n);
+#endif
+}
+OVL_HD void fx_words(double x, int& hi, unsigned& lo) {
+#if defined(__CUDA_ARCH__)
+  hi = __double2hiint(x);
+  lo = (unsigned)__double2loint(x);
+#else
+  unsigned long long b;
+  std::memcpy(&b, &x, 8);
+  hi = (int)(b >> 32);
+  lo = (unsigned)b;
+#endif
+}
+OVL_HD double fx_pow2(int biased) {  // 2^(biased - 1023), 0 < biased < 2047
+#if defined(__CUDA_ARCH__)
+  return __hiloint2double(biased << 20, 0);
+#else
+  return std::ldexp(1.0, biased - 1023);
+#endif
+}
+
+// Limbs of x in units of 2^-59 2^(e-1022), e >= 64 at least x's biased exponent (smaller values are
+// shifted out; zeros and subnormals, biased exponent 0, give 0).
+OVL_HD void fx_limbs(int hi, unsigned lo, int e, int& h, int& l) {
+  const unsigned mh = ((unsigned)hi & 0xfffffu) | 0x100000u;
+  const int d = e - (int)(((unsigned)hi >> 20) & 0x7ffu);
+  const unsigned long long m = ((unsigned long long)mh << 32 | lo) << 6;
+  const unsigned long long q = fx_shr(m, d);
+  const fx64 s = (fx64)(hi >> 31);
+  const fx64 v = ((fx64)q ^ s) - s;
+  h = (int)(v >> 30);
+  l = (int)((unsigned)v & 0x3fffffffu);
+}
+
+struct FxHalf {  // projected half spinor: limbs of [2 spins][3 colours] complex
+  int rh[2][3], rl[2][3], ih[2][3], il[2][3];
+};
+
+struct FxAcc {  // accumulators of a site: sums of hops in units of 2^-56 2^(E-1022)
+  fx64 re[4][3], im[4][3];
+  int E;     // common biased exponent (+1)
+  int emax;  // largest biased exponent of a neighbour
+};
+
+OVL_HD void fx_clear(FxAcc& a) {
+#pragma unroll
+  for (int i = 0; i < 12; ++i) a.re[i / 3][i % 3] = a.im[i / 3][i % 3] = 0;
+  a.E = 0;
+  a.emax = 0;
+}
+
+struct FxSpin {  // limbs of a site's 12 complex components relative to one exponent
+  int rh[4][3], rl[4][3], ih[4][3], il[4][3];
+};
+
+// Biased exponent of the site's largest component.
+OVL_HD int fx_exponent(const Spin<double>& p) {
+  int m = 0;
+#pragma unroll
+  for (int i = 0; i < 12; ++i) {
+    int w;
+    unsigned z;
+    fx_words(p.c[i / 3][i % 3].re, w, z);
+    m = m > (w & 0x7fffffff) ? m : (w & 0x7fffffff);
+    fx_words(p.c[i / 3][i % 3].im, w, z);
+    m = m > (w & 0x7fffffff) ? m : (w & 0x7fffffff);
+  }
+  return m >> 20;
+}
+
+OVL_HD void fx_spin(const Spin<double>& p, int e, FxSpin& o) {
+#pragma unroll
+  for (int i = 0; i < 12; ++i) {
+    int w;
+    unsigned z;
+    fx_words(p.c[i / 3][i % 3].re, w, z);
+    fx_limbs(w, z, e, o.rh[i / 3][i % 3], o.rl[i / 3][i % 3]);
+    fx_words(p.c[i / 3][i % 3].im, w, z);
+    fx_limbs(w, z, e, o.ih[i / 3][i % 3], o.il[i / 3][i % 3]);
+  }
+}
+
+// h_s = p_s + rot p_q with rot = 1 (ROT 0), i (1), -1 (2), -i (3); CONJ: its complex conjugate.
+template <int ROT, bool CONJ>
+OVL_HD void fx_row(const FxSpin& p, int s, int q, FxHalf& h) {
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    int rh, rl, ih, il;  // rot p_q
+    if (ROT == 0) rh = p.rh[q][a], rl = p.rl[q][a], ih = p.ih[q][a], il = p.il[q][a];
+    if (ROT == 1) rh = -p.ih[q][a], rl = -p.il[q][a], ih = p.rh[q][a], il = p.rl[q][a];
+    if (ROT == 2) rh = -p.rh[q][a], rl = -p.rl[q][a], ih = -p.ih[q][a], il = -p.il[q][a];
+    if (ROT == 3) rh = p.ih[q][a], rl = p.il[q][a], ih = -p.rh[q][a], il = -p.rl[q][a];
+    h.rh[s][a] = p.rh[s][a] + rh;
+    h.rl[s][a] = p.rl[s][a] + rl;
+    h.ih[s][a] = CONJ ? -(p.ih[s][a] + ih) : p.ih[s][a] + ih;
+    h.il[s][a] = CONJ ? -(p.il[s][a] + il) : p.il[s][a] + il;
+  }
+}
+
+// Half spinor of (1 - g_mu) p (MINUS) or (1 + g_mu) p (see project()).
+template <int MU, bool MINUS, bool CONJ>
+OVL_HD void fx_project(const FxSpin& p, FxHalf& h) {
+  constexpr int r0 = MU == 0 ? (MINUS ? 1 : 3) : MU == 1 ? (MINUS ? 0 : 2) : MU == 2 ? (MINUS ? 1 : 3) : (MINUS ? 2 : 0);
+  constexpr int r1 = MU == 0 ? (MINUS ? 1 : 3) : MU == 1 ? (MINUS ? 2 : 0) : MU == 2 ? (MINUS ? 3 : 1) : (MINUS ? 2 : 0);
+  fx_row<r0, CONJ>(p, 0, MU < 2 ? 3 : 2, h);
+  fx_row<r1, CONJ>(p, 1, MU < 2 ? 2 : 3, h);
+}
+
+// a + rot (re, im), rot = 1 (ROT 0), i (1), -1 (2), -i (3)
+template <int ROT>
+OVL_HD void fx_add_rot(fx64& re, fx64& im, fx64 tr, fx64 ti) {
+  re += ROT == 0 ? tr : ROT == 1 ? -ti : ROT == 2 ? -tr : ti;
+  im += ROT == 0 ? ti : ROT == 1 ? tr : ROT == 2 ? -ti : -tr;
+}
+
+// acc += (t, -/+ N t) for the half spinor t of a hop (see reconstruct_add).
+template <int MU, bool FWD>
+OVL_HD void fx_reconstruct(FxAcc& acc, const fx64 (&tr)[2][3], const fx64 (&ti)[2][3]) {
+  constexpr int i2 = MU < 2 ? 1 : 0, i3 = MU < 2 ? 0 : 1;
+  constexpr int r2 = MU == 0 ? (FWD ? 3 : 1) : MU == 1 ? (FWD ? 2 : 0) : MU == 2 ? (FWD ? 3 : 1) : (FWD ? 2 : 0);
+  constexpr int r3 = MU == 0 ? (FWD ? 3 : 1) : MU == 1 ? (FWD ? 0 : 2) : MU == 2 ? (FWD ? 1 : 3) : (FWD ? 2 : 0);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {  // the backward hop's t is conjugated
+    fx_add_rot<0>(acc.re[0][a], acc.im[0][a], tr[0][a], FWD ? ti[0][a] : -ti[0][a]);
+    fx_add_rot<0>(acc.re[1][a], acc.im[1][a], tr[1][a], FWD ? ti[1][a] : -ti[1][a]);
+    fx_add_rot<r2>(acc.re[2][a], acc.im[2][a], tr[i2][a], FWD ? ti[i2][a] : -ti[i2][a]);
+    fx_add_rot<r3>(acc.re[3][a], acc.im[3][a], tr[i3][a], FWD ? ti[i3][a] : -ti[i3][a]);
+  }
+}
+
+// T (|T| < 2^60.4 in units of 2^-58) times the fraction (h 2^30 + l) 2^-59, in units of 2^-56.
+OVL_HD fx64 fx_scale(fx64 t, int h, int l) {
+  const fx64 t2 = (t + 2) >> 2;
+  const int th = (int)(t2 >> 30), tl = (int)((unsigned)t2 & 0x3fffffffu);
+  const fx64 x = (fx64)th * l + (fx64)tl * h;
+  return 2 * ((fx64)th * h) + (x >> 29);
+}
+
+// Adds hop k = 2 mu (forward, U) or 2 mu + 1 (backward, U^H) of the neighbour spinor p to the
+// accumulators; U points at the link's entry [0][0], its entries `stride` apart. g5in: the input is
+// gamma5 p (the lower spins change sign, which exchanges the two projectors). flip: the hop crosses an
+// antiperiodic boundary. The direction is a run-time value (uniform over a warp) so that the hops share
+// one copy of the conversion and the product: unrolled over the eight hops the kernel was 100 KB of
+// code and took minutes to compile.
+OVL_HD void fx_hop(int k, const Spin<double>& p, const FxC* U, size_t stride, const FxCoef& c, bool g5in, bool flip,
+                   FxAcc& acc) {
+  const bool fwd = !(k & 1), time = k >= 6;
+  const int eb = fx_exponent(p);
+  acc.emax = acc.emax > eb ? acc.emax : eb;
+  const int e = eb > 64 ? eb : 64;
+  FxHalf h;
+  {
+    FxSpin q;
+    fx_spin(p, e, q);
+    // the backward hop multiplies by U^H = conj(U^T): conj(U^T conj(h)) conjugated at the end
+    switch (g5in ? k + 8 : k) {
+      case 0: fx_project<0, true, false>(q, h); break;
+      case 1: fx_project<0, false, true>(q, h); break;
+      case 2: fx_project<1, true, false>(q, h); break;
+      case 3: fx_project<1, false, true>(q, h); break;
+      case 4: fx_project<2, true, false>(q, h); break;
+      case 5: fx_project<2, false, true>(q, h); break;
+      case 6: fx_project<3, true, false>(q, h); break;
+      case 7: fx_project<3, false, true>(q, h); break;
+      case 8: fx_project<0, false, false>(q, h); break;
+      case 9: fx_project<0, true, true>(q, h); break;
+      case 10: fx_project<1, false, false>(q, h); break;
+      case 11: fx_project<1, true, true>(q, h); break;
+      case 12: fx_project<2, false, false>(q, h); break;
+      case 13: fx_project<2, true, true>(q, h); break;
+      case 14: fx_project<3, false, false>(q, h); break;
+      default: fx_project<3, true, true>(q, h); break;
+    }
+  }
+  const int eh = e + (time ? (fwd ? c.fe : c.be) : 0);  // exponent of this hop's contribution
+  if (eh > acc.E) {  // first hop, or a larger neighbour than any before
+    const int E = eh + 1;
+    if (acc.E != 0) {
+#pragma unroll
+      for (int i = 0; i < 12; ++i) {
+        acc.re[i / 3][i % 3] = fx_sar(acc.re[i / 3][i % 3], E - acc.E);
+        acc.im[i / 3][i % 3] = fx_sar(acc.im[i / 3][i % 3], E - acc.E);
+      }
+    }
+    acc.E = E;
+  }
+  const int d = acc.E - eh;
+  const bool scaled = time && !c.unit;
+  const int sh = scaled ? (d < 60 ? d : 60) : (d < 58 ? d + 2 : 60);
+  const fx64 half = sh > 0 ? (fx64)1 << (sh - 1) : 0;  // rounds the shift
+  const fx64 seed = scaled ? 0 : half;
+  const size_t sa = fwd ? 3 * stride : stride, sb = fwd ? stride : 3 * stride;  // U[a][b] or U[b][a]
+  fx64 tr[2][3], ti[2][3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    fx64 hr0 = seed, hi0 = seed, hr1 = seed, hi1 = seed, xr0 = 0, xi0 = 0, xr1 = 0, xi1 = 0;
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      const FxC u = U[a * sa + b * sb];
+      const int nh = -u.ih, nl = -u.il;
+      hr0 += (fx64)u.rh * h.rh[0][b];
+      hr0 += (fx64)nh * h.ih[0][b];
+      hi0 += (fx64)u.rh * h.ih[0][b];
+      hi0 += (fx64)u.ih * h.rh[0][b];
+      xr0 += (fx64)u.rh * h.rl[0][b];
+      xr0 += (fx64)u.rl * h.rh[0][b];
+      xr0 += (fx64)nh * h.il[0][b];
+      xr0 += (fx64)nl * h.ih[0][b];
+      xi0 += (fx64)u.rh * h.il[0][b];
+      xi0 += (fx64)u.rl * h.ih[0][b];
+      xi0 += (fx64)u.ih * h.rl[0][b];
+      xi0 += (fx64)u.il * h.rh[0][b];
+      hr1 += (fx64)u.rh * h.rh[1][b];
+      hr1 += (fx64)nh * h.ih[1][b];
+      hi1 += (fx64)u.rh * h.ih[1][b];
+      hi1 += (fx64)u.ih * h.rh[1][b];
+      xr1 += (fx64)u.rh * h.rl[1][b];
+      xr1 += (fx64)u.rl * h.rh[1][b];
+      xr1 += (fx64)nh * h.il[1][b];
+      xr1 += (fx64)nl * h.ih[1][b];
+      xi1 += (fx64)u.rh * h.il[1][b];
+      xi1 += (fx64)u.rl * h.ih[1][b];
+      xi1 += (fx64)u.ih * h.rl[1][b];
+      xi1 += (fx64)u.il * h.rh[1][b];
+    }
+    tr[0][a] = hr0 + (xr0 >> 30);
+    ti[0][a] = hi0 + (xi0 >> 30);
+    tr[1][a] = hr1 + (xr1 >> 30);
+    ti[1][a] = hi1 + (xi1 >> 30);
+  }
+  if (scaled) {
+    const int fh = fwd ? c.fh : c.bh, fl = fwd ? c.fl : c.bl;
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+      tr[i / 3][i % 3] = fx_scale(tr[i / 3][i % 3], fh, fl) + half;
+      ti[i / 3][i % 3] = fx_scale(ti[i / 3][i % 3], fh, fl) + half;
+    }
+  }
+  const fx64 fm = flip ? -1 : 0;
+#pragma unroll
+  for (int i = 0; i < 6; ++i) {
+    tr[i / 3][i % 3] = (fx_sar(tr[i / 3][i % 3], sh) ^ fm) - fm;
+    ti[i / 3][i % 3] = (fx_sar(ti[i / 3][i % 3], sh) ^ fm) - fm;
+  }
+  switch (k) {
+    case 0: fx_reconstruct<0, true>(acc, tr, ti); break;
+    case 1: fx_reconstruct<0, false>(acc, tr, ti); break;
+    case 2: fx_reconstruct<1, true>(acc, tr, ti); break;
+    case 3: fx_reconstruct<1, false>(acc, tr, ti); break;
+    case 4: fx_reconstruct<2, true>(acc, tr, ti); break;
+    case 5: fx_reconstruct<2, false>(acc, tr, ti); break;
+    case 6: fx_reconstruct<3, true>(acc, tr, ti); break;
+    default: fx_reconstruct<3, false>(acc, tr, ti); break;
+  }
+}
+
+// Field-wide scale of the fixed-point links, kept in device memory beside them (a later ovl_set_links
+// rewrites both in place, so captured graphs stay valid).
+struct FxField {
+  int ok;    // the links share a scale (see above)
+  int uexp;  // the scale is 2^uexp
+  unsigned long long lo, hi;  // bits of the smallest of the links' largest components and of the largest
+                              // of the links' scales (fx_link_range), over the field
+};
+
+// Largest component of a link, and the scale it needs: the largest of that and its row and column sums of
+// |re| + |im| over sqrt(6) (rounded up: 1 for SU(3) to rounding).
+OVL_HD void fx_link_range(const Mat3<double>& u, double& top, double& need) {
+  double row[3] = {0, 0, 0}, col[3] = {0, 0, 0};
+  top = need = 0;
+  bool nan = false;
+#pragma unroll
+  for (int i = 0; i < 9; ++i) {
+    const double a = std::fabs(u.m[i / 3][i % 3].re), b = std::fabs(u.m[i / 3][i % 3].im);
+    nan = nan || a != a || b != b;
+    top = a > top ? a : top;
+    top = b > top ? b : top;
+    row[i / 3] += a + b;
+    col[i % 3] += a + b;
+  }
+  need = top;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    need = row[i] / 2.4495 > need ? row[i] / 2.4495 : need;
+    need = col[i] / 2.4495 > need ? col[i] / 2.4495 : need;
+  }
+  if (nan) need = 1e308 * 10;  // infinity: the field is not usable
+}
+
+// Scale exponent of a field with these ranges; false: the FP64 hops.
+OVL_HD bool fx_field_scale(double lo, double hi, int* uexp) {
+  *uexp = 0;
+  if (!(hi > 0.0) || !(hi < 1e100) || !(lo >= 0.25 * hi)) return false;
+  std::frexp(hi * (1.0 - 1e-6), uexp);  // a scale of 1 (+ rounding) is 2^0
+  return *uexp >= -8 && *uexp <= 8;
+}
+
+OVL_HD FxC fx_link_entry(cplx<double> u, int uexp) {
+  const fx64 qr = std::llrint(std::ldexp(u.re, 59 - uexp)), qi = std::llrint(std::ldexp(u.im, 59 - uexp));
+  FxC r;
+  r.rh = (int)((qr + (1 << 29)) >> 30);
+  r.rl = (int)(qr - ((fx64)r.rh << 30));
+  r.ih = (int)((qi + (1 << 29)) >> 30);
+  r.il = (int)(qi - ((fx64)r.ih << 30));
+  return r;
+}
+
+// Neighbour of site s for hop k, and whether the hop crosses the time boundary.
+OVL_HD int fx_neighbour(const Geom& g, int s, int k, bool* wraps) {
+  const int mu = k >> 1;
+  const int st = mu == 0 ? 1 : mu == 1 ? g.sy : mu == 2 ? g.sz : g.st;
+  const int len = mu == 0 ? g.lx : mu == 1 ? g.ly : mu == 2 ? g.lz : g.lt;
+  const int x = (s / st) % len;
+  const bool edge = x == ((k & 1) ? 0 : len - 1);
+  *wraps = mu == 3 && edge;
+  const int step = edge ? (1 - len) * st : st;
+  return (k & 1) ? s - step : s + step;
+}
+
+// Hops k0 .. k1-1 of site s, psi loaded through `ld`.
+template <class Load>
+OVL_HD void fx_hops(const Geom& g, const FxC* U, int s, int k0, int k1, const FxCoef& c, Load ld, bool g5in, FxAcc& acc) {
+#pragma unroll 1
+  for (int k = k0; k < k1; ++k) {
+    bool wraps;
+    const int nb = fx_neighbour(g, s, k, &wraps);
+    Spin<double> p;
+    ld(nb, p);
+    fx_hop(k, p, U + (size_t)(k >> 1) * 9 * g.vol + ((k & 1) ? nb : s), (size_t)g.vol, c, g5in, wraps && g.t_bc < 0, acc);
+  }
+}
+
+// Whether the accumulators hold the hop sum: no infinity or NaN among the neighbours, and not only
+// components too small for the common exponent (all zero is fine: the sum is 0).
+OVL_HD bool fx_usable(const FxAcc& a) { return a.emax < 0x7ff && a.E < 2000 && (a.emax == 0 || a.emax >= 64); }
+
+// FP64 value of one unit of the accumulators times the hop coefficient ks and the links' scale.
+OVL_HD double fx_unit(const FxAcc& a, const FxCoef& c, int uexp) { return c.k.ks * fx_pow2(a.E - 55 + uexp); }
+
+}  // namespace ovl

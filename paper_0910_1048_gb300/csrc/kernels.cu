@@ -183,31 +183,88 @@ __global__ void k_ingest_links(int vol, const double2* ucan, double2* u64, float
   }
 }
 
-cudaError_t launch_ingest_links(const Geom& g, const double* ucan, double2* u64, float2* u32, uint32_t* u16, cudaStream_t st) {
+// Ranges of the links for their fixed-point copy: bits of non-negative doubles order like the values.
+__global__ void __launch_bounds__(256) k_fx_range(int vol, const double2* ucan, FxField* f) {
+  const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;  // over 4 V links
+  unsigned long long lo = ~0ull, hi = 0ull;
+  if (e < (size_t)4 * vol) {
+    Mat3<double> u;
+    for (int k = 0; k < 9; ++k) u.m[k / 3][k % 3] = ldc<double>(ucan, e * 9 + k);
+    double top, need;
+    fx_link_range(u, top, need);
+    lo = (unsigned long long)__double_as_longlong(top);
+    hi = (unsigned long long)__double_as_longlong(need);
+  }
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    const unsigned long long l2 = __shfl_xor_sync(0xffffffffu, lo, off), h2 = __shfl_xor_sync(0xffffffffu, hi, off);
+    lo = l2 < lo ? l2 : lo;
+    hi = h2 > hi ? h2 : hi;
+  }
+  if ((threadIdx.x & 31) == 0) {
+    atomicMin(&f->lo, lo);
+    atomicMax(&f->hi, hi);
+  }
+}
+
+__global__ void __launch_bounds__(256) k_fx_links(int vol, const double2* u64, FxField* f, FxC* ufx) {
+  const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;  // over 4*9*V
+  int uexp;
+  const bool ok = fx_field_scale(__longlong_as_double((long long)f->lo), __longlong_as_double((long long)f->hi), &uexp);
+  if (e == 0) {
+    f->ok = ok ? 1 : 0;
+    f->uexp = uexp;
+  }
+  if (ok && e < (size_t)36 * vol) ufx[e] = fx_link_entry(ldc<double>(u64, e), uexp);
+}
+
+size_t fx_field_bytes() { return sizeof(FxField); }
+
+cudaError_t launch_ingest_links(const Geom& g, const double* ucan, double2* u64, FxC* ufx, FxField* fxf, float2* u32,
+                                uint32_t* u16, cudaStream_t st) {
   size_t n = (size_t)36 * g.vol;
   k_ingest_links<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(g.vol, (const double2*)ucan, u64, u32, u16);
+  cudaError_t e;
+  if ((e = cudaMemsetAsync(fxf, 0, sizeof(FxField), st))) return e;
+  if ((e = cudaMemsetAsync(&fxf->lo, 0xff, sizeof(fxf->lo), st))) return e;
+  k_fx_range<<<(unsigned)(((size_t)4 * g.vol + 255) / 256), 256, 0, st>>>(g.vol, (const double2*)ucan, fxf);
+  k_fx_links<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(g.vol, u64, fxf, ufx);
   return cudaGetLastError();
 }
 
 // ------------------------------------------------------------------ apply D_W
-// G5IN (gamma5 on the input, the adjoint's form) is a template parameter so that the common
+// FP32: G5IN (gamma5 on the input, the adjoint's form) is a template parameter so that the common
 // case carries no per-neighbour branch: 32^4 FP32 4.7 -> 5.2 TB/s in a probe without it.
-template <class R, int LF, bool NIN, bool NOUT, bool G5IN>
-__global__ void __launch_bounds__(kBlock, sizeof(R) == 4 ? (LF == LINK_F16R12 ? 6 : 7) : 1)
-    k_dslash(Geom g, Links U, HopCoef<R> c, bool g5_out, const typename V2<R>::T* in, typename V2<R>::T* out) {
+template <int LF, bool NATIVE, bool G5IN>
+__global__ void __launch_bounds__(kBlock, LF == LINK_F16R12 ? 6 : 7)
+    k_dslash(Geom g, Links U, HopCoef<float> c, bool g5_out, const float2* in, float2* out) {
   int s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= g.vol) return;
   size_t off = (size_t)blockIdx.y * 12 * g.vol;
-  Loader<R, NIN> ld{in + off, g.vol, G5IN};
-  Spin<R> o;
-  dslash_site<LF, R>(g, U, s, c, ld, o);
-  const R sg = g5_out ? (R)-1 : (R)1;  // gamma5 = diag(1, 1, -1, -1) on the output, without a branch
+  Loader<float, NATIVE> ld{in + off, g.vol, G5IN};
+  Spin<float> o;
+  dslash_site<LF, float>(g, U, s, c, ld, o);
+  const float sg = g5_out ? -1.f : 1.f;  // gamma5 = diag(1, 1, -1, -1) on the output, without a branch
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     o.c[2][a] = sg * o.c[2][a];
     o.c[3][a] = sg * o.c[3][a];
   }
-  store_spin<R, NOUT>(out + off, g.vol, s, o);
+  store_spin<float, NATIVE>(out + off, g.vol, s, o);
+}
+
+// FP64 (fixed-point hops, see fixedpt.cuh): the layout and gamma5 are run-time values.
+__global__ void __launch_bounds__(kBlock, 3)
+    k_dslash_f64(Geom g, Links U, FxCoef c, bool native, bool g5_in, bool g5_out, const double2* in, double2* out) {
+  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+  if (s >= g.vol) return;
+  const size_t off = (size_t)blockIdx.y * 12 * g.vol;
+  const int ss = native ? 1 : 12, cs = native ? g.vol : 1;
+  Spin<double> o;
+  add_hops(g, U, s, 0, 8, c, StrideLoader{in + off, ss, cs}, g5_in, true, o);
+  if (g5_out) gamma5_inplace(o);
+#pragma unroll
+  for (int q = 0; q < 12; ++q) stc<double>(out + off, (size_t)s * ss + (size_t)q * cs, o.c[q / 3][q % 3]);
 }
 
 // The FP32 operator on a batch of sources, native layout in and out. A thread applies the links of
@@ -245,30 +302,22 @@ __global__ void __launch_bounds__(kBlock, G == 1 ? 7 : (G == 2 ? 4 : 2))
   }
 }
 
-template <class R, int LF, bool G5IN>
-static cudaError_t dslash_g(dim3 grid, const Geom& g, const Links& U, HopCoef<R> c, bool go, bool nin, bool nout,
-                            const typename V2<R>::T* i, typename V2<R>::T* o, cudaStream_t st) {
-  if (nin && nout)
-    k_dslash<R, LF, true, true, G5IN><<<grid, kBlock, 0, st>>>(g, U, c, go, i, o);
-  else if (nin)
-    k_dslash<R, LF, true, false, G5IN><<<grid, kBlock, 0, st>>>(g, U, c, go, i, o);
-  else if (nout)
-    k_dslash<R, LF, false, true, G5IN><<<grid, kBlock, 0, st>>>(g, U, c, go, i, o);
-  else
-    k_dslash<R, LF, false, false, G5IN><<<grid, kBlock, 0, st>>>(g, U, c, go, i, o);
-  return cudaGetLastError();
-}
-
-template <class R, int LF>
-static cudaError_t dslash_t(const Geom& g, const Links& U, double m_w, double mu, bool gi, bool go, bool nin, bool nout,
+template <int LF>
+static cudaError_t dslash_t(const Geom& g, const Links& U, double m_w, double mu, bool gi, bool go, bool native,
                             int nrhs, const void* in, void* out, cudaStream_t st) {
-  HopCoef<R> c = hop_coef<R>(m_w, mu);
-  dim3 grid((g.vol + kBlock - 1) / kBlock, nrhs);
-  using T = typename V2<R>::T;
-  const T* i = (const T*)in;
-  T* o = (T*)out;
-  return gi ? dslash_g<R, LF, true>(grid, g, U, c, go, nin, nout, i, o, st)
-            : dslash_g<R, LF, false>(grid, g, U, c, go, nin, nout, i, o, st);
+  const HopCoef<float> c = hop_coef<float>(m_w, mu);
+  const dim3 grid((g.vol + kBlock - 1) / kBlock, nrhs);
+  const float2* i = (const float2*)in;
+  float2* o = (float2*)out;
+  if (native && gi)
+    k_dslash<LF, true, true><<<grid, kBlock, 0, st>>>(g, U, c, go, i, o);
+  else if (native)
+    k_dslash<LF, true, false><<<grid, kBlock, 0, st>>>(g, U, c, go, i, o);
+  else if (gi)
+    k_dslash<LF, false, true><<<grid, kBlock, 0, st>>>(g, U, c, go, i, o);
+  else
+    k_dslash<LF, false, false><<<grid, kBlock, 0, st>>>(g, U, c, go, i, o);
+  return cudaGetLastError();
 }
 
 template <int LF, int G>
@@ -326,16 +375,19 @@ static cudaError_t dslash_group_t(const Geom& g, const Links& U, double m_w, dou
 }
 
 cudaError_t launch_dslash(const Geom& g, const Links& U, int lf, bool f64, double m_w, double mu, bool g5_in,
-                          bool g5_out, bool native_in, bool native_out, int nrhs, const void* in, void* out,
-                          cudaStream_t st) {
-  if (f64) return dslash_t<double, LINK_F64>(g, U, m_w, mu, g5_in, g5_out, native_in, native_out, nrhs, in, out, st);
-  if (nrhs > 1 && native_in && native_out) {  // a batch: links once per group of sources
+                          bool g5_out, bool native, int nrhs, const void* in, void* out, cudaStream_t st) {
+  if (f64) {
+    const dim3 grid((g.vol + kBlock - 1) / kBlock, nrhs);
+    k_dslash_f64<<<grid, kBlock, 0, st>>>(g, U, fx_coef(m_w, mu), native, g5_in, g5_out, (const double2*)in,
+                                          (double2*)out);
+    return cudaGetLastError();
+  }
+  if (nrhs > 1 && native) {  // a batch: links once per group of sources
     if (lf == LINK_F16R12) return dslash_group_t<LINK_F16R12>(g, U, m_w, mu, g5_in, g5_out, nrhs, in, out, st);
     return dslash_group_t<LINK_F32>(g, U, m_w, mu, g5_in, g5_out, nrhs, in, out, st);
   }
-  if (lf == LINK_F16R12)
-    return dslash_t<float, LINK_F16R12>(g, U, m_w, mu, g5_in, g5_out, native_in, native_out, nrhs, in, out, st);
-  return dslash_t<float, LINK_F32>(g, U, m_w, mu, g5_in, g5_out, native_in, native_out, nrhs, in, out, st);
+  if (lf == LINK_F16R12) return dslash_t<LINK_F16R12>(g, U, m_w, mu, g5_in, g5_out, native, nrhs, in, out, st);
+  return dslash_t<LINK_F32>(g, U, m_w, mu, g5_in, g5_out, native, nrhs, in, out, st);
 }
 
 // ------------------------------------------------------------------ Lanczos: start
@@ -610,8 +662,9 @@ __device__ __forceinline__ void st_release(int* p, int v) {
 // ONE_ROLE: one warp-uniform half per block instead (block (PS, 1), even blocks H(mu) vhat, odd
 // blocks H(-mu) what), twice the blocks at half the size: 12^4 with 32 sites is 1296 one-warp
 // blocks, at most 9 on an SM against a mean of 8.53 (with both halves per block: 5 against 4.26).
-template <class R, int LF, int PS, bool ONE_ROLE = false>
-__global__ void __launch_bounds__(ONE_ROLE ? PS : 2 * PS) k_lz_pair(Geom g, Links U, HopCoef<R> cp, HopCoef<R> cm, LzDev lz,
+template <class R, int LF, bool ONE_ROLE = false>
+__global__ void __launch_bounds__(ONE_ROLE ? 32 : 2 * kPairSites) k_lz_pair(Geom g, Links U, typename HopsOf<R>::T cp,
+                                                            typename HopsOf<R>::T cm, LzDev lz,
                                                             const typename V2<R>::T* vh, const typename V2<R>::T* wh,
                                                             typename V2<R>::T* av, typename V2<R>::T* aw) {
   using T = typename V2<R>::T;
@@ -623,7 +676,7 @@ __global__ void __launch_bounds__(ONE_ROLE ? PS : 2 * PS) k_lz_pair(Geom g, Link
   const double2 swd = lz.sw[o + j];
   const T* vj = vh + vcol(lz, rhs, j, n);
   const T* wj = wh + ((size_t)(j & 1) * lz.nrhs + rhs) * n;
-  const int s = (ONE_ROLE ? (int)(blockIdx.x >> 1) : (int)blockIdx.x) * PS + threadIdx.x;
+  const int s = (ONE_ROLE ? (int)(blockIdx.x >> 1) : (int)blockIdx.x) * blockDim.x + threadIdx.x;
   const bool is_w = ONE_ROLE ? (blockIdx.x & 1) != 0 : threadIdx.y == 1;
   const double sd[3] = {lz.sv[o + j], swd.x, swd.y};
   R sc[3];
@@ -632,7 +685,7 @@ __global__ void __launch_bounds__(ONE_ROLE ? PS : 2 * PS) k_lz_pair(Geom g, Link
   if (s < g.vol) {
     Spin<R> ov;
     if (!is_w) {
-      dslash_site<LF, R>(g, U, s, cp, Loader<R, true>{vj, g.vol, false}, ov);
+      stencil_site<LF, R>(g, U, s, cp, vj, ov);
       const R sv = sc[0];
       // all loads of w_j before the stores of Av (the compiler cannot reorder them across stores
       // that might alias, which would serialise twelve memory round trips)
@@ -650,7 +703,7 @@ __global__ void __launch_bounds__(ONE_ROLE ? PS : 2 * PS) k_lz_pair(Geom g, Link
       acc[0].add(a.re);
       acc[1].add(a.im);
     } else {
-      dslash_site<LF, R>(g, U, s, cm, Loader<R, true>{wj, g.vol, false}, ov);
+      stencil_site<LF, R>(g, U, s, cm, wj, ov);
       const cplx<R> sw = mk<R>(sc[1], sc[2]);
 #pragma unroll
       for (int c = 0; c < 12; ++c) {
@@ -674,7 +727,8 @@ __global__ void __launch_bounds__(ONE_ROLE ? PS : 2 * PS) k_lz_pair(Geom g, Link
 // one spin (three colours) of its site: scale, gamma5, store, and for the v half the partial of
 // alpha_j. SITES sites per block, at least MINB blocks per SM.
 template <class R, int LF, int MINB = 1, int SITES = kSplitSites>
-__global__ void __launch_bounds__(8 * SITES, MINB) k_lz_pair_split(Geom g, Links U, HopCoef<R> cp, HopCoef<R> cm,
+__global__ void __launch_bounds__(8 * SITES, MINB) k_lz_pair_split(Geom g, Links U, typename HopsOf<R>::T cp,
+                                                                   typename HopsOf<R>::T cm,
                                                                    LzDev lz, const typename V2<R>::T* vh,
                                                                    const typename V2<R>::T* wh,
                                                                    typename V2<R>::T* av, typename V2<R>::T* aw) {
@@ -734,7 +788,8 @@ __global__ void __launch_bounds__(8 * SITES, MINB) k_lz_pair_split(Geom g, Links
 constexpr int kDynMaxWarps = 12;  // warps per block at most
 
 template <class R, int LF>
-__global__ void __launch_bounds__(32 * kDynMaxWarps, 1) k_lz_pair_dyn(Geom g, Links U, HopCoef<R> cp, HopCoef<R> cm,
+__global__ void __launch_bounds__(32 * kDynMaxWarps, 1) k_lz_pair_dyn(Geom g, Links U, typename HopsOf<R>::T cp,
+                                                                 typename HopsOf<R>::T cm,
                                                                  LzDev lz, const typename V2<R>::T* vh,
                                                                  const typename V2<R>::T* wh,
                                                                  typename V2<R>::T* av, typename V2<R>::T* aw) {
@@ -787,7 +842,7 @@ __global__ void __launch_bounds__(32 * kDynMaxWarps, 1) k_lz_pair_dyn(Geom g, Li
     Red<R> acc[2];
     const bool live = s < g.vol;
     Spin<R> ov;
-    if (live) dslash_site<LF, R>(g, U, s, is_w ? cm : cp, Loader<R, true>{is_w ? wj : vj, g.vol, false}, ov);
+    if (live) stencil_site<LF, R>(g, U, s, is_w ? cm : cp, is_w ? wj : vj, ov);
     if (!waited) scales();  // warp-uniform: every lane reaches it, the status load is one value
     if (stop) break;
     if (live) {
@@ -1167,7 +1222,8 @@ static bool fp64_update_balanced() {
 // In the deferred FP64 step the settle kernel (the previous update's finish) runs first and the
 // stencil is launched early behind it (see k_lz_pair_dyn); `first` is recorded between them.
 template <class R, int LF>
-static cudaError_t pair_dyn_launch(const Geom& g, const Links& U, const HopCoef<R>& cp, const HopCoef<R>& cm,
+static cudaError_t pair_dyn_launch(const Geom& g, const Links& U, const typename HopsOf<R>::T& cp,
+                                   const typename HopsOf<R>::T& cm,
                                    const LzDev& lz, const LzVecs& vec, cudaStream_t st, cudaEvent_t first,
                                    cudaEvent_t mid) {
   const int nsm = std::max(1, sm_count());
@@ -1187,24 +1243,24 @@ static cudaError_t pair_dyn_launch(const Geom& g, const Links& U, const HopCoef<
 }
 
 template <int PS, bool ONE_ROLE = false>
-static cudaError_t pair_unsplit(const Geom& g, const Links& U, int lf, bool f64, HopCoef<double> dp, HopCoef<double> dm,
+static cudaError_t pair_unsplit(const Geom& g, const Links& U, int lf, bool f64, FxCoef dp, FxCoef dm,
                                 HopCoef<float> fp, HopCoef<float> fm, const LzDev& lz, const LzVecs& vec,
                                 cudaStream_t st) {
   const unsigned nb = (unsigned)((g.vol + PS - 1) / PS);
   dim3 grid(ONE_ROLE ? 2 * nb : nb, lz.nrhs), block(PS, ONE_ROLE ? 1 : 2);
   if (f64)
-    return launch_plain(k_lz_pair<double, LINK_F64, PS, ONE_ROLE>, grid, block, st, g, U, dp, dm, lz,
+    return launch_plain(k_lz_pair<double, LINK_F64, ONE_ROLE>, grid, block, st, g, U, dp, dm, lz,
                         (const double2*)vec.vh, (const double2*)vec.wh, (double2*)vec.av, (double2*)vec.aw);
   if (lf == LINK_F16R12)
-    return launch_plain(k_lz_pair<float, LINK_F16R12, PS, ONE_ROLE>, grid, block, st, g, U, fp, fm, lz,
+    return launch_plain(k_lz_pair<float, LINK_F16R12, ONE_ROLE>, grid, block, st, g, U, fp, fm, lz,
                         (const float2*)vec.vh, (const float2*)vec.wh, (float2*)vec.av, (float2*)vec.aw);
-  return launch_plain(k_lz_pair<float, LINK_F32, PS, ONE_ROLE>, grid, block, st, g, U, fp, fm, lz,
+  return launch_plain(k_lz_pair<float, LINK_F32, ONE_ROLE>, grid, block, st, g, U, fp, fm, lz,
                       (const float2*)vec.vh, (const float2*)vec.wh, (float2*)vec.av, (float2*)vec.aw);
 }
 
 template <int MINB, int SITES>
-static cudaError_t pair_split_launch(const Geom& g, const Links& U, int lf, bool f64, const HopCoef<double>& dp,
-                                     const HopCoef<double>& dm, const HopCoef<float>& fp, const HopCoef<float>& fm,
+static cudaError_t pair_split_launch(const Geom& g, const Links& U, int lf, bool f64, const FxCoef& dp,
+                                     const FxCoef& dm, const HopCoef<float>& fp, const HopCoef<float>& fm,
                                      const LzDev& lz, const LzVecs& vec, cudaStream_t st) {
   dim3 grid((g.vol + SITES - 1) / SITES, lz.nrhs), block(SITES, 8);
   if (f64)
@@ -1229,10 +1285,8 @@ cudaError_t launch_lanczos_pair(const Geom& g, const Links& U, int lf, bool f64,
                                 const LzDev& lz, const LzVecs& vec, cudaStream_t st, int variant, cudaEvent_t mid,
                                 cudaEvent_t first) {
   if (variant < 0) variant = resolve_pair_variant(g, lf, f64);
-  const HopCoef<double> dp = hop_coef<double>(m_w, mu), dm = hop_coef<double>(m_w, -mu);
+  const FxCoef dp = fx_coef(m_w, mu), dm = fx_coef(m_w, -mu);
   const HopCoef<float> fp = hop_coef<float>(m_w, mu), fm = hop_coef<float>(m_w, -mu);
-  const double2 *dv = (const double2*)vec.vh, *dw = (const double2*)vec.wh;
-  const float2 *fv = (const float2*)vec.vh, *fw = (const float2*)vec.wh;
   cudaError_t e;
   if (variant != 7 && first && (e = record_timing(first, st))) return e;
   if (variant == 1) {

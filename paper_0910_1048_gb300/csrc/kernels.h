@@ -109,13 +109,15 @@ struct LzDev {
 cudaError_t launch_to_native(const Geom& g, int nrhs, bool in_f64, const void* in, bool out_f64, void* out, cudaStream_t st);
 cudaError_t launch_from_native(const Geom& g, int nrhs, bool in_f64, const void* in, bool out_f64, void* out, cudaStream_t st);
 
-// Links: canonical complex128 [4][V][3][3] (device) -> [4][9][V] f64 / f32, [4][6][V] f16 rows 0-1.
-cudaError_t launch_ingest_links(const Geom& g, const double* ucan, double2* u64, float2* u32, uint32_t* u16, cudaStream_t st);
+// Links: canonical complex128 [4][V][3][3] (device) -> [4][9][V] f64 / f32, [4][6][V] f16 rows 0-1, and
+// the fixed-point copy of the FP64 links with its scale (fixedpt.cuh).
+cudaError_t launch_ingest_links(const Geom& g, const double* ucan, double2* u64, FxC* ufx, FxField* fxf, float2* u32,
+                                uint32_t* u16, cudaStream_t st);
+size_t fx_field_bytes();  // sizeof(FxField)
 
 // out = [g5^go] D_W(sign*mu) [g5^gi] in; dtype f64 (FP64 links) or f32 (lf = F32 / F16R12).
 cudaError_t launch_dslash(const Geom& g, const Links& U, int lf, bool f64, double m_w, double mu,
-                          bool g5_in, bool g5_out, bool native_in, bool native_out, int nrhs,
-                          const void* in, void* out, cudaStream_t st);
+                          bool g5_in, bool g5_out, bool native, int nrhs, const void* in, void* out, cudaStream_t st);
 
 // ---- direct two-sided Lanczos (Algorithm 4), per-step kernels
 // vh: [nrhs][kmax+1][12][V], wh: [2][nrhs][12][V], av/aw: [nrhs][12][V]; element type by f64.

@@ -167,7 +167,8 @@ __device__ __forceinline__ void ms_alpha_and_shifts(MsDev& ms, int rhs, const do
 
 // pair1 (MODE 0): t = A p, t~ = A^H p~.  pair2 (MODE 1): q = A t - s1 p, q~ = A^H t~ - s1 p~, p~^H q.
 template <class R, int LF, int MODE>
-__global__ void __launch_bounds__(2 * kPairSites) k_ms_pair(Geom g, Links U, HopCoef<R> cp, HopCoef<R> cm, MsDev ms,
+__global__ void __launch_bounds__(2 * kPairSites) k_ms_pair(Geom g, Links U, typename HopsOf<R>::T cp,
+                                                            typename HopsOf<R>::T cm, MsDev ms,
                                                             MsVecs v) {
   using T = typename V2<R>::T;
   const int rhs = blockIdx.y;
@@ -184,7 +185,7 @@ __global__ void __launch_bounds__(2 * kPairSites) k_ms_pair(Geom g, Links U, Hop
   Red<R> acc[2];
   if (s < g.vol) {
     Spin<R> o;
-    dslash_site<LF, R>(g, U, s, is_t ? cm : cp, Loader<R, true>{in, g.vol, false}, o);
+    stencil_site<LF, R>(g, U, s, is_t ? cm : cp, in, o);
     const R s1 = s1v[0];
     const T* pp = (const T*)(is_t ? v.pt : v.p) + voff<R>(rhs, n);
     const T* ptl = (const T*)v.pt + voff<R>(rhs, n);
@@ -227,7 +228,8 @@ __global__ void __launch_bounds__(2 * kPairSites) k_ms_pair(Geom g, Links U, Hop
 
 // pair1 / pair2 with 8 threads per site (small lattices): see pair_split.
 template <class R, int LF, int MODE>
-__global__ void __launch_bounds__(8 * kSplitSites) k_ms_pair_split(Geom g, Links U, HopCoef<R> cp, HopCoef<R> cm,
+__global__ void __launch_bounds__(8 * kSplitSites) k_ms_pair_split(Geom g, Links U, typename HopsOf<R>::T cp,
+                                                                   typename HopsOf<R>::T cm,
                                                                    MsDev ms, MsVecs v) {
   using T = typename V2<R>::T;
   __shared__ SplitSmem<R> sm;
@@ -497,7 +499,7 @@ static cudaError_t ms_step_t(const Geom& g, const Links& U, double m_w, double m
                              cudaStream_t st, cudaEvent_t* ev) {
   dim3 grid(vec_blocks(g), ms.nrhs);
   dim3 pgrid((g.vol + kPairSites - 1) / kPairSites, ms.nrhs), pblock(kPairSites, 2);
-  HopCoef<R> cp = hop_coef<R>(m_w, mu), cm = hop_coef<R>(m_w, -mu);
+  const typename HopsOf<R>::T cp = hops_of<R>(m_w, mu), cm = hops_of<R>(m_w, -mu);
   dim3 sgrid((g.vol + kSplitSites - 1) / kSplitSites, ms.nrhs), sblock(kSplitSites, 8);
   const bool split = ms_pair_split(g, sizeof(R) == 8 ? 0 : LF);
   const int elt = vec_elts(g, ms.nrhs, sizeof(R) == 8);

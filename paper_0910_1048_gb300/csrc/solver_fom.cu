@@ -174,15 +174,15 @@ ovl_status solve_fom(ovl_lattice* lat, const ovl_sign_params* p, int nrhs, const
   r0 = beta;
   // the batched reduced-precision stencil picks its link-group size on its first call (it
   // synchronises): make that call before the cycle is captured
-  OVL_CHECK_CUDA(launch_dslash(g, U, lf, f64, p->m_W, p->mu, false, true, true, true, nrhs, f.V, tmp, st));
+  OVL_CHECK_CUDA(launch_dslash(g, U, lf, f64, p->m_W, p->mu, false, true, true, nrhs, f.V, tmp, st));
   // ---- one cycle of k Arnoldi steps, captured once and replayed
   auto arnoldi_step = [&](int j, cudaEvent_t* ev) -> cudaError_t {
     cudaError_t e;
     void* vj = (char*)f.V + (size_t)j * nr * n * elt;
     void* vn = (char*)f.V + (size_t)(j + 1) * nr * n * elt;
     if (ev && (e = cudaEventRecord(ev[0], st))) return e;
-    if ((e = launch_dslash(g, U, lf, f64, p->m_W, p->mu, false, true, true, true, nrhs, vj, tmp, st))) return e;
-    if ((e = launch_dslash(g, U, lf, f64, p->m_W, p->mu, false, true, true, true, nrhs, tmp, vn, st))) return e;
+    if ((e = launch_dslash(g, U, lf, f64, p->m_W, p->mu, false, true, true, nrhs, vj, tmp, st))) return e;
+    if ((e = launch_dslash(g, U, lf, f64, p->m_W, p->mu, false, true, true, nrhs, tmp, vn, st))) return e;
     if (ev && (e = cudaEventRecord(ev[1], st))) return e;
     for (int pass = 0; pass < 3; ++pass)
       if ((e = launch_fom_gs(f, f64, j, pass, st))) return e;
@@ -292,7 +292,7 @@ ovl_status solve_fom(ovl_lattice* lat, const ovl_sign_params* p, int nrhs, const
     launches += 1;
   }
   // x = x_P + H_W X: one FP64 stencil with the FP64 links, then the canonical layout
-  OVL_CHECK_CUDA(launch_dslash(g, U, LINK_F64, true, p->m_W, p->mu, false, true, true, true, nrhs, X, ax, st));
+  OVL_CHECK_CUDA(launch_dslash(g, U, LINK_F64, true, p->m_W, p->mu, false, true, true, nrhs, X, ax, st));
   double2* xd = p->host_io ? (double2*)(base + o_xd) : x;
   OVL_CHECK_CUDA(launch_ms_finish(g, nrhs, ax, m > 0 ? xp : nullptr, xd, st));
   launches += 2;

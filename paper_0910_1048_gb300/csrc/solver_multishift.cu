@@ -468,8 +468,8 @@ ovl_status solve_multishift(ovl_lattice* lat, const ovl_sign_params* p, int nrhs
       std::vector<double> resn(gn, 0.0), r0(gn);
       for (int j = 0; j < gn; ++j) r0[j] = seed[(size_t)((j0 + j) / s) * 8 + 4].x;
       for (int sweep = 0;; ++sweep) {
-        OVL_CHECK_CUDA(launch_dslash(g, U, LINK_F64, true, p->m_W, p->mu, false, true, true, true, gn, xg, w->t1, st));
-        OVL_CHECK_CUDA(launch_dslash(g, U, LINK_F64, true, p->m_W, p->mu, false, true, true, true, gn, w->t1, w->t2, st));
+        OVL_CHECK_CUDA(launch_dslash(g, U, LINK_F64, true, p->m_W, p->mu, false, true, true, gn, xg, w->t1, st));
+        OVL_CHECK_CUDA(launch_dslash(g, U, LINK_F64, true, p->m_W, p->mu, false, true, true, gn, w->t1, w->t2, st));
         OVL_CHECK_CUDA(launch_ms_residual_batch(g, j0, gn, s, v.r64, w->t2, xg, w->sg_all, w->res, w->rpart,
                                                 w->rcount, w->rout, st));
         launches += 3;
@@ -566,7 +566,7 @@ ovl_status solve_multishift(ovl_lattice* lat, const ovl_sign_params* p, int nrhs
     launches += 1;
   }
   // x = x_P + A X (FP64 stencil, native layout)
-  OVL_CHECK_CUDA(launch_dslash(g, U, LINK_F64, true, p->m_W, p->mu, false, true, true, true, nrhs, v.X, w->ax, st));
+  OVL_CHECK_CUDA(launch_dslash(g, U, LINK_F64, true, p->m_W, p->mu, false, true, true, nrhs, v.X, w->ax, st));
   double2* xd = p->host_io ? w->xdev : x;
   OVL_CHECK_CUDA(launch_ms_finish(g, nrhs, w->ax, v.xp, xd, st));
   if (p->host_io) OVL_CHECK_CUDA(cudaMemcpyAsync(x, w->xdev, (size_t)nrhs * n * 16, cudaMemcpyDeviceToHost, st));
