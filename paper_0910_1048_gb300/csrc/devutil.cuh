@@ -374,14 +374,14 @@ __device__ __forceinline__ void add_hops(const Geom& g, const Links& U, int s, i
                                          StrideLoader ld, bool g5in, bool self, Spin<double>& out) {
   FxAcc acc;
   fx_clear(acc);
-  const bool fx = c.ok && U.fxf->ok;
-  if (fx) fx_hops(g, U.fx, s, k0, k1, c, ld, g5in, acc);
+  int E = 0;
+  const bool fx = c.ok && U.fxf->ok && fx_hops(g, U.fx, s, k0, k1, c, ld, g5in, acc, E);
   if (self) {
     ld(s, out);
     if (g5in) gamma5_inplace(out);
   }
-  if (fx && fx_usable(acc)) {
-    const double f = fx_unit(acc, c, U.fxf->uexp);
+  if (fx) {
+    const double f = fx_unit(E, c, U.fxf->uexp);
 #pragma unroll
     for (int i = 0; i < 12; ++i) {
       cplx<double>& o = out.c[i / 3][i % 3];

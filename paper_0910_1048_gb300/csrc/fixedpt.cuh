@@ -83,6 +83,24 @@ OVL_HD fx64 fx_sar(fx64 v, int n) {
   return v >> (n > 63 ? 63 : n);
 #endif
 }
+// acc + a b in one instruction. (Written out: the compiler turns a negated factor into a product and a
+// 64-bit subtraction, three instructions.)
+OVL_HD void fx_mad(fx64& acc, int a, int b) {
+#if defined(__CUDA_ARCH__)
+  asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(acc) : "r"(a), "r"(b));
+#else
+  acc += (fx64)a * b;
+#endif
+}
+OVL_HD fx64 fx_mul(int a, int b) {
+#if defined(__CUDA_ARCH__)
+  fx64 r;
+  asm("mul.wide.s32 %0, %1, %2;" : "=l"(r) : "r"(a), "r"(b));
+  return r;
+#else
+  return (fx64)a * b;
+#endif
+}
 OVL_HD void fx_words(double x, int& hi, unsigned& lo) {
 #if defined(__CUDA_ARCH__)
   hi = __double2hiint(x);
@@ -103,33 +121,28 @@ OVL_HD double fx_pow2(int biased) {  // 2^(biased - 1023), 0 < biased < 2047
 }
 
 // Limbs of x in units of 2^-59 2^(e-1022), e >= 64 at least x's biased exponent (smaller values are
-// shifted out; zeros and subnormals, biased exponent 0, give 0).
+// shifted out; zeros and subnormals, biased exponent 0, give 0 or -1 unit). A negative value is the one's
+// complement of its 59-bit magnitude: one unit off, and two instructions less per component.
 OVL_HD void fx_limbs(int hi, unsigned lo, int e, int& h, int& l) {
-  const unsigned mh = ((unsigned)hi & 0xfffffu) | 0x100000u;
   const int d = e - (int)(((unsigned)hi >> 20) & 0x7ffu);
-  const unsigned long long m = ((unsigned long long)mh << 32 | lo) << 6;
-  const unsigned long long q = fx_shr(m, d);
-  const fx64 s = (fx64)(hi >> 31);
-  const fx64 v = ((fx64)q ^ s) - s;
-  h = (int)(v >> 30);
-  l = (int)((unsigned)v & 0x3fffffffu);
+  const unsigned s = (unsigned)(hi >> 31);
+  const unsigned mh = (((unsigned)hi << 6 | lo >> 26) & 0x03ffffffu) ^ s ^ 0x04000000u;
+  const fx64 v = (fx64)((unsigned long long)mh << 32 | ((lo << 6) ^ s));
+  h = (int)fx_sar(v, d + 30);
+  l = (int)((unsigned)fx_sar(v, d) & 0x3fffffffu);
 }
 
 struct FxHalf {  // projected half spinor: limbs of [2 spins][3 colours] complex
   int rh[2][3], rl[2][3], ih[2][3], il[2][3];
 };
 
-struct FxAcc {  // accumulators of a site: sums of hops in units of 2^-56 2^(E-1022)
+struct FxAcc {  // accumulators of a site: sums of hops in units of 2^-56 2^(E-1022), E their biased exponent
   fx64 re[4][3], im[4][3];
-  int E;     // common biased exponent (+1)
-  int emax;  // largest biased exponent of a neighbour
 };
 
 OVL_HD void fx_clear(FxAcc& a) {
 #pragma unroll
   for (int i = 0; i < 12; ++i) a.re[i / 3][i % 3] = a.im[i / 3][i % 3] = 0;
-  a.E = 0;
-  a.emax = 0;
 }
 
 struct FxSpin {  // limbs of a site's 12 complex components relative to one exponent
@@ -219,55 +232,39 @@ OVL_HD fx64 fx_scale(fx64 t, int h, int l) {
   return 2 * ((fx64)th * h) + (x >> 29);
 }
 
-// Adds hop k = 2 mu (forward, U) or 2 mu + 1 (backward, U^H) of the neighbour spinor p to the
-// accumulators; U points at the link's entry [0][0], its entries `stride` apart. g5in: the input is
-// gamma5 p (the lower spins change sign, which exchanges the two projectors). flip: the hop crosses an
-// antiperiodic boundary. The direction is a run-time value (uniform over a warp) so that the hops share
-// one copy of the conversion and the product: unrolled over the eight hops the kernel was 100 KB of
-// code and took minutes to compile.
-OVL_HD void fx_hop(int k, const Spin<double>& p, const FxC* U, size_t stride, const FxCoef& c, bool g5in, bool flip,
-                   FxAcc& acc) {
+// Half spinor of hop k = 2 mu (forward, U) or 2 mu + 1 (backward, U^H) from the neighbour's limbs.
+// g5in: the input is gamma5 p (the lower spins change sign, which exchanges the two projectors). The
+// direction is a run-time value (uniform over a warp) so that the hops share one copy of the conversion
+// and the product: unrolled over the eight hops the kernel was 100 KB of code and took minutes to compile.
+OVL_HD void fx_half(int k, const FxSpin& q, bool g5in, FxHalf& h) {
+  // the backward hop multiplies by U^H = conj(U^T): conj(U^T conj(h)) conjugated at the end
+  switch (g5in ? k + 8 : k) {
+    case 0: fx_project<0, true, false>(q, h); break;
+    case 1: fx_project<0, false, true>(q, h); break;
+    case 2: fx_project<1, true, false>(q, h); break;
+    case 3: fx_project<1, false, true>(q, h); break;
+    case 4: fx_project<2, true, false>(q, h); break;
+    case 5: fx_project<2, false, true>(q, h); break;
+    case 6: fx_project<3, true, false>(q, h); break;
+    case 7: fx_project<3, false, true>(q, h); break;
+    case 8: fx_project<0, false, false>(q, h); break;
+    case 9: fx_project<0, true, true>(q, h); break;
+    case 10: fx_project<1, false, false>(q, h); break;
+    case 11: fx_project<1, true, true>(q, h); break;
+    case 12: fx_project<2, false, false>(q, h); break;
+    case 13: fx_project<2, true, true>(q, h); break;
+    case 14: fx_project<3, false, false>(q, h); break;
+    default: fx_project<3, true, true>(q, h); break;
+  }
+}
+
+// Exponent of hop k's contribution for a neighbour of exponent e.
+OVL_HD int fx_hop_exponent(int k, int e, const FxCoef& c) { return k < 6 ? e : e + ((k & 1) ? c.be : c.fe); }
+
+// Adds hop k of the half spinor h to the accumulators, d = E - (the hop's exponent) >= 0; U points at the
+// link's entry [0][0], its entries `stride` apart. flip: the hop crosses an antiperiodic boundary.
+OVL_HD void fx_hop(int k, int d, const FxHalf& h, const FxC* U, size_t stride, const FxCoef& c, bool flip, FxAcc& acc) {
   const bool fwd = !(k & 1), time = k >= 6;
-  const int eb = fx_exponent(p);
-  acc.emax = acc.emax > eb ? acc.emax : eb;
-  const int e = eb > 64 ? eb : 64;
-  FxHalf h;
-  {
-    FxSpin q;
-    fx_spin(p, e, q);
-    // the backward hop multiplies by U^H = conj(U^T): conj(U^T conj(h)) conjugated at the end
-    switch (g5in ? k + 8 : k) {
-      case 0: fx_project<0, true, false>(q, h); break;
-      case 1: fx_project<0, false, true>(q, h); break;
-      case 2: fx_project<1, true, false>(q, h); break;
-      case 3: fx_project<1, false, true>(q, h); break;
-      case 4: fx_project<2, true, false>(q, h); break;
-      case 5: fx_project<2, false, true>(q, h); break;
-      case 6: fx_project<3, true, false>(q, h); break;
-      case 7: fx_project<3, false, true>(q, h); break;
-      case 8: fx_project<0, false, false>(q, h); break;
-      case 9: fx_project<0, true, true>(q, h); break;
-      case 10: fx_project<1, false, false>(q, h); break;
-      case 11: fx_project<1, true, true>(q, h); break;
-      case 12: fx_project<2, false, false>(q, h); break;
-      case 13: fx_project<2, true, true>(q, h); break;
-      case 14: fx_project<3, false, false>(q, h); break;
-      default: fx_project<3, true, true>(q, h); break;
-    }
-  }
-  const int eh = e + (time ? (fwd ? c.fe : c.be) : 0);  // exponent of this hop's contribution
-  if (eh > acc.E) {  // first hop, or a larger neighbour than any before
-    const int E = eh + 1;
-    if (acc.E != 0) {
-#pragma unroll
-      for (int i = 0; i < 12; ++i) {
-        acc.re[i / 3][i % 3] = fx_sar(acc.re[i / 3][i % 3], E - acc.E);
-        acc.im[i / 3][i % 3] = fx_sar(acc.im[i / 3][i % 3], E - acc.E);
-      }
-    }
-    acc.E = E;
-  }
-  const int d = acc.E - eh;
   const bool scaled = time && !c.unit;
   const int sh = scaled ? (d < 60 ? d : 60) : (d < 58 ? d + 2 : 60);
   const fx64 half = sh > 0 ? (fx64)1 << (sh - 1) : 0;  // rounds the shift
@@ -276,40 +273,45 @@ OVL_HD void fx_hop(int k, const Spin<double>& p, const FxC* U, size_t stride, co
   fx64 tr[2][3], ti[2][3];
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    fx64 hr0 = seed, hi0 = seed, hr1 = seed, hi1 = seed, xr0 = 0, xi0 = 0, xr1 = 0, xi1 = 0;
+    fx64 hr[2], hi[2], xr[2], xi[2];
 #pragma unroll
     for (int b = 0; b < 3; ++b) {
       const FxC u = U[a * sa + b * sb];
       const int nh = -u.ih, nl = -u.il;
-      hr0 += (fx64)u.rh * h.rh[0][b];
-      hr0 += (fx64)nh * h.ih[0][b];
-      hi0 += (fx64)u.rh * h.ih[0][b];
-      hi0 += (fx64)u.ih * h.rh[0][b];
-      xr0 += (fx64)u.rh * h.rl[0][b];
-      xr0 += (fx64)u.rl * h.rh[0][b];
-      xr0 += (fx64)nh * h.il[0][b];
-      xr0 += (fx64)nl * h.ih[0][b];
-      xi0 += (fx64)u.rh * h.il[0][b];
-      xi0 += (fx64)u.rl * h.ih[0][b];
-      xi0 += (fx64)u.ih * h.rl[0][b];
-      xi0 += (fx64)u.il * h.rh[0][b];
-      hr1 += (fx64)u.rh * h.rh[1][b];
-      hr1 += (fx64)nh * h.ih[1][b];
-      hi1 += (fx64)u.rh * h.ih[1][b];
-      hi1 += (fx64)u.ih * h.rh[1][b];
-      xr1 += (fx64)u.rh * h.rl[1][b];
-      xr1 += (fx64)u.rl * h.rh[1][b];
-      xr1 += (fx64)nh * h.il[1][b];
-      xr1 += (fx64)nl * h.ih[1][b];
-      xi1 += (fx64)u.rh * h.il[1][b];
-      xi1 += (fx64)u.rl * h.ih[1][b];
-      xi1 += (fx64)u.ih * h.rl[1][b];
-      xi1 += (fx64)u.il * h.rh[1][b];
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        if (b == 0) {
+          hr[r] = hi[r] = seed;
+          xr[r] = fx_mul(u.rh, h.rl[r][b]);
+          xi[r] = fx_mul(u.rh, h.il[r][b]);
+        } else {
+          fx_mad(xr[r], u.rh, h.rl[r][b]);
+          fx_mad(xi[r], u.rh, h.il[r][b]);
+        }
+        fx_mad(hr[r], u.rh, h.rh[r][b]);
+        fx_mad(hi[r], u.rh, h.ih[r][b]);
+        fx_mad(xr[r], u.rl, h.rh[r][b]);
+        fx_mad(xi[r], u.rl, h.ih[r][b]);
+        fx_mad(hr[r], nh, h.ih[r][b]);
+        fx_mad(hi[r], u.ih, h.rh[r][b]);
+        fx_mad(xr[r], nh, h.il[r][b]);
+        fx_mad(xi[r], u.ih, h.rl[r][b]);
+        fx_mad(xr[r], nl, h.ih[r][b]);
+        fx_mad(xi[r], u.il, h.rh[r][b]);
+      }
     }
-    tr[0][a] = hr0 + (xr0 >> 30);
-    ti[0][a] = hi0 + (xi0 >> 30);
-    tr[1][a] = hr1 + (xr1 >> 30);
-    ti[1][a] = hi1 + (xi1 >> 30);
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      tr[r][a] = hr[r] + (xr[r] >> 30);
+      ti[r][a] = hi[r] + (xi[r] >> 30);
+    }
+  }
+  if (time && flip) {
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+      tr[i / 3][i % 3] = -tr[i / 3][i % 3];
+      ti[i / 3][i % 3] = -ti[i / 3][i % 3];
+    }
   }
   if (scaled) {
     const int fh = fwd ? c.fh : c.bh, fl = fwd ? c.fl : c.bl;
@@ -319,11 +321,10 @@ OVL_HD void fx_hop(int k, const Spin<double>& p, const FxC* U, size_t stride, co
       ti[i / 3][i % 3] = fx_scale(ti[i / 3][i % 3], fh, fl) + half;
     }
   }
-  const fx64 fm = flip ? -1 : 0;
 #pragma unroll
   for (int i = 0; i < 6; ++i) {
-    tr[i / 3][i % 3] = (fx_sar(tr[i / 3][i % 3], sh) ^ fm) - fm;
-    ti[i / 3][i % 3] = (fx_sar(ti[i / 3][i % 3], sh) ^ fm) - fm;
+    tr[i / 3][i % 3] = fx_sar(tr[i / 3][i % 3], sh);
+    ti[i / 3][i % 3] = fx_sar(ti[i / 3][i % 3], sh);
   }
   switch (k) {
     case 0: fx_reconstruct<0, true>(acc, tr, ti); break;
@@ -388,36 +389,71 @@ OVL_HD FxC fx_link_entry(cplx<double> u, int uexp) {
   return r;
 }
 
+// The coordinates of a site in 16-bit fields (extents are at most 4096).
+OVL_HD unsigned long long fx_coords(const Geom& g, int s) {
+  const int x = s % g.lx;
+  int r = s / g.lx;
+  const int y = r % g.ly;
+  r /= g.ly;
+  const int z = r % g.lz, t = r / g.lz;
+  return (unsigned long long)(t << 16 | z) << 32 | (unsigned)(y << 16 | x);
+}
+
 // Neighbour of site s for hop k, and whether the hop crosses the time boundary.
-OVL_HD int fx_neighbour(const Geom& g, int s, int k, bool* wraps) {
+OVL_HD int fx_neighbour(const Geom& g, int s, unsigned long long xyzt, int k, bool* wraps) {
   const int mu = k >> 1;
   const int st = mu == 0 ? 1 : mu == 1 ? g.sy : mu == 2 ? g.sz : g.st;
   const int len = mu == 0 ? g.lx : mu == 1 ? g.ly : mu == 2 ? g.lz : g.lt;
-  const int x = (s / st) % len;
+  const int x = (int)(fx_shr(xyzt, 16 * mu) & 0xffff);
   const bool edge = x == ((k & 1) ? 0 : len - 1);
   *wraps = mu == 3 && edge;
   const int step = edge ? (1 - len) * st : st;
   return (k & 1) ? s - step : s + step;
 }
 
-// Hops k0 .. k1-1 of site s, psi loaded through `ld`.
+// Hops k0 .. k1-1 of site s, psi in FP64 loaded through `ld` and converted on the way. E: the largest
+// exponent met so far (+1). Returns whether the accumulators hold the hop sum: no infinity or NaN among
+// the neighbours, and not only components too small for the common exponent (all zero is fine).
 template <class Load>
-OVL_HD void fx_hops(const Geom& g, const FxC* U, int s, int k0, int k1, const FxCoef& c, Load ld, bool g5in, FxAcc& acc) {
+OVL_HD bool fx_hops(const Geom& g, const FxC* U, int s, int k0, int k1, const FxCoef& c, Load ld, bool g5in, FxAcc& acc,
+                    int& E) {
+  const unsigned long long xyzt = fx_coords(g, s);
+  int emax = 0;
+  E = 0;
 #pragma unroll 1
   for (int k = k0; k < k1; ++k) {
     bool wraps;
-    const int nb = fx_neighbour(g, s, k, &wraps);
-    Spin<double> p;
-    ld(nb, p);
-    fx_hop(k, p, U + (size_t)(k >> 1) * 9 * g.vol + ((k & 1) ? nb : s), (size_t)g.vol, c, g5in, wraps && g.t_bc < 0, acc);
+    const int nb = fx_neighbour(g, s, xyzt, k, &wraps);
+    FxHalf h;
+    int e;
+    {
+      Spin<double> p;
+      ld(nb, p);
+      const int eb = fx_exponent(p);
+      emax = emax > eb ? emax : eb;
+      e = eb > 64 ? eb : 64;
+      FxSpin q;
+      fx_spin(p, e, q);
+      fx_half(k, q, g5in, h);
+    }
+    const int eh = fx_hop_exponent(k, e, c);
+    if (eh > E) {  // first hop, or a larger neighbour than any before
+      if (E != 0) {
+#pragma unroll
+        for (int i = 0; i < 12; ++i) {
+          acc.re[i / 3][i % 3] = fx_sar(acc.re[i / 3][i % 3], eh + 1 - E);
+          acc.im[i / 3][i % 3] = fx_sar(acc.im[i / 3][i % 3], eh + 1 - E);
+        }
+      }
+      E = eh + 1;
+    }
+    fx_hop(k, E - eh, h, U + (size_t)(k >> 1) * 9 * g.vol + ((k & 1) ? nb : s), (size_t)g.vol, c, wraps && g.t_bc < 0,
+           acc);
   }
+  return emax < 0x7ff && E < 2000 && (emax == 0 || emax >= 64);
 }
 
-// Whether the accumulators hold the hop sum: no infinity or NaN among the neighbours, and not only
-// components too small for the common exponent (all zero is fine: the sum is 0).
-OVL_HD bool fx_usable(const FxAcc& a) { return a.emax < 0x7ff && a.E < 2000 && (a.emax == 0 || a.emax >= 64); }
-
 // FP64 value of one unit of the accumulators times the hop coefficient ks and the links' scale.
-OVL_HD double fx_unit(const FxAcc& a, const FxCoef& c, int uexp) { return c.k.ks * fx_pow2(a.E - 55 + uexp); }
+OVL_HD double fx_unit(int E, const FxCoef& c, int uexp) { return c.k.ks * fx_pow2(E - 55 + uexp); }
 
 }  // namespace ovl

@@ -35,16 +35,14 @@ void run(const Geom& g, double m_w, double mu, const FxC* fx, int uexp, const do
          int* usable) {
   const FxCoef c = fx_coef(m_w, mu);
   for (int s = 0; s < g.vol; ++s) {
-    Nbr n;
-    neighbours(g, s, n);
     FxAcc a;
+    int E;
     fx_clear(a);
     const Load<double> ld{psi, g.vol, false};
-    fx_hops(g, fx, s, 0, 8, c, ld, g5in, a);
-    usable[s] = c.ok && fx_usable(a);
+    usable[s] = c.ok && fx_hops(g, fx, s, 0, 8, c, ld, g5in, a, E);
     Spin<double> o;
     Load<double>{psi, g.vol, g5in}(s, o);
-    const double f = usable[s] ? fx_unit(a, c, uexp) : 0.0;
+    const double f = usable[s] ? fx_unit(E, c, uexp) : 0.0;
     for (int i = 0; i < 12; ++i) {
       double* q = out + 2 * ((size_t)i * g.vol + s);
       q[0] = std::fma(f, (double)a.re[i / 3][i % 3], o.c[i / 3][i % 3].re);
