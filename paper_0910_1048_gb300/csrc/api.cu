@@ -178,9 +178,12 @@ ovl_status ovl_set_links(ovl_lattice* lat, const void* U, int32_t U_on_device, u
   }
   cudaError_t e = launch_ingest_links(lat->g, src, lat->u64, lat->ufx, lat->fxf, (formats & OVL_F32) ? lat->u32 : nullptr,
                                       (formats & OVL_F16R12) ? lat->u16 : nullptr, st);
+  char field[64];
+  if (e == cudaSuccess) e = cudaMemcpyAsync(field, lat->fxf, fx_field_bytes(), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (tmp) cudaFree(tmp);
   OVL_CHECK_CUDA(e);
+  lat->fx_ok = fx_field_ok(field);
   lat->formats |= formats;
   return OVL_OK;
 }

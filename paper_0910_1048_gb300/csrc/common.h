@@ -160,6 +160,7 @@ struct ovl_lattice {
   double2* u64 = nullptr;
   ovl::FxC* ufx = nullptr;        // fixed-point copy of u64 and its scale (one allocation)
   ovl::FxField* fxf = nullptr;
+  bool fx_ok = false;             // the fixed-point copy is usable (FxField::ok)
   float2* u32 = nullptr;
   uint32_t* u16 = nullptr;
   ovl_deflation defl;

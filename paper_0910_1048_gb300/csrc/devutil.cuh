@@ -1,6 +1,8 @@
 // Device helpers shared by the kernel translation units.
 #pragma once
 
+#include <type_traits>
+
 #include "fixedpt.cuh"
 #include "wilson.cuh"
 
@@ -316,7 +318,7 @@ __device__ __forceinline__ void store_spin(typename V2<R>::T* p, int vol, int s,
 
 
 // ------------------------------------------------------------------ hops of a site
-// Hop coefficients by precision: the FP64 stencil runs in fixed point (fixedpt.cuh).
+// Hop coefficients by precision: the FP64 stencils run in fixed point (fixedpt.cuh).
 template <class R> struct HopsOf { using T = HopCoef<R>; };
 template <> struct HopsOf<double> { using T = FxCoef; };
 template <class R>
@@ -422,34 +424,35 @@ struct SplitSmem {
   cplx<R> part[2][3][12][SITES];  // [which][slot of the contributing direction][component][site]
 };
 
-template <class R, int LF, int SITES = kSplitSites, class Emit>
-__device__ __forceinline__ void pair_split(const Geom& g, const Links& U, const typename HopsOf<R>::T& c0,
-                                           const typename HopsOf<R>::T& c1,
+template <class R, int LF, class Coef, int SITES = kSplitSites, class Emit>
+__device__ __forceinline__ void pair_split(const Geom& g, const Links& U, const Coef& c0, const Coef& c1,
                                            const typename V2<R>::T* in0, const typename V2<R>::T* in1,
                                            SplitSmem<R, SITES>& sm, Emit emit) {
   const int tx = threadIdx.x, which = threadIdx.y >> 2, dir = threadIdx.y & 3;
   const int s = blockIdx.x * SITES + tx;
   const typename V2<R>::T* in = which ? in1 : in0;
-  const typename HopsOf<R>::T& c = which ? c1 : c0;
-  Loader<R, true> ld{in, g.vol, false};
+  const Coef& c = which ? c1 : c0;
   Spin<R> acc;
 #pragma unroll
   for (int q = 0; q < 12; ++q) acc.c[q / 3][q % 3] = mk<R>(0, 0);
   if (s < g.vol) {
-    Nbr n;
-    neighbours(g, s, n);
-    if constexpr (sizeof(R) == 8) {
+    if constexpr (std::is_same_v<Coef, FxCoef>) {
       add_hops(g, U, s, 2 * dir, 2 * dir + 2, c, StrideLoader{in, 1, g.vol}, false, false, acc);
-    } else if (dir == 0) {
-      hop_dir<0, LF>(g, U, s, n, c.ks, c.ks, ld, acc);
-    } else if (dir == 1) {
-      hop_dir<1, LF>(g, U, s, n, c.ks, c.ks, ld, acc);
-    } else if (dir == 2) {
-      hop_dir<2, LF>(g, U, s, n, c.ks, c.ks, ld, acc);
     } else {
-      R ktf = (n.t == g.lt - 1) ? (R)g.t_bc * c.ktf : c.ktf;
-      R ktb = (n.t == 0) ? (R)g.t_bc * c.ktb : c.ktb;
-      hop_dir<3, LF>(g, U, s, n, ktf, ktb, ld, acc);
+      Nbr n;
+      neighbours(g, s, n);
+      Loader<R, true> ld{in, g.vol, false};
+      if (dir == 0) {
+        hop_dir<0, LF>(g, U, s, n, c.ks, c.ks, ld, acc);
+      } else if (dir == 1) {
+        hop_dir<1, LF>(g, U, s, n, c.ks, c.ks, ld, acc);
+      } else if (dir == 2) {
+        hop_dir<2, LF>(g, U, s, n, c.ks, c.ks, ld, acc);
+      } else {
+        R ktf = (n.t == g.lt - 1) ? (R)g.t_bc * c.ktf : c.ktf;
+        R ktb = (n.t == 0) ? (R)g.t_bc * c.ktb : c.ktb;
+        hop_dir<3, LF>(g, U, s, n, ktf, ktb, ld, acc);
+      }
     }
     // contributions to the spins finalised by the other three threads; slot = this direction's
     // index among the three

@@ -15,6 +15,7 @@
 
 #include "devutil.cuh"
 #include "kernels.h"
+#include "lzscalars.cuh"
 
 namespace ovl {
 
@@ -219,6 +220,7 @@ __global__ void __launch_bounds__(256) k_fx_links(int vol, const double2* u64, F
 }
 
 size_t fx_field_bytes() { return sizeof(FxField); }
+bool fx_field_ok(const void* host_copy) { return ((const FxField*)host_copy)->ok != 0; }
 
 cudaError_t launch_ingest_links(const Geom& g, const double* ucan, double2* u64, FxC* ufx, FxField* fxf, float2* u32,
                                 uint32_t* u16, cudaStream_t st) {
@@ -253,9 +255,7 @@ __global__ void __launch_bounds__(kBlock, LF == LINK_F16R12 ? 6 : 7)
   store_spin<float, NATIVE>(out + off, g.vol, s, o);
 }
 
-// FP64 (fixed-point hops, see fixedpt.cuh): the layout and gamma5 are run-time values.
-
-// Three blocks per SM (168 registers): 16^4 x 8 sources 271 us; two (198 registers) 328, four (128,
+// FP64 (fixed-point hops, see fixedpt.cuh): the layout and gamma5 are run-time values. Three blocks per SM (168 registers): 16^4 x 8 sources 271 us; two (198 registers) 328, four (128,
 // spilled) 277.
 __global__ void __launch_bounds__(kBlock, 3)
     k_dslash_f64(Geom g, Links U, FxCoef c, bool native, bool g5_in, bool g5_out, const double2* in, double2* out) {
@@ -596,46 +596,6 @@ __device__ __forceinline__ void lz_alpha_finish(const LzDev& lz, int rhs, size_t
   lz_alpha_store(lz, rhs, o, j, alpha, c);
 }
 
-struct BetaVals {
-  bool ok;    // false: breakdown (or a non-finite value)
-  double d;   // delta_j
-  double id;  // 1/delta_j = sv_{j+1}
-  zd bt;      // beta_j
-  zd swv;     // 1/conj(beta_j) = sw_{j+1}
-  double vn;  // |v_{j+1}|
-};
-
-__device__ __forceinline__ BetaVals lz_beta_vals(const double (&sums)[4]) {
-  // few FP64 operations in one dependent chain (each is slow on this GPU's FP64 pipe): with
-  // r = |ip|^-1 and id = r^(1/2) = 1/delta_j, delta_j = |ip| id, beta_j = id ip, and
-  // 1/conj(beta_j) = beta_j / |beta_j|^2 = id r ip (|beta_j|^2 = |ip|); the breakdown test on squares
-  BetaVals b{};
-  const zd ip = mk(sums[0], sums[1]);
-  const double n2 = norm2(ip);
-  b.ok = (n2 > 1e-28 * (sums[2] * sums[3])) && (n2 <= 1.7976931348623157e308);
-  if (!b.ok) return b;
-  const double r = rsqrt(n2), id = sqrt(r), idp = id * r;
-  b.id = id;
-  b.d = n2 * r * id;  // |ip| / delta_j = delta_j
-  b.bt = id * ip;
-  b.swv = mk(idp * ip.re, idp * ip.im);
-  b.vn = sqrt(sums[2]) * id;
-  return b;
-}
-
-// Stores the values of step j (b.ok) or marks the breakdown.
-__device__ __forceinline__ void lz_beta_store(const LzDev& lz, int rhs, size_t o, int j, const BetaVals& b) {
-  if (!b.ok) {
-    lz.status[rhs] = 1;
-    return;
-  }
-  lz.delta[o + j] = b.d;
-  lz.beta[o + j] = make_double2(b.bt.re, b.bt.im);
-  lz.sv[o + j + 1] = b.id;
-  lz.sw[o + j + 1] = make_double2(b.swv.re, b.swv.im);
-  lz.vnorm[o + j + 1] = b.vn;
-}
-
 // From sums = (what^H vhat re, im, |vhat|^2, |what|^2) of step j: delta_j = sqrt|what^H vhat|,
 // beta_j = what^H vhat / delta_j, the next column scales and |v_{j+1}|; j advances. A relative
 // breakdown (or a non-finite value) sets status 1 instead.
@@ -666,8 +626,7 @@ __device__ __forceinline__ void st_release(int* p, int v) {
 // blocks H(-mu) what), twice the blocks at half the size: 12^4 with 32 sites is 1296 one-warp
 // blocks, at most 9 on an SM against a mean of 8.53 (with both halves per block: 5 against 4.26).
 template <class R, int LF, bool ONE_ROLE = false>
-__global__ void __launch_bounds__(ONE_ROLE ? 32 : 2 * kPairSites) k_lz_pair(Geom g, Links U, typename HopsOf<R>::T cp,
-                                                            typename HopsOf<R>::T cm, LzDev lz,
+__global__ void __launch_bounds__(ONE_ROLE ? 32 : 2 * kPairSites) k_lz_pair(Geom g, Links U, HopCoef<R> cp, HopCoef<R> cm, LzDev lz,
                                                             const typename V2<R>::T* vh, const typename V2<R>::T* wh,
                                                             typename V2<R>::T* av, typename V2<R>::T* aw) {
   using T = typename V2<R>::T;
@@ -688,7 +647,7 @@ __global__ void __launch_bounds__(ONE_ROLE ? 32 : 2 * kPairSites) k_lz_pair(Geom
   if (s < g.vol) {
     Spin<R> ov;
     if (!is_w) {
-      stencil_site<LF, R>(g, U, s, cp, vj, ov);
+      dslash_site<LF, R>(g, U, s, cp, Loader<R, true>{vj, g.vol, false}, ov);
       const R sv = sc[0];
       // all loads of w_j before the stores of Av (the compiler cannot reorder them across stores
       // that might alias, which would serialise twelve memory round trips)
@@ -706,7 +665,7 @@ __global__ void __launch_bounds__(ONE_ROLE ? 32 : 2 * kPairSites) k_lz_pair(Geom
       acc[0].add(a.re);
       acc[1].add(a.im);
     } else {
-      stencil_site<LF, R>(g, U, s, cm, wj, ov);
+      dslash_site<LF, R>(g, U, s, cm, Loader<R, true>{wj, g.vol, false}, ov);
       const cplx<R> sw = mk<R>(sc[1], sc[2]);
 #pragma unroll
       for (int c = 0; c < 12; ++c) {
@@ -730,8 +689,7 @@ __global__ void __launch_bounds__(ONE_ROLE ? 32 : 2 * kPairSites) k_lz_pair(Geom
 // one spin (three colours) of its site: scale, gamma5, store, and for the v half the partial of
 // alpha_j. SITES sites per block, at least MINB blocks per SM.
 template <class R, int LF, int MINB = 1, int SITES = kSplitSites>
-__global__ void __launch_bounds__(8 * SITES, MINB) k_lz_pair_split(Geom g, Links U, typename HopsOf<R>::T cp,
-                                                                   typename HopsOf<R>::T cm,
+__global__ void __launch_bounds__(8 * SITES, MINB) k_lz_pair_split(Geom g, Links U, HopCoef<R> cp, HopCoef<R> cm,
                                                                    LzDev lz, const typename V2<R>::T* vh,
                                                                    const typename V2<R>::T* wh,
                                                                    typename V2<R>::T* av, typename V2<R>::T* aw) {
@@ -751,7 +709,7 @@ __global__ void __launch_bounds__(8 * SITES, MINB) k_lz_pair_split(Geom g, Links
   const R sv = sc[0];
   const cplx<R> sw = mk<R>(sc[1], sc[2]);
   Red<R> acc[2];
-  pair_split<R, LF, SITES>(g, U, cp, cm, vj, wj, sm, [&](int which, int s, int sp, cplx<R> (&x)[3]) {
+  pair_split<R, LF, HopCoef<R>, SITES>(g, U, cp, cm, vj, wj, sm, [&](int which, int s, int sp, cplx<R> (&x)[3]) {
     const R g5 = sp >= 2 ? (R)-1 : (R)1;
     if (which == 0) {
       cplx<R> wv[3];  // loads first (see k_lz_pair)
@@ -791,8 +749,7 @@ __global__ void __launch_bounds__(8 * SITES, MINB) k_lz_pair_split(Geom g, Links
 constexpr int kDynMaxWarps = 12;  // warps per block at most
 
 template <class R, int LF>
-__global__ void __launch_bounds__(32 * kDynMaxWarps, 1) k_lz_pair_dyn(Geom g, Links U, typename HopsOf<R>::T cp,
-                                                                 typename HopsOf<R>::T cm,
+__global__ void __launch_bounds__(32 * kDynMaxWarps, 1) k_lz_pair_dyn(Geom g, Links U, HopCoef<R> cp, HopCoef<R> cm,
                                                                  LzDev lz, const typename V2<R>::T* vh,
                                                                  const typename V2<R>::T* wh,
                                                                  typename V2<R>::T* av, typename V2<R>::T* aw) {
@@ -845,7 +802,7 @@ __global__ void __launch_bounds__(32 * kDynMaxWarps, 1) k_lz_pair_dyn(Geom g, Li
     Red<R> acc[2];
     const bool live = s < g.vol;
     Spin<R> ov;
-    if (live) stencil_site<LF, R>(g, U, s, is_w ? cm : cp, is_w ? wj : vj, ov);
+    if (live) dslash_site<LF, R>(g, U, s, is_w ? cm : cp, Loader<R, true>{is_w ? wj : vj, g.vol, false}, ov);
     if (!waited) scales();  // warp-uniform: every lane reaches it, the status load is one value
     if (stop) break;
     if (live) {
@@ -1225,8 +1182,7 @@ static bool fp64_update_balanced() {
 // In the deferred FP64 step the settle kernel (the previous update's finish) runs first and the
 // stencil is launched early behind it (see k_lz_pair_dyn); `first` is recorded between them.
 template <class R, int LF>
-static cudaError_t pair_dyn_launch(const Geom& g, const Links& U, const typename HopsOf<R>::T& cp,
-                                   const typename HopsOf<R>::T& cm,
+static cudaError_t pair_dyn_launch(const Geom& g, const Links& U, const HopCoef<R>& cp, const HopCoef<R>& cm,
                                    const LzDev& lz, const LzVecs& vec, cudaStream_t st, cudaEvent_t first,
                                    cudaEvent_t mid) {
   const int nsm = std::max(1, sm_count());
@@ -1246,7 +1202,7 @@ static cudaError_t pair_dyn_launch(const Geom& g, const Links& U, const typename
 }
 
 template <int PS, bool ONE_ROLE = false>
-static cudaError_t pair_unsplit(const Geom& g, const Links& U, int lf, bool f64, FxCoef dp, FxCoef dm,
+static cudaError_t pair_unsplit(const Geom& g, const Links& U, int lf, bool f64, HopCoef<double> dp, HopCoef<double> dm,
                                 HopCoef<float> fp, HopCoef<float> fm, const LzDev& lz, const LzVecs& vec,
                                 cudaStream_t st) {
   const unsigned nb = (unsigned)((g.vol + PS - 1) / PS);
@@ -1262,8 +1218,8 @@ static cudaError_t pair_unsplit(const Geom& g, const Links& U, int lf, bool f64,
 }
 
 template <int MINB, int SITES>
-static cudaError_t pair_split_launch(const Geom& g, const Links& U, int lf, bool f64, const FxCoef& dp,
-                                     const FxCoef& dm, const HopCoef<float>& fp, const HopCoef<float>& fm,
+static cudaError_t pair_split_launch(const Geom& g, const Links& U, int lf, bool f64, const HopCoef<double>& dp,
+                                     const HopCoef<double>& dm, const HopCoef<float>& fp, const HopCoef<float>& fm,
                                      const LzDev& lz, const LzVecs& vec, cudaStream_t st) {
   dim3 grid((g.vol + SITES - 1) / SITES, lz.nrhs), block(SITES, 8);
   if (f64)
@@ -1288,7 +1244,7 @@ cudaError_t launch_lanczos_pair(const Geom& g, const Links& U, int lf, bool f64,
                                 const LzDev& lz, const LzVecs& vec, cudaStream_t st, int variant, cudaEvent_t mid,
                                 cudaEvent_t first) {
   if (variant < 0) variant = resolve_pair_variant(g, lf, f64);
-  const FxCoef dp = fx_coef(m_w, mu), dm = fx_coef(m_w, -mu);
+  const HopCoef<double> dp = hop_coef<double>(m_w, mu), dm = hop_coef<double>(m_w, -mu);
   const HopCoef<float> fp = hop_coef<float>(m_w, mu), fm = hop_coef<float>(m_w, -mu);
   cudaError_t e;
   if (variant != 7 && first && (e = record_timing(first, st))) return e;

@@ -114,6 +114,7 @@ cudaError_t launch_from_native(const Geom& g, int nrhs, bool in_f64, const void*
 cudaError_t launch_ingest_links(const Geom& g, const double* ucan, double2* u64, FxC* ufx, FxField* fxf, float2* u32,
                                 uint32_t* u16, cudaStream_t st);
 size_t fx_field_bytes();  // sizeof(FxField)
+bool fx_field_ok(const void* host_copy);  // FxField::ok of a copy of it in host memory
 
 // out = [g5^go] D_W(sign*mu) [g5^gi] in; dtype f64 (FP64 links) or f32 (lf = F32 / F16R12).
 cudaError_t launch_dslash(const Geom& g, const Links& U, int lf, bool f64, double m_w, double mu,
@@ -128,6 +129,30 @@ struct LzVecs {
   void* aw = nullptr;
   double2* xp = nullptr;    // [nrhs][12][V] FP64 deflated part x_P (nullptr without deflation)
 };
+
+// ---- the FP64 step in fixed point (kernels_fx.cu), for fields and coefficients that fit it
+// Limbs of the recurrence vectors, [nrhs][12][V], and their exponents, [nrhs][V]: column j in slot j & 1.
+struct FxVecs {
+  FxC *v[2] = {nullptr, nullptr}, *w[2] = {nullptr, nullptr};
+  FxC *av = nullptr, *aw = nullptr;  // H(mu) vhat_j and H(-mu) what_j over their common factor
+  int *ev[2] = {nullptr, nullptr}, *ew[2] = {nullptr, nullptr}, *eav = nullptr, *eaw = nullptr;
+  int store = 1;                     // write the basis columns (0: two-pass)
+};
+constexpr size_t kFxExponents = 6;   // int arrays of FxVecs per site and rhs
+// Whether (m_W, mu) fit (the field: ovl_lattice::fx_ok).
+bool fx_step_usable(double m_w, double mu);
+// After launch_lanczos_start: slot 1 from vhat_1 (basis column 1) and what_1 (FP64 in w1).
+cudaError_t launch_fx_begin(const Geom& g, const LzDev& lz, const FxVecs& fx, const void* vh, const void* w1,
+                            cudaStream_t st);
+// A step = the finish of the previous one (k_fx_settle) with the pair stencil launched early behind it,
+// then the update; launch_fx_settle after a chunk's last step. `variant`: 1, 4, 5 four threads per site and
+// role, else one. Events as for launch_lanczos_pair.
+cudaError_t launch_fx_pair(const Geom& g, const Links& U, double m_w, double mu, const LzDev& lz, const FxVecs& fx,
+                           cudaStream_t st, int variant, cudaEvent_t mid = nullptr, cudaEvent_t first = nullptr);
+cudaError_t launch_fx_update(const Geom& g, const Links& U, double m_w, const LzDev& lz, const FxVecs& fx, void* vh,
+                             cudaStream_t st, cudaEvent_t mid = nullptr);
+cudaError_t launch_fx_settle(const Geom& g, const LzDev& lz, cudaStream_t st);
+constexpr int kFxStepLaunches = 3;
 
 // c_i = l_i^H b, d_i = r_i^H b (dots[rhs][0..m) = c, [m..2m) = d); part >= nrhs*m*ceil(V/128)*4.
 cudaError_t launch_defl_dots(const Geom& g, int nrhs, int m, const double2* b, const double2* R, const double2* L,

@@ -245,7 +245,7 @@ __global__ void __launch_bounds__(8 * kSplitSites) k_ms_pair_split(Geom g, Links
   const R s1 = s1v[0];
   Red<R> acc[2];
   // each thread finishes one spin (three colours) of its site: see pair_split
-  pair_split<R, LF>(g, U, cp, cm, in0, in1, sm, [&](int which, int s, int sp, cplx<R> (&o)[3]) {
+  pair_split<R, LF, typename HopsOf<R>::T>(g, U, cp, cm, in0, in1, sm, [&](int which, int s, int sp, cplx<R> (&o)[3]) {
     T* out = (T*)(MODE == 0 ? (which ? v.tt : v.t) : (which ? v.qt : v.q)) + voff<R>(rhs, n);
     const T* pp = (const T*)(which ? v.pt : v.p) + voff<R>(rhs, n);
     const T* ptl = (const T*)v.pt + voff<R>(rhs, n);

@@ -34,15 +34,23 @@ namespace {
 constexpr size_t kStaticScratchBytes = (size_t)64 << 20;  // 64 MiB
 constexpr int kMaxDevices = 128;
 
+// Vectors of the fixed-point FP64 step that have no place in the layout below (2 x 12 complex and six
+// exponents per site and rhs): a layout that fits the 64 MiB holds at least seven FP64 vectors, so this
+// is at most 408 / 1344 of it.
+constexpr size_t kStaticFxBytes = (size_t)20 << 20;
+static_assert(kStaticFxBytes * 1344 >= kStaticScratchBytes * 408, "the fixed-point vectors of every layout that fits");
+
 __device__ __align__(256) unsigned char g_static_scratch[kStaticScratchBytes];
+__device__ __align__(256) unsigned char g_static_fx[kStaticFxBytes];
 
 std::mutex g_addr_mu;
 char* g_addr[kMaxDevices] = {nullptr};
+char* g_fx_addr[kMaxDevices] = {nullptr};
 
 // Device address of the static array on device `dev` (current). Looked up again on every call
 // made outside a stream capture, so that an address cached before a device reset is never
 // reused; inside a capture the address cached by an earlier call is used.
-ovl_status static_scratch(int dev, cudaStream_t st, char** out) {
+ovl_status static_scratch(int dev, cudaStream_t st, char** out, char** fx) {
   std::lock_guard<std::mutex> lk(g_addr_mu);
   if (dev < 0 || dev >= kMaxDevices) {
     set_error("apply_sign_noalloc: device ordinal %d out of range", dev);
@@ -54,15 +62,18 @@ ovl_status static_scratch(int dev, cudaStream_t st, char** out) {
     cs = cudaStreamCaptureStatusActive;  // unknown: keep the cached address if there is one
   }
   if (!g_addr[dev] || cs == cudaStreamCaptureStatusNone) {
-    void* p = nullptr;
+    void *p = nullptr, *q = nullptr;
     cudaError_t e = cudaGetSymbolAddress(&p, g_static_scratch);  // the device is current here
-    if (e != cudaSuccess || !p) {
+    if (e == cudaSuccess) e = cudaGetSymbolAddress(&q, g_static_fx);
+    if (e != cudaSuccess || !p || !q) {
       set_error("apply_sign_noalloc: cudaGetSymbolAddress failed: %s", cudaGetErrorString(e));
       return OVL_ECUDA;
     }
     g_addr[dev] = (char*)p;
+    g_fx_addr[dev] = (char*)q;
   }
   *out = g_addr[dev];
+  *fx = g_fx_addr[dev];
   return OVL_OK;
 }
 
@@ -116,8 +127,8 @@ extern "C" ovl_status ovl_apply_sign_noalloc(ovl_lattice* lat, const ovl_sign_pa
     OVL_REQUIRE(sdev == lat->ctx->device, "apply_sign_noalloc: the stream belongs to device %d, the lattice to %d",
                 sdev, lat->ctx->device);
   }
-  char* base = nullptr;
-  OVL_TRY(static_scratch(lat->ctx->device, st, &base));
+  char *base = nullptr, *fxbase = nullptr;
+  OVL_TRY(static_scratch(lat->ctx->device, st, &base, &fxbase));
   const Geom& g = lat->g;
   const size_t n = (size_t)12 * g.vol, elt = f64 ? 16 : 8;
   const int nblk = partial_slots(g), ks = kmax + 2;
@@ -187,9 +198,30 @@ extern "C" ovl_status ovl_apply_sign_noalloc(ovl_lattice* lat, const ovl_sign_pa
   std::vector<double> ls(std::max(m, 1));
   for (int i = 0; i < m; ++i) ls[i] = lat->src()->defl.lam[2 * i] >= 0 ? 1.0 : -1.0;
   if (m > 0) OVL_CHECK_CUDA(cudaMemcpyAsync(lam_sign, ls.data(), m * 8, cudaMemcpyHostToDevice, st));
-  OVL_CHECK_CUDA(launch_lanczos_start(g, f64, lz, vec, (const double2*)b, m, lat->src()->defl.R, lat->src()->defl.L, lam_sign,
-                                      dots, st));
   const Links U = lat->src()->links();
+  // the FP64 step in fixed point as in ovl_apply_sign
+  const bool fxs = f64 && lat->src()->fx_ok && fx_step_usable(p->m_W, p->mu);
+  FxVecs fx;
+  if (fxs) {
+    const size_t nv = (size_t)nrhs * n * 16, ne = (size_t)nrhs * g.vol;
+    fx.v[0] = (FxC*)fxbase;
+    fx.v[1] = (FxC*)(fxbase + nv);
+    int* fe = (int*)(fxbase + 2 * nv);
+    fx.w[0] = (FxC*)vec.wh;
+    fx.w[1] = (FxC*)((char*)vec.wh + nv);
+    fx.av = (FxC*)vec.av;
+    fx.aw = (FxC*)vec.aw;
+    for (int q = 0; q < 2; ++q) fx.ev[q] = fe + q * ne, fx.ew[q] = fe + (2 + q) * ne;
+    fx.eav = fe + 4 * ne;
+    fx.eaw = fe + 5 * ne;
+  }
+  {
+    LzVecs v = vec;
+    if (fxs) v.wh = (char*)vec.aw - (size_t)nrhs * n * 16;  // what_1 (slot 1 of wh) goes to aw, in FP64
+    OVL_CHECK_CUDA(launch_lanczos_start(g, f64, lz, v, (const double2*)b, m, lat->src()->defl.R, lat->src()->defl.L,
+                                        lam_sign, dots, st));
+    if (fxs) OVL_CHECK_CUDA(launch_fx_begin(g, lz, fx, vec.vh, vec.aw, st));
+  }
   const int chunk = std::max(1, std::min(p->check_every > 0 ? p->check_every : 20, kmax));
   const bool fixed = p->fixed_k > 0;
   // host copies of the scalars (pageable: the copies complete before the host reads them)
@@ -268,15 +300,23 @@ extern "C" ovl_status ovl_apply_sign_noalloc(ovl_lattice* lat, const ovl_sign_pa
       if (kk[r] > 0) rs[r].est = out[2 * r + 1] > 0 ? std::sqrt(out[2 * r] / out[2 * r + 1]) : 1e300;
     return OVL_OK;
   };
-  int queued = 0, launches = 1 + (m > 0 ? 1 : 0) + 1;
+  int queued = 0, launches = 1 + (m > 0 ? 1 : 0) + (fxs ? 1 : 0) + 1;
   const int pvar = resolve_pair_variant(g, lf, f64);  // one shape for every step of this call
   while (queued < kmax) {
     int ns = std::min(chunk, kmax - queued);
-    for (int i = 0; i < ns; ++i)
-      OVL_CHECK_CUDA(launch_lanczos_step(g, U, lf, f64, p->m_W, p->mu, lz, vec, st, pvar));
-    OVL_CHECK_CUDA(launch_lanczos_settle(g, f64, lz, st, pvar));  // before the scalars are read
+    for (int i = 0; i < ns; ++i) {
+      if (fxs) {
+        OVL_CHECK_CUDA(launch_fx_pair(g, U, p->m_W, p->mu, lz, fx, st, pvar));
+        OVL_CHECK_CUDA(launch_fx_update(g, U, p->m_W, lz, fx, vec.vh, st));
+      } else {
+        OVL_CHECK_CUDA(launch_lanczos_step(g, U, lf, f64, p->m_W, p->mu, lz, vec, st, pvar));
+      }
+    }
+    // before the scalars are read
+    OVL_CHECK_CUDA(fxs ? launch_fx_settle(g, lz, st) : launch_lanczos_settle(g, f64, lz, st, pvar));
     queued += ns;
-    launches += lanczos_step_launches(g, lf, f64, pvar) * ns + lanczos_settle_launches(f64, pvar);
+    launches += fxs ? kFxStepLaunches * ns + 1
+                    : lanczos_step_launches(g, lf, f64, pvar) * ns + lanczos_settle_launches(f64, pvar);
     if (fixed) continue;
     OVL_CHECK_CUDA(snapshot());
     const bool final_snapshot = queued >= kmax;

@@ -29,6 +29,7 @@ struct DirectWS {
   int nrhs = 0, kmax = 0, f64 = -1, m = 0, vol = 0, prio = 0, two_pass = 0;
   LzDev lz;
   LzVecs vec;
+  FxVecs fx;  // FP64: the fixed-point step's vectors (its v slots share bdev and xdev, w and A v, A w share vec's)
   void* dev_block = nullptr;  // one allocation for everything
   size_t dev_bytes = 0;
   double2* dots = nullptr;
@@ -62,6 +63,7 @@ struct DirectWS {
   int gchunk = 0;
   double g_mw = 0, g_mu = 0;
   int g_lf = -1;
+  int g_fx = -1;   // whether the graphs launch the fixed-point step
   int g_var = -1;  // the pair-stencil shape the graphs launch (a pinned shape may change between solves)
   cudaStream_t stream = nullptr;
   cudaEvent_t ev = nullptr;
@@ -152,6 +154,7 @@ static ovl_status ensure_ws(ovl_lattice* lat, int nrhs, int kmax, bool f64, int 
   size_t o_n1 = take((size_t)nrhs * kmax * 16), o_n2 = take((size_t)nrhs * kmax * 16);
   size_t o_nk = take((size_t)nrhs * 4), o_np = take((size_t)nrhs * 2 * vec_blocks(lat->g) * 8);
   size_t o_nc = take((size_t)nrhs * 4), o_no = take((size_t)nrhs * 2 * 8);
+  size_t o_fe = take(f64 ? kFxExponents * nrhs * vol * 4 : 0);
   size_t o_xa = take(two_pass ? (size_t)nrhs * n * 16 : 0), o_xc = take(two_pass ? (size_t)nrhs * ks * 16 : 0);
   // stream priority: 0 the default; p > 0 asks for p levels more urgent (numerically lower,
   // clamped to the device's range), so that concurrent solves can favour the longest one
@@ -212,6 +215,20 @@ static ovl_status ensure_ws(ovl_lattice* lat, int nrhs, int kmax, bool f64, int 
   w->npart = (double*)(base + o_np);
   w->ncount = (unsigned*)(base + o_nc);
   w->nout = (double*)(base + o_no);
+  if (f64) {
+    int* fe = (int*)(base + o_fe);
+    const size_t ne = (size_t)nrhs * vol;
+    w->fx.v[0] = (FxC*)w->bdev;
+    w->fx.v[1] = (FxC*)w->xdev;
+    w->fx.w[0] = (FxC*)w->vec.wh;
+    w->fx.w[1] = (FxC*)((char*)w->vec.wh + (size_t)nrhs * n * 16);
+    w->fx.av = (FxC*)w->vec.av;
+    w->fx.aw = (FxC*)w->vec.aw;
+    for (int q = 0; q < 2; ++q) w->fx.ev[q] = fe + q * ne, w->fx.ew[q] = fe + (2 + q) * ne;
+    w->fx.eav = fe + 4 * ne;
+    w->fx.eaw = fe + 5 * ne;
+    w->fx.store = two_pass ? 0 : 1;
+  }
   if (two_pass) {
     w->xacc = (double2*)(base + o_xa);
     w->xcoef = (double2*)(base + o_xc);
@@ -417,20 +434,39 @@ ovl_status solve_direct(ovl_lattice* lat, const ovl_sign_params* p, int nrhs, co
   }
   LzVecs vec = w->vec;
   if (m == 0) vec.xp = nullptr;
-  OVL_CHECK_CUDA(launch_lanczos_start(g, f64, w->lz, vec, bd, m, lat->src()->defl.R, lat->src()->defl.L, w->lam_sign, w->dots, st));
   const Links U = lat->src()->links();
+  // the FP64 step in fixed point where the field and the coefficients fit it (kernels_fx.cu)
+  const bool fxs = f64 && lat->src()->fx_ok && fx_step_usable(p->m_W, p->mu);
+  auto start = [&](const LzDev& lz) -> cudaError_t {
+    LzVecs v = vec;
+    if (fxs) v.wh = (char*)vec.aw - (size_t)nrhs * n * 16;  // what_1 (slot 1 of wh) goes to aw, in FP64
+    cudaError_t e = launch_lanczos_start(g, f64, lz, v, bd, m, lat->src()->defl.R, lat->src()->defl.L, w->lam_sign,
+                                         w->dots, st);
+    return e != cudaSuccess || !fxs ? e : launch_fx_begin(g, lz, w->fx, vec.vh, vec.aw, st);
+  };
+  auto pair = [&](const LzDev& lz, int var, cudaEvent_t mid, cudaEvent_t first) -> cudaError_t {
+    return fxs ? launch_fx_pair(g, U, p->m_W, p->mu, lz, w->fx, st, var, mid, first)
+               : launch_lanczos_pair(g, U, lf, f64, p->m_W, p->mu, lz, vec, st, var, mid, first);
+  };
+  auto update = [&](const LzDev& lz, int var, cudaEvent_t mid) -> cudaError_t {
+    return fxs ? launch_fx_update(g, U, p->m_W, lz, w->fx, vec.vh, st, mid)
+               : launch_lanczos_update(g, f64, lz, vec, st, var, mid);
+  };
+  auto settle = [&](const LzDev& lz, int var) -> cudaError_t {
+    return fxs ? launch_fx_settle(g, lz, st) : launch_lanczos_settle(g, f64, lz, st, var);
+  };
+  auto step_launches = [&](int var) { return fxs ? kFxStepLaunches : lanczos_step_launches(g, lf, f64, var); };
+  auto settle_launches = [&](int var) { return fxs ? 1 : lanczos_settle_launches(f64, var); };
+  OVL_CHECK_CUDA(start(w->lz));
   // autotuner: on first use of (volume, precision) time every pair-stencil variant on this
   // solve's step-1 data (the real step-1 launch below recomputes everything they write)
+  // (the fixed-point step has two shapes: one thread per site and role, or four)
+  auto launch_shape = [&](int var) { return pair(w->lz, var, nullptr, nullptr); };
   struct TuneArg {
-    const Geom* g;
-    const Links* U;
-    int lf;
-    bool f64;
-    const ovl_sign_params* p;
-    const LzDev* lz;
-    const LzVecs* vec;
+    decltype(launch_shape)* launch;
     cudaStream_t st;
-  } targ{&g, &U, lf, f64, p, &w->lz, &vec, st};
+    int shapes;
+  } targ{&launch_shape, st, fxs ? 2 : kPairVariants};
   auto measure = [](void* v) -> int {
     TuneArg& t = *(TuneArg*)v;
     float best[kPairVariants];
@@ -443,10 +479,8 @@ ovl_status solve_direct(ovl_lattice* lat, const ovl_sign_params* p, int nrhs, co
     }
     bool ok = true;
     for (int rep = 0; rep < 4 && ok; ++rep)
-      for (int var = 0; var < kPairVariants && ok; ++var) {
-        ok = cudaEventRecord(a, t.st) == cudaSuccess &&
-             launch_lanczos_pair(*t.g, *t.U, t.lf, t.f64, t.p->m_W, t.p->mu, *t.lz, *t.vec, t.st, var) ==
-                 cudaSuccess &&
+      for (int var = 0; var < t.shapes && ok; ++var) {
+        ok = cudaEventRecord(a, t.st) == cudaSuccess && (*t.launch)(var) == cudaSuccess &&
              cudaEventRecord(b2, t.st) == cudaSuccess && cudaEventSynchronize(b2) == cudaSuccess;
         float ms_ = 0;
         if (ok && rep > 0 && cudaEventElapsedTime(&ms_, a, b2) == cudaSuccess) best[var] = std::min(best[var], ms_);
@@ -455,7 +489,7 @@ ovl_status solve_direct(ovl_lattice* lat, const ovl_sign_params* p, int nrhs, co
     cudaEventDestroy(b2);
     cudaGetLastError();
     int pick = 0;
-    for (int var = 1; var < kPairVariants; ++var)
+    for (int var = 1; var < t.shapes; ++var)
       if (best[var] < best[pick]) pick = var;
     return ok ? pick : -1;
   };
@@ -466,12 +500,10 @@ ovl_status solve_direct(ovl_lattice* lat, const ovl_sign_params* p, int nrhs, co
   auto step = [&](cudaEvent_t* tev) -> cudaError_t {
     cudaError_t e;
     if (tev && (e = record_timing(tev[0], st))) return e;
-    if ((e = launch_lanczos_pair(g, U, lf, f64, p->m_W, p->mu, w->lz, vec, st, pvar, tev ? tev[4] : nullptr,
-                                 tev ? tev[6] : nullptr)))
-      return e;
+    if ((e = pair(w->lz, pvar, tev ? tev[4] : nullptr, tev ? tev[6] : nullptr))) return e;
     if (tev && (e = record_timing(tev[1], st))) return e;
     if (tev && (e = record_timing(tev[2], st))) return e;
-    if ((e = launch_lanczos_update(g, f64, w->lz, vec, st, pvar, tev ? tev[5] : nullptr))) return e;
+    if ((e = update(w->lz, pvar, tev ? tev[5] : nullptr))) return e;
     if (tev && (e = record_timing(tev[3], st))) return e;
     return cudaSuccess;
   };
@@ -482,7 +514,7 @@ ovl_status solve_direct(ovl_lattice* lat, const ovl_sign_params* p, int nrhs, co
   // step instead.
   bool use_graph = p->use_graphs != 0 && chunk > 1;
   if (use_graph && !(w->graph[0] && w->graph[1] && w->gchunk == chunk && w->g_mw == p->m_W && w->g_mu == p->mu &&
-                     w->g_lf == lf && w->g_var == pvar)) {
+                     w->g_lf == lf && w->g_var == pvar && w->g_fx == (int)fxs)) {
     const int mid = std::max(1, chunk / 2);
     for (int q = 0; q < 2; ++q) {
       if (w->graph[q]) cudaGraphExecDestroy(w->graph[q]);
@@ -506,11 +538,12 @@ ovl_status solve_direct(ovl_lattice* lat, const ovl_sign_params* p, int nrhs, co
     w->g_mu = p->mu;
     w->g_lf = lf;
     w->g_var = pvar;
+    w->g_fx = fxs;
   }
-  int launches = 1 + (m > 0 ? 1 : 0) + 1;  // start (+ deflation dots) and the combine
+  int launches = 1 + (m > 0 ? 1 : 0) + (fxs ? 1 : 0) + 1;  // start (+ deflation dots, limbs) and the combine
   // the chunk's steps, then the finish of a deferred last step (before the scalars are read)
   auto run_steps = [&](int nsteps, int q) -> cudaError_t {
-    launches += lanczos_step_launches(g, lf, f64, pvar) * nsteps + lanczos_settle_launches(f64, pvar);
+    launches += step_launches(pvar) * nsteps + settle_launches(pvar);
     const bool graph = use_graph && nsteps == chunk;
     cudaError_t e = step(graph ? nullptr : w->tev[q]);
     if (e != cudaSuccess) return e;
@@ -520,7 +553,7 @@ ovl_status solve_direct(ovl_lattice* lat, const ovl_sign_params* p, int nrhs, co
       for (int i = 1; i < nsteps; ++i)
         if ((e = step(nullptr)) != cudaSuccess) return e;
     }
-    return launch_lanczos_settle(g, f64, w->lz, st, pvar);
+    return settle(w->lz, pvar);
   };
   double t_pair = 0, t_upd = 0, t_fin = 0;
   int nsamp = 0;
@@ -732,9 +765,10 @@ ovl_status solve_direct(ovl_lattice* lat, const ovl_sign_params* p, int nrhs, co
     LzDev lz2 = w->lz;
     lz2.xacc = w->xacc;
     lz2.xcoef = w->xcoef;
-    OVL_CHECK_CUDA(launch_lanczos_start(g, f64, lz2, vec, bd, m, lat->src()->defl.R, lat->src()->defl.L, w->lam_sign,
-                                        w->dots, st));
-    launches += 1 + (m > 0 ? 1 : 0);
+    if (p->host_io && fxs)  // the staged b made room for the step's vectors
+      OVL_CHECK_CUDA(cudaMemcpyAsync(w->bdev, b, (size_t)nrhs * n * 16, cudaMemcpyHostToDevice, st));
+    OVL_CHECK_CUDA(start(lz2));
+    launches += 1 + (m > 0 ? 1 : 0) + (fxs ? 1 : 0);
     auto retire = [&](int jdone) -> cudaError_t {  // rhs whose last column is jdone
       for (int r = 0; r < nrhs; ++r)
         if (rs[r].k == jdone) {
@@ -745,13 +779,13 @@ ovl_status solve_direct(ovl_lattice* lat, const ovl_sign_params* p, int nrhs, co
     };
     OVL_CHECK_CUDA(retire(1));
     for (int j = 1; j < kmax2; ++j) {  // step j adds column j + 1
-      OVL_CHECK_CUDA(launch_lanczos_pair(g, U, lf, f64, p->m_W, p->mu, lz2, vec, st, pvar));
-      OVL_CHECK_CUDA(launch_lanczos_update(g, f64, lz2, vec, st, pvar));
-      launches += lanczos_step_launches(g, lf, f64, pvar);
+      OVL_CHECK_CUDA(pair(lz2, pvar, nullptr, nullptr));
+      OVL_CHECK_CUDA(update(lz2, pvar, nullptr));
+      launches += step_launches(pvar);
       OVL_CHECK_CUDA(retire(j + 1));
     }
-    OVL_CHECK_CUDA(launch_lanczos_settle(g, f64, lz2, st, pvar));
-    launches += lanczos_settle_launches(f64, pvar);
+    OVL_CHECK_CUDA(settle(lz2, pvar));
+    launches += settle_launches(pvar);
     OVL_CHECK_CUDA(launch_ms_finish(g, nrhs, w->xacc, vec.xp, xd, st));
   }
   if (p->host_io) OVL_CHECK_CUDA(cudaMemcpyAsync(x, w->xdev, (size_t)nrhs * n * 16, cudaMemcpyDeviceToHost, st));
