@@ -136,23 +136,25 @@ struct FxVecs {
   FxC *v[2] = {nullptr, nullptr}, *w[2] = {nullptr, nullptr};
   FxC *av = nullptr, *aw = nullptr;  // H(mu) vhat_j and H(-mu) what_j over their common factor
   int *ev[2] = {nullptr, nullptr}, *ew[2] = {nullptr, nullptr}, *eav = nullptr, *eaw = nullptr;
+  void* step = nullptr;              // [nrhs] fx_step_bytes(): coefficients of the next update
   int store = 1;                     // write the basis columns (0: two-pass)
 };
 constexpr size_t kFxExponents = 6;   // int arrays of FxVecs per site and rhs
+size_t fx_step_bytes();
 // Whether (m_W, mu) fit (the field: ovl_lattice::fx_ok).
 bool fx_step_usable(double m_w, double mu);
 // After launch_lanczos_start: slot 1 from vhat_1 (basis column 1) and what_1 (FP64 in w1).
-cudaError_t launch_fx_begin(const Geom& g, const LzDev& lz, const FxVecs& fx, const void* vh, const void* w1,
-                            cudaStream_t st);
-// A step = the finish of the previous one (k_fx_settle) with the pair stencil launched early behind it,
-// then the update; launch_fx_settle after a chunk's last step. `variant`: 1, 4, 5 four threads per site and
-// role, else one. Events as for launch_lanczos_pair.
+cudaError_t launch_fx_begin(const Geom& g, const Links& U, double m_w, const LzDev& lz, const FxVecs& fx, const void* vh,
+                            const void* w1, cudaStream_t st);
+// A step = the pair stencil, one block of which ends the previous step, then the update; launch_fx_settle ends
+// a chunk's last step before the host reads the scalars. `variant`: 1, 4, 5 four threads per site and role,
+// else one.
 cudaError_t launch_fx_pair(const Geom& g, const Links& U, double m_w, double mu, const LzDev& lz, const FxVecs& fx,
-                           cudaStream_t st, int variant, cudaEvent_t mid = nullptr, cudaEvent_t first = nullptr);
-cudaError_t launch_fx_update(const Geom& g, const Links& U, double m_w, const LzDev& lz, const FxVecs& fx, void* vh,
-                             cudaStream_t st, cudaEvent_t mid = nullptr);
-cudaError_t launch_fx_settle(const Geom& g, const LzDev& lz, cudaStream_t st);
-constexpr int kFxStepLaunches = 3;
+                           cudaStream_t st, int variant);
+cudaError_t launch_fx_update(const Geom& g, const LzDev& lz, const FxVecs& fx, void* vh, cudaStream_t st);
+cudaError_t launch_fx_settle(const Geom& g, const Links& U, double m_w, const LzDev& lz, const FxVecs& fx,
+                             cudaStream_t st);
+constexpr int kFxStepLaunches = 2;
 
 // c_i = l_i^H b, d_i = r_i^H b (dots[rhs][0..m) = c, [m..2m) = d); part >= nrhs*m*ceil(V/128)*4.
 cudaError_t launch_defl_dots(const Geom& g, int nrhs, int m, const double2* b, const double2* R, const double2* L,

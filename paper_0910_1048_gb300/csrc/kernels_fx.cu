@@ -11,10 +11,17 @@
 //
 // Step j:
 //   k_fx_pair:   A v = H(mu) vhat_j / k, A w = H(-mu) what_j / k (k = the hop coefficient ks times the links'
-//                scale; unscaled otherwise), normalised per site, and the chunk sums of what_j^H (A v)
+//                scale; unscaled otherwise), normalised per site, and the chunk sums of what_j^H (A v). It
+//                needs none of the step's scalars, so one more block settles the previous step
+//                meanwhile: delta, beta, the next scales and the coefficients the update needs
 //   k_fx_update: alpha_j from the chunk sums; vhat_{j+1}, what_{j+1} in place of vhat_{j-1}, what_{j-1}, the
 //                basis column in FP64, and the chunk sums of what^H vhat, |vhat|^2, |what|^2
-//   k_fx_settle: delta_j, beta_j, the next scales (behind the next pair stencil, which needs none of them)
+// Both are launched early (programmatic dependent launch). Each waits for its predecessor, then lets its
+// successor launch; what comes before the wait reads only what the kernel before the predecessor has
+// finished (vectors, exponents, links, j).
+#include <map>
+#include <mutex>
+
 #include "devutil.cuh"
 #include "kernels.h"
 #include "lzscalars.cuh"
@@ -102,10 +109,145 @@ __device__ __forceinline__ FxParts fx_parts(const LzDev& lz, int rhs, int nchunk
   return f;
 }
 
+// ------------------------------------------------------------------ sums over chunks
+// Sum over the chunks c = q 32 + lane, + 32 nshare, ... of t(c) 2^e(c), by one warp: the terms aligned to the
+// largest exponent met and added as two words, exactly. In units of 2^k; every lane gets it.
+template <class LoadT, class LoadE>
+__device__ __forceinline__ double fx_warp_sum_chunks(int nchunk, int q, int nshare, LoadT tv, LoadE ev, int k) {
+  const int first = q * 32 + (threadIdx.x & 31), step = 32 * nshare;
+  constexpr int NK = 4;  // terms kept in registers: one round trip for most lattices
+  fx64 t[NK];
+  int e[NK], em = kFxNone;
+#pragma unroll
+  for (int i = 0; i < NK; ++i) {
+    const int c = first + i * step;
+    t[i] = c < nchunk ? tv(c) : 0;
+    e[i] = c < nchunk ? ev(c) : kFxNone;
+  }
+#pragma unroll
+  for (int i = 0; i < NK; ++i) em = max(em, e[i]);
+  for (int c = first + NK * step; c < nchunk; c += step) em = max(em, ev(c));
+  em = __reduce_max_sync(0xffffffffu, em);
+  fx64 hi = 0, lo = 0;
+#pragma unroll
+  for (int i = 0; i < NK; ++i) {
+    const fx64 a = fx_align(t[i], em - e[i]);
+    hi += a >> 31;
+    lo += a & 0x7fffffff;
+  }
+#pragma unroll 4
+  for (int c = first + NK * step; c < nchunk; c += step) {
+    const fx64 a = fx_align(tv(c), em - ev(c));
+    hi += a >> 31;
+    lo += a & 0x7fffffff;
+  }
+  hi = warp_sum(hi);
+  lo = warp_sum(lo);
+  return fx_scalb(fma((double)hi, 2147483648.0, (double)lo), em + k);
+}
+
+// ------------------------------------------------------------------ settle
+// A complex coefficient in limbs, |components| < 2^(e - 1022).
+struct FxCoefSh {
+  FxC c;
+  int e;
+};
+__device__ __forceinline__ FxCoefSh fx_coefficient(zd r) {
+  FxCoefSh d;
+  int hr, hi;
+  unsigned lr, li;
+  fx_words(r.re, hr, lr);
+  fx_words(r.im, hi, li);
+  const int e = max(max(hr & 0x7fffffff, hi & 0x7fffffff) >> 20, 64);
+  fx_limbs(hr, lr, e, d.c.rh, d.c.rl);
+  fx_limbs(hi, li, e, d.c.ih, d.c.il);
+  d.e = r.re == 0.0 && r.im == 0.0 ? kFxNone : e;  // (the vectors before the first may hold anything)
+  return d;
+}
+
+// What the update of step j needs beside alpha_j (formed where sv_j, sw_j are):
+//   vhat_{j+1} = c0 A v + (kv a) vhat_j + c2 vhat_{j-1}, what_{j+1} = c0w A w + (kw conj(a)) what_j + c2w what_{j-1},
+//   alpha_j = k1 a, a the sum of what_j^H A v.
+struct FxStep {
+  FxCoefSh c[4];    // c0, c2, c0w, c2w
+  double2 k[3];     // kv, kw, k1
+};
+size_t fx_step_bytes() { return (sizeof(FxStep) + 255) & ~(size_t)255; }
+
+__device__ __forceinline__ FxStep* fx_step(const FxVecs& fx, int rhs) {
+  return (FxStep*)((char*)fx.step + (size_t)rhs * ((sizeof(FxStep) + 255) & ~(size_t)255));
+}
+
+// By one warp: lane i < 4 one coefficient, lane 4 the factors of the sum.
+__device__ __forceinline__ void fx_step_store(FxStep* st, double kse, double sv, zd sw, double svp, zd bt, double dp,
+                                              zd swp) {
+  const int lane = threadIdx.x & 31;
+  if (lane < 4) {
+    const zd p = lane == 0 ? mk(sv, 0.0) : lane == 1 ? mk(-svp, 0.0) : lane == 2 ? sw : mk(-dp, 0.0);
+    const zd q = lane == 1 ? bt : lane == 3 ? swp : mk(kse, 0.0);
+    st->c[lane] = fx_coefficient(p * q);
+  } else if (lane == 4) {
+    const zd k1 = (sv * kse) * conj(sw), kv = -(sv * k1), kw = -(sw * conj(k1));
+    st->k[0] = make_double2(kv.re, kv.im);
+    st->k[1] = make_double2(kw.re, kw.im);
+    st->k[2] = make_double2(k1.re, k1.im);
+  }
+}
+
+// Ends the update of step j - 1 (j has been advanced): its sums, delta, beta, the scales of column j, the
+// coefficients of the update of step j. By one block.
+__device__ __forceinline__ void fx_settle(const LzDev& lz, const FxVecs& fx, int rhs, int nchunk, double ks,
+                                          const FxField* fxf) {
+  __shared__ double sh[4][8];
+  const int t = lin_tid(), warp = t >> 5, lane = t & 31, nw = lin_nthreads() >> 5;
+  const int go = lz.pending[rhs] && !lz.status[rhs];
+  const int j = lz.j[rhs];
+  const size_t o = (size_t)rhs * (lz.kmax + 2);
+  const double svp = j > 1 ? lz.sv[o + j - 1] : 0.0;
+  const zd swp = j > 1 ? ldc<double>(lz.sw, o + j - 1) : mk(0.0, 0.0);
+  const FxParts f = fx_parts(lz, rhs, nchunk);
+  const int nshare = max(1, min(8, nw / 4));
+  if (go)
+    for (int i = warp; i < 4 * nshare; i += nw) {
+      const int v = i & 3, q = i >> 2;
+      const double x = fx_warp_sum_chunks(
+          nchunk, q, nshare, [&](int c) { return f.u[(size_t)v * nchunk + c]; },
+          [&](int c) { return f.ue[(size_t)v * nchunk + c]; }, -58 - 2044);
+      if (lane == 0) sh[v][q] = x;
+    }
+  __syncthreads();
+  if (!go || warp != 0) return;
+  double sums[4];
+#pragma unroll
+  for (int v = 0; v < 4; ++v) {
+    sums[v] = sh[v][0];
+    for (int q = 1; q < nshare; ++q) sums[v] += sh[v][q];
+  }
+  const BetaVals b = lz_beta_vals(sums);
+  if (b.ok) fx_step_store(fx_step(fx, rhs), fx_scalb(ks, fxf->uexp), b.id, b.swv, svp, b.bt, b.d, swp);
+  if (lane == 0) {
+    lz_beta_store(lz, rhs, o, j - 1, b);
+    if (!b.ok) lz.j[rhs] = j - 1;
+    lz.pending[rhs] = 0;
+  }
+}
+
+constexpr int kFxSettle = 512;
+__global__ void __launch_bounds__(kFxSettle) k_fx_settle(LzDev lz, const __grid_constant__ FxVecs fx, int nchunk, double ks,
+                                                        const FxField* fxf) {
+  fx_settle(lz, fx, blockIdx.y, nchunk, ks, fxf);
+}
+
 // ------------------------------------------------------------------ start
 // vhat_1 (basis column 1) and what_1 (FP64, in `w1`) to limbs in slot 1. One thread per site.
-__global__ void __launch_bounds__(64) k_fx_begin(Geom g, LzDev lz, FxVecs fx, const double2* vh, const double2* w1) {
+__global__ void __launch_bounds__(64) k_fx_begin(Geom g, LzDev lz, FxVecs fx, const double2* vh, const double2* w1,
+                                                 double ks, const FxField* fxf) {
   const int rhs = blockIdx.y, s = blockIdx.x * blockDim.x + threadIdx.x;
+  if (blockIdx.x == 0 && threadIdx.x < 32) {
+    const size_t o = (size_t)rhs * (lz.kmax + 2) + 1;
+    fx_step_store(fx_step(fx, rhs), fx_scalb(ks, fxf->uexp), lz.sv[o], ldc<double>(lz.sw, o), 0.0, mk(0.0, 0.0), 0.0,
+                  mk(0.0, 0.0));
+  }
   if (s >= g.vol) return;
   const size_t n = (size_t)12 * g.vol;
 #pragma unroll 1
@@ -127,89 +269,158 @@ __global__ void __launch_bounds__(64) k_fx_begin(Geom g, LzDev lz, FxVecs fx, co
 // ------------------------------------------------------------------ pair stencil
 // Block (32 sites, 2 T): warp y computes the hops of role y / T (0: H(mu) vhat_j, 1: H(-mu) what_j) whose
 // index is in [8 t / T, 8 (t+1) / T), t = y % T. T = 1: one thread per site and role; T = 4: one direction
-// per thread, for lattices too small to fill the GPU with one (each thread finishes one spin).
+// per thread, for lattices too small to fill the GPU with one (each thread finishes one spin). Block 0
+// settles the previous step, block b > 0 takes chunk b - 1.
+// With 8.5 warps per SM (12^4) the latency of the loads is not hidden by other warps, so a hop's inputs are
+// copied to shared memory while the previous one is computed: the neighbour's 12 components per thread,
+// and the link's nine once for the two roles.
 struct FxSelf {
   int h, l, e;  // 1 / ks = (h 2^30 + l) 2^-59 2^e
 };
+struct FxPairArgs {  // indexed by the role
+  FxCoef c[2];
+  const FxC* q[2][2];  // [role][slot]
+  const int* e[2][2];
+  FxC* out[2];
+  int* eo[2];
+};
+
+__device__ __forceinline__ void copy_async(void* smem, const void* gmem) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(smem)), "l"(gmem)
+               : "memory");
+}
+__device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 template <int T>
-__global__ void __launch_bounds__(64 * T, T == 1 ? 6 : 1)
-    k_fx_pair(Geom g, Links U, FxCoef cp, FxCoef cm, FxSelf self, LzDev lz, FxVecs fx) {
+struct FxPairSmem {
+  FxC q[2][12][64 * T];   // [stage][component][thread]
+  FxC u[2][T][9][32];     // [stage][direction set][entry][site]
+  fx64 part[T > 1 ? 2 : 1][T > 1 ? T - 1 : 1][12][2][T > 1 ? 32 : 1];  // [role][slot][component][re, im][site]
+  int top[2][T][32];
+  fx64 dot[T][2][32];
+};
+
+template <int T>
+__global__ void __launch_bounds__(64 * T, T == 1 ? 5 : 1)
+    k_fx_pair(Geom g, Links U, const __grid_constant__ FxPairArgs args, FxSelf self, LzDev lz,
+              const __grid_constant__ FxVecs fx, double ks) {
+  extern __shared__ __align__(16) unsigned char raw[];
+  FxPairSmem<T>& sm = *reinterpret_cast<FxPairSmem<T>*>(raw);
   const int rhs = blockIdx.y;
-  const int lane = threadIdx.x, role = threadIdx.y / T, t = threadIdx.y % T;
-  // launched early behind k_fx_settle (programmatic dependent launch): status and j are final since the
-  // update, and the step's scalars are not used here, so the only wait is the one at the end
-  const bool run = lz.status[rhs] == 0;
-  const int j = lz.j[rhs];
-  const int s = blockIdx.x * 32 + lane;
-  const bool live = run && s < g.vol;
+  if (blockIdx.x == 0) {
+    grid_wait();
+    grid_launch();
+    fx_settle(lz, fx, rhs, gridDim.x - 1, ks, U.fxf);
+    return;
+  }
+  const int chunk = blockIdx.x - 1;
+  const int lane = threadIdx.x, role = threadIdx.y / T, t = threadIdx.y % T, tid = lin_tid();
+  const bool live = chunk * 32 + lane < g.vol;
+  const int s = live ? chunk * 32 + lane : g.vol - 1;  // (a lane past the end repeats the last site)
   const size_t n = (size_t)12 * g.vol;
-  const FxCoef& c = role ? cm : cp;
-  const FxC* q = (role ? fx.w : fx.v)[j & 1] + (size_t)rhs * n;
-  const int* ex = (role ? fx.ew : fx.ev)[j & 1] + (size_t)rhs * g.vol;
+  const FxCoef& c = args.c[role];
+  constexpr int NH = 8 / T;
+  const unsigned long long xyzt = fx_coords(g, s);
+  auto fetch_link = [&](int k, int nb) {  // the roles share the nine rows
+    const FxC* u = U.fx + (size_t)(k >> 1) * 9 * g.vol + ((k & 1) ? nb : s);
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+      const int row = role * 5 + i;
+      if (row < 9) copy_async(&sm.u[k & 1][t][row][lane], u + (size_t)row * g.vol);
+    }
+  };
+  bool wraps;
+  int nb = fx_neighbour(g, s, xyzt, t * NH, &wraps);
+  fetch_link(t * NH, nb);
+  grid_wait();
+  grid_launch();
+  const int status = lz.status[rhs], j = lz.j[rhs];
+  const FxC* q = args.q[role][j & 1] + (size_t)rhs * n;
+  const int* ex = args.e[role][j & 1] + (size_t)rhs * g.vol;
+  auto fetch_spinor = [&](int stage, const FxC* p) {
+#pragma unroll
+    for (int i = 0; i < 12; ++i) copy_async(&sm.q[stage][i][tid], p + (size_t)i * g.vol);
+  };
+  fetch_spinor(0, q + nb);
   FxAcc acc;
   fx_clear(acc);
-  int E = 0, es = 0;
   const int se = self.e - U.fxf->uexp;  // exponent of the diagonal's coefficient
-  if (live) {
-    const unsigned long long xyzt = fx_coords(g, s);
-    es = ex[s];
-    int en[8];
-    bool wraps;
+  const int es = ex[s], ew = args.e[1][j & 1][(size_t)rhs * g.vol + s];
+  // the diagonal's scale is at most 2^5 of the hops': |A| < 2^61.8 units
+  int E = es + se - 3;
 #pragma unroll
-    for (int k = 0; k < 8; ++k) en[k] = ex[fx_neighbour(g, s, xyzt, k, &wraps)];
-    // the diagonal's scale is at most 2^5 of the hops': |A| < 2^61.8 units
-    E = es + se - 3;
-#pragma unroll
-    for (int k = 0; k < 8; ++k) E = max(E, fx_hop_exponent(k, en[k], c));
-#pragma unroll 1
-    for (int k = t * (8 / T); k < (t + 1) * (8 / T); ++k) {
-      const int nb = fx_neighbour(g, s, xyzt, k, &wraps);
-      const int eh = fx_hop_exponent(k, ex[nb], c);
-      FxHalf h;
-      {
-        FxSpin p;
-#pragma unroll
-        for (int i = 0; i < 12; ++i) {
-          const FxC x = q[(size_t)i * g.vol + nb];
-          p.rh[i / 3][i % 3] = x.rh;
-          p.rl[i / 3][i % 3] = x.rl;
-          p.ih[i / 3][i % 3] = x.ih;
-          p.il[i / 3][i % 3] = x.il;
-        }
-        fx_half(k, p, false, h);
-      }
-      fx_hop(k, E - eh, h, U.fx + (size_t)(k >> 1) * 9 * g.vol + ((k & 1) ? nb : s), (size_t)g.vol, c,
-             wraps && g.t_bc < 0, acc);
-    }
+  for (int k = 0; k < 8; ++k) {
+    bool w;
+    E = max(E, fx_hop_exponent(k, ex[fx_neighbour(g, s, xyzt, k, &w)], c));
   }
+  const FxC* w = args.q[1][j & 1] + (size_t)rhs * n + s;
+#pragma unroll 1
+  for (int i = 0; i < NH; ++i) {
+    const int k = t * NH + i, eh = fx_hop_exponent(k, ex[nb], c);
+    const bool flip = wraps && g.t_bc < 0;
+    copy_wait();
+    __syncthreads();  // hop k's inputs are there, and the other stage has been read
+    if (i + 1 < NH) {
+      nb = fx_neighbour(g, s, xyzt, k + 1, &wraps);
+      fetch_spinor((i + 1) & 1, q + nb);
+      fetch_link(k + 1, nb);
+    } else if (T == 1) {  // the site's own components, for the diagonal
+      fetch_spinor(0, q + s);
+    } else {  // of the thread's spin, and of what_j
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        copy_async(&sm.q[0][a][tid], q + (size_t)(t * 3 + a) * g.vol + s);
+        copy_async(&sm.q[0][3 + a][tid], w + (size_t)(t * 3 + a) * g.vol);
+      }
+    }
+    FxHalf h;
+    {
+      FxSpin p;
+#pragma unroll
+      for (int r = 0; r < 12; ++r) {
+        const FxC x = sm.q[i & 1][r][tid];
+        p.rh[r / 3][r % 3] = x.rh;
+        p.rl[r / 3][r % 3] = x.rl;
+        p.ih[r / 3][r % 3] = x.ih;
+        p.il[r / 3][r % 3] = x.il;
+      }
+      fx_half(k, p, false, h);
+    }
+    fx_hop(k, E - eh, h, &sm.u[k & 1][t][0][lane], 32, c, flip, acc);
+  }
+  copy_wait();
   // the diagonal psi / ks, and gamma5: A of spin sp
-  auto finish = [&](int sp, fx64 (&ar)[3], fx64 (&ai)[3]) {
-    const int sh = E - es - se + 3;  // from units of 2^-59 2^(es + se - 1022)
+  const int sh = E - es - se + 3;  // from units of 2^-59 2^(es + se - 1022)
+  const int shc = min(sh, 61);
+  const fx64 half = shc > 0 ? (fx64)1 << (shc - 1) : 0;
+  auto finish = [&](int sp, int row, fx64 (&ar)[3], fx64 (&ai)[3]) {
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      const FxC x = q[(size_t)(sp * 3 + a) * g.vol + s];
+      const FxC x = sm.q[0][row + a][tid];
       fx64 xr = fx_mul(x.rh, self.l), xi = fx_mul(x.ih, self.l);
       fx_mad(xr, x.rl, self.h);
       fx_mad(xi, x.il, self.h);
-      ar[a] += fx_align(2 * fx_mul(x.rh, self.h) + (xr >> 29), sh);
-      ai[a] += fx_align(2 * fx_mul(x.ih, self.h) + (xi >> 29), sh);
+      ar[a] += fx_sar(2 * fx_mul(x.rh, self.h) + (xr >> 29) + half, shc);
+      ai[a] += fx_sar(2 * fx_mul(x.ih, self.h) + (xi >> 29) + half, shc);
       if (sp >= 2) ar[a] = -ar[a], ai[a] = -ai[a];
     }
   };
   // normalised A of spin sp to HBM; what_j^H (A v) of the spin in units of 2^-58
-  FxC* out = (role ? fx.aw : fx.av) + (size_t)rhs * n;
+  FxC* out = args.out[role] + (size_t)rhs * n;
   auto emit = [&](int sp, int r, const fx64 (&ar)[3], const fx64 (&ai)[3], fx64& dr, fx64& di) {
-    const FxC* w = fx.w[j & 1] + (size_t)rhs * n;
+    const int rr = max(r, 0), rl = max(-r, 0);
+    const fx64 hn = rr > 0 ? (fx64)1 << (rr - 1) : 0;
     fx64 hr = 0, hi = 0, xr = 0, xi = 0;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
       FxC y;
-      fx_split(fx_normalise(ar[a], r), y.rh, y.rl);
-      fx_split(fx_normalise(ai[a], r), y.ih, y.il);
-      out[(size_t)(sp * 3 + a) * g.vol + s] = y;
+      fx_split(((ar[a] + hn) >> rr) << rl, y.rh, y.rl);
+      fx_split(((ai[a] + hn) >> rr) << rl, y.ih, y.il);
+      if (live) out[(size_t)(sp * 3 + a) * g.vol + s] = y;
       if (role == 0) {
-        const FxC x = w[(size_t)(sp * 3 + a) * g.vol + s];
+        const FxC x = T == 1 ? w[(size_t)(sp * 3 + a) * g.vol] : sm.q[0][3 + a][tid];
         const int nh = -x.ih, nl = -x.il;  // conj(what)
         fx_mad(hr, x.rh, y.rh);
         fx_mad(hr, x.ih, y.ih);
@@ -229,289 +440,259 @@ __global__ void __launch_bounds__(64 * T, T == 1 ? 6 : 1)
     di = hi + (xi >> 30);
   };
   fx64 dr = 0, di = 0;
-  int de = kFxNone;
+  int ea;
   if constexpr (T == 1) {
-    if (live) {
-      int m = 0;
+    int m = 0;
 #pragma unroll
-      for (int sp = 0; sp < 4; ++sp) {
-        finish(sp, acc.re[sp], acc.im[sp]);
+    for (int sp = 0; sp < 4; ++sp) {
+      finish(sp, sp * 3, acc.re[sp], acc.im[sp]);
 #pragma unroll
-        for (int a = 0; a < 3; ++a) m = fx_top(fx_top(m, acc.re[sp][a]), acc.im[sp][a]);
-      }
-      const int r = fx_norm_shift(m), ea = E + r + 3;
+      for (int a = 0; a < 3; ++a) m = fx_top(fx_top(m, acc.re[sp][a]), acc.im[sp][a]);
+    }
+    const int r = fx_norm_shift(m);
+    ea = E + r + 3;
 #pragma unroll
-      for (int sp = 0; sp < 4; ++sp) {
-        fx64 x, y;
-        emit(sp, r, acc.re[sp], acc.im[sp], x, y);
-        dr += x;
-        di += y;
-      }
-      (role ? fx.eaw : fx.eav)[(size_t)rhs * g.vol + s] = ea;
-      if (role == 0) de = ea + fx.ew[j & 1][(size_t)rhs * g.vol + s];
+    for (int sp = 0; sp < 4; ++sp) {
+      fx64 x, y;
+      emit(sp, r, acc.re[sp], acc.im[sp], x, y);
+      dr += x;
+      di += y;
     }
   } else {
     // each thread keeps its own direction's part of spin t and hands the other spins over
-    __shared__ fx64 part[2][3][12][2][32];  // [role][slot of the contributing thread][component][re, im][site]
-    __shared__ int top[2][4][32];
-    __shared__ fx64 dot[4][2][32];
-    if (live) {
 #pragma unroll
-      for (int sp = 0; sp < 4; ++sp)
-        if (sp != t)
+    for (int sp = 0; sp < 4; ++sp)
+      if (sp != t)
 #pragma unroll
-          for (int a = 0; a < 3; ++a) {
-            part[role][t < sp ? t : t - 1][sp * 3 + a][0][lane] = acc.re[sp][a];
-            part[role][t < sp ? t : t - 1][sp * 3 + a][1][lane] = acc.im[sp][a];
-          }
-    }
+        for (int a = 0; a < 3; ++a) {
+          sm.part[role][t < sp ? t : t - 1][sp * 3 + a][0][lane] = acc.re[sp][a];
+          sm.part[role][t < sp ? t : t - 1][sp * 3 + a][1][lane] = acc.im[sp][a];
+        }
     __syncthreads();
     fx64 ar[3] = {0, 0, 0}, ai[3] = {0, 0, 0};
-    if (live) {
 #pragma unroll
-      for (int sp = 0; sp < 4; ++sp)
-        if (sp == t)
+    for (int sp = 0; sp < 4; ++sp)
+      if (sp == t)
 #pragma unroll
-          for (int a = 0; a < 3; ++a) {
-            ar[a] = acc.re[sp][a] + part[role][0][sp * 3 + a][0][lane] + part[role][1][sp * 3 + a][0][lane] +
-                    part[role][2][sp * 3 + a][0][lane];
-            ai[a] = acc.im[sp][a] + part[role][0][sp * 3 + a][1][lane] + part[role][1][sp * 3 + a][1][lane] +
-                    part[role][2][sp * 3 + a][1][lane];
-          }
-      finish(t, ar, ai);
-      int m = 0;
+        for (int a = 0; a < 3; ++a) ar[a] = acc.re[sp][a], ai[a] = acc.im[sp][a];
 #pragma unroll
-      for (int a = 0; a < 3; ++a) m = fx_top(fx_top(m, ar[a]), ai[a]);
-      top[role][t][lane] = m;
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+      for (int p = 0; p < T - 1; ++p) {
+        ar[a] += sm.part[role][p][t * 3 + a][0][lane];
+        ai[a] += sm.part[role][p][t * 3 + a][1][lane];
+      }
+    finish(t, 0, ar, ai);
+    int m = 0;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) m = fx_top(fx_top(m, ar[a]), ai[a]);
+    sm.top[role][t][lane] = m;
+    __syncthreads();
+#pragma unroll
+    for (int p = 0; p < T; ++p) m = max(m, sm.top[role][p][lane]);
+    const int r = fx_norm_shift(m);
+    ea = E + r + 3;
+    fx64 x, y;
+    emit(t, r, ar, ai, x, y);
+    if (role == 0) {
+      sm.dot[t][0][lane] = x;
+      sm.dot[t][1][lane] = y;
     }
     __syncthreads();
-    if (live) {
-      const int m = max(max(top[role][0][lane], top[role][1][lane]), max(top[role][2][lane], top[role][3][lane]));
-      const int r = fx_norm_shift(m), ea = E + r + 3;
-      fx64 x, y;
-      emit(t, r, ar, ai, x, y);
-      if (role == 0) {
-        dot[t][0][lane] = x;
-        dot[t][1][lane] = y;
+    if (role == 0 && t == 0)
+#pragma unroll
+      for (int p = 0; p < T; ++p) {
+        dr += sm.dot[p][0][lane];
+        di += sm.dot[p][1][lane];
       }
-      if (t == 0) {
-        (role ? fx.eaw : fx.eav)[(size_t)rhs * g.vol + s] = ea;
-        if (role == 0) de = ea + fx.ew[j & 1][(size_t)rhs * g.vol + s];
-      }
-    }
-    __syncthreads();
-    if (role == 0 && t == 0 && live) {
-      dr = dot[0][0][lane] + dot[1][0][lane] + dot[2][0][lane] + dot[3][0][lane];
-      di = dot[0][1][lane] + dot[1][1][lane] + dot[2][1][lane] + dot[3][1][lane];
-    }
   }
-  if (role == 0 && t == 0 && run) {  // the chunk's sum
+  if (live && t == 0) args.eo[role][(size_t)rhs * g.vol + s] = ea;
+  if (role == 0 && t == 0 && status == 0) {  // the chunk's sum
+    const int de = live ? ea + ew : kFxNone;
     const int em = __reduce_max_sync(0xffffffffu, de), d = em - de + 5;
-    dr = warp_sum(fx_align(dr, d));
-    di = warp_sum(fx_align(di, d));
+    dr = warp_sum(live ? fx_align(dr, d) : 0);
+    di = warp_sum(live ? fx_align(di, d) : 0);
     if (lane == 0) {
-      const FxParts f = fx_parts(lz, rhs, gridDim.x);
-      f.a[blockIdx.x] = make_longlong2(dr, di);
-      f.ae[blockIdx.x] = em + 5;
+      const FxParts f = fx_parts(lz, rhs, gridDim.x - 1);
+      f.a[chunk] = make_longlong2(dr, di);
+      f.ae[chunk] = em + 5;
     }
   }
-  asm volatile("griddepcontrol.wait;" ::: "memory");  // the settle kernel has finished before this one does
-}
-
-// ------------------------------------------------------------------ sums over chunks
-// Sums of NV values over the chunk partials: value v of chunk c is t(v, c) 2^e(v, c). Every thread of the
-// block takes chunks tid, tid + nthreads, ...; the terms are aligned to the largest exponent and added
-// as two words, exactly. Results (sum hi, sum lo with 2^31 between them, exponent) in all lanes of warp 0.
-struct FxSum {
-  fx64 hi, lo;
-  int e;
-  __device__ __forceinline__ double get(int k) const {  // (hi 2^31 + lo) 2^(e + k)
-    return fx_scalb(fma((double)hi, 2147483648.0, (double)lo), e + k);
-  }
-};
-
-template <int NV, class LoadT, class LoadE>
-__device__ __forceinline__ void fx_sum_chunks(int nchunk, LoadT tv, LoadE ev, FxSum (&out)[NV]) {
-  __shared__ int se[NV][32];
-  __shared__ fx64 sh[NV][2][32];
-  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
-  fx64 t0[NV];
-  int e0[NV], em[NV];
-#pragma unroll
-  for (int v = 0; v < NV; ++v) {  // the first chunk's values: one round trip for most lattices
-    t0[v] = tid < nchunk ? tv(v, tid) : 0;
-    em[v] = e0[v] = tid < nchunk ? ev(v, tid) : kFxNone;
-  }
-  for (int c = tid + nt; c < nchunk; c += nt)
-#pragma unroll
-    for (int v = 0; v < NV; ++v) em[v] = max(em[v], ev(v, c));
-#pragma unroll
-  for (int v = 0; v < NV; ++v) {
-    em[v] = __reduce_max_sync(0xffffffffu, em[v]);
-    if (lane == 0) se[v][warp] = em[v];
-  }
-  __syncthreads();
-#pragma unroll
-  for (int v = 0; v < NV; ++v) {
-    em[v] = __reduce_max_sync(0xffffffffu, lane < nw ? se[v][lane] : kFxNone);
-    fx64 a = fx_align(t0[v], em[v] - e0[v]);
-    fx64 hi = a >> 31, lo = a & 0x7fffffff;
-    for (int c = tid + nt; c < nchunk; c += nt) {
-      a = fx_align(tv(v, c), em[v] - ev(v, c));
-      hi += a >> 31;
-      lo += a & 0x7fffffff;
-    }
-    hi = warp_sum(hi);
-    lo = warp_sum(lo);
-    if (lane == 0) sh[v][0][warp] = hi, sh[v][1][warp] = lo;
-  }
-  __syncthreads();
-  if (warp == 0)
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      out[v].hi = warp_sum(lane < nw ? sh[v][0][lane] : 0);
-      out[v].lo = warp_sum(lane < nw ? sh[v][1][lane] : 0);
-      out[v].e = em[v];
-    }
 }
 
 // ------------------------------------------------------------------ update
 // One block per SM, block b taking the chunks [nchunk b / G, nchunk (b+1) / G); a group of four warps per
 // chunk, warp sp of the group its spin sp. Groups synchronise by themselves (named barriers).
-// Every block forms the coefficients from the pair stencil's chunk sums (a microsecond, instead of a
-// one-block kernel between the two). The block that takes the last ticket at the start (every block
-// has read j by then) advances j and marks the step pending for k_fx_settle.
+// A chunk's inputs are copied to shared memory asynchronously, the first chunk's before anything else,
+// so that their latency passes during the prologue: every block forms the coefficients from the pair
+// stencil's chunk sums (a microsecond, instead of a one-block kernel between the two). The block that takes
+// the last ticket at the start (every block has read j by then) advances j and marks the step pending
+// for k_fx_settle.
 constexpr int kFxGroups = 5;  // chunks in flight per block (96 registers a thread)
-
-struct FxCoefSh {
-  FxC c;
-  int e;
-};
+constexpr int kFxRows = 18;   // 16-byte inputs per thread: three colours of A, column j, column j-1, twice
 
 __device__ __forceinline__ void group_sync(int grp) { asm volatile("bar.sync %0, 128;" ::"r"(grp + 1) : "memory"); }
 
+// (a b) >> d, rounded, for complex limbs; d in [0, 61].
+__device__ __forceinline__ void fx_cmul_shift(const FxC& a, const FxC& b, int d, fx64 half, fx64& re, fx64& im) {
+  const int nh = -a.ih, nl = -a.il;
+  fx64 hr = half, hi = half, xr = fx_mul(a.rh, b.rl), xi = fx_mul(a.rh, b.il);
+  fx_mad(hr, a.rh, b.rh);
+  fx_mad(hi, a.rh, b.ih);
+  fx_mad(xr, a.rl, b.rh);
+  fx_mad(xi, a.rl, b.ih);
+  fx_mad(hr, nh, b.ih);
+  fx_mad(hi, a.ih, b.rh);
+  fx_mad(xr, nh, b.il);
+  fx_mad(xi, a.ih, b.rl);
+  fx_mad(xr, nl, b.ih);
+  fx_mad(xi, a.il, b.rh);
+  re = fx_sar(hr + (xr >> 30), d);
+  im = fx_sar(hi + (xi >> 30), d);
+}
+
 template <bool STORE, bool XACC>
 __global__ void __launch_bounds__(128 * kFxGroups, 1)
-    k_fx_update(Geom g, double ks, const FxField* fxf, LzDev lz, FxVecs fx, double2* vh) {
+    k_fx_update(Geom g, LzDev lz, const __grid_constant__ FxVecs fx, double2* vh) {
+  extern __shared__ FxC rows[];  // [row][thread]
   const int rhs = blockIdx.y;
-  if (lz.status[rhs]) return;
-  __shared__ int jsh;
-  __shared__ FxCoefSh cs[6];
+  __shared__ FxCoefSh cs[6];  // c0, (kv a), c2, c0w, (kw conj(a)), c2w
+  __shared__ double ash[2][4];
   __shared__ fx64 dots[kFxGroups][4][4][32];
   __shared__ int tops[kFxGroups][2][4][32];
-  const int tid = threadIdx.x, lane = tid & 31;
-  if (tid == 0) {
-    jsh = lz.j[rhs];
-    __threadfence();  // this block's read of j completes before its ticket
-    if (atomicAdd(lz.count + rhs, 1u) == gridDim.x - 1) {
-      lz.count[rhs] = 0u;
-      lz.j[rhs] = jsh + 1;
-      lz.pending[rhs] = 1;
-    }
-  }
-  __syncthreads();
-  const int j = jsh;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nt = blockDim.x;
+  const int j = lz.j[rhs];  // (the settle block may take it back, with a status: see below)
   const int nchunk = (g.vol + 31) >> 5;
   const size_t n = (size_t)12 * g.vol, o = (size_t)rhs * (lz.kmax + 2);
+  const int grp = tid >> 7, sp = (tid >> 5) & 3, ngrp = nt >> 7;
+  const int c0 = (int)((long long)nchunk * blockIdx.x / gridDim.x), c1 = (int)((long long)nchunk * (blockIdx.x + 1) / gridDim.x);
+  // rows 0..2 and 9..11: A (after the wait); 3..8, 12..17: columns j and j - 1 (before it)
+  const FxC* in[6] = {fx.av, fx.v[j & 1], fx.v[(j + 1) & 1], fx.aw, fx.w[j & 1], fx.w[(j + 1) & 1]};
+  auto fetch = [&](int ch, bool a) {  // this thread's inputs of chunk ch (a lane past the end takes the last site's)
+    const size_t base = (size_t)rhs * n + (size_t)sp * 3 * g.vol + min(ch * 32 + lane, g.vol - 1);
+#pragma unroll
+    for (int i = 0; i < kFxRows; ++i)
+      if ((i % 9 < 3) == a) copy_async(rows + i * nt + tid, in[i / 3] + base + (size_t)(i % 3) * g.vol);
+  };
+  const bool any = c0 + grp < c1;
+  const size_t es0 = (size_t)rhs * g.vol + min((c0 + grp) * 32 + lane, g.vol - 1);
+  int ex[6] = {0, 0, 0, 0, 0, 0};  // exponents of A, columns j and j - 1, twice
+  auto fetch_e = [&](size_t es, bool a) {
+    if (a)
+      ex[0] = fx.eav[es], ex[3] = fx.eaw[es];
+    else
+      ex[1] = fx.ev[j & 1][es], ex[2] = fx.ev[(j + 1) & 1][es], ex[4] = fx.ew[j & 1][es], ex[5] = fx.ew[(j + 1) & 1][es];
+  };
+  if (any) {
+    fetch(c0 + grp, false);
+    fetch_e(es0, false);
+  }
+  grid_wait();
+  grid_launch();
+  if (lz.status[rhs]) {
+    copy_wait();
+    return;
+  }
+  if (any) {
+    fetch(c0 + grp, true);
+    fetch_e(es0, true);
+  }
   const FxParts parts = fx_parts(lz, rhs, nchunk);
   {
-    // warp 0, one coefficient per lane (lanes 0..5: A v, vhat_j, vhat_{j-1}, A w, what_j, what_{j-1}; 6: alpha_j)
-    zd p = mk(0.0, 0.0), q = mk(0.0, 0.0);
-    if (tid < 32) {
-      const double kse = fx_scalb(ks, fxf->uexp), sv = lz.sv[o + j];
-      const zd sw = ldc<double>(lz.sw, o + j);
-      const zd k1 = (sv * kse) * conj(sw);  // alpha_j = k1 (sum of what^H A v)
-      if (lane == 0) p = mk(sv, 0.0), q = mk(kse, 0.0);
-      if (lane == 1) p = -(sv * k1);
-      if (lane == 2 && j > 1) p = mk(-lz.sv[o + j - 1], 0.0), q = ldc<double>(lz.beta, o + j - 1);
-      if (lane == 3) p = sw, q = mk(kse, 0.0);
-      if (lane == 4) p = -(sw * conj(k1));
-      if (lane == 5 && j > 1) p = mk(-lz.delta[o + j - 1], 0.0), q = ldc<double>(lz.sw, o + j - 1);
-      if (lane == 6) p = k1;
+    const FxStep* st = fx_step(fx, rhs);
+    const int nshare = min(4, nt >> 6);
+    zd k = mk(0.0, 0.0);
+    if (warp == 0 && lane < 3) k = mk(st->k[lane].x, st->k[lane].y);
+    if (warp == 1 && lane < 4) cs[lane < 2 ? 2 * lane : 2 * lane - 1] = st->c[lane];
+    if (warp < 2 * nshare) {  // the sum of what^H A v: warp (value, share)
+      const int v = warp & 1, q = warp >> 1;
+      const double x = fx_warp_sum_chunks(
+          nchunk, q, nshare, [&](int c) { return v ? parts.a[c].y : parts.a[c].x; }, [&](int c) { return parts.ae[c]; },
+          -58 - 2044);
+      if (lane == 0) ash[v][q] = x;
     }
-    FxSum sum[2];
-    fx_sum_chunks<2>(
-        nchunk, [&](int v, int c) { return v ? parts.a[c].y : parts.a[c].x; }, [&](int, int c) { return parts.ae[c]; }, sum);
-    if (tid < 7) {
-      const zd al = mk(sum[0].get(-58 - 2044), sum[1].get(-58 - 2044));
-      if (lane == 1 || lane == 6) q = al;
-      if (lane == 4) q = conj(al);
-      const zd r = p * q;
-      if (lane < 6) {
-        int hr, hi;
-        unsigned lr, li;
-        fx_words(r.re, hr, lr);
-        fx_words(r.im, hi, li);
-        const int e = max(max(hr & 0x7fffffff, hi & 0x7fffffff) >> 20, 64);
-        FxCoefSh& d = cs[lane];
-        fx_limbs(hr, lr, e, d.c.rh, d.c.rl);
-        fx_limbs(hi, li, e, d.c.ih, d.c.il);
-        d.e = r.re == 0.0 && r.im == 0.0 ? kFxNone : e;  // (the vectors before the first may hold anything)
-      } else if (blockIdx.x == 0) {
-        lz.alpha[o + j] = make_double2(r.re, r.im);
+    __syncthreads();
+    if (warp == 0) {
+      zd a = mk(ash[0][0], ash[1][0]);
+      for (int q = 1; q < nshare; ++q) a = a + mk(ash[0][q], ash[1][q]);
+      const zd r = k * (lane == 1 ? conj(a) : a);
+      if (lane < 2) cs[3 * lane + 1] = fx_coefficient(r);
+      if (lane == 2 && blockIdx.x == 0) lz.alpha[o + j] = make_double2(r.re, r.im);
+    }
+    if (tid == 32) {
+      // (every thread of the block has read j: the barrier above)
+      __threadfence();
+      if (atomicAdd(lz.count + rhs, 1u) == gridDim.x - 1) {
+        lz.count[rhs] = 0u;
+        lz.j[rhs] = j + 1;
+        lz.pending[rhs] = 1;
       }
     }
     __syncthreads();
   }
-  const int grp = tid >> 7, sp = (tid >> 5) & 3;
-  const int ngrp = blockDim.x >> 7;
-  const int c0 = (int)((long long)nchunk * blockIdx.x / gridDim.x), c1 = (int)((long long)nchunk * (blockIdx.x + 1) / gridDim.x);
   const zd xc = XACC ? ldc<double>(lz.xcoef, o + j + 1) : mk(0.0, 0.0);
 #pragma unroll 1
   for (int ch = c0 + grp; ch < c1; ch += ngrp) {
     const bool live = ch * 32 + lane < g.vol;
-    const int s = live ? ch * 32 + lane : g.vol - 1;  // (a lane past the end reads the chunk's last site)
+    const int s = live ? ch * 32 + lane : g.vol - 1;
     const size_t base = (size_t)rhs * n + (size_t)sp * 3 * g.vol + s;
     const size_t es = (size_t)rhs * g.vol + s;
-    FxC nv[2][3];  // new limbs of vhat and what
+    fx64 x[2][3][2];
     int en[2];
 #pragma unroll
     for (int role = 0; role < 2; ++role) {
-      const FxC* A = (role ? fx.aw : fx.av) + base;
-      const FxC* V = (role ? fx.w : fx.v)[j & 1] + base;
-      FxC* P = (role ? fx.w : fx.v)[(j + 1) & 1] + base;  // column j-1, overwritten
-      int* pe = (role ? fx.ew : fx.ev)[(j + 1) & 1] + es;
       const FxCoefSh& k0 = cs[3 * role];
       const FxCoefSh& k1 = cs[3 * role + 1];
       const FxCoefSh& k2 = cs[3 * role + 2];
       const bool prev = k2.e != kFxNone;
       // biased exponents of the three products
-      const int e0 = (role ? fx.eaw : fx.eav)[es] + k0.e - 1022, e1 = (role ? fx.ew : fx.ev)[j & 1][es] + k1.e - 1022;
-      const int e2 = prev ? *pe + k2.e - 1022 : kFxNone;
+      const int e0 = ex[3 * role] + k0.e - 1022, e1 = ex[3 * role + 1] + k1.e - 1022;
+      const int e2 = prev ? ex[3 * role + 2] + k2.e - 1022 : kFxNone;
       const int E = max(max(e0, e1), e2);
-      fx64 x[3][2];
+      const int d0 = min(E - e0, 61), d1 = min(E - e1, 61), d2 = min(E - e2, 61);
+      const fx64 h0 = d0 > 0 ? (fx64)1 << (d0 - 1) : 0, h1 = d1 > 0 ? (fx64)1 << (d1 - 1) : 0,
+                 h2 = d2 > 0 ? (fx64)1 << (d2 - 1) : 0;
+      if (role == 0) copy_wait();
       int m = 0;
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
-        const FxC va = A[(size_t)a * g.vol], vv = V[(size_t)a * g.vol];
-        const FxC vp = prev ? P[(size_t)a * g.vol] : FxC{0, 0, 0, 0};
-        fx64 r, i;
+        const FxC va = rows[(role * 9 + a) * nt + tid], vv = rows[(role * 9 + 3 + a) * nt + tid];
+        fx64 xr, xi, r, i;
         if (role == 0) {  // a real coefficient
-          r = fx_rmul(k0.c.rh, k0.c.rl, va.rh, va.rl);
-          i = fx_rmul(k0.c.rh, k0.c.rl, va.ih, va.il);
+          xr = fx_sar(fx_rmul(k0.c.rh, k0.c.rl, va.rh, va.rl) + h0, d0);
+          xi = fx_sar(fx_rmul(k0.c.rh, k0.c.rl, va.ih, va.il) + h0, d0);
         } else {
-          fx_cmul<false>(k0.c, va, r, i);
+          fx_cmul_shift(k0.c, va, d0, h0, xr, xi);
         }
-        fx64 xr = fx_align(r, E - e0), xi = fx_align(i, E - e0);
-        fx_cmul<false>(k1.c, vv, r, i);
-        xr += fx_align(r, E - e1);
-        xi += fx_align(i, E - e1);
-        fx_cmul<false>(k2.c, vp, r, i);
-        xr += fx_align(r, E - e2);
-        xi += fx_align(i, E - e2);
-        x[a][0] = xr;
-        x[a][1] = xi;
+        fx_cmul_shift(k1.c, vv, d1, h1, r, i);
+        xr += r;
+        xi += i;
+        if (prev) {
+          fx_cmul_shift(k2.c, rows[(role * 9 + 6 + a) * nt + tid], d2, h2, r, i);
+          xr += r;
+          xi += i;
+        }
+        x[role][a][0] = xr;
+        x[role][a][1] = xi;
         m = fx_top(fx_top(m, xr), xi);
       }
       tops[grp][role][sp][lane] = m;
-      group_sync(grp);
-      m = max(max(tops[grp][role][0][lane], tops[grp][role][1][lane]),
-              max(tops[grp][role][2][lane], tops[grp][role][3][lane]));
-      const int r = fx_norm_shift(m);
-      en[role] = E + r + 1;
+      en[role] = E;
+    }
+    group_sync(grp);
+    FxC nv[2][3];  // new limbs of vhat and what
+#pragma unroll
+    for (int role = 0; role < 2; ++role) {
+      const int m = max(max(tops[grp][role][0][lane], tops[grp][role][1][lane]),
+                        max(tops[grp][role][2][lane], tops[grp][role][3][lane]));
+      const int r = fx_norm_shift(m), rr = max(r, 0), rl = max(-r, 0);
+      const fx64 half = rr > 0 ? (fx64)1 << (rr - 1) : 0;
+      en[role] += r + 1;
+      FxC* P = (role ? fx.w : fx.v)[(j + 1) & 1] + base;  // in place of column j-1
+      const int k = en[role] - 1022 - 59;
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
-        const fx64 qr = fx_normalise(x[a][0], r), qi = fx_normalise(x[a][1], r);
+        const fx64 qr = ((x[role][a][0] + half) >> rr) << rl, qi = ((x[role][a][1] + half) >> rr) << rl;
         FxC y;
         fx_split(qr, y.rh, y.rl);
         fx_split(qi, y.ih, y.il);
@@ -519,7 +700,7 @@ __global__ void __launch_bounds__(128 * kFxGroups, 1)
         if (live) {
           P[(size_t)a * g.vol] = y;
           if (role == 0 && (STORE || XACC)) {
-            const zd d = mk(fx_scalb((double)qr, en[0] - 1022 - 59), fx_scalb((double)qi, en[0] - 1022 - 59));
+            const zd d = mk(fx_scalb((double)qr, k), fx_scalb((double)qi, k));
             const size_t at = (size_t)(sp * 3 + a) * g.vol + s;
             if (STORE) stc<double>(vh, ((size_t)rhs * lz.vcols + j) * n + at, d);  // column j + 1
             if (XACC) {
@@ -529,30 +710,37 @@ __global__ void __launch_bounds__(128 * kFxGroups, 1)
           }
         }
       }
-      if (live && sp == 0) *pe = en[role];
+      if (live && sp == 0) (role ? fx.ew : fx.ev)[(j + 1) & 1][es] = en[role];
+    }
+    if (ch + ngrp < c1) {  // (this thread has read its rows)
+      const size_t nx = (size_t)rhs * g.vol + min((ch + ngrp) * 32 + lane, g.vol - 1);
+      fetch(ch + ngrp, false);
+      fetch(ch + ngrp, true);
+      fetch_e(nx, false);
+      fetch_e(nx, true);
     }
     // what^H vhat, |vhat|^2, |what|^2 of this spin
     fx64 h[4] = {0, 0, 0, 0}, xx[4] = {0, 0, 0, 0};
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      const FxC x = nv[0][a], y = nv[1][a];
+      const FxC u = nv[0][a], y = nv[1][a];
       const int nh = -y.ih, nl = -y.il;
-      fx_mad(h[0], y.rh, x.rh);
-      fx_mad(h[0], y.ih, x.ih);
-      fx_mad(xx[0], y.rh, x.rl);
-      fx_mad(xx[0], y.rl, x.rh);
-      fx_mad(xx[0], y.ih, x.il);
-      fx_mad(xx[0], y.il, x.ih);
-      fx_mad(h[1], y.rh, x.ih);
-      fx_mad(h[1], nh, x.rh);
-      fx_mad(xx[1], y.rh, x.il);
-      fx_mad(xx[1], y.rl, x.ih);
-      fx_mad(xx[1], nh, x.rl);
-      fx_mad(xx[1], nl, x.rh);
-      fx_mad(h[2], x.rh, x.rh);
-      fx_mad(h[2], x.ih, x.ih);
-      fx_mad(xx[2], x.rh, x.rl);
-      fx_mad(xx[2], x.ih, x.il);
+      fx_mad(h[0], y.rh, u.rh);
+      fx_mad(h[0], y.ih, u.ih);
+      fx_mad(xx[0], y.rh, u.rl);
+      fx_mad(xx[0], y.rl, u.rh);
+      fx_mad(xx[0], y.ih, u.il);
+      fx_mad(xx[0], y.il, u.ih);
+      fx_mad(h[1], y.rh, u.ih);
+      fx_mad(h[1], nh, u.rh);
+      fx_mad(xx[1], y.rh, u.il);
+      fx_mad(xx[1], y.rl, u.ih);
+      fx_mad(xx[1], nh, u.rl);
+      fx_mad(xx[1], nl, u.rh);
+      fx_mad(h[2], u.rh, u.rh);
+      fx_mad(h[2], u.ih, u.ih);
+      fx_mad(xx[2], u.rh, u.rl);
+      fx_mad(xx[2], u.ih, u.il);
       fx_mad(h[3], y.rh, y.rh);
       fx_mad(h[3], y.ih, y.ih);
       fx_mad(xx[3], y.rh, y.rl);
@@ -566,7 +754,7 @@ __global__ void __launch_bounds__(128 * kFxGroups, 1)
     {  // warp v of the group sums value v over the chunk
       const int v = sp;
       const fx64 d = dots[grp][0][v][lane] + dots[grp][1][v][lane] + dots[grp][2][v][lane] + dots[grp][3][v][lane];
-      const int e = !live ? kFxNone : v < 2 ? en[0] + en[1] : 2 * en[v - 2];
+      const int e = !live ? kFxNone : v < 2 ? en[0] + en[1] : v == 2 ? 2 * en[0] : 2 * en[1];
       const int em = __reduce_max_sync(0xffffffffu, e);
       const fx64 t = warp_sum(live ? fx_align(d, em - e + 5) : 0);
       if (lane == 0) {
@@ -574,36 +762,8 @@ __global__ void __launch_bounds__(128 * kFxGroups, 1)
         parts.ue[(size_t)v * nchunk + ch] = em + 5;
       }
     }
-    group_sync(grp);  // dots and tops are free again
-  }
-}
-
-// ------------------------------------------------------------------ settle
-constexpr int kFxSettle = 512;
-
-__global__ void __launch_bounds__(kFxSettle) k_fx_settle(LzDev lz, int nchunk) {
-  asm volatile("griddepcontrol.launch_dependents;");  // the pair stencil that follows may start
-  const int rhs = blockIdx.y;
-  __shared__ int go, jsh;
-  if (threadIdx.x == 0) {
-    go = lz.pending[rhs] && !lz.status[rhs];
-    jsh = lz.j[rhs];
-  }
-  __syncthreads();
-  if (!go) return;
-  const int j = jsh;
-  const FxParts f = fx_parts(lz, rhs, nchunk);
-  FxSum sum[4];
-  fx_sum_chunks<4>(
-      nchunk, [&](int v, int c) { return f.u[(size_t)v * nchunk + c]; },
-      [&](int v, int c) { return f.ue[(size_t)v * nchunk + c]; }, sum);
-  if (threadIdx.x == 0) {
-    const double sums[4] = {sum[0].get(-58 - 2044), sum[1].get(-58 - 2044), sum[2].get(-58 - 2044),
-                            sum[3].get(-58 - 2044)};
-    const BetaVals b = lz_beta_vals(sums);
-    lz_beta_store(lz, rhs, (size_t)rhs * (lz.kmax + 2), j - 1, b);
-    if (!b.ok) lz.j[rhs] = j - 1;
-    lz.pending[rhs] = 0;
+    // (the next chunk's tops are written before its first barrier, which every warp reaches only after
+    // reading this chunk's dots; its dots are written after that barrier)
   }
 }
 
@@ -623,42 +783,64 @@ bool fx_step_usable(double m_w, double mu) {
   return c.ok && k >= 0x1p-10 && k <= 0x1p10;
 }
 
-cudaError_t launch_fx_begin(const Geom& g, const LzDev& lz, const FxVecs& fx, const void* vh, const void* w1,
-                            cudaStream_t st) {
+cudaError_t launch_fx_begin(const Geom& g, const Links& U, double m_w, const LzDev& lz, const FxVecs& fx, const void* vh,
+                            const void* w1, cudaStream_t st) {
   return launch_plain(k_fx_begin, dim3((g.vol + 63) / 64, lz.nrhs), dim3(64), st, g, lz, fx, (const double2*)vh,
-                      (const double2*)w1);
+                      (const double2*)w1, hop_coef<double>(m_w, 0.0).ks, U.fxf);
 }
 
-cudaError_t launch_fx_settle(const Geom& g, const LzDev& lz, cudaStream_t st) {
-  return launch_plain(k_fx_settle, dim3(1, lz.nrhs), dim3(kFxSettle), st, lz, (g.vol + 31) >> 5);
+cudaError_t launch_fx_settle(const Geom& g, const Links& U, double m_w, const LzDev& lz, const FxVecs& fx,
+                             cudaStream_t st) {
+  return launch_plain(k_fx_settle, dim3(1, lz.nrhs), dim3(kFxSettle), st, lz, fx, (g.vol + 31) >> 5,
+                      hop_coef<double>(m_w, 0.0).ks, U.fxf);
 }
 
-cudaError_t launch_fx_pair(const Geom& g, const Links& U, double m_w, double mu, const LzDev& lz, const FxVecs& fx,
-                           cudaStream_t st, int variant, cudaEvent_t mid, cudaEvent_t first) {
-  cudaError_t e;
-  if ((e = launch_fx_settle(g, lz, st))) return e;
-  if (first && (e = record_timing(first, st))) return e;
-  const FxCoef cp = fx_coef(m_w, mu), cm = fx_coef(m_w, -mu);
-  const bool split = variant == 1 || variant == 4 || variant == 5;
+// Early launch behind the previous kernel of the stream, with dynamic shared memory.
+template <typename... KArgs, typename... Args>
+static cudaError_t launch_early(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  {  // once per kernel and device and size
+    static std::mutex mu;
+    static std::map<std::pair<const void*, int>, size_t> allowed;
+    std::lock_guard<std::mutex> lk(mu);
+    size_t& a = allowed[{(const void*)kern, dev}];
+    if (a < smem) {
+      if ((e = cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))) return e;
+      a = smem;
+    }
+  }
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((g.vol + 31) / 32, lz.nrhs);
-  cfg.blockDim = dim3(32, split ? 8 : 2);
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
-  if (!first) {  // (a timing event between the two kernels orders them anyway)
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-  }
-  e = split ? cudaLaunchKernelEx(&cfg, k_fx_pair<4>, g, U, cp, cm, fx_self(cp.k.ks), lz, fx)
-            : cudaLaunchKernelEx(&cfg, k_fx_pair<1>, g, U, cp, cm, fx_self(cp.k.ks), lz, fx);
-  if (e == cudaSuccess && mid) e = record_timing(mid, st);
-  return e;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
-cudaError_t launch_fx_update(const Geom& g, const Links& U, double m_w, const LzDev& lz, const FxVecs& fx, void* vh,
-                             cudaStream_t st, cudaEvent_t mid) {
+cudaError_t launch_fx_pair(const Geom& g, const Links& U, double m_w, double mu, const LzDev& lz, const FxVecs& fx,
+                           cudaStream_t st, int variant) {
+  const FxCoef cp = fx_coef(m_w, mu), cm = fx_coef(m_w, -mu);
+  const bool split = variant == 1 || variant == 4 || variant == 5;
+  const dim3 grid((g.vol + 31) / 32 + 1, lz.nrhs);
+  const FxPairArgs args{{cp, cm},
+                        {{fx.v[0], fx.v[1]}, {fx.w[0], fx.w[1]}},
+                        {{fx.ev[0], fx.ev[1]}, {fx.ew[0], fx.ew[1]}},
+                        {fx.av, fx.aw},
+                        {fx.eav, fx.eaw}};
+  return split ? launch_early(k_fx_pair<4>, grid, dim3(32, 8), sizeof(FxPairSmem<4>), st, g, U, args, fx_self(cp.k.ks), lz,
+                              fx, cp.k.ks)
+               : launch_early(k_fx_pair<1>, grid, dim3(32, 2), sizeof(FxPairSmem<1>), st, g, U, args, fx_self(cp.k.ks), lz,
+                              fx, cp.k.ks);
+}
+
+cudaError_t launch_fx_update(const Geom& g, const LzDev& lz, const FxVecs& fx, void* vh, cudaStream_t st) {
   int dev = 0, nsm = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
@@ -666,14 +848,10 @@ cudaError_t launch_fx_update(const Geom& g, const Links& U, double m_w, const Lz
   const int nchunk = (g.vol + 31) >> 5;
   const int nb = std::min(nsm, nchunk);
   const int grp = std::min(kFxGroups, (nchunk + nb - 1) / nb);
-  const dim3 grid(nb, lz.nrhs), block(128 * grp);
-  const double ks = hop_coef<double>(m_w, 0.0).ks;
-  const bool store = fx.store != 0, xacc = lz.xacc != nullptr;
-  e = xacc    ? launch_plain(k_fx_update<false, true>, grid, block, st, g, ks, U.fxf, lz, fx, (double2*)vh)
-      : store ? launch_plain(k_fx_update<true, false>, grid, block, st, g, ks, U.fxf, lz, fx, (double2*)vh)
-              : launch_plain(k_fx_update<false, false>, grid, block, st, g, ks, U.fxf, lz, fx, (double2*)vh);
-  if (e == cudaSuccess && mid) e = record_timing(mid, st);
-  return e;
+  using Kern = void (*)(Geom, LzDev, FxVecs, double2*);
+  const Kern kern = lz.xacc ? k_fx_update<false, true> : fx.store ? k_fx_update<true, false> : k_fx_update<false, false>;
+  return launch_early(kern, dim3(nb, lz.nrhs), dim3(128 * grp), (size_t)128 * grp * kFxRows * 16, st, g, lz, fx,
+                      (double2*)vh);
 }
 
 }  // namespace ovl

@@ -38,7 +38,8 @@ constexpr int kMaxDevices = 128;
 // exponents per site and rhs): a layout that fits the 64 MiB holds at least seven FP64 vectors, so this
 // is at most 408 / 1344 of it.
 constexpr size_t kStaticFxBytes = (size_t)20 << 20;
-static_assert(kStaticFxBytes * 1344 >= kStaticScratchBytes * 408, "the fixed-point vectors of every layout that fits");
+static_assert((kStaticFxBytes - 64 * 256) * 1344 >= kStaticScratchBytes * 408,
+              "the fixed-point vectors of every layout that fits, and the step coefficients of 64 rhs at the end");
 
 __device__ __align__(256) unsigned char g_static_scratch[kStaticScratchBytes];
 __device__ __align__(256) unsigned char g_static_fx[kStaticFxBytes];
@@ -203,6 +204,7 @@ extern "C" ovl_status ovl_apply_sign_noalloc(ovl_lattice* lat, const ovl_sign_pa
   const bool fxs = f64 && lat->src()->fx_ok && fx_step_usable(p->m_W, p->mu);
   FxVecs fx;
   if (fxs) {
+    OVL_REQUIRE(fx_step_bytes() <= 256, "apply_sign_noalloc: step coefficients");
     const size_t nv = (size_t)nrhs * n * 16, ne = (size_t)nrhs * g.vol;
     fx.v[0] = (FxC*)fxbase;
     fx.v[1] = (FxC*)(fxbase + nv);
@@ -214,13 +216,14 @@ extern "C" ovl_status ovl_apply_sign_noalloc(ovl_lattice* lat, const ovl_sign_pa
     for (int q = 0; q < 2; ++q) fx.ev[q] = fe + q * ne, fx.ew[q] = fe + (2 + q) * ne;
     fx.eav = fe + 4 * ne;
     fx.eaw = fe + 5 * ne;
+    fx.step = fxbase + kStaticFxBytes - (size_t)64 * 256;
   }
   {
     LzVecs v = vec;
     if (fxs) v.wh = (char*)vec.aw - (size_t)nrhs * n * 16;  // what_1 (slot 1 of wh) goes to aw, in FP64
     OVL_CHECK_CUDA(launch_lanczos_start(g, f64, lz, v, (const double2*)b, m, lat->src()->defl.R, lat->src()->defl.L,
                                         lam_sign, dots, st));
-    if (fxs) OVL_CHECK_CUDA(launch_fx_begin(g, lz, fx, vec.vh, vec.aw, st));
+    if (fxs) OVL_CHECK_CUDA(launch_fx_begin(g, U, p->m_W, lz, fx, vec.vh, vec.aw, st));
   }
   const int chunk = std::max(1, std::min(p->check_every > 0 ? p->check_every : 20, kmax));
   const bool fixed = p->fixed_k > 0;
@@ -307,13 +310,13 @@ extern "C" ovl_status ovl_apply_sign_noalloc(ovl_lattice* lat, const ovl_sign_pa
     for (int i = 0; i < ns; ++i) {
       if (fxs) {
         OVL_CHECK_CUDA(launch_fx_pair(g, U, p->m_W, p->mu, lz, fx, st, pvar));
-        OVL_CHECK_CUDA(launch_fx_update(g, U, p->m_W, lz, fx, vec.vh, st));
+        OVL_CHECK_CUDA(launch_fx_update(g, lz, fx, vec.vh, st));
       } else {
         OVL_CHECK_CUDA(launch_lanczos_step(g, U, lf, f64, p->m_W, p->mu, lz, vec, st, pvar));
       }
     }
     // before the scalars are read
-    OVL_CHECK_CUDA(fxs ? launch_fx_settle(g, lz, st) : launch_lanczos_settle(g, f64, lz, st, pvar));
+    OVL_CHECK_CUDA(fxs ? launch_fx_settle(g, U, p->m_W, lz, fx, st) : launch_lanczos_settle(g, f64, lz, st, pvar));
     queued += ns;
     launches += fxs ? kFxStepLaunches * ns + 1
                     : lanczos_step_launches(g, lf, f64, pvar) * ns + lanczos_settle_launches(f64, pvar);

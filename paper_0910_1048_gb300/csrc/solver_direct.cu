@@ -154,7 +154,7 @@ static ovl_status ensure_ws(ovl_lattice* lat, int nrhs, int kmax, bool f64, int 
   size_t o_n1 = take((size_t)nrhs * kmax * 16), o_n2 = take((size_t)nrhs * kmax * 16);
   size_t o_nk = take((size_t)nrhs * 4), o_np = take((size_t)nrhs * 2 * vec_blocks(lat->g) * 8);
   size_t o_nc = take((size_t)nrhs * 4), o_no = take((size_t)nrhs * 2 * 8);
-  size_t o_fe = take(f64 ? kFxExponents * nrhs * vol * 4 : 0);
+  size_t o_fe = take(f64 ? kFxExponents * nrhs * vol * 4 : 0), o_fs = take(f64 ? nrhs * fx_step_bytes() : 0);
   size_t o_xa = take(two_pass ? (size_t)nrhs * n * 16 : 0), o_xc = take(two_pass ? (size_t)nrhs * ks * 16 : 0);
   // stream priority: 0 the default; p > 0 asks for p levels more urgent (numerically lower,
   // clamped to the device's range), so that concurrent solves can favour the longest one
@@ -227,6 +227,7 @@ static ovl_status ensure_ws(ovl_lattice* lat, int nrhs, int kmax, bool f64, int 
     for (int q = 0; q < 2; ++q) w->fx.ev[q] = fe + q * ne, w->fx.ew[q] = fe + (2 + q) * ne;
     w->fx.eav = fe + 4 * ne;
     w->fx.eaw = fe + 5 * ne;
+    w->fx.step = base + o_fs;
     w->fx.store = two_pass ? 0 : 1;
   }
   if (two_pass) {
@@ -442,18 +443,25 @@ ovl_status solve_direct(ovl_lattice* lat, const ovl_sign_params* p, int nrhs, co
     if (fxs) v.wh = (char*)vec.aw - (size_t)nrhs * n * 16;  // what_1 (slot 1 of wh) goes to aw, in FP64
     cudaError_t e = launch_lanczos_start(g, f64, lz, v, bd, m, lat->src()->defl.R, lat->src()->defl.L, w->lam_sign,
                                          w->dots, st);
-    return e != cudaSuccess || !fxs ? e : launch_fx_begin(g, lz, w->fx, vec.vh, vec.aw, st);
+    return e != cudaSuccess || !fxs ? e : launch_fx_begin(g, U, p->m_W, lz, w->fx, vec.vh, vec.aw, st);
   };
   auto pair = [&](const LzDev& lz, int var, cudaEvent_t mid, cudaEvent_t first) -> cudaError_t {
-    return fxs ? launch_fx_pair(g, U, p->m_W, p->mu, lz, w->fx, st, var, mid, first)
-               : launch_lanczos_pair(g, U, lf, f64, p->m_W, p->mu, lz, vec, st, var, mid, first);
+    if (fxs) {
+      cudaError_t e = first ? record_timing(first, st) : cudaSuccess;
+      if (e == cudaSuccess) e = launch_fx_pair(g, U, p->m_W, p->mu, lz, w->fx, st, var);
+      return e == cudaSuccess && mid ? record_timing(mid, st) : e;
+    }
+    return launch_lanczos_pair(g, U, lf, f64, p->m_W, p->mu, lz, vec, st, var, mid, first);
   };
   auto update = [&](const LzDev& lz, int var, cudaEvent_t mid) -> cudaError_t {
-    return fxs ? launch_fx_update(g, U, p->m_W, lz, w->fx, vec.vh, st, mid)
-               : launch_lanczos_update(g, f64, lz, vec, st, var, mid);
+    if (fxs) {
+      const cudaError_t e = launch_fx_update(g, lz, w->fx, vec.vh, st);
+      return e == cudaSuccess && mid ? record_timing(mid, st) : e;
+    }
+    return launch_lanczos_update(g, f64, lz, vec, st, var, mid);
   };
   auto settle = [&](const LzDev& lz, int var) -> cudaError_t {
-    return fxs ? launch_fx_settle(g, lz, st) : launch_lanczos_settle(g, f64, lz, st, var);
+    return fxs ? launch_fx_settle(g, U, p->m_W, lz, w->fx, st) : launch_lanczos_settle(g, f64, lz, st, var);
   };
   auto step_launches = [&](int var) { return fxs ? kFxStepLaunches : lanczos_step_launches(g, lf, f64, var); };
   auto settle_launches = [&](int var) { return fxs ? 1 : lanczos_settle_launches(f64, var); };
