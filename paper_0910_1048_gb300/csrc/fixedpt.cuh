@@ -10,17 +10,19 @@
 //  - Spinors: S is 2^(e+1) for e the exponent of the site's largest component (block floating point:
 //    one S for the 24 reals of a neighbour), |h| <= 2^29, 0 <= l < 2^30. A component is cut at
 //    2^-59 S; FP64 arithmetic on the same site rounds every partial sum at about 2^-54 S.
-//  - Links: S is one power of two for the field, at least its largest component and its largest row or
-//    column sum of moduli of components over sqrt(6) (1 for SU(3)), l balanced in [-2^29, 2^29), so
-//    that the dropped l l products have mean zero.
+//  - Links: (h 2^30 + l) 2^-58 S, S one power of two for the field, at least its largest component and its
+//    largest row or column sum of moduli of components over sqrt(6) (1 for SU(3)), l balanced in
+//    [-2^29, 2^29), so that the dropped l l products have mean zero.
 //  - Projected half spinors are limb-wise sums: |h| <= 2^30, l in (-2^30, 2^31).
-//  - Products: H = sum h_u h, X = sum (h_u l + l_u h) over a row's six components, |H| < 2^60.4 and
+//  - Products: H = sum h_u h, X = sum (h_u l + l_u h) over a row's six components, |H| < 2^59.4 and
 //    |X| < 2^62.5; the l_u l terms, below 2^-59 of full scale, are dropped.
-//  - A hop's 12 reals T = H + (X >> 30) are rounded once, to the common unit 2^-56 2^(E-1022) of
-//    the site's accumulators, E the largest exponent among its neighbours met so far (+1); eight
-//    hops stay below 2^61.4.
-// The error of a hop sum is about 2^-56 of the largest neighbouring component (the rounding of eight
-// hops and the dropped products), against about 2^-52 for the FP64 chains it replaces.
+//  - A hop's 12 reals T = H + (X >> 30) are in units of 2^-57 of the neighbour's scale. The site's
+//    accumulators are in units of 2^-57 2^(E-1022), E at least every hop's exponent; a hop whose
+//    exponent is smaller is shifted (rounded). Six hops and two with factors below 4 stay below 2^62.7.
+// The error of a hop sum is about 2^-55 of the neighbours' common scale (the cuts of eight hops and the
+// dropped products), against about 2^-52 of their largest component for the FP64 chains it replaces.
+// On GB300 a 32 x 32 + 64 bit multiply-add, a logic operation and a shift all take two issue cycles of a
+// scheduler (measured), so a hop is about 600 cycles a warp, 432 of them its 216 products.
 //
 // Integer sums do not depend on their order, so every shape of the stencil gives the same hop sums
 // up to that rounding. Sites next to an infinity, a NaN or only components below 2^-959 (E < 64), and
@@ -38,10 +40,11 @@ struct alignas(16) FxC {  // a complex link entry: limbs of its real and imagina
   int rh, rl, ih, il;
 };
 
-// Hop coefficients of the fixed-point stencil: the time hops' factors e^{+-mu} as 59-bit fractions of 2^e.
+// Hop coefficients of the fixed-point stencil: the time hops' factors e^{+-mu} as 2^-57 fractions (below 4) of
+// a power of two, 2^0 for |mu| < 1.38.
 struct FxCoef {
   HopCoef<double> k;
-  int fh, fl, fe;  // forward: (fh 2^30 + fl) 2^-59 2^fe
+  int fh, fl, fe;  // forward: (fh 2^30 + fl) 2^-57 2^fe
   int bh, bl, be;  // backward
   int unit;        // 1: both factors are 1 (mu = 0)
   int ok;          // 0: a factor is outside the fixed-point range (FP64 path)
@@ -53,14 +56,15 @@ inline FxCoef fx_coef(double m_w, double mu) {
   c.unit = mu == 0.0;
   c.ok = std::fabs(mu) <= 16.0;
   auto split = [&](double f, int& h, int& l, int& e) {
-    const double m = std::frexp(c.ok ? f : 1.0, &e);
-    const fx64 q = std::llrint(std::ldexp(m, 59));
+    int x;
+    const double m = std::frexp(c.ok ? f : 1.0, &x);
+    e = x > 2 ? x - 2 : 0;
+    const fx64 q = std::llrint(std::ldexp(m, 57 + x - e));
     h = (int)(q >> 30);
     l = (int)(q & ((1 << 30) - 1));
   };
   split(std::exp(mu), c.fh, c.fl, c.fe);
   split(std::exp(-mu), c.bh, c.bl, c.be);
-  if (c.unit) c.fe = c.be = 0;  // not applied
   return c;
 }
 
@@ -90,6 +94,16 @@ OVL_HD void fx_mad(fx64& acc, int a, int b) {
   asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(acc) : "r"(a), "r"(b));
 #else
   acc += (fx64)a * b;
+#endif
+}
+// a b + c (c kept)
+OVL_HD fx64 fx_mad_to(int a, int b, fx64 c) {
+#if defined(__CUDA_ARCH__)
+  fx64 r;
+  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+  return r;
+#else
+  return c + (fx64)a * b;
 #endif
 }
 OVL_HD fx64 fx_mul(int a, int b) {
@@ -136,7 +150,7 @@ struct FxHalf {  // projected half spinor: limbs of [2 spins][3 colours] complex
   int rh[2][3], rl[2][3], ih[2][3], il[2][3];
 };
 
-struct FxAcc {  // accumulators of a site: sums of hops in units of 2^-56 2^(E-1022), E their biased exponent
+struct FxAcc {  // accumulators of a site: sums of hops in units of 2^-57 2^(E-1022), E their biased exponent
   fx64 re[4][3], im[4][3];
 };
 
@@ -224,12 +238,12 @@ OVL_HD void fx_reconstruct(FxAcc& acc, const fx64 (&tr)[2][3], const fx64 (&ti)[
   }
 }
 
-// T (|T| < 2^60.4 in units of 2^-58) times the fraction (h 2^30 + l) 2^-59, in units of 2^-56.
+// T (|T| < 2^59.4) times the factor (h 2^30 + l) 2^-57.
 OVL_HD fx64 fx_scale(fx64 t, int h, int l) {
-  const fx64 t2 = (t + 2) >> 2;
-  const int th = (int)(t2 >> 30), tl = (int)((unsigned)t2 & 0x3fffffffu);
-  const fx64 x = (fx64)th * l + (fx64)tl * h;
-  return 2 * ((fx64)th * h) + (x >> 29);
+  const int th = (int)(t >> 30), tl = (int)((unsigned)t & 0x3fffffffu);
+  fx64 x = fx_mad_to(th, l, (fx64)1 << 26);
+  fx_mad(x, tl, h);
+  return (fx_mul(th, h) << 3) + (x >> 27);
 }
 
 // Half spinor of hop k = 2 mu (forward, U) or 2 mu + 1 (backward, U^H) from the neighbour's limbs.
@@ -261,35 +275,33 @@ OVL_HD void fx_half(int k, const FxSpin& q, bool g5in, FxHalf& h) {
 // Exponent of hop k's contribution for a neighbour of exponent e.
 OVL_HD int fx_hop_exponent(int k, int e, const FxCoef& c) { return k < 6 ? e : e + ((k & 1) ? c.be : c.fe); }
 
-// Adds hop k of the half spinor h to the accumulators, d = E - (the hop's exponent) >= 0; U points at the
-// link's entry [0][0], its entries `stride` apart. flip: the hop crosses an antiperiodic boundary.
-OVL_HD void fx_hop(int k, int d, const FxHalf& h, const FxC* U, size_t stride, const FxCoef& c, bool flip, FxAcc& acc) {
-  const bool fwd = !(k & 1), time = k >= 6;
-  const bool scaled = time && !c.unit;
-  const int sh = scaled ? (d < 60 ? d : 60) : (d < 58 ? d + 2 : 60);
-  const fx64 half = sh > 0 ? (fx64)1 << (sh - 1) : 0;  // rounds the shift
-  const fx64 seed = scaled ? 0 : half;
-  const size_t sa = fwd ? 3 * stride : stride, sb = fwd ? stride : 3 * stride;  // U[a][b] or U[b][a]
+// Adds hop k of the half spinor h to the accumulators, d = E - (the hop's exponent) >= 0, `shift` whether any
+// lane of the warp has d > 0. link(a, b): entry U[a][b], or U[b][a] for a backward hop. flip: the hop
+// crosses an antiperiodic boundary.
+template <class Link>
+OVL_HD void fx_hop(int k, int d, bool shift, const FxHalf& h, Link link, const FxCoef& c, bool flip, FxAcc& acc) {
+  const bool fwd = !(k & 1);
   fx64 tr[2][3], ti[2][3];
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     fx64 hr[2], hi[2], xr[2], xi[2];
 #pragma unroll
     for (int b = 0; b < 3; ++b) {
-      const FxC u = U[a * sa + b * sb];
+      const FxC u = link(a, b);
       const int nh = -u.ih, nl = -u.il;
 #pragma unroll
       for (int r = 0; r < 2; ++r) {
         if (b == 0) {
-          hr[r] = hi[r] = seed;
-          xr[r] = fx_mul(u.rh, h.rl[r][b]);
-          xi[r] = fx_mul(u.rh, h.il[r][b]);
+          hr[r] = fx_mul(u.rh, h.rh[r][b]);
+          hi[r] = fx_mul(u.rh, h.ih[r][b]);
+          xr[r] = fx_mad_to(u.rh, h.rl[r][b], (fx64)1 << 29);  // (rounds the shift of X)
+          xi[r] = fx_mad_to(u.rh, h.il[r][b], (fx64)1 << 29);
         } else {
+          fx_mad(hr[r], u.rh, h.rh[r][b]);
+          fx_mad(hi[r], u.rh, h.ih[r][b]);
           fx_mad(xr[r], u.rh, h.rl[r][b]);
           fx_mad(xi[r], u.rh, h.il[r][b]);
         }
-        fx_mad(hr[r], u.rh, h.rh[r][b]);
-        fx_mad(hi[r], u.rh, h.ih[r][b]);
         fx_mad(xr[r], u.rl, h.rh[r][b]);
         fx_mad(xi[r], u.rl, h.ih[r][b]);
         fx_mad(hr[r], nh, h.ih[r][b]);
@@ -306,25 +318,31 @@ OVL_HD void fx_hop(int k, int d, const FxHalf& h, const FxC* U, size_t stride, c
       ti[r][a] = hi[r] + (xi[r] >> 30);
     }
   }
-  if (time && flip) {
+  if (k >= 6) {
+    if (!c.unit) {
+      const int fh = fwd ? c.fh : c.bh, fl = fwd ? c.fl : c.bl;
 #pragma unroll
-    for (int i = 0; i < 6; ++i) {
-      tr[i / 3][i % 3] = -tr[i / 3][i % 3];
-      ti[i / 3][i % 3] = -ti[i / 3][i % 3];
+      for (int i = 0; i < 6; ++i) {
+        tr[i / 3][i % 3] = fx_scale(tr[i / 3][i % 3], fh, fl);
+        ti[i / 3][i % 3] = fx_scale(ti[i / 3][i % 3], fh, fl);
+      }
+    }
+    if (flip) {
+#pragma unroll
+      for (int i = 0; i < 6; ++i) {
+        tr[i / 3][i % 3] = -tr[i / 3][i % 3];
+        ti[i / 3][i % 3] = -ti[i / 3][i % 3];
+      }
     }
   }
-  if (scaled) {
-    const int fh = fwd ? c.fh : c.bh, fl = fwd ? c.fl : c.bl;
+  if (shift) {
+    const int n = d < 62 ? d : 62;
+    const fx64 half = n > 0 ? (fx64)1 << (n - 1) : 0;
 #pragma unroll
     for (int i = 0; i < 6; ++i) {
-      tr[i / 3][i % 3] = fx_scale(tr[i / 3][i % 3], fh, fl) + half;
-      ti[i / 3][i % 3] = fx_scale(ti[i / 3][i % 3], fh, fl) + half;
+      tr[i / 3][i % 3] = fx_sar(tr[i / 3][i % 3] + half, n);
+      ti[i / 3][i % 3] = fx_sar(ti[i / 3][i % 3] + half, n);
     }
-  }
-#pragma unroll
-  for (int i = 0; i < 6; ++i) {
-    tr[i / 3][i % 3] = fx_sar(tr[i / 3][i % 3], sh);
-    ti[i / 3][i % 3] = fx_sar(ti[i / 3][i % 3], sh);
   }
   switch (k) {
     case 0: fx_reconstruct<0, true>(acc, tr, ti); break;
@@ -380,7 +398,7 @@ OVL_HD bool fx_field_scale(double lo, double hi, int* uexp) {
 }
 
 OVL_HD FxC fx_link_entry(cplx<double> u, int uexp) {
-  const fx64 qr = std::llrint(std::ldexp(u.re, 59 - uexp)), qi = std::llrint(std::ldexp(u.im, 59 - uexp));
+  const fx64 qr = std::llrint(std::ldexp(u.re, 58 - uexp)), qi = std::llrint(std::ldexp(u.im, 58 - uexp));
   FxC r;
   r.rh = (int)((qr + (1 << 29)) >> 30);
   r.rl = (int)(qr - ((fx64)r.rh << 30));
@@ -411,9 +429,10 @@ OVL_HD int fx_neighbour(const Geom& g, int s, unsigned long long xyzt, int k, bo
   return (k & 1) ? s - step : s + step;
 }
 
-// Hops k0 .. k1-1 of site s, psi in FP64 loaded through `ld` and converted on the way. E: the largest
-// exponent met so far (+1). Returns whether the accumulators hold the hop sum: no infinity or NaN among
-// the neighbours, and not only components too small for the common exponent (all zero is fine).
+// Hops k0 .. k1-1 of site s, psi in FP64 loaded through `ld` and converted on the way, to limbs relative to the
+// largest exponent E met so far (+1), so that no hop is shifted afterwards. Returns whether the
+// accumulators hold the hop sum: no infinity or NaN among the neighbours, and not only components too
+// small for the common exponent (all zero is fine).
 template <class Load>
 OVL_HD bool fx_hops(const Geom& g, const FxC* U, int s, int k0, int k1, const FxCoef& c, Load ld, bool g5in, FxAcc& acc,
                     int& E) {
@@ -425,35 +444,34 @@ OVL_HD bool fx_hops(const Geom& g, const FxC* U, int s, int k0, int k1, const Fx
     bool wraps;
     const int nb = fx_neighbour(g, s, xyzt, k, &wraps);
     FxHalf h;
-    int e;
     {
       Spin<double> p;
       ld(nb, p);
       const int eb = fx_exponent(p);
       emax = emax > eb ? emax : eb;
-      e = eb > 64 ? eb : 64;
+      const int fe = fx_hop_exponent(k, 0, c), eh = (eb > 64 ? eb : 64) + fe;
+      if (eh > E) {  // first hop, or a larger neighbour than any before
+        if (E != 0) {
+#pragma unroll
+          for (int i = 0; i < 12; ++i) {
+  acc.re[i / 3][i % 3] = fx_sar(acc.re[i / 3][i % 3], eh + 1 - E);
+            acc.im[i / 3][i % 3] = fx_sar(acc.im[i / 3][i % 3], eh + 1 - E);
+          }
+        }
+        E = eh + 1;
+      }
       FxSpin q;
-      fx_spin(p, e, q);
+      fx_spin(p, E - fe, q);
       fx_half(k, q, g5in, h);
     }
-    const int eh = fx_hop_exponent(k, e, c);
-    if (eh > E) {  // first hop, or a larger neighbour than any before
-      if (E != 0) {
-#pragma unroll
-        for (int i = 0; i < 12; ++i) {
-          acc.re[i / 3][i % 3] = fx_sar(acc.re[i / 3][i % 3], eh + 1 - E);
-          acc.im[i / 3][i % 3] = fx_sar(acc.im[i / 3][i % 3], eh + 1 - E);
-        }
-      }
-      E = eh + 1;
-    }
-    fx_hop(k, E - eh, h, U + (size_t)(k >> 1) * 9 * g.vol + ((k & 1) ? nb : s), (size_t)g.vol, c, wraps && g.t_bc < 0,
-           acc);
+    const FxC* u = U + (size_t)(k >> 1) * 9 * g.vol + ((k & 1) ? nb : s);
+    const size_t sa = (k & 1) ? (size_t)g.vol : (size_t)3 * g.vol, sb = (k & 1) ? (size_t)3 * g.vol : (size_t)g.vol;
+    fx_hop(k, 0, false, h, [&](int a, int b) { return u[a * sa + b * sb]; }, c, wraps && g.t_bc < 0, acc);
   }
   return emax < 0x7ff && E < 2000 && (emax == 0 || emax >= 64);
 }
 
 // FP64 value of one unit of the accumulators times the hop coefficient ks and the links' scale.
-OVL_HD double fx_unit(int E, const FxCoef& c, int uexp) { return c.k.ks * fx_pow2(E - 55 + uexp); }
+OVL_HD double fx_unit(int E, const FxCoef& c, int uexp) { return c.k.ks * fx_pow2(E - 56 + uexp); }
 
 }  // namespace ovl

@@ -55,31 +55,6 @@ __device__ __forceinline__ int fx_top(int m, fx64 v) {
 }
 // Shift that takes values whose largest high word is m to at most 2^59: right if positive, left if not.
 __device__ __forceinline__ int fx_norm_shift(int m) { return 5 - __clz(m); }  // (32 - clz) + 32 - 59
-__device__ __forceinline__ fx64 fx_normalise(fx64 v, int r) { return r > 0 ? fx_sar_round(v, r) : v << -r; }
-
-// Product of two complex numbers in limbs, T = H + (X >> 30), in units of 2^-58 of their scales' product.
-// CONJ: conj(a) b.
-template <bool CONJ>
-__device__ __forceinline__ void fx_cmul(const FxC& a, const FxC& b, fx64& re, fx64& im) {
-  const int ih = CONJ ? -a.ih : a.ih, il = CONJ ? -a.il : a.il, nh = -ih, nl = -il;
-  fx64 hr = fx_mul(a.rh, b.rh), hi = fx_mul(a.rh, b.ih), xr = fx_mul(a.rh, b.rl), xi = fx_mul(a.rh, b.il);
-  fx_mad(hr, nh, b.ih);
-  fx_mad(hi, ih, b.rh);
-  fx_mad(xr, a.rl, b.rh);
-  fx_mad(xi, a.rl, b.ih);
-  fx_mad(xr, nh, b.il);
-  fx_mad(xi, ih, b.rl);
-  fx_mad(xr, nl, b.ih);
-  fx_mad(xi, il, b.rh);
-  re = hr + (xr >> 30);
-  im = hi + (xi >> 30);
-}
-__device__ __forceinline__ fx64 fx_rmul(int ah, int al, int bh, int bl) {
-  fx64 x = fx_mul(ah, bl);
-  fx_mad(x, al, bh);
-  return fx_mul(ah, bh) + (x >> 30);
-}
-
 // ------------------------------------------------------------------ chunk sums
 // A chunk is 32 consecutive sites (a warp). Its sum: the sites' values aligned to the chunk's largest
 // exponent with five bits of headroom, each rounded once; stored as an integer and that exponent.
@@ -171,6 +146,8 @@ __device__ __forceinline__ FxCoefSh fx_coefficient(zd r) {
 struct FxStep {
   FxCoefSh c[4];    // c0, c2, c0w, c2w
   double2 k[3];     // kv, kw, k1
+  // largest site exponent of column j of vhat and what, slot j & 1 (see k_fx_update)
+  int emax[2][2];
 };
 size_t fx_step_bytes() { return (sizeof(FxStep) + 255) & ~(size_t)255; }
 
@@ -229,6 +206,8 @@ __device__ __forceinline__ void fx_settle(const LzDev& lz, const FxVecs& fx, int
     lz_beta_store(lz, rhs, o, j - 1, b);
     if (!b.ok) lz.j[rhs] = j - 1;
     lz.pending[rhs] = 0;
+    fx_step(fx, rhs)->emax[0][(j + 1) & 1] = kFxNone;  // column j - 1's, replaced by the next update
+    fx_step(fx, rhs)->emax[1][(j + 1) & 1] = kFxNone;
   }
 }
 
@@ -244,6 +223,7 @@ __global__ void __launch_bounds__(64) k_fx_begin(Geom g, LzDev lz, FxVecs fx, co
                                                  double ks, const FxField* fxf) {
   const int rhs = blockIdx.y, s = blockIdx.x * blockDim.x + threadIdx.x;
   if (blockIdx.x == 0 && threadIdx.x < 32) {
+    if (threadIdx.x < 4) fx_step(fx, rhs)->emax[threadIdx.x >> 1][threadIdx.x & 1] = kFxNone;
     const size_t o = (size_t)rhs * (lz.kmax + 2) + 1;
     fx_step_store(fx_step(fx, rhs), fx_scalb(ks, fxf->uexp), lz.sv[o], ldc<double>(lz.sw, o), 0.0, mk(0.0, 0.0), 0.0,
                   mk(0.0, 0.0));
@@ -327,8 +307,8 @@ __global__ void __launch_bounds__(64 * T, T == 1 ? 5 : 1)
     const FxC* u = U.fx + (size_t)(k >> 1) * 9 * g.vol + ((k & 1) ? nb : s);
 #pragma unroll
     for (int i = 0; i < 5; ++i) {
-      const int row = role * 5 + i;
-      if (row < 9) copy_async(&sm.u[k & 1][t][row][lane], u + (size_t)row * g.vol);
+      const int row = role * 5 + i;  // of a backward hop's link, transposed
+      if (row < 9) copy_async(&sm.u[k & 1][t][row][lane], u + (size_t)((k & 1) ? (row % 3) * 3 + row / 3 : row) * g.vol);
     }
   };
   bool wraps;
@@ -348,8 +328,8 @@ __global__ void __launch_bounds__(64 * T, T == 1 ? 5 : 1)
   fx_clear(acc);
   const int se = self.e - U.fxf->uexp;  // exponent of the diagonal's coefficient
   const int es = ex[s], ew = args.e[1][j & 1][(size_t)rhs * g.vol + s];
-  // the diagonal's scale is at most 2^5 of the hops': |A| < 2^61.8 units
-  int E = es + se - 3;
+  // the diagonal's scale is at most 2^2 of the hops': |A| < 2^62.8 units
+  int E = es + se - 2;
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
     bool w;
@@ -388,18 +368,20 @@ __global__ void __launch_bounds__(64 * T, T == 1 ? 5 : 1)
       }
       fx_half(k, p, false, h);
     }
-    fx_hop(k, E - eh, h, &sm.u[k & 1][t][0][lane], 32, c, flip, acc);
+    const FxC* u = &sm.u[k & 1][t][0][lane];
+    fx_hop(k, E - eh, __any_sync(0xffffffffu, E != eh), h, [&](int a, int b) { return u[(a * 3 + b) * 32]; }, c, flip,
+           acc);
   }
   copy_wait();
   // the diagonal psi / ks, and gamma5: A of spin sp
-  const int sh = E - es - se + 3;  // from units of 2^-59 2^(es + se - 1022)
+  const int sh = E - es - se + 2;  // from units of 2^-59 2^(es + se - 1022)
   const int shc = min(sh, 61);
   const fx64 half = shc > 0 ? (fx64)1 << (shc - 1) : 0;
   auto finish = [&](int sp, int row, fx64 (&ar)[3], fx64 (&ai)[3]) {
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
       const FxC x = sm.q[0][row + a][tid];
-      fx64 xr = fx_mul(x.rh, self.l), xi = fx_mul(x.ih, self.l);
+      fx64 xr = fx_mad_to(x.rh, self.l, (fx64)1 << 28), xi = fx_mad_to(x.ih, self.l, (fx64)1 << 28);
       fx_mad(xr, x.rl, self.h);
       fx_mad(xi, x.il, self.h);
       ar[a] += fx_sar(2 * fx_mul(x.rh, self.h) + (xr >> 29) + half, shc);
@@ -450,7 +432,7 @@ __global__ void __launch_bounds__(64 * T, T == 1 ? 5 : 1)
       for (int a = 0; a < 3; ++a) m = fx_top(fx_top(m, acc.re[sp][a]), acc.im[sp][a]);
     }
     const int r = fx_norm_shift(m);
-    ea = E + r + 3;
+    ea = E + r + 2;
 #pragma unroll
     for (int sp = 0; sp < 4; ++sp) {
       fx64 x, y;
@@ -491,7 +473,7 @@ __global__ void __launch_bounds__(64 * T, T == 1 ? 5 : 1)
 #pragma unroll
     for (int p = 0; p < T; ++p) m = max(m, sm.top[role][p][lane]);
     const int r = fx_norm_shift(m);
-    ea = E + r + 3;
+    ea = E + r + 2;
     fx64 x, y;
     emit(t, r, ar, ai, x, y);
     if (role == 0) {
@@ -533,12 +515,12 @@ constexpr int kFxRows = 18;   // 16-byte inputs per thread: three colours of A, 
 
 __device__ __forceinline__ void group_sync(int grp) { asm volatile("bar.sync %0, 128;" ::"r"(grp + 1) : "memory"); }
 
-// (a b) >> d, rounded, for complex limbs; d in [0, 61].
-__device__ __forceinline__ void fx_cmul_shift(const FxC& a, const FxC& b, int d, fx64 half, fx64& re, fx64& im) {
-  const int nh = -a.ih, nl = -a.il;
-  fx64 hr = half, hi = half, xr = fx_mul(a.rh, b.rl), xi = fx_mul(a.rh, b.il);
+// H and X of a b (complex limbs) added to hr, hi, xr, xi.
+__device__ __forceinline__ void fx_cmad(const FxC& a, int nh, int nl, const FxC& b, fx64& hr, fx64& hi, fx64& xr, fx64& xi) {
   fx_mad(hr, a.rh, b.rh);
   fx_mad(hi, a.rh, b.ih);
+  fx_mad(xr, a.rh, b.rl);
+  fx_mad(xi, a.rh, b.il);
   fx_mad(xr, a.rl, b.rh);
   fx_mad(xi, a.rl, b.ih);
   fx_mad(hr, nh, b.ih);
@@ -547,8 +529,15 @@ __device__ __forceinline__ void fx_cmul_shift(const FxC& a, const FxC& b, int d,
   fx_mad(xi, a.ih, b.rl);
   fx_mad(xr, nl, b.ih);
   fx_mad(xi, a.il, b.rh);
-  re = fx_sar(hr + (xr >> 30), d);
-  im = fx_sar(hi + (xi >> 30), d);
+}
+// A coefficient's limbs moved down by d bits (to another exponent).
+__device__ __forceinline__ FxC fx_lower(const FxC& c, int d) {
+  const int n = min(d, 62);
+  const fx64 half = n > 0 ? (fx64)1 << (n - 1) : 0;
+  FxC r;
+  fx_split(fx_sar(((fx64)c.rh << 30) + c.rl + half, n), r.rh, r.rl);
+  fx_split(fx_sar(((fx64)c.ih << 30) + c.il + half, n), r.ih, r.il);
+  return r;
 }
 
 template <bool STORE, bool XACC>
@@ -589,27 +578,29 @@ __global__ void __launch_bounds__(128 * kFxGroups, 1)
   }
   grid_wait();
   grid_launch();
-  if (lz.status[rhs]) {
-    copy_wait();
-    return;
-  }
-  if (any) {
-    fetch(c0 + grp, true);
-    fetch_e(es0, true);
-  }
+  const int status = lz.status[rhs];
   const FxParts parts = fx_parts(lz, rhs, nchunk);
+  const FxStep* st = fx_step(fx, rhs);
+  const int er0 = st->emax[0][j & 1], er1 = st->emax[1][j & 1];
   {
-    const FxStep* st = fx_step(fx, rhs);
     const int nshare = min(4, nt >> 6);
     zd k = mk(0.0, 0.0);
     if (warp == 0 && lane < 3) k = mk(st->k[lane].x, st->k[lane].y);
     if (warp == 1 && lane < 4) cs[lane < 2 ? 2 * lane : 2 * lane - 1] = st->c[lane];
+    if (any) {
+      fetch(c0 + grp, true);
+      fetch_e(es0, true);
+    }
     if (warp < 2 * nshare) {  // the sum of what^H A v: warp (value, share)
       const int v = warp & 1, q = warp >> 1;
       const double x = fx_warp_sum_chunks(
           nchunk, q, nshare, [&](int c) { return v ? parts.a[c].y : parts.a[c].x; }, [&](int c) { return parts.ae[c]; },
           -58 - 2044);
       if (lane == 0) ash[v][q] = x;
+    }
+    if (status) {  // (uniform)
+      copy_wait();
+      return;
     }
     __syncthreads();
     if (warp == 0) {
@@ -631,6 +622,7 @@ __global__ void __launch_bounds__(128 * kFxGroups, 1)
     __syncthreads();
   }
   const zd xc = XACC ? ldc<double>(lz.xcoef, o + j + 1) : mk(0.0, 0.0);
+  const int eref[2] = {er0, er1};
 #pragma unroll 1
   for (int ch = c0 + grp; ch < c1; ch += ngrp) {
     const bool live = ch * 32 + lane < g.vol;
@@ -645,51 +637,60 @@ __global__ void __launch_bounds__(128 * kFxGroups, 1)
       const FxCoefSh& k1 = cs[3 * role + 1];
       const FxCoefSh& k2 = cs[3 * role + 2];
       const bool prev = k2.e != kFxNone;
-      // biased exponents of the three products
+      // biased exponents of the three products; the coefficients are moved to the largest, so that the
+      // products add up without shifts
       const int e0 = ex[3 * role] + k0.e - 1022, e1 = ex[3 * role + 1] + k1.e - 1022;
       const int e2 = prev ? ex[3 * role + 2] + k2.e - 1022 : kFxNone;
       const int E = max(max(e0, e1), e2);
-      const int d0 = min(E - e0, 61), d1 = min(E - e1, 61), d2 = min(E - e2, 61);
-      const fx64 h0 = d0 > 0 ? (fx64)1 << (d0 - 1) : 0, h1 = d1 > 0 ? (fx64)1 << (d1 - 1) : 0,
-                 h2 = d2 > 0 ? (fx64)1 << (d2 - 1) : 0;
+      const FxC q0 = fx_lower(k0.c, E - e0), q1 = fx_lower(k1.c, E - e1), q2 = fx_lower(k2.c, E - e2);
       if (role == 0) copy_wait();
       int m = 0;
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
         const FxC va = rows[(role * 9 + a) * nt + tid], vv = rows[(role * 9 + 3 + a) * nt + tid];
-        fx64 xr, xi, r, i;
-        if (role == 0) {  // a real coefficient
-          xr = fx_sar(fx_rmul(k0.c.rh, k0.c.rl, va.rh, va.rl) + h0, d0);
-          xi = fx_sar(fx_rmul(k0.c.rh, k0.c.rl, va.ih, va.il) + h0, d0);
-        } else {
-          fx_cmul_shift(k0.c, va, d0, h0, xr, xi);
+        fx64 hr = fx_mul(q0.rh, va.rh), hi = fx_mul(q0.rh, va.ih), xr = fx_mad_to(q0.rh, va.rl, (fx64)1 << 29),
+             xi = fx_mad_to(q0.rh, va.il, (fx64)1 << 29);
+        fx_mad(xr, q0.rl, va.rh);
+        fx_mad(xi, q0.rl, va.ih);
+        if (role == 1) {  // (vhat's coefficient of A v is real)
+          fx_mad(hr, -q0.ih, va.ih);
+          fx_mad(hi, q0.ih, va.rh);
+          fx_mad(xr, -q0.ih, va.il);
+          fx_mad(xi, q0.ih, va.rl);
+          fx_mad(xr, -q0.il, va.ih);
+          fx_mad(xi, q0.il, va.rh);
         }
-        fx_cmul_shift(k1.c, vv, d1, h1, r, i);
-        xr += r;
-        xi += i;
-        if (prev) {
-          fx_cmul_shift(k2.c, rows[(role * 9 + 6 + a) * nt + tid], d2, h2, r, i);
-          xr += r;
-          xi += i;
-        }
-        x[role][a][0] = xr;
-        x[role][a][1] = xi;
-        m = fx_top(fx_top(m, xr), xi);
+        fx_cmad(q1, -q1.ih, -q1.il, vv, hr, hi, xr, xi);
+        if (prev) fx_cmad(q2, -q2.ih, -q2.il, rows[(role * 9 + 6 + a) * nt + tid], hr, hi, xr, xi);
+        hr += xr >> 30;
+        hi += xi >> 30;
+        x[role][a][0] = hr;
+        x[role][a][1] = hi;
+        m = fx_top(fx_top(m, hr), hi);
       }
       tops[grp][role][sp][lane] = m;
       en[role] = E;
     }
     group_sync(grp);
     FxC nv[2][3];  // new limbs of vhat and what
+    int em[2];     // largest exponent of the chunk's sites
 #pragma unroll
     for (int role = 0; role < 2; ++role) {
       const int m = max(max(tops[grp][role][0][lane], tops[grp][role][1][lane]),
                         max(tops[grp][role][2][lane], tops[grp][role][3][lane]));
-      const int r = fx_norm_shift(m), rr = max(r, 0), rl = max(-r, 0);
-      const fx64 half = rr > 0 ? (fx64)1 << (rr - 1) : 0;
+      int r = fx_norm_shift(m);
+      const int e = en[role] + r + 1;
+      em[role] = __reduce_max_sync(0xffffffffu, live ? e : kFxNone);
+      // sites within three bits of the largest exponent of the previous column take that one: nearly all
+      // sites of a vector then share it, and the next pair stencil's hops need no shift
+      const int up = eref[role] - e;
+      if (up > 0 && up <= 3) r += up;
       en[role] += r + 1;
+      const int rr = max(r, 0), rl = max(-r, 0);
+      const fx64 half = rr > 0 ? (fx64)1 << (rr - 1) : 0;
       FxC* P = (role ? fx.w : fx.v)[(j + 1) & 1] + base;  // in place of column j-1
       const int k = en[role] - 1022 - 59;
+      const bool normal = k > -1000 && k < 900;
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
         const fx64 qr = ((x[role][a][0] + half) >> rr) << rl, qi = ((x[role][a][1] + half) >> rr) << rl;
@@ -700,7 +701,13 @@ __global__ void __launch_bounds__(128 * kFxGroups, 1)
         if (live) {
           P[(size_t)a * g.vol] = y;
           if (role == 0 && (STORE || XACC)) {
-            const zd d = mk(fx_scalb((double)qr, k), fx_scalb((double)qi, k));
+            zd d = mk((double)qr, (double)qi);
+            if (normal) {  // q is 0 or between 1 and 2^59: the exponent field moves
+              d.re = __hiloint2double(__double2hiint(d.re) + (qr ? k * (1 << 20) : 0), __double2loint(d.re));
+              d.im = __hiloint2double(__double2hiint(d.im) + (qi ? k * (1 << 20) : 0), __double2loint(d.im));
+            } else {
+              d = mk(fx_scalb(d.re, k), fx_scalb(d.im, k));
+            }
             const size_t at = (size_t)(sp * 3 + a) * g.vol + s;
             if (STORE) stc<double>(vh, ((size_t)rhs * lz.vcols + j) * n + at, d);  // column j + 1
             if (XACC) {
@@ -712,6 +719,7 @@ __global__ void __launch_bounds__(128 * kFxGroups, 1)
       }
       if (live && sp == 0) (role ? fx.ew : fx.ev)[(j + 1) & 1][es] = en[role];
     }
+    if (lane == 0 && sp < 2) atomicMax(&fx_step(fx, rhs)->emax[sp][(j + 1) & 1], sp ? em[1] : em[0]);
     if (ch + ngrp < c1) {  // (this thread has read its rows)
       const size_t nx = (size_t)rhs * g.vol + min((ch + ngrp) * 32 + lane, g.vol - 1);
       fetch(ch + ngrp, false);
