@@ -397,49 +397,77 @@ bool choose_scale(const std::vector<cz>& lam, double eps, int s_max, double* c_o
   return true;
 }
 
-// |re| + |im|: the pivoting magnitude of the tridiagonal solves (no square root).
-inline double abs1(cz z) { return std::fabs(z.real()) + std::fabs(z.imag()); }
-inline cz cinv(cz z) { return std::conj(z) * (1.0 / std::norm(z)); }
+// kLanes complex numbers side by side: one tridiagonal solve is a chain of dependent reciprocals (tens of
+// cycles per row), so two shifts are solved in lockstep in one vector register, the pivot choice a select per
+// lane. On 16 Grace cores thirteen evaluations from k = 25 to 1300 (296 poles) take 12.8 ms against 28.3
+// with one shift at a time and a thread per 40000 rows; four or eight lanes took 17 to 19.
+constexpr int kLanes = 2;
+typedef double LaneVec __attribute__((vector_size(kLanes * sizeof(double))));  // (split to the host's vector width)
+struct Lanes {
+  LaneVec re, im;
+};
+inline Lanes lanes_mul(const Lanes& a, const Lanes& b) {
+  return Lanes{a.re * b.re - a.im * b.im, a.re * b.im + a.im * b.re};
+}
+inline Lanes lanes_fnma(const Lanes& c, const Lanes& a, const Lanes& b) {  // c - a b
+  const Lanes p = lanes_mul(a, b);
+  return Lanes{c.re - p.re, c.im - p.im};
+}
+inline LaneVec lanes_abs(LaneVec x) { return x < 0.0 ? -x : x; }
 
-// Solve (c H + z) x = b in place (b -> x) for tridiagonal H (diag al, super be, sub de) by
-// Gaussian elimination with partial pivoting (one row interchange at most per step; the
-// interchange fills a second superdiagonal). d, du, dl, du2 are scratch of length k.
-// Returns false if a pivot is zero.
-inline bool tri_solve(int k, const cz* al, const cz* be, const cz* de, double c, cz z, cz* b, cz* d, cz* du, cz* dl,
-                      cz* du2) {
+// Solve (c H + i t_w) x_w = b_w in place (b -> x) for tridiagonal H (diag al, super be, sub de) and kLanes
+// shifts by Gaussian elimination with partial pivoting by |re| + |im| (one row interchange at most per
+// step; the interchange fills a second superdiagonal). inv, du, du2 are scratch of length k. Returns false
+// if a pivot is zero.
+bool tri_solve(int k, const cz* al, const cz* be, const cz* de, double c, LaneVec t, Lanes* b, Lanes* inv, Lanes* du,
+               Lanes* du2) {
+  const LaneVec zero = t - t;
+  // first two entries of the row being eliminated with
+  Lanes d{zero + c * al[0].real(), t + c * al[0].imag()};
+  Lanes u{zero + (k > 1 ? c * be[0].real() : 0.0), zero + (k > 1 ? c * be[0].imag() : 0.0)};
+  Lanes bi = b[0];
+  bool bad = false;
   for (int i = 0; i < k; ++i) {
-    d[i] = c * al[i] + z;
-    if (i + 1 < k) {
-      du[i] = c * be[i];
-      dl[i] = c * de[i];
+    if (i + 1 == k) {
+      const LaneVec n2 = d.re * d.re + d.im * d.im, r = 1.0 / n2;
+      for (int w = 0; w < kLanes; ++w) bad = bad || n2[w] == 0.0;
+      inv[i] = Lanes{d.re * r, -d.im * r};
+      du[i] = du2[i] = Lanes{zero, zero};
+      b[i] = bi;
+      break;
     }
-    du2[i] = 0.0;
+    const LaneVec lr = zero + c * de[i].real(), li = zero + c * de[i].imag();  // the next row
+    const LaneVec nr = zero + c * al[i + 1].real(), ni = t + c * al[i + 1].imag();
+    const double mr = i + 2 < k ? c * be[i + 1].real() : 0.0, mi = i + 2 < k ? c * be[i + 1].imag() : 0.0;
+    const auto sw = lanes_abs(d.re) + lanes_abs(d.im) < lanes_abs(lr) + lanes_abs(li);
+    const Lanes bn = b[i + 1];
+    const LaneVec vr = zero + mr, vi = zero + mi;
+    // the pivot row (p) and the other one (q)
+    const Lanes pf{sw ? lr : d.re, sw ? li : d.im}, qf{sw ? d.re : lr, sw ? d.im : li};
+    const Lanes ps{sw ? nr : u.re, sw ? ni : u.im}, qs{sw ? u.re : nr, sw ? u.im : ni};
+    const Lanes pt{sw ? vr : zero, sw ? vi : zero}, qt{sw ? zero : vr, sw ? zero : vi};
+    const Lanes pb{sw ? bn.re : bi.re, sw ? bn.im : bi.im}, qb{sw ? bi.re : bn.re, sw ? bi.im : bn.im};
+    const LaneVec n2 = pf.re * pf.re + pf.im * pf.im, r = 1.0 / n2;
+    for (int w = 0; w < kLanes; ++w) bad = bad || n2[w] == 0.0;
+    const Lanes iv{pf.re * r, -pf.im * r};
+    inv[i] = iv;
+    du[i] = ps;
+    du2[i] = pt;
+    b[i] = pb;
+    const Lanes f = lanes_mul(qf, iv);
+    d = lanes_fnma(qs, f, ps);
+    u = lanes_fnma(qt, f, pt);
+    bi = lanes_fnma(qb, f, pb);
   }
-  for (int i = 0; i + 1 < k; ++i) {
-    if (abs1(d[i]) >= abs1(dl[i])) {
-      if (d[i] == cz(0.0)) return false;
-      const cz f = dl[i] * cinv(d[i]);
-      d[i + 1] -= f * du[i];
-      b[i + 1] -= f * b[i];
-    } else {  // interchange rows i and i+1
-      const cz f = d[i] * cinv(dl[i]);
-      d[i] = dl[i];
-      const cz t = d[i + 1];
-      d[i + 1] = du[i] - f * t;
-      if (i + 2 < k) {
-        du2[i] = du[i + 1];
-        du[i + 1] = -f * du2[i];
-      }
-      du[i] = t;
-      const cz bi = b[i];
-      b[i] = b[i + 1];
-      b[i + 1] = bi - f * b[i + 1];
-    }
+  if (bad) return false;
+  Lanes x1 = lanes_mul(b[k - 1], inv[k - 1]), x2{zero, zero};  // x_{i+1}, x_{i+2}
+  b[k - 1] = x1;
+  for (int i = k - 2; i >= 0; --i) {
+    const Lanes x = lanes_mul(lanes_fnma(lanes_fnma(b[i], du[i], x1), du2[i], x2), inv[i]);
+    b[i] = x;
+    x2 = x1;
+    x1 = x;
   }
-  if (d[k - 1] == cz(0.0)) return false;
-  b[k - 1] *= cinv(d[k - 1]);
-  if (k > 1) b[k - 2] = (b[k - 2] - du[k - 2] * b[k - 1]) * cinv(d[k - 2]);
-  for (int i = k - 3; i >= 0; --i) b[i] = (b[i] - du[i] * b[i + 1] - du2[i] * b[i + 2]) * cinv(d[i]);
   return true;
 }
 
@@ -452,23 +480,35 @@ bool rational_apply(int k, const cz* al, const cz* be, const cz* de, double c, i
   // the s shifted solves are independent: split them over host threads, each summing its
   // own shifts in order, then add the per-thread sums in thread order (deterministic)
   const int hw = std::max(1, (int)std::thread::hardware_concurrency() / std::max(1, g_sign_concurrency));
-  const int nth = std::max(1, std::min({hw, 16, s, (int)((size_t)s * k / 40000 + 1)}));
+  // (a thread takes whole groups of kLanes shifts; from about 5000 rows each it pays to start one)
+  const int ngroup = (s + kLanes - 1) / kLanes;
+  const int nth = std::max(1, std::min({hw, 16, ngroup, (int)((size_t)s * k / 5000 + 1)}));
   std::vector<std::vector<cz>> part(nth, std::vector<cz>(k, 0.0));
   std::vector<char> ok(nth, 1);
   auto work = [&](int tid) {
     std::vector<cz>& acc = part[tid];
-    std::vector<cz> x(k), d(k), du(k), dl(k), du2(k);
-    for (int sh = 1 + tid; sh <= s; sh += nth) {
-      const double th = 3.14159265358979323846 / (2.0 * s) * (sh - 0.5);
-      const double om = 1.0 / (s * std::cos(th) * std::cos(th));
-      const double t = std::tan(th);  // sigma = -t^2
-      std::copy(v, v + k, x.begin());
-      if (!tri_solve(k, al, be, de, c, cz(0.0, -t), x.data(), d.data(), du.data(), dl.data(), du2.data()) ||
-          !tri_solve(k, al, be, de, c, cz(0.0, t), x.data(), d.data(), du.data(), dl.data(), du2.data())) {
+    std::vector<Lanes> x(k), inv(k), du(k), du2(k);
+    for (int gr = tid; gr < ngroup; gr += nth) {
+      LaneVec om, tp;
+      for (int w = 0; w < kLanes; ++w) {
+        const int sh = std::min(s, gr * kLanes + w + 1);  // (lanes past the last shift repeat it, weight 0)
+        const double th = 3.14159265358979323846 / (2.0 * s) * (sh - 0.5);
+        om[w] = gr * kLanes + w < s ? 1.0 / (s * std::cos(th) * std::cos(th)) : 0.0;
+        tp[w] = std::tan(th);  // sigma = -t^2
+      }
+      const LaneVec zero = tp - tp;
+      for (int i = 0; i < k; ++i) x[i] = Lanes{zero + v[i].real(), zero + v[i].imag()};
+      if (!tri_solve(k, al, be, de, c, -tp, x.data(), inv.data(), du.data(), du2.data()) ||
+          !tri_solve(k, al, be, de, c, tp, x.data(), inv.data(), du.data(), du2.data())) {
         ok[tid] = 0;
         return;
       }
-      for (int i = 0; i < k; ++i) acc[i] += om * x[i];
+      for (int i = 0; i < k; ++i) {
+        const LaneVec r = om * x[i].re, m = om * x[i].im;
+        double re = 0, im = 0;
+        for (int w = 0; w < kLanes; ++w) re += r[w], im += m[w];
+        acc[i] += cz(re, im);
+      }
     }
   };
   if (nth == 1) {
