@@ -475,6 +475,56 @@ __global__ void __launch_bounds__(kVecBlock) k_ms_dirs(Geom g, MsDev ms, MsVecs 
   }
 }
 
+// float -> double by its bits (normal numbers; the conversion instruction runs on the FP64 pipe, four of
+// whose operations per component bound the kernel below).
+__device__ __forceinline__ double widen(float x) {
+  const unsigned u = __float_as_uint(x), e = (u >> 23) & 0xffu;
+  if (e == 0u || e == 0xffu) return (double)x;
+  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (896u << 20))), (int)(u << 29));
+}
+
+// dirs for one system without shifts (the FP32 corrections of the reliable updates: s = 1, dsig = 0, so
+// p^1 = p, alpha^1 = alpha and omega = 1): X += alpha p; p = r + beta p, p~ = r~ + conj(beta) p~. Two elements
+// per thread and pass. HBM-bound: 80 bytes an element. The general kernel, which carries p^1 beside p and
+// spent eight FP64 operations an element on X, took 526 us on average over the 80 systems of 16^4 (at most a
+// third running at a time), this one 249.
+constexpr int kSeedBlock = 256, kSeedPasses = 4;
+__global__ void __launch_bounds__(kSeedBlock) k_ms_dirs_seed(Geom g, MsDev ms, MsVecs v) {
+  const int rhs = blockIdx.y;
+  const int st = ms.status[rhs];
+  if (st != 0 && st != 4) return;
+  const size_t n = (size_t)12 * g.vol;  // a multiple of 192: pairs stay aligned and inside one system
+  const double2* sd = ms.seed + (size_t)rhs * 8;
+  const double src[4] = {sd[1].x, sd[1].y, sd[5].x, sd[5].y};
+  float c[4];
+  scalars_in<float, 4>(src, c);
+  const float4* r = (const float4*)((const float2*)v.r + voff<float>(rhs, n));
+  const float4* rt = (const float4*)((const float2*)v.rt + voff<float>(rhs, n));
+  float4* p = (float4*)((float2*)v.p + voff<float>(rhs, n));
+  float4* pt = (float4*)((float2*)v.pt + voff<float>(rhs, n));
+  double2* X = v.X + voff<float>(rhs, n);
+  const cplx<float> al = mk<float>(c[0], c[1]), be = mk<float>(c[2], c[3]), bc = mk<float>(c[2], -c[3]);
+#pragma unroll
+  for (int q = 0; q < kSeedPasses; ++q) {
+    const size_t i = ((size_t)blockIdx.x * kSeedPasses + q) * kSeedBlock + threadIdx.x;
+    if (i >= n / 2) break;
+    const float4 pv = p[i];
+    const cplx<float> p0 = mk<float>(pv.x, pv.y), p1 = mk<float>(pv.z, pv.w);
+    const double2 x0 = X[2 * i], x1 = X[2 * i + 1];
+    const cplx<float> a0 = al * p0, a1 = al * p1;
+    X[2 * i] = make_double2(x0.x + widen(a0.re), x0.y + widen(a0.im));
+    X[2 * i + 1] = make_double2(x1.x + widen(a1.re), x1.y + widen(a1.im));
+    if (st == 0) {
+      const float4 rv = r[i], rtv = rt[i], qv = pt[i];
+      const cplx<float> n0 = mk<float>(rv.x, rv.y) + be * p0, n1 = mk<float>(rv.z, rv.w) + be * p1;
+      const cplx<float> m0 = mk<float>(rtv.x, rtv.y) + bc * mk<float>(qv.x, qv.y);
+      const cplx<float> m1 = mk<float>(rtv.z, rtv.w) + bc * mk<float>(qv.z, qv.w);
+      p[i] = make_float4(n0.re, n0.im, n1.re, n1.im);
+      pt[i] = make_float4(m0.re, m0.im, m1.re, m1.im);
+    }
+  }
+}
+
 cudaError_t launch_ms_start(const Geom& g, bool f64, const MsDev& ms, const MsVecs& v, const double2* b, int m,
                             const double2* R, const double2* L, const double* lam_sign, double2* dots, cudaStream_t st) {
   dim3 grid((g.vol + kBlock - 1) / kBlock, ms.nrhs);
@@ -514,9 +564,15 @@ static cudaError_t ms_step_t(const Geom& g, const Links& U, double m_w, double m
   if (e) return e;
   if ((e = launch_plain(k_ms_update<R>, dim3(vec_blocks(g, elt), ms.nrhs), dim3(kVecBlock), st, g, ms, v, elt))) return e;
   if (ev && (e = record_timing(ev[2], st))) return e;
-  if ((e = v.xs ? launch_plain(k_ms_dirs<R, true>, grid, dim3(kVecBlock), st, g, ms, v)
-                : launch_plain(k_ms_dirs<R, false>, grid, dim3(kVecBlock), st, g, ms, v)))
-    return e;
+  if (sizeof(R) == 4 && ms.s == 1 && ms.sig1v) {  // a correction batch (each system its own shift as the seed)
+    const size_t pairs = (size_t)6 * g.vol;
+    const unsigned nb = (unsigned)((pairs + (size_t)kSeedBlock * kSeedPasses - 1) / ((size_t)kSeedBlock * kSeedPasses));
+    e = launch_plain(k_ms_dirs_seed, dim3(nb, ms.nrhs), dim3(kSeedBlock), st, g, ms, v);
+  } else {
+    e = v.xs ? launch_plain(k_ms_dirs<R, true>, grid, dim3(kVecBlock), st, g, ms, v)
+             : launch_plain(k_ms_dirs<R, false>, grid, dim3(kVecBlock), st, g, ms, v);
+  }
+  if (e) return e;
   if (ev && (e = record_timing(ev[3], st))) return e;
   return cudaGetLastError();
 }
