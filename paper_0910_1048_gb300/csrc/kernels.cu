@@ -270,6 +270,81 @@ __global__ void __launch_bounds__(kBlock, 3)
   for (int q = 0; q < 12; ++q) stc<double>(out + off, (size_t)s * ss + (size_t)q * cs, o.c[q / 3][q % 3]);
 }
 
+// The same with four threads per site (block (32 sites, 4)), one direction's two hops each, for fields too
+// small to fill the GPU with one thread per site: a site's eight hops in a row are about 16 K cycles of one
+// warp's latency. The directions' sums are aligned to their largest exponent and exchanged as integers;
+// thread t finishes spin t.
+__global__ void __launch_bounds__(128, 3)
+    k_dslash_f64_split(Geom g, Links U, FxCoef c, bool native, bool g5_in, bool g5_out, const double2* in, double2* out) {
+  __shared__ fx64 part[4][3][6][32];  // [receiving spin][slot of the sender][component][site]
+  __shared__ int expo[4][32];
+  const int lane = threadIdx.x, t = threadIdx.y;
+  const bool live = (int)blockIdx.x * 32 + lane < g.vol;
+  const int s = live ? blockIdx.x * 32 + lane : g.vol - 1;
+  const size_t off = (size_t)blockIdx.y * 12 * g.vol;
+  const int ss = native ? 1 : 12, cs = native ? g.vol : 1;
+  const StrideLoader ld{in + off, ss, cs};
+  FxAcc acc;
+  fx_clear(acc);
+  int E = 0;
+  const bool fx = c.ok && U.fxf->ok && fx_hops(g, U.fx, s, 2 * t, 2 * t + 2, c, ld, g5_in, acc, E);
+  expo[t][lane] = fx ? E : 1 << 20;
+  __syncthreads();
+  const int Em = max(max(expo[0][lane], expo[1][lane]), max(expo[2][lane], expo[3][lane]));
+  const bool all = Em < 1 << 20;  // no direction needs the FP64 hops
+  const int d = min(Em - E, 62);
+  if (__any_sync(0xffffffffu, d > 0)) {
+    const fx64 half = d > 0 ? (fx64)1 << (d - 1) : 0;
+#pragma unroll
+    for (int i = 0; i < 12; ++i) {
+      acc.re[i / 3][i % 3] = fx_sar(acc.re[i / 3][i % 3] + half, d);
+      acc.im[i / 3][i % 3] = fx_sar(acc.im[i / 3][i % 3] + half, d);
+    }
+  }
+  fx64 ar[3], ai[3];
+#pragma unroll
+  for (int sp = 0; sp < 4; ++sp)
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      if (sp == t) {
+        ar[a] = acc.re[sp][a];
+        ai[a] = acc.im[sp][a];
+      } else {
+        part[sp][t < sp ? t : t - 1][2 * a][lane] = acc.re[sp][a];
+        part[sp][t < sp ? t : t - 1][2 * a + 1][lane] = acc.im[sp][a];
+      }
+    }
+  __syncthreads();
+  if (!live) return;
+  if (!all) {  // the whole site in FP64, by one thread
+    if (t != 0) return;
+    Spin<double> o;
+    ld(s, o);
+    if (g5_in) gamma5_inplace(o);
+    hops_f64(g, U.f64, s, c.k, 0, 8, ld, g5_in, o);
+    if (g5_out) gamma5_inplace(o);
+#pragma unroll
+    for (int q = 0; q < 12; ++q) stc<double>(out + off, (size_t)s * ss + (size_t)q * cs, o.c[q / 3][q % 3]);
+    return;
+  }
+  const double f = fx_unit(Em, c, U.fxf->uexp);
+  const double gi = g5_in && t >= 2 ? -1.0 : 1.0;
+  const bool flip = g5_out && t >= 2;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+#pragma unroll
+    for (int p = 0; p < 3; ++p) {
+      ar[a] += part[t][p][2 * a][lane];
+      ai[a] += part[t][p][2 * a + 1][lane];
+    }
+    const size_t i = (size_t)s * ss + (size_t)(t * 3 + a) * cs;
+    const zd x = ldc<double>(in + off, i);
+    zd o = mk(fma(f, (double)ar[a], gi * x.re), fma(f, (double)ai[a], gi * x.im));
+    if (flip) o = -o;
+    stc<double>(out + off, i, o);
+  }
+}
+
 // The FP32 operator on a batch of sources, native layout in and out. A thread applies the links of
 // its site to a group of G sources (each link loaded once per group), and the grid is ordered
 // group-fastest (block b: site tile b / ngroups, group b % ngroups), so that the blocks of all
@@ -380,9 +455,15 @@ static cudaError_t dslash_group_t(const Geom& g, const Links& U, double m_w, dou
 cudaError_t launch_dslash(const Geom& g, const Links& U, int lf, bool f64, double m_w, double mu, bool g5_in,
                           bool g5_out, bool native, int nrhs, const void* in, void* out, cudaStream_t st) {
   if (f64) {
-    const dim3 grid((g.vol + kBlock - 1) / kBlock, nrhs);
-    k_dslash_f64<<<grid, kBlock, 0, st>>>(g, U, fx_coef(m_w, mu), native, g5_in, g5_out, (const double2*)in,
-                                          (double2*)out);
+    const FxCoef c = fx_coef(m_w, mu);
+    // one source at 8^4 22.8 -> 13.4 us and 12^4 29.7 -> 22.7 with four threads per site; 14^4 30.8 against
+    // 33.4. By the volume alone, so that a source's result is the same alone and in a batch.
+    if (g.vol <= 28672)
+      k_dslash_f64_split<<<dim3((g.vol + 31) / 32, nrhs), dim3(32, 4), 0, st>>>(g, U, c, native, g5_in, g5_out,
+                                                                               (const double2*)in, (double2*)out);
+    else
+      k_dslash_f64<<<dim3((g.vol + kBlock - 1) / kBlock, nrhs), kBlock, 0, st>>>(g, U, c, native, g5_in, g5_out,
+                                                                               (const double2*)in, (double2*)out);
     return cudaGetLastError();
   }
   if (nrhs > 1 && native) {  // a batch: links once per group of sources
