@@ -15,75 +15,97 @@
 namespace ovl {
 
 // One Gram-Schmidt pass over columns 0..j for every rhs (blockIdx.y): block partials only.
-// PASS 0: dots of w; PASS 1: w -= V c1, dots of the new w; PASS 2: w -= V c2, |w|^2. E elements per
-// thread. j = -1 (PASS 2): |v_0|^2.
+// PASS 0: dots of w; PASS 1: w -= V c1, dots of the new w; PASS 2: w -= V c2, |w|^2. j = -1 (PASS 2):
+// |v_0|^2. A block takes a tile of 128 E elements. w stays in shared memory; in the update the columns
+// of an element are shared by 2 / E threads (added in column-group order); in the dots every warp takes
+// whole columns of the tile, so a column costs one butterfly per block. (With the block reducing every
+// column together, two barriers and twenty FP64 instructions each, the three passes of a step took 83,
+// 120 and 52 us on average at 2304 sites and k = 40, bound by those; now 12, 17 and 11.) FP64: the pipe's 16 (j + 1) operations per
+// element and step, 16 us on average there.
+constexpr int kGsThreads = 256;
+
+// Sum of (re, im) over a warp: lanes below 16 keep re, the others im; result in lanes 0 and 16.
+template <class R>
+__device__ __forceinline__ double warp_sum2(const Red<R>& re, const Red<R>& im) {
+  const bool hi = threadIdx.x & 16;
+  Red<R> k = hi ? im : re;
+  const Red<R> s = hi ? re : im;
+  k.add(s.shfl_xor(16));
+#pragma unroll
+  for (int off = 8; off > 0; off >>= 1) k.add(k.shfl_xor(off));
+  return k.get();
+}
+
 template <class R, int PASS>
-__global__ void __launch_bounds__(kFomBlock) k_fom_gs(FomDev f, int j, int E) {
+__global__ void __launch_bounds__(kGsThreads) k_fom_gs(FomDev f, int j, int E) {
   using T = typename V2<R>::T;
   const int rhs = blockIdx.y;
   if (f.status[rhs]) return;
   const size_t n = f.n;
   const int nc = j + 1;  // columns v_0..v_j
   __shared__ cplx<R> cs[kFomMaxK + 1];
+  __shared__ cplx<R> ws[kFomBlock * kFomMaxE];
   const T* V = (const T*)f.V;
   T* w = (T*)f.V + ((size_t)(j + 1) * f.nrhs + rhs) * n;
   const size_t cstride = (size_t)f.nrhs * n;  // between columns
   const T* v0 = V + (size_t)rhs * n;
+  const int tid = threadIdx.x, tile = kFomBlock * E;
+  const size_t base = (size_t)blockIdx.x * tile;
+  const int len = (int)(n - base < (size_t)tile ? n - base : (size_t)tile);  // elements of the tile
   if (PASS > 0 && nc > 0) {
     const double2* c = (PASS == 1 ? f.c1 : f.c2) + (size_t)rhs * (f.kcap + 1);
-    for (int i = threadIdx.x; i < nc; i += blockDim.x) cs[i] = mk<R>((R)c[i].x, (R)c[i].y);
-    __syncthreads();
+    for (int i = tid; i < nc; i += kGsThreads) cs[i] = mk<R>((R)c[i].x, (R)c[i].y);
   }
-  // this thread's elements: E runs of the block, each coalesced
-  const size_t base = (size_t)blockIdx.x * blockDim.x * E + threadIdx.x;
-  cplx<R> wl[kFomMaxE];
-#pragma unroll
-  for (int q = 0; q < kFomMaxE; ++q) {
-    const size_t e = base + (size_t)q * blockDim.x;
-    wl[q] = (q < E && e < n) ? ldc<R>(w, e) : mk<R>(0, 0);
-  }
+  for (int q = tid; q < tile; q += kGsThreads) ws[q] = q < len ? ldc<R>(w, base + q) : mk<R>(0, 0);
+  __syncthreads();
   if (PASS > 0 && nc > 0) {
-    for (int i = 0; i < nc; ++i) {
-      const cplx<R> ci = cs[i];
-#pragma unroll
-      for (int q = 0; q < kFomMaxE; ++q) {
-        const size_t e = base + (size_t)q * blockDim.x;
-        if (q < E && e < n) wl[q] = cmsub(wl[q], ci, ldc<R>(v0 + (size_t)i * cstride, e));
+    if (E == 1) {  // two threads per element, even and odd columns
+      __shared__ cplx<R> half[kFomBlock];
+      const int q = tid & (kFomBlock - 1), odd = tid / kFomBlock;
+      cplx<R> a = odd ? mk<R>(0, 0) : ws[q];
+      if (q < len) {
+#pragma unroll 4
+        for (int i = odd; i < nc; i += 2) a = cmsub(a, cs[i], ldc<R>(v0 + (size_t)i * cstride, base + q));
+      }
+      if (odd) half[q] = a;
+      __syncthreads();
+      if (!odd && q < len) {
+        a = a + half[q];
+        ws[q] = a;
+        stc<R>(w, base + q, a);
+      }
+    } else {
+      for (int q = tid; q < len; q += kGsThreads) {
+        cplx<R> a = ws[q];
+#pragma unroll 4
+        for (int i = 0; i < nc; ++i) a = cmsub(a, cs[i], ldc<R>(v0 + (size_t)i * cstride, base + q));
+        ws[q] = a;
+        stc<R>(w, base + q, a);
       }
     }
-#pragma unroll
-    for (int q = 0; q < kFomMaxE; ++q) {
-      const size_t e = base + (size_t)q * blockDim.x;
-      if (q < E && e < n) stc<R>(w, e, wl[q]);
-    }
+    __syncthreads();
   }
   double* part = f.part + ((size_t)rhs * f.nblk + blockIdx.x) * f.pstride;
   if (PASS < 2) {
-    for (int i = 0; i < nc; ++i) {
-      Red<R> acc[2];
-#pragma unroll
-      for (int q = 0; q < kFomMaxE; ++q) {
-        const size_t e = base + (size_t)q * blockDim.x;
-        if (q < E && e < n) {
-          const cplx<R> v = ldc<R>(v0 + (size_t)i * cstride, e);
-          acc[0].dot2(v.re, wl[q].re, v.im, wl[q].im);   // (v^H w).re
-          acc[1].dot2(v.re, wl[q].im, -v.im, wl[q].re);  // (v^H w).im
-        }
+    const int lane = tid & 31;
+    for (int i = tid >> 5; i < nc; i += kGsThreads / 32) {
+      const T* vi = v0 + (size_t)i * cstride + base;
+      Red<R> re, im;
+#pragma unroll 4
+      for (int q = lane; q < len; q += 32) {
+        const cplx<R> v = ldc<R>(vi, q), x = ws[q];
+        re.dot2(v.re, x.re, v.im, x.im);   // (v^H w).re
+        im.dot2(v.re, x.im, -v.im, x.re);  // (v^H w).im
       }
-      double tot[2];
-      block_reduce<R, 2>(acc, tot);
-      if (threadIdx.x == 0) {
-        part[2 * i] = tot[0];
-        part[2 * i + 1] = tot[1];
-      }
+      const double t = warp_sum2<R>(re, im);
+      if ((lane & 15) == 0) part[2 * i + (lane >> 4)] = t;
     }
   } else {
     Red<R> acc[1];
-#pragma unroll
-    for (int q = 0; q < kFomMaxE; ++q) acc[0].dot2(wl[q].re, wl[q].re, wl[q].im, wl[q].im);
+    for (int q = tid; q < len; q += kGsThreads) acc[0].dot2(ws[q].re, ws[q].re, ws[q].im, ws[q].im);
     double tot[1];
     block_reduce<R, 1>(acc, tot);
-    if (threadIdx.x == 0) part[0] = tot[0];
+    if (tid == 0) part[0] = tot[0];
   }
 }
 
@@ -154,13 +176,13 @@ cudaError_t launch_fom_gs(const FomDev& f, bool f64, int j, int pass, cudaStream
   const unsigned nb = (unsigned)((f.n + (size_t)kFomBlock * E - 1) / ((size_t)kFomBlock * E));
   dim3 grid(nb, f.nrhs);
   if (f64) {
-    if (pass == 0) k_fom_gs<double, 0><<<grid, kFomBlock, 0, st>>>(f, j, E);
-    else if (pass == 1) k_fom_gs<double, 1><<<grid, kFomBlock, 0, st>>>(f, j, E);
-    else k_fom_gs<double, 2><<<grid, kFomBlock, 0, st>>>(f, j, E);
+    if (pass == 0) k_fom_gs<double, 0><<<grid, kGsThreads, 0, st>>>(f, j, E);
+    else if (pass == 1) k_fom_gs<double, 1><<<grid, kGsThreads, 0, st>>>(f, j, E);
+    else k_fom_gs<double, 2><<<grid, kGsThreads, 0, st>>>(f, j, E);
   } else {
-    if (pass == 0) k_fom_gs<float, 0><<<grid, kFomBlock, 0, st>>>(f, j, E);
-    else if (pass == 1) k_fom_gs<float, 1><<<grid, kFomBlock, 0, st>>>(f, j, E);
-    else k_fom_gs<float, 2><<<grid, kFomBlock, 0, st>>>(f, j, E);
+    if (pass == 0) k_fom_gs<float, 0><<<grid, kGsThreads, 0, st>>>(f, j, E);
+    else if (pass == 1) k_fom_gs<float, 1><<<grid, kGsThreads, 0, st>>>(f, j, E);
+    else k_fom_gs<float, 2><<<grid, kGsThreads, 0, st>>>(f, j, E);
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
