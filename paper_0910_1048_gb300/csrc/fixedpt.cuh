@@ -163,8 +163,8 @@ struct FxSpin {  // limbs of a site's 12 complex components relative to one expo
   int rh[4][3], rl[4][3], ih[4][3], il[4][3];
 };
 
-// Biased exponent of the site's largest component.
-OVL_HD int fx_exponent(const Spin<double>& p) {
+// High word of the site's largest component's modulus (its biased exponent is the word >> 20).
+OVL_HD int fx_top_word(const Spin<double>& p) {
   int m = 0;
 #pragma unroll
   for (int i = 0; i < 12; ++i) {
@@ -175,7 +175,7 @@ OVL_HD int fx_exponent(const Spin<double>& p) {
     fx_words(p.c[i / 3][i % 3].im, w, z);
     m = m > (w & 0x7fffffff) ? m : (w & 0x7fffffff);
   }
-  return m >> 20;
+  return m;
 }
 
 OVL_HD void fx_spin(const Spin<double>& p, int e, FxSpin& o) {
@@ -432,12 +432,12 @@ OVL_HD int fx_neighbour(const Geom& g, int s, unsigned long long xyzt, int k, bo
 // Hops k0 .. k1-1 of site s, psi in FP64 loaded through `ld` and converted on the way, to limbs relative to the
 // largest exponent E met so far (+1), so that no hop is shifted afterwards. Returns whether the
 // accumulators hold the hop sum: no infinity or NaN among the neighbours, and not only components too
-// small for the common exponent (all zero is fine).
+// small for the common exponent (all zero, or below 2^-1042, is fine: the sum is zero).
 template <class Load>
 OVL_HD bool fx_hops(const Geom& g, const FxC* U, int s, int k0, int k1, const FxCoef& c, Load ld, bool g5in, FxAcc& acc,
                     int& E) {
   const unsigned long long xyzt = fx_coords(g, s);
-  int emax = 0;
+  int top = 0;
   E = 0;
 #pragma unroll 1
   for (int k = k0; k < k1; ++k) {
@@ -447,14 +447,14 @@ OVL_HD bool fx_hops(const Geom& g, const FxC* U, int s, int k0, int k1, const Fx
     {
       Spin<double> p;
       ld(nb, p);
-      const int eb = fx_exponent(p);
-      emax = emax > eb ? emax : eb;
+      const int w = fx_top_word(p), eb = w >> 20;
+      top = top > w ? top : w;
       const int fe = fx_hop_exponent(k, 0, c), eh = (eb > 64 ? eb : 64) + fe;
       if (eh > E) {  // first hop, or a larger neighbour than any before
         if (E != 0) {
 #pragma unroll
           for (int i = 0; i < 12; ++i) {
-  acc.re[i / 3][i % 3] = fx_sar(acc.re[i / 3][i % 3], eh + 1 - E);
+            acc.re[i / 3][i % 3] = fx_sar(acc.re[i / 3][i % 3], eh + 1 - E);
             acc.im[i / 3][i % 3] = fx_sar(acc.im[i / 3][i % 3], eh + 1 - E);
           }
         }
@@ -468,7 +468,8 @@ OVL_HD bool fx_hops(const Geom& g, const FxC* U, int s, int k0, int k1, const Fx
     const size_t sa = (k & 1) ? (size_t)g.vol : (size_t)3 * g.vol, sb = (k & 1) ? (size_t)3 * g.vol : (size_t)g.vol;
     fx_hop(k, 0, false, h, [&](int a, int b) { return u[a * sa + b * sb]; }, c, wraps && g.t_bc < 0, acc);
   }
-  return emax < 0x7ff && E < 2000 && (emax == 0 || emax >= 64);
+  if (top == 0) fx_clear(acc);  // (a negative zero left one unit)
+  return top < (0x7ff << 20) && E < 2000 && (top == 0 || top >= (64 << 20));
 }
 
 // FP64 value of one unit of the accumulators times the hop coefficient ks and the links' scale.
