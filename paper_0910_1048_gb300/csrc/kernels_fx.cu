@@ -175,7 +175,7 @@ __device__ __forceinline__ void fx_step_store(FxStep* st, double kse, double sv,
 // coefficients of the update of step j. By one block.
 __device__ __forceinline__ void fx_settle(const LzDev& lz, const FxVecs& fx, int rhs, int nchunk, double ks,
                                           const FxField* fxf) {
-  __shared__ double sh[4][8];
+  __shared__ double sh[4][2];
   const int t = lin_tid(), warp = t >> 5, lane = t & 31, nw = lin_nthreads() >> 5;
   const int go = lz.pending[rhs] && !lz.status[rhs];
   const int j = lz.j[rhs];
@@ -183,7 +183,7 @@ __device__ __forceinline__ void fx_settle(const LzDev& lz, const FxVecs& fx, int
   const double svp = j > 1 ? lz.sv[o + j - 1] : 0.0;
   const zd swp = j > 1 ? ldc<double>(lz.sw, o + j - 1) : mk(0.0, 0.0);
   const FxParts f = fx_parts(lz, rhs, nchunk);
-  const int nshare = max(1, min(8, nw / 4));
+  constexpr int nshare = 2;  // per sum, whatever the block: the shares are added in FP64
   if (go)
     for (int i = warp; i < 4 * nshare; i += nw) {
       const int v = i & 3, q = i >> 2;
@@ -211,7 +211,7 @@ __device__ __forceinline__ void fx_settle(const LzDev& lz, const FxVecs& fx, int
   }
 }
 
-constexpr int kFxSettle = 512;
+constexpr int kFxSettle = 256;
 __global__ void __launch_bounds__(kFxSettle) k_fx_settle(LzDev lz, const __grid_constant__ FxVecs fx, int nchunk, double ks,
                                                         const FxField* fxf) {
   fx_settle(lz, fx, blockIdx.y, nchunk, ks, fxf);
@@ -235,7 +235,7 @@ __global__ void __launch_bounds__(64) k_fx_begin(Geom g, LzDev lz, FxVecs fx, co
     const double2* in = role ? w1 + (size_t)rhs * n : vh + (size_t)rhs * lz.vcols * n;
     Spin<double> p;
     StrideLoader{in, 1, g.vol}(s, p);
-    const int e = max(fx_exponent(p), 64);
+    const int e = max(fx_top_word(p) >> 20, 64);
     FxSpin q;
     fx_spin(p, e, q);
     FxC* out = (role ? fx.w[1] : fx.v[1]) + (size_t)rhs * n;
