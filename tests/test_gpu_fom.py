@@ -157,3 +157,18 @@ def test_batch_equals_single(ovl, p4f):
         st1, info1, x1 = _solve(ovl, lat, b2[r], **kw)
         assert info1[0]["iterations"] == info[r]["iterations"]
         assert np.array_equal(x1, x2[r])
+
+
+@pytest.mark.parametrize("dims,k", [((2, 2, 2, 2), 33), ((2, 2, 2, 2), 2), ((6, 10, 10, 12), 9), ((10, 10, 10, 10), 8)])
+def test_gram_schmidt_tiles(ovl, ctx, dims, k):
+    """Tiles of one, two and three elements per thread with a remainder, and column counts around the
+    block's eight warps: one cycle at equal k, to the other cycles' 1e-10."""
+    u = synth.gauge_links(dims, 15)
+    b = synth.gaussian_source(dims, 16)
+    lat = ovl.ovl_create_lattice(ctx, dims, -1)
+    ovl.ovl_set_links(lat, u, ovl.OVL_F64)
+    st, info, x = _solve(ovl, lat, b, mu=0.3, tol=0.0, k_max=k, restart_k=k, spec_lo=0.05, spec_hi=2.7, s=6)
+    ovl.ovl_destroy_lattice(lat)
+    w, sg = rational.neuberger_scaled(6, rational.scale_and_d(*rational.circle_from_gap(0.05, 2.7))[0])
+    xo, _ = fom.sign_fom_lr(lambda v: krylov.apply_hw(u, dims, -2.0, 0.3, v), b, w, sg, k, tol=0.0, max_cycles=1)
+    assert _rel(x, xo) < 1e-10

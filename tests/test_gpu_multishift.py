@@ -182,3 +182,19 @@ def test_reliable_updates_reach_fp64_accuracy(ovl, p4m, prec):
     xg = lanczos.rational_sign_dense(p["h"], p["b"].ravel(), w, sg)
     assert _rel(x.ravel(), xg) < 2e-9
     assert _rel(x.ravel(), p["xstar"].ravel()) < 1e-8
+
+
+@pytest.mark.parametrize("dims", [(2, 2, 2, 2), (2, 4, 6, 6)])
+def test_corrections_on_ragged_volumes(ovl, ctx, dims):
+    """The corrections' direction kernel with a block less than half filled and one and a remainder: FP32 with
+    reliable updates against FP64 on the same poles; each is within 2e-9 of g(A) b at eps = 1e-10."""
+    u = synth.gauge_links(dims, 17)
+    b = synth.gaussian_source(dims, 18, nrhs=2)
+    lat = ovl.ovl_create_lattice(ctx, dims, -1)
+    ovl.ovl_set_links(lat, u, ovl.OVL_F64 | ovl.OVL_F32)
+    kw = dict(mu=0.3, tol=1e-10, k_max=5000, spec_lo=0.05, spec_hi=2.7, s=8)
+    st, info, x = _solve(ovl, lat, b, precision=ovl.OVL_PREC_F32, **kw)
+    st64, _, x64 = _solve(ovl, lat, b, **kw)
+    assert st == st64 == ovl.OVL_OK, info
+    assert _rel(x, x64) < 4e-9
+    ovl.ovl_destroy_lattice(lat)
