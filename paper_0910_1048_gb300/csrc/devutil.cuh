@@ -307,6 +307,32 @@ struct Loader {
   }
 };
 
+// A canonical FP32 spinor (96 consecutive bytes) by 16 bytes at a time; p on a 16-byte boundary.
+struct Loader16 {
+  const float2* p;
+  int vol;
+  bool g5;
+  __device__ __forceinline__ void operator()(int s, Spin<float>& o) const {
+    const float4* q = (const float4*)p + (size_t)s * 6;
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+      const float4 v = q[c];
+      o.c[2 * c / 3][2 * c % 3] = mk<float>(v.x, v.y);
+      o.c[(2 * c + 1) / 3][(2 * c + 1) % 3] = mk<float>(v.z, v.w);
+    }
+    if (g5) gamma5_inplace(o);
+  }
+};
+
+__device__ __forceinline__ void store_spin16(float2* p, int s, const Spin<float>& o) {
+  float4* q = (float4*)p + (size_t)s * 6;
+#pragma unroll
+  for (int c = 0; c < 6; ++c) {
+    const cplx<float> a = o.c[2 * c / 3][2 * c % 3], b = o.c[(2 * c + 1) / 3][(2 * c + 1) % 3];
+    q[c] = make_float4(a.re, a.im, b.re, b.im);
+  }
+}
+
 template <class R, bool NATIVE>
 __device__ __forceinline__ void store_spin(typename V2<R>::T* p, int vol, int s, const Spin<R>& o) {
 #pragma unroll

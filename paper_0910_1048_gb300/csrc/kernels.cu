@@ -12,6 +12,7 @@
 #include <mutex>
 #include <set>
 #include <tuple>
+#include <type_traits>
 
 #include "devutil.cuh"
 #include "kernels.h"
@@ -237,13 +238,19 @@ cudaError_t launch_ingest_links(const Geom& g, const double* ucan, double2* u64,
 // ------------------------------------------------------------------ apply D_W
 // FP32: G5IN (gamma5 on the input, the adjoint's form) is a template parameter so that the common
 // case carries no per-neighbour branch: 32^4 FP32 4.7 -> 5.2 TB/s in a probe without it.
-template <int LF, bool NATIVE, bool G5IN>
-__global__ void __launch_bounds__(kBlock, LF == LINK_F16R12 ? 6 : 7)
+// Canonical fields are read and written 16 bytes at a time where both buffers start on such a boundary (a
+// caller's view may start on 8): with 8, a warp's request touches 24 lines for 256 bytes and the L1 is 84%
+// busy with them. FP16 links, 28 x 20 x 12 x 30: 34.9 -> 26.7 us, FP32 24^4 62 -> 50.5, five sources at 12^4
+// 23 -> 18.6 from the loads alone, 22.6, 43.1 and 16.5 with the stores. (Copies of a warp's 32 neighbours to
+// shared memory, 16 bytes per lane and transposed there, stores by whole lines: 26.8, 47.7 and 18.6.)
+enum { kCanonical = 0, kNative = 1, kCanonical16 = 2 };
+template <int LF, int LAYOUT, bool G5IN>
+__global__ void __launch_bounds__(kBlock, (LF == LINK_F16R12 ? 6 : 7) - (LAYOUT == kCanonical16))
     k_dslash(Geom g, Links U, HopCoef<float> c, bool g5_out, const float2* in, float2* out) {
   int s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= g.vol) return;
   size_t off = (size_t)blockIdx.y * 12 * g.vol;
-  Loader<float, NATIVE> ld{in + off, g.vol, G5IN};
+  std::conditional_t<LAYOUT == kCanonical16, Loader16, Loader<float, LAYOUT == kNative>> ld{in + off, g.vol, G5IN};
   Spin<float> o;
   dslash_site<LF, float>(g, U, s, c, ld, o);
   const float sg = g5_out ? -1.f : 1.f;  // gamma5 = diag(1, 1, -1, -1) on the output, without a branch
@@ -252,7 +259,10 @@ __global__ void __launch_bounds__(kBlock, LF == LINK_F16R12 ? 6 : 7)
     o.c[2][a] = sg * o.c[2][a];
     o.c[3][a] = sg * o.c[3][a];
   }
-  store_spin<float, NATIVE>(out + off, g.vol, s, o);
+  if (LAYOUT == kCanonical16)
+    store_spin16(out + off, s, o);
+  else
+    store_spin<float, LAYOUT == kNative>(out + off, g.vol, s, o);
 }
 
 // FP64 (fixed-point hops, see fixedpt.cuh): the layout and gamma5 are run-time values. Three blocks per SM (168 registers): 16^4 x 8 sources 271 us; two (198 registers) 328, four (128,
@@ -387,14 +397,20 @@ static cudaError_t dslash_t(const Geom& g, const Links& U, double m_w, double mu
   const dim3 grid((g.vol + kBlock - 1) / kBlock, nrhs);
   const float2* i = (const float2*)in;
   float2* o = (float2*)out;
-  if (native && gi)
-    k_dslash<LF, true, true><<<grid, kBlock, 0, st>>>(g, U, c, go, i, o);
-  else if (native)
-    k_dslash<LF, true, false><<<grid, kBlock, 0, st>>>(g, U, c, go, i, o);
-  else if (gi)
-    k_dslash<LF, false, true><<<grid, kBlock, 0, st>>>(g, U, c, go, i, o);
+  const bool wide = (((uintptr_t)in | (uintptr_t)out) & 15) == 0;
+  auto run = [&](auto layout) {
+    constexpr int L = decltype(layout)::value;
+    if (gi)
+      k_dslash<LF, L, true><<<grid, kBlock, 0, st>>>(g, U, c, go, i, o);
+    else
+      k_dslash<LF, L, false><<<grid, kBlock, 0, st>>>(g, U, c, go, i, o);
+  };
+  if (native)
+    run(std::integral_constant<int, kNative>());
+  else if (wide)
+    run(std::integral_constant<int, kCanonical16>());
   else
-    k_dslash<LF, false, false><<<grid, kBlock, 0, st>>>(g, U, c, go, i, o);
+    run(std::integral_constant<int, kCanonical>());
   return cudaGetLastError();
 }
 

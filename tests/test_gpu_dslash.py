@@ -193,3 +193,29 @@ def test_full_size_sampled_sites(ovl, ctx, dims):
         got = can.reshape(vol, 4, 3)[torch.from_numpy(sites).cuda()].cpu().numpy()
         assert np.abs(got - ref).max() <= tol * scale, (dt, flags)
     ovl.ovl_destroy_lattice(lat)
+
+
+@pytest.mark.parametrize("links,tol", [("f32", 2e-6), ("f16", 3e-3)])
+def test_dslash_f32_canonical_alignment(ovl, ctx, links, tol):
+    """Canonical single-precision fields that start on 16 bytes, and views that start on 8: the same arithmetic, so
+    the same bits; both to the other single-precision bounds."""
+    dims = (6, 4, 2, 6)
+    lat, u = _lattice(ovl, ctx, dims, 17)
+    psi = synth.gaussian_source(dims, 18, nrhs=3)
+    n = psi.size
+    room = torch.empty(n + 1, dtype=torch.complex64, device="cuda")
+    room_out = torch.empty(n + 1, dtype=torch.complex64, device="cuda")
+    got = []
+    for i, o in ((0, 0), (1, 0), (0, 1), (1, 1)):
+        inp, out = room[i:n + i].view(psi.shape), room_out[o:n + o].view(psi.shape)
+        inp.copy_(torch.from_numpy(psi).to(torch.complex64))
+        for flags in (ovl.OVL_GAMMA5, ovl.OVL_DAGGER):
+            ovl.ovl_apply_DW(lat, -2.0, 0.3, flags | (ovl.OVL_LINKS_F16R12 if links == "f16" else ovl.OVL_LINKS_F32),
+                             inp, out)
+            got.append((flags, out.cpu().numpy()))
+    for flags, y in got[:2]:
+        ref = np.stack([_ref(u, psi[r], 0.3, flags, ovl, -1) for r in range(3)])
+        assert np.abs(y - ref).max() / np.abs(ref).max() < tol
+    for i in range(2, 8):
+        assert np.array_equal(got[i][1], got[i % 2][1])
+    ovl.ovl_destroy_lattice(lat)
