@@ -355,38 +355,122 @@ __global__ void __launch_bounds__(128, 3)
   }
 }
 
-// The FP32 operator on a batch of sources, native layout in and out. A thread applies the links of
-// its site to a group of G sources (each link loaded once per group), and the grid is ordered
-// group-fastest (block b: site tile b / ngroups, group b % ngroups), so that the blocks of all
-// groups of one site tile run together and a tile's link lines come from DRAM once and from L2
-// for the other groups. G = 1 is the single-source kernel in that order.
-template <int LF, bool G5IN, int G>
-__global__ void __launch_bounds__(kBlock, G == 1 ? 7 : (G == 2 ? 4 : 2))
-    k_dslash_group(Geom g, Links U, HopCoef<float> c, bool g5_out, int nrhs,
-                                                         const float2* in, float2* out) {
-  const int ngroups = (nrhs + G - 1) / G;
-  const int tile = blockIdx.x / ngroups, grp = blockIdx.x % ngroups;
-  const int s = tile * blockDim.x + threadIdx.x;
-  if (s >= g.vol) return;
-  const int r0 = grp * G;
-  const int nact = min(G, nrhs - r0);
-  const size_t n = (size_t)12 * g.vol;
-  Loader<float, true> ld[G];
+// The FP32 operator on a batch of sources, native layout in and out: two sites s, s + 1 per thread (s even: in one x
+// row), so that a request carries 16 bytes per lane (FP16 links: 8), the pair's inner x neighbours are its own
+// values, and the neighbours' indices are found once for both. The kernel with one site and, autotuned, 1, 2 or
+// 4 sources per thread kept the L1 data path 62% busy, the issue slots 54% and HBM 50%: no single bound.
+// The grid is ordered source-fastest, so that a tile's links come from HBM once and from L2 for the other
+// sources; sources in sets whose three time slices stay in L2 (kSetBytes; at 24^4, 16 sources: one set of 16
+// read 0.6 GB of spinors again). 24^4, 16 sources 423 -> 371 us in sets of 8 (389 in one, 377 in fours); 16^4, 8
+// sources 45.1 -> 42.9, 16 79.2 -> 74.9 (one set; 77.9 in eights); 32^4, 4 sources 322 -> 305;
+// 28 x 20 x 12 x 30 with FP16 links, 13 sources 192 -> 178. A single source gains at 24^4 (37.1 -> 35.0) and loses at
+// 20^4 (18.6 -> 19.1), and keeps one site per thread. 168 registers; at 128 the spills cost 4%.
+template <int LF>
+__device__ __forceinline__ void load_link2(const Links& U, int mu, int s, int vol, Mat3<float> (&u)[2]) {
+  if (LF == LINK_F32) {
+    const float2* p = U.f32 + (size_t)mu * 9 * vol + s;
 #pragma unroll
-  for (int r = 0; r < G; ++r) ld[r] = Loader<float, true>{in + (size_t)(r0 + (r < nact ? r : 0)) * n, g.vol, G5IN};
-  Spin<float> o[G];
-  dslash_site_g<LF, G>(g, U, s, c, ld, nact, o);
+    for (int k = 0; k < 9; ++k) {
+      const float4 v = *(const float4*)(p + (size_t)k * vol);
+      u[0].m[k / 3][k % 3] = mk<float>(v.x, v.y);
+      u[1].m[k / 3][k % 3] = mk<float>(v.z, v.w);
+    }
+  } else {
+    const uint32_t* p = U.f16 + (size_t)mu * 6 * vol + s;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+      const uint2 v = *(const uint2*)(p + (size_t)k * vol);
+      const float2 a = __half22float2(*(const __half2*)&v.x), b = __half22float2(*(const __half2*)&v.y);
+      u[0].m[k / 3][k % 3] = mk<float>(a.x, a.y);
+      u[1].m[k / 3][k % 3] = mk<float>(b.x, b.y);
+    }
+    complete_link(u[0]);
+    complete_link(u[1]);
+  }
+}
+__device__ __forceinline__ void load_spin2(const float2* p, int vol, int s, bool g5, Spin<float> (&o)[2]) {
+#pragma unroll
+  for (int c = 0; c < 12; ++c) {
+    const float4 v = *(const float4*)(p + (size_t)c * vol + s);
+    o[0].c[c / 3][c % 3] = mk<float>(v.x, v.y);
+    o[1].c[c / 3][c % 3] = mk<float>(v.z, v.w);
+  }
+  if (g5) {
+    gamma5_inplace(o[0]);
+    gamma5_inplace(o[1]);
+  }
+}
+template <int MU, bool FWD, int LF>
+__device__ __forceinline__ void hop2(const Links& U, int vol, int s, int nb, float k, const float2* in, bool g5,
+                                     Spin<float> (&acc)[2]) {
+  Half<float> h[2], hu;
+  Mat3<float> u[2];
+  {
+    Spin<float> p[2];
+    load_spin2(in, vol, nb, g5, p);
+    project<MU, FWD>(p[0], h[0]);
+    project<MU, FWD>(p[1], h[1]);
+  }
+  load_link2<LF>(U, MU, FWD ? s : nb, vol, u);
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    su3_mul<!FWD>(u[i], h[i], hu);
+    reconstruct_add<MU, FWD>(acc[i], hu, k);
+  }
+}
+
+constexpr int kPairBlock = 64;
+constexpr size_t kSetBytes = 40u << 20;
+
+template <int LF, bool G5IN>
+__global__ void __launch_bounds__(kPairBlock, 6)
+    k_dslash2(Geom g, Links U, HopCoef<float> c, bool g5_out, int nrhs, int set, const float2* in, float2* out) {
+  const int tiles = (g.vol / 2 + kPairBlock - 1) / kPairBlock;
+  const int r0 = blockIdx.x / (tiles * set) * set, b = blockIdx.x - r0 * tiles, w = min(set, nrhs - r0);
+  const int s = 2 * (b / w * kPairBlock + threadIdx.x), rhs = r0 + b % w;
+  if (s >= g.vol) return;
+  in += (size_t)rhs * 12 * g.vol;
+  out += (size_t)rhs * 12 * g.vol;
+  Nbr n;
+  neighbours(g, s, n);
+  Spin<float> o[2];
+  load_spin2(in, g.vol, s, G5IN, o);
+  {  // x: the inner neighbours are the pair itself
+    Half<float> hf[2], hb[2], hu;
+    Mat3<float> u[2], ub;
+    Spin<float> p;
+    const Loader<float, true> ld{in, g.vol, G5IN};
+    project<0, true>(o[1], hf[0]);
+    project<0, false>(o[0], hb[1]);
+    const int nf = s % g.lx + 2 == g.lx ? s + 2 - g.lx : s + 2;
+    ld(nf, p);
+    project<0, true>(p, hf[1]);
+    load_link2<LF>(U, 0, s, g.vol, u);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      su3_mul<false>(u[i], hf[i], hu);
+      reconstruct_add<0, true>(o[i], hu, c.ks);
+    }
+    ld(n.b[0], p);
+    project<0, false>(p, hb[0]);
+    load_link<LF>(U, 0, n.b[0], g.vol, ub);
+    su3_mul<true>(ub, hb[0], hu);
+    reconstruct_add<0, false>(o[0], hu, c.ks);
+    su3_mul<true>(u[0], hb[1], hu);
+    reconstruct_add<0, false>(o[1], hu, c.ks);
+  }
+  hop2<1, true, LF>(U, g.vol, s, n.f[1], c.ks, in, G5IN, o);
+  hop2<1, false, LF>(U, g.vol, s, n.b[1], c.ks, in, G5IN, o);
+  hop2<2, true, LF>(U, g.vol, s, n.f[2], c.ks, in, G5IN, o);
+  hop2<2, false, LF>(U, g.vol, s, n.b[2], c.ks, in, G5IN, o);
+  hop2<3, true, LF>(U, g.vol, s, n.f[3], n.t == g.lt - 1 ? (float)g.t_bc * c.ktf : c.ktf, in, G5IN, o);
+  hop2<3, false, LF>(U, g.vol, s, n.b[3], n.t == 0 ? (float)g.t_bc * c.ktb : c.ktb, in, G5IN, o);
   const float sg = g5_out ? -1.f : 1.f;
 #pragma unroll
-  for (int r = 0; r < G; ++r) {
-    if (r < nact) {
-#pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        o[r].c[2][a] = sg * o[r].c[2][a];
-        o[r].c[3][a] = sg * o[r].c[3][a];
-      }
-      store_spin<float, true>(out + (size_t)(r0 + r) * n, g.vol, s, o[r]);
-    }
+  for (int q = 0; q < 12; ++q) {
+    const float f = q < 6 ? 1.f : sg;
+    const cplx<float> a = f * o[0].c[q / 3][q % 3], b = f * o[1].c[q / 3][q % 3];
+    *(float4*)(out + (size_t)q * g.vol + s) = make_float4(a.re, a.im, b.re, b.im);
   }
 }
 
@@ -414,58 +498,18 @@ static cudaError_t dslash_t(const Geom& g, const Links& U, double m_w, double mu
   return cudaGetLastError();
 }
 
-template <int LF, int G>
-static cudaError_t dslash_group_g(const Geom& g, const Links& U, HopCoef<float> c, bool gi, bool go, int nrhs,
-                                  const void* in, void* out, cudaStream_t st) {
-  const unsigned tiles = (unsigned)((g.vol + kBlock - 1) / kBlock), ngroups = (unsigned)((nrhs + G - 1) / G);
-  if (gi)
-    k_dslash_group<LF, true, G><<<tiles * ngroups, kBlock, 0, st>>>(g, U, c, go, nrhs, (const float2*)in, (float2*)out);
-  else
-    k_dslash_group<LF, false, G><<<tiles * ngroups, kBlock, 0, st>>>(g, U, c, go, nrhs, (const float2*)in,
-                                                                      (float2*)out);
-  return cudaGetLastError();
-}
-
-// Sources per link load of the batched stencil (1, 2 or 4), chosen per (volume, links, batch) by
-// timing the three on the first call (the real launch follows and rewrites `out`).
-static std::mutex g_group_mu;
-static std::map<std::tuple<int, int, int>, int> g_group;
-
 template <int LF>
-static cudaError_t dslash_group_t(const Geom& g, const Links& U, double m_w, double mu, bool gi, bool go, int nrhs,
-                                  const void* in, void* out, cudaStream_t st) {
+static cudaError_t dslash_batch(const Geom& g, const Links& U, double m_w, double mu, bool gi, bool go, int nrhs,
+                                const void* in, void* out, cudaStream_t st) {
   const HopCoef<float> c = hop_coef<float>(m_w, mu);
-  auto run = [&](int G) {
-    return G == 4 ? dslash_group_g<LF, 4>(g, U, c, gi, go, nrhs, in, out, st)
-                  : G == 2 ? dslash_group_g<LF, 2>(g, U, c, gi, go, nrhs, in, out, st)
-                           : dslash_group_g<LF, 1>(g, U, c, gi, go, nrhs, in, out, st);
-  };
-  int G = 0;
-  {
-    std::lock_guard<std::mutex> lk(g_group_mu);
-    auto it = g_group.find({g.vol, LF, nrhs});
-    if (it != g_group.end()) G = it->second;
-    if (!G) {
-      cudaEvent_t a, b;
-      if (cudaEventCreate(&a) == cudaSuccess && cudaEventCreate(&b) == cudaSuccess) {
-        float best = 1e30f;
-        bool ok = true;
-        for (int rep = 0; rep < 3 && ok; ++rep)
-          for (int cand : {1, 2, 4}) {
-            ok = ok && cudaEventRecord(a, st) == cudaSuccess && run(cand) == cudaSuccess &&
-                 cudaEventRecord(b, st) == cudaSuccess && cudaEventSynchronize(b) == cudaSuccess;
-            float ms = 0;
-            if (ok && rep > 0 && cudaEventElapsedTime(&ms, a, b) == cudaSuccess && ms < best) best = ms, G = cand;
-          }
-        cudaEventDestroy(a);
-        cudaEventDestroy(b);
-        if (!ok) G = 0;
-      }
-      cudaGetLastError();
-      if (G) g_group[{g.vol, LF, nrhs}] = G;
-    }
-  }
-  return run(G ? G : kLinkGroup);
+  const int most = (int)std::max<size_t>(1, kSetBytes / ((size_t)3 * g.st * 96));
+  const int sets = (nrhs + most - 1) / most, set = (nrhs + sets - 1) / sets;
+  const unsigned nb = (unsigned)((g.vol / 2 + kPairBlock - 1) / kPairBlock) * nrhs;
+  if (gi)
+    k_dslash2<LF, true><<<nb, kPairBlock, 0, st>>>(g, U, c, go, nrhs, set, (const float2*)in, (float2*)out);
+  else
+    k_dslash2<LF, false><<<nb, kPairBlock, 0, st>>>(g, U, c, go, nrhs, set, (const float2*)in, (float2*)out);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_dslash(const Geom& g, const Links& U, int lf, bool f64, double m_w, double mu, bool g5_in,
@@ -482,9 +526,9 @@ cudaError_t launch_dslash(const Geom& g, const Links& U, int lf, bool f64, doubl
                                                                                (const double2*)in, (double2*)out);
     return cudaGetLastError();
   }
-  if (nrhs > 1 && native) {  // a batch: links once per group of sources
-    if (lf == LINK_F16R12) return dslash_group_t<LINK_F16R12>(g, U, m_w, mu, g5_in, g5_out, nrhs, in, out, st);
-    return dslash_group_t<LINK_F32>(g, U, m_w, mu, g5_in, g5_out, nrhs, in, out, st);
+  if (nrhs > 1 && native && (((uintptr_t)in | (uintptr_t)out) & 15) == 0) {  // (a view may start on 8 bytes)
+    if (lf == LINK_F16R12) return dslash_batch<LINK_F16R12>(g, U, m_w, mu, g5_in, g5_out, nrhs, in, out, st);
+    return dslash_batch<LINK_F32>(g, U, m_w, mu, g5_in, g5_out, nrhs, in, out, st);
   }
   if (lf == LINK_F16R12) return dslash_t<LINK_F16R12>(g, U, m_w, mu, g5_in, g5_out, native, nrhs, in, out, st);
   return dslash_t<LINK_F32>(g, U, m_w, mu, g5_in, g5_out, native, nrhs, in, out, st);

@@ -9,7 +9,6 @@ namespace ovl {
 
 constexpr int kBlock = 128;     // threads per block of the site-parallel kernels
 constexpr int kPairSites = 64;  // sites per block of the pair stencil (x2 threads)
-constexpr int kLinkGroup = 4;     // sources that share one load of a site's links in the batched FP32 kernels
 constexpr int kSplitVolume = 32768;  // below this many sites the pair stencils split each site over 8 threads
 inline bool use_split(const Geom& g) { return g.vol < kSplitVolume; }
 // Plain launch through cudaLaunchKernelEx (one call site per kernel shape, error returned).

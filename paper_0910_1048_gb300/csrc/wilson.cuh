@@ -113,6 +113,14 @@ OVL_HD void su3_mul(const Mat3<R>& u, const Half<R>& h, Half<R>& out) {
 }
 
 // ------------------------------------------------------------------ link loads
+// Third row of an SU(3) matrix: conj(row0 x row1).
+template <class R>
+OVL_HD void complete_link(Mat3<R>& u) {
+  u.m[2][0] = conj(u.m[0][1] * u.m[1][2] - u.m[0][2] * u.m[1][1]);
+  u.m[2][1] = conj(u.m[0][2] * u.m[1][0] - u.m[0][0] * u.m[1][2]);
+  u.m[2][2] = conj(u.m[0][0] * u.m[1][1] - u.m[0][1] * u.m[1][0]);
+}
+
 template <int LF, class R>
 OVL_HD void load_link(const Links& U, int mu, int site, int vol, Mat3<R>& u) {
   if (LF == LINK_F64) {
@@ -139,10 +147,7 @@ OVL_HD void load_link(const Links& U, int mu, int site, int vol, Mat3<R>& u) {
       float2 f = __half22float2(hv);
       u.m[k / 3][k % 3] = mk<R>((R)f.x, (R)f.y);
     }
-    // third row of an SU(3) matrix: conj(row0 x row1)
-    u.m[2][0] = conj(u.m[0][1] * u.m[1][2] - u.m[0][2] * u.m[1][1]);
-    u.m[2][1] = conj(u.m[0][2] * u.m[1][0] - u.m[0][0] * u.m[1][2]);
-    u.m[2][2] = conj(u.m[0][0] * u.m[1][1] - u.m[0][1] * u.m[1][0]);
+    complete_link(u);
 #endif
   }
 }

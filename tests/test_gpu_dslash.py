@@ -219,3 +219,29 @@ def test_dslash_f32_canonical_alignment(ovl, ctx, links, tol):
     for i in range(2, 8):
         assert np.array_equal(got[i][1], got[i % 2][1])
     ovl.ovl_destroy_lattice(lat)
+
+
+@pytest.mark.parametrize("dims,nrhs", [((2, 2, 2, 2), 3), ((2, 6, 4, 4), 2), ((6, 4, 2, 6), 5), ((12, 10, 6, 8), 4)])
+@pytest.mark.parametrize("links,tol", [("f32", 2e-6), ("f16", 3e-3)])
+def test_dslash_f32_native_batch(ovl, ctx, dims, nrhs, links, tol):
+    """Batches in the native layout (two sites per thread): rows of two sites, blocks partly filled, views that start
+    on 8 bytes; to the other single-precision bounds, and equal to the sources alone to a rounding per hop."""
+    lat, u = _lattice(ovl, ctx, dims, 19)
+    psi = synth.gaussian_source(dims, 20, nrhs=nrhs)
+    vol = int(np.prod(dims))
+    nat = torch.from_numpy(np.ascontiguousarray(psi.reshape(nrhs, vol, 12).transpose(0, 2, 1))).to(torch.complex64)
+    lf = ovl.OVL_NATIVE | (ovl.OVL_LINKS_F16R12 if links == "f16" else ovl.OVL_LINKS_F32)
+    for flags in (ovl.OVL_GAMMA5, ovl.OVL_DAGGER):
+        ref = np.stack([_ref(u, psi[r], 0.3, flags, ovl, -1) for r in range(nrhs)]).reshape(nrhs, vol, 12)
+        for skip in (0, 1):
+            inp = torch.empty(nat.numel() + skip, dtype=torch.complex64, device="cuda")[skip:].view(nat.shape)
+            out = torch.empty(nat.numel() + skip, dtype=torch.complex64, device="cuda")[skip:].view(nat.shape)
+            inp.copy_(nat)
+            ovl.ovl_apply_DW(lat, -2.0, 0.3, flags | lf, inp, out)
+            got = out.cpu().numpy().transpose(0, 2, 1)
+            assert np.abs(got - ref).max() / np.abs(ref).max() < tol
+            for r in range(nrhs):
+                one = torch.empty_like(inp[r])
+                ovl.ovl_apply_DW(lat, -2.0, 0.3, flags | lf, inp[r].clone(), one)
+                assert np.abs(one.cpu().numpy().T - got[r]).max() <= 8 * 2.0 ** -23 * np.abs(ref).max()
+    ovl.ovl_destroy_lattice(lat)
