@@ -244,7 +244,7 @@ struct MsDev {
 
 struct MsVecs {
   void *r = nullptr, *rt = nullptr, *p = nullptr, *pt = nullptr;  // [nrhs][12][V]
-  void *t = nullptr, *tt = nullptr, *q = nullptr, *qt = nullptr;  // [nrhs][12][V]
+  void *t = nullptr, *tt = nullptr;                               // [nrhs][12][V]
   void* ps = nullptr;          // [nrhs][s][12][V] shifted directions
   double2* X = nullptr;        // [nrhs][12][V] FP64 sum_i omega_i x^(i)
   double2* xp = nullptr;       // [nrhs][12][V] FP64 x_P (nullptr without deflation)
@@ -255,7 +255,7 @@ struct MsVecs {
 
 cudaError_t launch_ms_start(const Geom& g, bool f64, const MsDev& ms, const MsVecs& v, const double2* b, int m,
                             const double2* R, const double2* L, const double* lam_sign, double2* dots, cudaStream_t st);
-// One iteration (four launches). With timing events (may be null): ev[0] before the first
+// One iteration (three launches). With timing events (may be null): ev[0] before the first
 // pair stencil, ev[1] after it, ev[2] before the direction update, ev[3] after it.
 // Whether the multishift iteration uses the eight-threads-per-site stencils (from the pair shape of
 // (volume, key), key = link format, 0 for FP64); the solvers key their cached graphs on it.

@@ -1,11 +1,10 @@
 // Multishift BiCG kernels (Algorithm 3 on M = A^2, A = H_W(mu); Section 5's rational sign).
 //
-// One iteration k is four launches:
-//   pair1:  t = A p,  t~ = A^H p~                                   (A^H = H_W(-mu))
-//   pair2:  q = A t - s1 p = (M - s1) p,  q~ = A^H t~ - s1 p~;  alpha_k = rho / (p~^H q);
+// One iteration k is three launches:
+//   pair1:  t = A p,  t~ = A^H p~  (A^H = H_W(-mu));  alpha_k = rho / (t~^H t - s1 p~^H p);
 //           last block: zeta^i_{k+1}, alpha^i_k for every live shift
-//   update: r -= alpha_k q,  r~ -= conj(alpha_k) q~;  rho' = r~^H r, |r|;
-//           last block: beta_k = rho'/rho, beta^i_k = beta_k (zeta^i_{k+1}/zeta^i_k)^2,
+//   pair2:  r -= alpha_k q, q = A t - s1 p = (M - s1) p;  r~ -= conj(alpha_k) q~, q~ = A^H t~ - s1 p~;
+//           rho' = r~^H r, |r|; last block: beta_k = rho'/rho, beta^i_k = beta_k (zeta^i_{k+1}/zeta^i_k)^2,
 //           shifts with |zeta^i_{k+1}| |r| <= tol |r_0| are retired after this step
 //   dirs:   X += sum_i omega_i alpha^i_k p^i;  p^i = zeta^i_{k+1} r + beta^i_k p^i;
 //           p = r + beta_k p,  p~ = r~ + conj(beta_k) p~
@@ -118,7 +117,7 @@ __device__ __forceinline__ MsAlphaIn ms_alpha_inputs(const MsDev& ms, int rhs) {
   return in;
 }
 
-// last block of pair2: alpha_k, then zeta^i_{k+1} and alpha^i_k of the live shifts
+// last block of pair1: alpha_k, then zeta^i_{k+1} and alpha^i_k of the live shifts
 __device__ __forceinline__ void ms_alpha_and_shifts(MsDev& ms, int rhs, const double (&pv)[4], const MsAlphaIn& in) {
   __shared__ zd alpha_sh;
   __shared__ int bad;
@@ -165,217 +164,270 @@ __device__ __forceinline__ void ms_alpha_and_shifts(MsDev& ms, int rhs, const do
   }
 }
 
-// pair1 (MODE 0): t = A p, t~ = A^H p~.  pair2 (MODE 1): q = A t - s1 p, q~ = A^H t~ - s1 p~, p~^H q.
+struct MsBetaIn {
+  double tol, r0;
+  zd rho, z1, z2;  // rho_k, zeta^t_k, zeta^t_{k+1}
+  int act;
+};
+__device__ __forceinline__ MsBetaIn ms_beta_inputs(const MsDev& ms, int rhs) {
+  MsBetaIn in{};
+  const double2* sd = ms.seed + (size_t)rhs * 8;
+  const int t = lin_tid();
+  in.tol = ms.tolv ? ms.tolv[rhs] : ms.tol;
+  in.rho = ldc<double>(sd, 0);
+  in.r0 = sd[4].x;
+  if (t < ms.s) {
+    const size_t si = (size_t)rhs * ms.s + t;
+    in.act = ms.active[si];
+    in.z1 = ldc<double>(ms.zeta + si * 3, 1);
+    in.z2 = ldc<double>(ms.zeta + si * 3, 2);
+  }
+  return in;
+}
+
+// last block of pair2: rho_{k+1} and |r_{k+1}| (pv), beta_k, the shifts' beta^i_k and states
+__device__ __forceinline__ void ms_beta_and_status(MsDev& ms, int rhs, const double (&pv)[4], const MsBetaIn& in) {
+  const int t = lin_tid();
+  double2* sd = ms.seed + (size_t)rhs * 8;
+  __shared__ zd beta_sh;
+  __shared__ double r2_sh;
+  __shared__ int live;
+  if (t == 0) {
+    zd rhon = mk(pv[0], pv[1]);
+    double rr = norm2(in.rho);
+    zd beta = rr > 0 ? (1.0 / rr) * (rhon * conj(in.rho)) : mk(0.0, 0.0);
+    double rn = sqrt(pv[2]);
+    beta_sh = beta;
+    r2_sh = pv[2];
+    live = 0;
+    sd[0] = make_double2(rhon.re, rhon.im);
+    sd[2] = sd[1];  // alpha_{k-1} <- alpha_k
+    sd[3] = make_double2(beta.re, beta.im);
+    sd[5] = make_double2(beta.re, beta.im);
+    sd[4].y = rn;
+    ms.k[rhs] += 1;
+    // breakdown of the BiCG recurrence (rho' = 0 while r is not small) or non-finite values
+    if (!(rn < 1e300) || !(norm2(rhon) < 1e300) || (norm2(rhon) == 0.0 && rn > in.tol * sd[4].x))
+      ms.status[rhs] = 1;
+  }
+  __syncthreads();
+  const zd beta = beta_sh;
+  const double r2 = r2_sh, lim = (in.tol * in.r0) * (in.tol * in.r0);
+  int mylive = 0;
+  for (int i = t; i < ms.s; i += lin_nthreads()) {
+    const size_t si = (size_t)rhs * ms.s + i;
+    const bool mine = i == t;
+    if (!(mine ? in.act : ms.active[si])) continue;
+    double2* z = ms.zeta + si * 3;
+    const zd z0 = mine ? in.z1 : ldc<double>(z, 1), zp = mine ? in.z2 : ldc<double>(z, 2);
+    double z0n = norm2(z0);
+    zd ratio = z0n > 0 ? (1.0 / z0n) * (zp * conj(z0)) : mk(0.0, 0.0);
+    zd bi = beta * (ratio * ratio);
+    ms.bsh[si] = make_double2(bi.re, bi.im);
+    z[0] = make_double2(z0.re, z0.im);
+    z[1] = make_double2(zp.re, zp.im);
+    if (norm2(zp) * r2 <= lim)  // |zeta^i_{k+1}| |r_{k+1}| <= tol |r_0|, on squares
+      ms.active[si] = 2;  // this step's direction update is its last
+    else
+      mylive = 1;
+  }
+  if (mylive) atomicOr(&live, 1);
+  __syncthreads();
+  if (t == 0 && !live && ms.status[rhs] == 0) ms.status[rhs] = 4;
+}
+
+// pair1 (MODE 0): t = A p, t~ = A^H p~, and the denominator of alpha: with q = (A^2 - s1) p,
+// p~^H q = t~^H t - s1 p~^H p, so alpha is known before q is.
+// pair2 (MODE 1): r -= alpha (A t - s1 p), r~ -= conj(alpha) (A^H t~ - s1 p~) as q comes out of the stencil, and
+// rho' = r~^H r, |r|^2. The two roles of a site (p and p~ side) exchange components through shared memory for
+// the products and share their float-float sums: the p side takes |r|^2 and colour 0, the other the rest.
+// With the denominator from q itself, q and q~ were written here and read back by a kernel of their own: 22 vector
+// passes a step in a correction instead of 18, and 16^4, 4 sources, 20 poles took 636 ms instead of 555 (FP32 with
+// 5 blocks per SM, 96 registers; 738 at 228 registers, 561 at 80).
+template <class R, int MODE>
+struct MsPairSum {
+  static constexpr int kValues = MODE == 0 ? 2 : 3;
+  Red<R> acc[kValues];
+  __device__ __forceinline__ void dot(cplx<R> y, cplx<R> x) {  // y^H x
+    acc[0].dot2(y.re, x.re, y.im, x.im);
+    acc[1].dot2(y.re, x.im, -y.im, x.re);
+  }
+  // The block's sums published, and the last block's share of the recurrence. (Its inputs are loaded after
+  // the sum: held across it they cost the whole stencil kernel registers, 80 -> 106, and occupancy.)
+  __device__ __forceinline__ void finish(MsDev& ms, int rhs) {
+    double tot[kValues];
+    block_reduce<R, kValues>(acc, tot);
+    double* part = ms.part + (size_t)rhs * ms.nblk * 4;
+    double pv[4] = {tot[0], tot[1], MODE == 0 ? 0.0 : tot[kValues - 1], 0.0};
+    if (publish_partials<4>(pv, part, ms.count + rhs)) {
+      reduce_partials<4>(part, gridDim.x, pv);
+      if (MODE == 0)
+        ms_alpha_and_shifts(ms, rhs, pv, ms_alpha_inputs(ms, rhs));
+      else
+        ms_beta_and_status(ms, rhs, pv, ms_beta_inputs(ms, rhs));
+    }
+  }
+};
+
 template <class R, int LF, int MODE>
-__global__ void __launch_bounds__(2 * kPairSites) k_ms_pair(Geom g, Links U, typename HopsOf<R>::T cp,
+__global__ void __launch_bounds__(2 * kPairSites, sizeof(R) == 8 ? 3 : 5) k_ms_pair(Geom g, Links U, typename HopsOf<R>::T cp,
                                                             typename HopsOf<R>::T cm, MsDev ms,
                                                             MsVecs v) {
   using T = typename V2<R>::T;
+  __shared__ cplx<R> xch[12][kPairSites];
   const int rhs = blockIdx.y;
   if (MODE == 0 && blockIdx.x == 0 && lin_tid() == 0 && ms.status[rhs] == 4) ms.status[rhs] = 2;
   if (ms.status[rhs] != 0) return;
   const size_t n = (size_t)12 * g.vol;
-  const int s = blockIdx.x * kPairSites + threadIdx.x;
-  const bool is_t = threadIdx.y == 1;
+  const int tx = threadIdx.x, s = blockIdx.x * kPairSites + tx;
+  const bool is_t = threadIdx.y == 1, live = s < g.vol;
   const T* in = (const T*)(MODE == 0 ? (is_t ? v.pt : v.p) : (is_t ? v.tt : v.t)) + voff<R>(rhs, n);
-  T* out = (T*)(MODE == 0 ? (is_t ? v.tt : v.t) : (is_t ? v.qt : v.q)) + voff<R>(rhs, n);
+  const T* p = (const T*)v.p + voff<R>(rhs, n);
+  const T* pt = (const T*)v.pt + voff<R>(rhs, n);
   const double s1d = ms.sig1v ? ms.sig1v[rhs] : ms.sigma1;
-  R s1v[1];
+  R s1v[1], akv[2];
   scalars_in<R, 1>(&s1d, s1v);
-  Red<R> acc[2];
-  if (s < g.vol) {
+  if (MODE == 1) scalars_in<R, 2>((const double*)(ms.seed + (size_t)rhs * 8 + 1), akv);
+  const R s1 = s1v[0];
+  MsPairSum<R, MODE> sum;
+  cplx<R> x[12];
+  if (live) {
     Spin<R> o;
     stencil_site<LF, R>(g, U, s, is_t ? cm : cp, in, o);
-    const R s1 = s1v[0];
-    const T* pp = (const T*)(is_t ? v.pt : v.p) + voff<R>(rhs, n);
-    const T* ptl = (const T*)v.pt + voff<R>(rhs, n);
-    // MODE 1: every load before the first store (stores that might alias would otherwise
-    // serialise twelve memory round trips)
-    cplx<R> pv[12], tv[12];
-    if (MODE == 1) {
+#pragma unroll
+    for (int c = 0; c < 12; ++c) x[c] = c >= 6 ? -o.c[c / 3][c % 3] : o.c[c / 3][c % 3];  // gamma5
+    if constexpr (MODE == 0) {
+      T* out = (T*)(is_t ? v.tt : v.t) + voff<R>(rhs, n);
+      if (is_t) {
+        if (s1 != (R)0) {
+          cplx<R> a = mk<R>(0, 0);
+#pragma unroll
+          for (int c = 0; c < 12; ++c)
+            a = a + cdot(ldc<R>(pt, (size_t)c * g.vol + s), ldc<R>(p, (size_t)c * g.vol + s));
+          sum.acc[0].add(-s1 * a.re);
+          sum.acc[1].add(-s1 * a.im);
+        }
+#pragma unroll
+        for (int c = 0; c < 12; ++c) xch[c][tx] = x[c];
+      }
+#pragma unroll
+      for (int c = 0; c < 12; ++c) stc<R>(out, (size_t)c * g.vol + s, x[c]);
+    } else {
+      const cplx<R> ak = mk<R>(akv[0], is_t ? -akv[1] : akv[1]);
+      const T* pp = is_t ? pt : p;
+      T* r = (T*)(is_t ? v.rt : v.r) + voff<R>(rhs, n);
+      // every load before the first store (stores that might alias would otherwise serialise twelve
+      // memory round trips)
+      cplx<R> pv[12], rv[12];
 #pragma unroll
       for (int c = 0; c < 12; ++c) {
         pv[c] = ldc<R>(pp, (size_t)c * g.vol + s);
-        tv[c] = is_t ? mk<R>(0, 0) : ldc<R>(ptl, (size_t)c * g.vol + s);
+        rv[c] = ldc<R>(r, (size_t)c * g.vol + s);
       }
-    }
-    cplx<R> a = mk<R>(0, 0);
 #pragma unroll
-    for (int c = 0; c < 12; ++c) {
-      cplx<R> x = o.c[c / 3][c % 3];
-      if (c >= 6) x = -x;  // gamma5
-      if (MODE == 1) {
-        x = x - s1 * pv[c];
-        if (!is_t) a = a + cdot(tv[c], x);
+      for (int c = 0; c < 12; ++c) {
+        x[c] = cmsub(rv[c], ak, x[c] - s1 * pv[c]);
+        stc<R>(r, (size_t)c * g.vol + s, x[c]);
+        if (is_t == (c % 3 == 0)) xch[c][tx] = x[c];
       }
-      stc<R>(out, (size_t)c * g.vol + s, x);
     }
-    acc[0].add(a.re);
-    acc[1].add(a.im);
   }
-  if (MODE == 0) return;
-  double tot[2];
-  block_reduce<R, 2>(acc, tot);
-  double* part = ms.part + (size_t)rhs * ms.nblk * 4;
-  double pv[4] = {tot[0], tot[1], 0, 0};
-  if (publish_partials<4>(pv, part, ms.count + rhs)) {
-    // (the inputs are loaded after the sum here: held across it they cost the whole stencil
-    // kernel registers, 80 -> 106, and occupancy)
-    reduce_partials<4>(part, gridDim.x, pv);
-    ms_alpha_and_shifts(ms, rhs, pv, ms_alpha_inputs(ms, rhs));
+  __syncthreads();
+  if (live) {
+    if constexpr (MODE == 0) {
+      if (!is_t) {
+        cplx<R> a = mk<R>(0, 0);
+#pragma unroll
+        for (int c = 0; c < 12; ++c) a = a + cdot(xch[c][tx], x[c]);
+        sum.acc[0].add(a.re);
+        sum.acc[1].add(a.im);
+      }
+    } else if (is_t) {
+#pragma unroll
+      for (int c = 0; c < 12; ++c)
+        if (c % 3 != 0) sum.dot(x[c], xch[c][tx]);
+    } else {
+#pragma unroll
+      for (int c = 0; c < 12; ++c) {
+        if (c % 3 == 0) sum.dot(xch[c][tx], x[c]);
+        sum.acc[2].dot2(x[c].re, x[c].re, x[c].im, x[c].im);
+      }
+    }
   }
+  sum.finish(ms, rhs);
 }
 
-// pair1 / pair2 with 8 threads per site (small lattices): see pair_split.
+// The same with eight threads per site (pair_split): each thread finishes one spin of its site.
 template <class R, int LF, int MODE>
 __global__ void __launch_bounds__(8 * kSplitSites) k_ms_pair_split(Geom g, Links U, typename HopsOf<R>::T cp,
                                                                    typename HopsOf<R>::T cm,
                                                                    MsDev ms, MsVecs v) {
   using T = typename V2<R>::T;
   __shared__ SplitSmem<R> sm;
+  __shared__ cplx<R> xch[12][kSplitSites];
   const int rhs = blockIdx.y;
   if (MODE == 0 && blockIdx.x == 0 && lin_tid() == 0 && ms.status[rhs] == 4) ms.status[rhs] = 2;
   if (ms.status[rhs] != 0) return;
   const size_t n = (size_t)12 * g.vol;
   const T* in0 = (const T*)(MODE == 0 ? v.p : v.t) + voff<R>(rhs, n);
   const T* in1 = (const T*)(MODE == 0 ? v.pt : v.tt) + voff<R>(rhs, n);
+  const T* p = (const T*)v.p + voff<R>(rhs, n);
+  const T* pt = (const T*)v.pt + voff<R>(rhs, n);
   const double s1d = ms.sig1v ? ms.sig1v[rhs] : ms.sigma1;
-  R s1v[1];
+  R s1v[1], akv[2];
   scalars_in<R, 1>(&s1d, s1v);
+  if (MODE == 1) scalars_in<R, 2>((const double*)(ms.seed + (size_t)rhs * 8 + 1), akv);
   const R s1 = s1v[0];
-  Red<R> acc[2];
-  // each thread finishes one spin (three colours) of its site: see pair_split
+  MsPairSum<R, MODE> sum;
+  cplx<R> x[3];
   pair_split<R, LF, typename HopsOf<R>::T>(g, U, cp, cm, in0, in1, sm, [&](int which, int s, int sp, cplx<R> (&o)[3]) {
-    T* out = (T*)(MODE == 0 ? (which ? v.tt : v.t) : (which ? v.qt : v.q)) + voff<R>(rhs, n);
-    const T* pp = (const T*)(which ? v.pt : v.p) + voff<R>(rhs, n);
-    const T* ptl = (const T*)v.pt + voff<R>(rhs, n);
     const R g5 = sp >= 2 ? (R)-1 : (R)1;
-    cplx<R> pv[3], tv[3];  // loads first (see k_ms_pair)
-    if (MODE == 1) {
+    if constexpr (MODE == 0) {
+      T* out = (T*)(which ? v.tt : v.t) + voff<R>(rhs, n);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        const size_t e = (size_t)(sp * 3 + a) * g.vol + s;
+        x[a] = g5 * o[a];
+        if (which) {
+          if (s1 != (R)0) sum.dot(-s1 * ldc<R>(pt, e), ldc<R>(p, e));
+          xch[sp * 3 + a][threadIdx.x] = x[a];
+        }
+        stc<R>(out, e, x[a]);
+      }
+    } else {
+      const cplx<R> ak = mk<R>(akv[0], which ? -akv[1] : akv[1]);
+      const T* pp = which ? pt : p;
+      T* r = (T*)(which ? v.rt : v.r) + voff<R>(rhs, n);
+      cplx<R> pv[3], rv[3];  // loads first (see k_ms_pair)
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
         pv[a] = ldc<R>(pp, (size_t)(sp * 3 + a) * g.vol + s);
-        tv[a] = which ? mk<R>(0, 0) : ldc<R>(ptl, (size_t)(sp * 3 + a) * g.vol + s);
+        rv[a] = ldc<R>(r, (size_t)(sp * 3 + a) * g.vol + s);
       }
-    }
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      cplx<R> x = g5 * o[a];
-      if (MODE == 1) {
-        x = x - s1 * pv[a];
-        if (!which) {
-          acc[0].dot2(tv[a].re, x.re, tv[a].im, x.im);
-          acc[1].dot2(tv[a].re, x.im, -tv[a].im, x.re);
-        }
+      for (int a = 0; a < 3; ++a) {
+        x[a] = cmsub(rv[a], ak, g5 * o[a] - s1 * pv[a]);
+        stc<R>(r, (size_t)(sp * 3 + a) * g.vol + s, x[a]);
+        if ((which == 1) == (a == 0)) xch[sp * 3 + a][threadIdx.x] = x[a];
       }
-      stc<R>(out, (size_t)(sp * 3 + a) * g.vol + s, x);
     }
   });
-  if (MODE == 0) return;
-  double tot[2];
-  block_reduce<R, 2>(acc, tot);
-  double* part = ms.part + (size_t)rhs * ms.nblk * 4;
-  double pv[4] = {tot[0], tot[1], 0, 0};
-  if (publish_partials<4>(pv, part, ms.count + rhs)) {
-    // (the inputs are loaded after the sum here: held across it they cost the whole stencil
-    // kernel registers, 80 -> 106, and occupancy)
-    reduce_partials<4>(part, gridDim.x, pv);
-    ms_alpha_and_shifts(ms, rhs, pv, ms_alpha_inputs(ms, rhs));
-  }
-}
-
-// update: r -= alpha q, r~ -= conj(alpha) q~; rho' = r~^H r, |r|^2 (elt elements per thread)
-template <class R>
-__global__ void __launch_bounds__(kVecBlock) k_ms_update(Geom g, MsDev ms, MsVecs v, int elt) {
-  using T = typename V2<R>::T;
-  const int rhs = blockIdx.y;
-  if (ms.status[rhs] != 0) return;
-  const size_t n = (size_t)12 * g.vol;
-  double2* sd = ms.seed + (size_t)rhs * 8;
-  R akr[2];
-  scalars_in<R, 2>((const double*)(sd + 1), akr);
-  const cplx<R> a = mk<R>(akr[0], akr[1]), ac = mk<R>(akr[0], -akr[1]);
-  T* r = (T*)v.r + voff<R>(rhs, n);
-  T* rt = (T*)v.rt + voff<R>(rhs, n);
-  const T* q = (const T*)v.q + voff<R>(rhs, n);
-  const T* qt = (const T*)v.qt + voff<R>(rhs, n);
-  Red<R> red[3];
-  for (int k = 0; k < elt; ++k) {
-    const size_t e = ((size_t)blockIdx.x * elt + k) * blockDim.x + threadIdx.x;
-    if (e >= n) break;
-    cplx<R> x = cmsub(ldc<R>(r, e), a, ldc<R>(q, e));
-    cplx<R> y = cmsub(ldc<R>(rt, e), ac, ldc<R>(qt, e));
-    stc<R>(r, e, x);
-    stc<R>(rt, e, y);
-    red[0].add(fma(y.re, x.re, y.im * x.im));  // (y^H x).re
-    red[1].add(fma(y.re, x.im, -(y.im * x.re)));
-    red[2].add(fma(x.re, x.re, x.im * x.im));
-  }
-  double acc[3];
-  block_reduce<R, 3>(red, acc);
-  double* part = ms.part + (size_t)rhs * ms.nblk * 4;
-  double pv[4] = {acc[0], acc[1], acc[2], 0};
-  if (publish_partials<4>(pv, part, ms.count + rhs)) {
-    // this block's inputs first (their latency overlaps the sum): rho_k, |r_0|, shift t's state
-    const int t = lin_tid();
-    const double tl = ms.tolv ? ms.tolv[rhs] : ms.tol;
-    const zd rho = ldc<double>(sd, 0);
-    const double r0 = sd[4].x;
-    int act0 = 0;
-    zd z1 = mk(0.0, 0.0), z2 = mk(0.0, 0.0);
-    if (t < ms.s) {
-      const size_t si = (size_t)rhs * ms.s + t;
-      act0 = ms.active[si];
-      z1 = ldc<double>(ms.zeta + si * 3, 1);
-      z2 = ldc<double>(ms.zeta + si * 3, 2);
+  __syncthreads();
+  if (blockIdx.x * kSplitSites + threadIdx.x < g.vol) {
+    const int which = threadIdx.y >> 2, c0 = (threadIdx.y & 3) * 3;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      const cplx<R> y = xch[c0 + a][threadIdx.x];
+      if constexpr (MODE == 0) {
+        if (!which) sum.dot(y, x[a]);
+      } else {
+        if (which && a != 0) sum.dot(x[a], y);
+        if (!which && a == 0) sum.dot(y, x[a]);
+        if (!which) sum.acc[2].dot2(x[a].re, x[a].re, x[a].im, x[a].im);
+      }
     }
-    reduce_partials<4>(part, gridDim.x, pv);
-    __shared__ zd beta_sh;
-    __shared__ double r2_sh;
-    __shared__ int live;
-    if (t == 0) {
-      zd rhon = mk(pv[0], pv[1]);
-      double rr = norm2(rho);
-      zd beta = rr > 0 ? (1.0 / rr) * (rhon * conj(rho)) : mk(0.0, 0.0);
-      double rn = sqrt(pv[2]);
-      beta_sh = beta;
-      r2_sh = pv[2];
-      live = 0;
-      sd[0] = make_double2(rhon.re, rhon.im);
-      sd[2] = sd[1];  // alpha_{k-1} <- alpha_k
-      sd[3] = make_double2(beta.re, beta.im);
-      sd[5] = make_double2(beta.re, beta.im);
-      sd[4].y = rn;
-      ms.k[rhs] += 1;
-      // breakdown of the BiCG recurrence (rho' = 0 while r is not small) or non-finite values
-      if (!(rn < 1e300) || !(norm2(rhon) < 1e300) || (norm2(rhon) == 0.0 && rn > tl * sd[4].x))
-        ms.status[rhs] = 1;
-    }
-    __syncthreads();
-    const zd beta = beta_sh;
-    const double r2 = r2_sh, lim = (tl * r0) * (tl * r0);
-    int mylive = 0;
-    for (int i = t; i < ms.s; i += lin_nthreads()) {
-      const size_t si = (size_t)rhs * ms.s + i;
-      const bool mine = i == t;
-      if (!(mine ? act0 : ms.active[si])) continue;
-      double2* z = ms.zeta + si * 3;
-      const zd z0 = mine ? z1 : ldc<double>(z, 1), zp = mine ? z2 : ldc<double>(z, 2);
-      double z0n = norm2(z0);
-      zd ratio = z0n > 0 ? (1.0 / z0n) * (zp * conj(z0)) : mk(0.0, 0.0);
-      zd bi = beta * (ratio * ratio);
-      ms.bsh[si] = make_double2(bi.re, bi.im);
-      z[0] = make_double2(z0.re, z0.im);
-      z[1] = make_double2(zp.re, zp.im);
-      if (norm2(zp) * r2 <= lim)  // |zeta^i_{k+1}| |r_{k+1}| <= tol |r_0|, on squares
-        ms.active[si] = 2;  // this step's direction update is its last
-      else
-        mylive = 1;
-    }
-    if (mylive) atomicOr(&live, 1);
-    __syncthreads();
-    if (t == 0 && !live && ms.status[rhs] == 0) ms.status[rhs] = 4;
   }
+  sum.finish(ms, rhs);
 }
 
 // dirs: X += sum_i omega_i alpha^i p^i; p^i = zeta^i r + beta^i p^i; p, p~ updates.
@@ -552,7 +604,6 @@ static cudaError_t ms_step_t(const Geom& g, const Links& U, double m_w, double m
   const typename HopsOf<R>::T cp = hops_of<R>(m_w, mu), cm = hops_of<R>(m_w, -mu);
   dim3 sgrid((g.vol + kSplitSites - 1) / kSplitSites, ms.nrhs), sblock(kSplitSites, 8);
   const bool split = ms_pair_split(g, sizeof(R) == 8 ? 0 : LF);
-  const int elt = vec_elts(g, ms.nrhs, sizeof(R) == 8);
   cudaError_t e;
   if (ev && (e = record_timing(ev[0], st))) return e;
   e = split ? launch_plain(k_ms_pair_split<R, LF, 0>, sgrid, sblock, st, g, U, cp, cm, ms, v)
@@ -562,7 +613,6 @@ static cudaError_t ms_step_t(const Geom& g, const Links& U, double m_w, double m
   e = split ? launch_plain(k_ms_pair_split<R, LF, 1>, sgrid, sblock, st, g, U, cp, cm, ms, v)
             : launch_plain(k_ms_pair<R, LF, 1>, pgrid, pblock, st, g, U, cp, cm, ms, v);
   if (e) return e;
-  if ((e = launch_plain(k_ms_update<R>, dim3(vec_blocks(g, elt), ms.nrhs), dim3(kVecBlock), st, g, ms, v, elt))) return e;
   if (ev && (e = record_timing(ev[2], st))) return e;
   if (sizeof(R) == 4 && ms.s == 1 && ms.sig1v) {  // a correction batch (each system its own shift as the seed)
     const size_t pairs = (size_t)6 * g.vol;

@@ -100,8 +100,8 @@ static ovl_status ensure_mws(ovl_lattice* lat, int nrhs, int s, bool f64, int m,
     off += al256(b);
     return o;
   };
-  size_t o_vec[8];
-  for (int i = 0; i < 8; ++i) o_vec[i] = take((size_t)nrhs * n * elt);
+  size_t o_vec[6];
+  for (int i = 0; i < 6; ++i) o_vec[i] = take((size_t)nrhs * n * elt);
   size_t o_ps = take((size_t)nrhs * s * n * elt);
   size_t o_X = take((size_t)nrhs * n * 16);
   size_t o_xp = take((size_t)nrhs * n * 16);
@@ -140,8 +140,8 @@ static ovl_status ensure_mws(ovl_lattice* lat, int nrhs, int s, bool f64, int m,
   size_t o_res = take(gq * rn * 16), o_t1 = take(gq * rn * 16), o_t2 = take(gq * rn * 16), o_ec = take(gq * rn * 16);
   size_t o_rp = take(std::max<size_t>(1, gq) * vec_blocks(lat->g) * 8), o_ro = take(std::max<size_t>(1, gq) * 8),
          o_oz = take(16), o_rc = take(std::max<size_t>(1, gq) * 4);
-  size_t o_gvec[9];
-  for (int i = 0; i < 9; ++i) o_gvec[i] = take(gq * rn * 8);
+  size_t o_gvec[7];
+  for (int i = 0; i < 7; ++i) o_gvec[i] = take(gq * rn * 8);
   size_t o_gX = take(gq * rn * 16), o_gk = take(gq * 4), o_gst = take(gq * 4), o_gseed = take(gq * 8 * 16),
          o_gz = take(gq * 3 * 16), o_ga = take(gq * 16), o_gb = take(gq * 16), o_gact = take(gq * 4),
          o_gpa = take(gq * nblk * 4 * 8), o_gcn = take(gq * 4), o_sga = take((size_t)s * 8), o_gsig = take(gq * 8),
@@ -163,8 +163,8 @@ static ovl_status ensure_mws(ovl_lattice* lat, int nrhs, int s, bool f64, int m,
     return OVL_ENOMEM;
   }
   char* b = w->dev;
-  void** vp[8] = {&w->v.r, &w->v.rt, &w->v.p, &w->v.pt, &w->v.t, &w->v.tt, &w->v.q, &w->v.qt};
-  for (int i = 0; i < 8; ++i) *vp[i] = b + o_vec[i];
+  void** vp[6] = {&w->v.r, &w->v.rt, &w->v.p, &w->v.pt, &w->v.t, &w->v.tt};
+  for (int i = 0; i < 6; ++i) *vp[i] = b + o_vec[i];
   w->v.ps = b + o_ps;
   w->v.X = (double2*)(b + o_X);
   w->v.xp = (double2*)(b + o_xp);
@@ -198,8 +198,8 @@ static ovl_status ensure_mws(ovl_lattice* lat, int nrhs, int s, bool f64, int m,
     w->t1 = (double2*)(b + o_t1);
     w->t2 = (double2*)(b + o_t2);
     w->ecan = (double2*)(b + o_ec);
-    void** gp[9] = {&w->gv.r, &w->gv.rt, &w->gv.p, &w->gv.pt, &w->gv.t, &w->gv.tt, &w->gv.q, &w->gv.qt, &w->gv.ps};
-    for (int i = 0; i < 9; ++i) *gp[i] = b + o_gvec[i];
+    void** gp[7] = {&w->gv.r, &w->gv.rt, &w->gv.p, &w->gv.pt, &w->gv.t, &w->gv.tt, &w->gv.ps};
+    for (int i = 0; i < 7; ++i) *gp[i] = b + o_gvec[i];
     w->gv.X = (double2*)(b + o_gX);
     MsDev& gm = w->gms;
     gm.nrhs = grp;
@@ -371,7 +371,7 @@ ovl_status solve_multishift(ovl_lattice* lat, const ovl_sign_params* p, int nrhs
   int launches = 1 + (m > 0 ? 1 : 0) + 2;  // start (+ deflation dots), final stencil and finish
   // a chunk = one iteration launched directly, then a graph of the rest (events: see above)
   auto run_chunk = [&](int ns, int q) -> cudaError_t {
-    launches += 4 * ns;
+    launches += 3 * ns;
     const bool graph = use_graph && ns == chunk;
     cudaError_t e = launch_ms_step(g, U, lf, f64, p->m_W, p->mu, ms, v, st, graph ? nullptr : w->tev[q]);
     if (e != cudaSuccess || ns == 1) return e;
@@ -533,7 +533,7 @@ ovl_status solve_multishift(ovl_lattice* lat, const ovl_sign_params* p, int nrhs
           }
           if (e) return e;
           it += ns;
-          launches += 4 * ns;
+          launches += 3 * ns;
           if ((e = cudaMemcpyAsync(w->h_gst + (size_t)slot * grp, gm.status, gn * 4, cudaMemcpyDeviceToHost, st)))
             return e;
           if ((e = cudaEventRecord(w->ev[slot], st))) return e;
@@ -622,10 +622,10 @@ ovl_status solve_multishift(ovl_lattice* lat, const ovl_sign_params* p, int nrhs
 size_t multishift_footprint(int vol, int nrhs, int s, bool f64, bool refine) {
   const size_t n = (size_t)12 * vol, elt = f64 ? 16 : 8, nr = (size_t)nrhs;
   const size_t slots = (n + kVecBlock - 1) / kVecBlock + kMaxFillSMs;  // partial_slots
-  size_t b = nr * n * (8 * elt + (size_t)s * elt + 5 * 16) + nr * 16 * slots * 32;  // (deflation dots: m <= 16)
+  size_t b = nr * n * (6 * elt + (size_t)s * elt + 5 * 16) + nr * 16 * slots * 32;  // (deflation dots: m <= 16)
   if (refine) {
     const size_t gq = std::min<size_t>(nr * s, kRefineGroup);
-    b += nr * s * n * 16 + nr * n * 16 + gq * n * (4 * 16 + 9 * 8 + 16) + gq * slots * 32;
+    b += nr * s * n * 16 + nr * n * 16 + gq * n * (4 * 16 + 7 * 8 + 16) + gq * slots * 32;
   }
   return b + ((size_t)1 << 20);
 }

@@ -198,3 +198,35 @@ def test_corrections_on_ragged_volumes(ovl, ctx, dims):
     assert st == st64 == ovl.OVL_OK, info
     assert _rel(x, x64) < 4e-9
     ovl.ovl_destroy_lattice(lat)
+
+
+@pytest.mark.parametrize("variant", [0, 1])
+@pytest.mark.parametrize("prec,k,tol", [("f64", 12, 1e-9), ("f32", 8, 1e-4), ("f16", 8, 1e-4)])
+def test_equal_k_both_stencil_shapes(ovl, ctx, variant, prec, k, tol):
+    """One and eight threads per site with the last block half filled, two sources, a seed shift: alpha from
+    (A^H p~)^H (A p) - s1 p~^H p and the residuals updated in the stencil, against the oracle's iterates at equal
+    k, to the bounds of the other equal-k comparisons (FP32: those of the direct method's)."""
+    dims = (2, 4, 6, 6)
+    u = synth.gauge_links(dims, 27)
+    b = synth.gaussian_source(dims, 28, nrhs=2)
+    lat = ovl.ovl_create_lattice(ctx, dims, -1)
+    ovl.ovl_set_links(lat, u, ovl.OVL_F64 | ovl.OVL_F32 | ovl.OVL_F16R12)
+    pr, key = {"f64": (ovl.OVL_PREC_F64, 0), "f32": (ovl.OVL_PREC_F32, 1), "f16": (ovl.OVL_PREC_F32_F16LINKS, 2)}[prec]
+    ovl.ovl_set_pair_variant(288, key, variant)
+    try:
+        # (single precision: a tolerance below its floor would start the reliable updates)
+        st, info, x = _solve(ovl, lat, b, mu=0.3, tol=0.0 if prec == "f64" else 1e-5, k_max=k, spec_lo=0.05,
+                             spec_hi=2.7, s=6, check_every=5, precision=pr)
+    finally:
+        ovl.ovl_set_pair_variant(288, key, -1)
+    ovl.ovl_destroy_lattice(lat)
+    from conftest import fp16_quantised
+    w, sg = rational.neuberger_scaled(6, rational.scale_and_d(*rational.circle_from_gap(0.05, 2.7))[0])
+    uq = fp16_quantised(u) if prec == "f16" else u
+    a, ah = deflation.sparse_hw(uq, dims, -2.0, 0.3), deflation.sparse_hw(uq, dims, -2.0, -0.3)
+    m, mh = a @ a, ah @ ah
+    last = deflation.sparse_hw(u, dims, -2.0, 0.3)  # x = A sum_i omega_i x^(i) is one FP64 stencil, FP64 links
+    for r in range(2):
+        assert info[r]["iterations"] == k
+        xs, _ = lanczos.multishift_iterates(lambda v: m @ v, lambda v: mh @ v, b[r].ravel(), b[r].ravel(), k, sg)
+        assert _rel(x[r].ravel(), last @ np.tensordot(w, xs, axes=1)) < tol
