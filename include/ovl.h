@@ -99,7 +99,10 @@ int64_t ovl_lattice_n(const ovl_lattice* lat);
  * into library-owned device copies in each format of the `formats` bit set (OVL_F64 is
  * always kept). Every format the lattice already holds from an earlier call is rewritten
  * from U as well, so no copy keeps the previous field. The caller's buffer may be freed on
- * return (the call synchronises).
+ * return (the call synchronises). Beside the FP64 links a fixed-point copy of the same size
+ * (576 bytes a site) is kept for the FP64 stencils; it is used if the field has a common scale:
+ * finite, every link's largest component at least a quarter of the largest of the field, and
+ * that within 2^-8 .. 2^8 (any SU(3) field). Other fields run FP64 arithmetic.
  * Errors: EINVAL, EBUSY (a solve is reading the links), ENOMEM, ECUDA. */
 ovl_status ovl_set_links(ovl_lattice* lat, const void* U, int32_t U_on_device, uint32_t formats);
 
@@ -211,8 +214,10 @@ ovl_status ovl_apply_sign(ovl_lattice* lat, const ovl_sign_params* p, int32_t nr
  * site's links loaded once per group (otherwise as 3). The multishift method runs 1, 4, 5 as its eight-thread stencil and the others as its
  * one-thread stencil. variant = -1
  * clears the entry: the next direct solve for that key times every shape on its own vectors and
- * keeps the fastest. Process-wide. All shapes compute the same step; results differ in the
- * rounding of the partial sums of alpha_j only.
+ * keeps the fastest. Process-wide. FP64 solves on fields with a common link scale (see
+ * ovl_set_links) keep their vectors in fixed point and have two shapes: 1, 4 and 5 four threads per
+ * site and stencil, the others one; results are the same bits. Otherwise all shapes compute the same
+ * step and results differ in the rounding of the partial sums of alpha_j only.
  * Errors: EINVAL (variant outside -1..8, volume < 1, unknown precision). */
 ovl_status ovl_set_pair_variant(int64_t volume, int32_t precision, int32_t variant);
 
@@ -225,7 +230,8 @@ int32_t ovl_get_pair_variant(int64_t volume, int32_t precision);
  * loops that must not call cudaMalloc/cudaFree. The paper has no counterpart: this is a
  * property of the library, not of the method. Same kernels and results as ovl_apply_sign
  * (method OVL_DIRECT_2SL); b and x are device buffers; runs on `stream` and synchronizes it.
- * All scratch lives in one static 64 MiB device array per GPU that loads the library, held
+ * All scratch lives in one static 64 MiB device array per GPU that loads the library (and 20 MiB
+ * beside it for the FP64 solve's fixed-point vectors, sized so as not to lower any limit), held
  * until the process exits; its address is looked up on the first call for each device (make
  * that first call before any stream capture) and again on each later call made outside a
  * capture. Calls share the array: calls that overlap on the GPU race. No CUDA graphs, streams,
