@@ -253,7 +253,10 @@ __global__ void __launch_bounds__(64) k_fx_begin(Geom g, LzDev lz, FxVecs fx, co
 // settles the previous step, block b > 0 takes chunk b - 1.
 // With 8.5 warps per SM (12^4) the latency of the loads is not hidden by other warps, so a hop's inputs are
 // copied to shared memory while the previous one is computed: the neighbour's 12 components per thread,
-// and the link's nine once for the two roles.
+// and the link's nine once for the two roles; what_j for the dot during the last hop (12^4 step 45.7 -> 44.2 us;
+// loaded where it is used, the end of the kernel took 9000 clocks instead of 4000). At 12^4 the pair takes
+// 34 us, two 20000-clock warps or three per scheduler. Two threads per site and role, or the last 40 of the 648
+// chunks split over twice the warps, were no faster (49.7, 44.5).
 struct FxSelf {
   int h, l, e;  // 1 / ks = (h 2^30 + l) 2^-59 2^e
 };
@@ -368,6 +371,9 @@ __global__ void __launch_bounds__(64 * T, T == 1 ? 5 : 1)
       }
       fx_half(k, p, false, h);
     }
+    if (T == 1 && i + 1 == NH && role == 0)  // what_j, in the thread's slots of the stage just read
+#pragma unroll
+      for (int a = 0; a < 12; ++a) copy_async(&sm.q[i & 1][a][tid], w + (size_t)a * g.vol);
     const FxC* u = &sm.u[k & 1][t][0][lane];
     fx_hop(k, E - eh, __any_sync(0xffffffffu, E != eh), h, [&](int a, int b) { return u[(a * 3 + b) * 32]; }, c, flip,
            acc);
@@ -402,7 +408,7 @@ __global__ void __launch_bounds__(64 * T, T == 1 ? 5 : 1)
       fx_split(((ai[a] + hn) >> rr) << rl, y.ih, y.il);
       if (live) out[(size_t)(sp * 3 + a) * g.vol + s] = y;
       if (role == 0) {
-        const FxC x = T == 1 ? w[(size_t)(sp * 3 + a) * g.vol] : sm.q[0][3 + a][tid];
+        const FxC x = T == 1 ? sm.q[(NH - 1) & 1][sp * 3 + a][tid] : sm.q[0][3 + a][tid];
         const int nh = -x.ih, nl = -x.il;  // conj(what)
         fx_mad(hr, x.rh, y.rh);
         fx_mad(hr, x.ih, y.ih);

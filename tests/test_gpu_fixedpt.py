@@ -109,7 +109,7 @@ def _solve(ovl, lat, b, variant, **kw):
     return xt.cpu().numpy(), [ovl.ovl_get_tridiag(lat, r) for r in range(len(b))]
 
 
-@pytest.mark.parametrize("dims", [(2, 2, 2, 2), (6, 2, 6, 6), (10, 8, 6, 12)])
+@pytest.mark.parametrize("dims", [(2, 2, 2, 2), (6, 2, 6, 6), (10, 8, 6, 12), (14, 10, 10, 10), (10, 10, 10, 10)])
 @pytest.mark.parametrize("two_pass", [0, 1])
 def test_lanczos_same_bits(ovl, ctx, dims, two_pass):
     k = 24
