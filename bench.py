@@ -155,9 +155,7 @@ FP64_PEAK_TFLOPS = 1.256
 # DRAM bytes (read + write) per launch of the dominant kernel from one ncu capture (cold L2, every
 # pass flushed), keyed (kernel, precision, lattice, nrhs, pair-stencil shape); the captures and their
 # commands are in profiles/. An entry is removed when its kernel changes.
-TRAFFIC = {
-    ("k_lz_pair", "f64", (12, 12, 12, 12), 1, 7): 20003840,  # k_lz_pair_dyn<double>: 20.003 MB read + 0.5 KB written
-}
+TRAFFIC = {}
 
 
 def _peaks():
@@ -524,8 +522,9 @@ def _roofline(wl, infos, fp64_peak, fp64_src):
                 "frac": (ach / fp64_peak) if ach else None, "traffic": traffic, "peak_source": fp64_src,
                 "algorithmic_flops_per_launch": flops,
                 "algorithmic_bytes_per_launch": pair_bytes("f64", vol, nr), "pair_variant": shape,
-                "note": "FP64 kernels are bound by GB300's FP64 pipe (ncu at 12^4: FP64 pipe 84% of active "
-                        "cycles in the pair stencil, 66-72% in the update)"}
+                "note": "the direct method's FP64 stencils run in fixed point on the integer pipe (FP64-accurate), "
+                        "so frac can exceed 1 of the FP64 pipe's peak; at 12^4 the pair stencil is bound by "
+                        "integer issue and load latency at two warps per scheduler"}
     byts = pair_bytes(prec, vol, nr)
     ach = byts / (t_pair * 1e-3) / 1e9 if t_pair else None
     return {"kernel": kernel, "bound": "hbm", "achieved": ach, "peak": peaks["hbm_gbs"], "unit": "GB/s",
