@@ -134,7 +134,6 @@ ovl_status ovl_destroy_lattice(ovl_lattice* lat) {
   free_multi_ws(lat->mws);
   if (lat->owns_links) {
     cudaFree(lat->u64);
-    cudaFree(lat->ufx);
     cudaFree(lat->u32);
     cudaFree(lat->u16);
     cudaFree(lat->defl.R);
@@ -161,10 +160,10 @@ ovl_status ovl_set_links(ovl_lattice* lat, const void* U, int32_t U_on_device, u
   // a copy held from an earlier call is refreshed too: no format may keep the previous field
   if (lat->u32) formats |= OVL_F32;
   if (lat->u16) formats |= OVL_F16R12;
-  if (!lat->u64) OVL_CHECK_CUDA(cudaMalloc(&lat->u64, nl * 16));
-  if (!lat->ufx) {
-    OVL_CHECK_CUDA(cudaMalloc(&lat->ufx, nl * 16 + fx_field_bytes()));
-    lat->fxf = (FxField*)((char*)lat->ufx + nl * 16);
+  if (!lat->u64) {  // one allocation: links, fixed-point copy, scale
+    OVL_CHECK_CUDA(cudaMalloc(&lat->u64, 2 * nl * 16 + fx_field_bytes()));
+    lat->ufx = (FxC*)((char*)lat->u64 + nl * 16);
+    lat->fxf = (FxField*)((char*)lat->u64 + 2 * nl * 16);
   }
   if ((formats & OVL_F32) && !lat->u32) OVL_CHECK_CUDA(cudaMalloc(&lat->u32, nl * 8));
   if ((formats & OVL_F16R12) && !lat->u16) OVL_CHECK_CUDA(cudaMalloc(&lat->u16, (size_t)24 * lat->g.vol * 4));

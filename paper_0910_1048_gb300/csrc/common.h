@@ -158,7 +158,7 @@ struct ovl_lattice {
   ovl::Geom g{};
   uint32_t formats = 0;
   double2* u64 = nullptr;
-  ovl::FxC* ufx = nullptr;        // fixed-point copy of u64 and its scale (one allocation)
+  ovl::FxC* ufx = nullptr;        // fixed-point copy of u64 and its scale (in u64's allocation)
   ovl::FxField* fxf = nullptr;
   bool fx_ok = false;             // the fixed-point copy is usable (FxField::ok)
   float2* u32 = nullptr;

@@ -186,12 +186,14 @@ __global__ void k_ingest_links(int vol, const double2* ucan, double2* u64, float
 }
 
 // Ranges of the links for their fixed-point copy: bits of non-negative doubles order like the values.
-__global__ void __launch_bounds__(256) k_fx_range(int vol, const double2* ucan, FxField* f) {
+__global__ void __launch_bounds__(256) k_fx_range(int vol, const double2* u64, FxField* f) {
   const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;  // over 4 V links
   unsigned long long lo = ~0ull, hi = 0ull;
   if (e < (size_t)4 * vol) {
     Mat3<double> u;
-    for (int k = 0; k < 9; ++k) u.m[k / 3][k % 3] = ldc<double>(ucan, e * 9 + k);
+    const double2* p = u64 + e / vol * 9 * vol + e % vol;  // [direction][9][site]
+#pragma unroll
+    for (int k = 0; k < 9; ++k) u.m[k / 3][k % 3] = ldc<double>(p, (size_t)k * vol);
     double top, need;
     fx_link_range(u, top, need);
     lo = (unsigned long long)__double_as_longlong(top);
@@ -230,7 +232,7 @@ cudaError_t launch_ingest_links(const Geom& g, const double* ucan, double2* u64,
   cudaError_t e;
   if ((e = cudaMemsetAsync(fxf, 0, sizeof(FxField), st))) return e;
   if ((e = cudaMemsetAsync(&fxf->lo, 0xff, sizeof(fxf->lo), st))) return e;
-  k_fx_range<<<(unsigned)(((size_t)4 * g.vol + 255) / 256), 256, 0, st>>>(g.vol, (const double2*)ucan, fxf);
+  k_fx_range<<<(unsigned)(((size_t)4 * g.vol + 255) / 256), 256, 0, st>>>(g.vol, u64, fxf);
   k_fx_links<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(g.vol, u64, fxf, ufx);
   return cudaGetLastError();
 }
