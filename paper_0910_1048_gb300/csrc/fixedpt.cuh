@@ -137,11 +137,12 @@ OVL_HD double fx_pow2(int biased) {  // 2^(biased - 1023), 0 < biased < 2047
 }
 
 // Limbs of x in units of 2^-59 2^(e-1022), e >= 64 at least x's biased exponent (smaller values are
-// shifted out; zeros and subnormals, biased exponent 0, give 0 or -1 unit). A negative value is the one's
-// complement of its 59-bit magnitude: one unit off, and two instructions less per component.
+// shifted out). A negative value is the one's complement of its 59-bit magnitude: one unit off, and two
+// instructions less per component. Zeros of either sign, and subnormals (biased exponent 0), give 0: their sign is
+// left out, so that components that are exactly zero add nothing.
 OVL_HD void fx_limbs(int hi, unsigned lo, int e, int& h, int& l) {
   const int d = e - (int)(((unsigned)hi >> 20) & 0x7ffu);
-  const unsigned s = (unsigned)(hi >> 31);
+  const unsigned s = (unsigned)hi >= 0x80100000u ? ~0u : 0u;
   const unsigned mh = (((unsigned)hi << 6 | lo >> 26) & 0x03ffffffu) ^ s ^ 0x04000000u;
   const fx64 v = (fx64)((unsigned long long)mh << 32 | ((lo << 6) ^ s));
   h = (int)fx_sar(v, d + 30);
@@ -493,7 +494,6 @@ OVL_HD bool fx_hops(const Geom& g, const FxC* U, int s, int k0, int k1, const Fx
     const size_t sa = (k & 1) ? (size_t)g.vol : (size_t)3 * g.vol, sb = (k & 1) ? (size_t)3 * g.vol : (size_t)g.vol;
     fx_hop(k, 0, false, h, [&](int a, int b) { return u[a * sa + b * sb]; }, c, wraps && g.t_bc < 0, acc);
   }
-  if (top == 0) fx_clear(acc);  // (a negative zero left one unit)
   return top < (0x7ff << 20) && E < 2000 && (top == 0 || top >= (64 << 20));
 }
 
