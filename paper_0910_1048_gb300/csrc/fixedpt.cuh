@@ -26,10 +26,16 @@
 // about 1300 it takes. Against the FP64 hops D_W at 12^4 takes 22.6 us instead of 65.5, eight sources at 16^4
 // 256 instead of 801; its error against 64 bits is 1.4e-16 instead of 1.8e-16.
 //
+// That is an error relative to the largest terms around a site, so it is kept for links that carry a large
+// colour's value into every colour. Where colours decouple (unit or diagonal links, SU(2) blocks), FP64 arithmetic
+// keeps a colour's 53 bits however much smaller than the others it is: on unit links a colour 1e-10 of the others
+// came out with an error of 2e-7 from these sums.
+//
 // Integer sums do not depend on their order, so every shape of the stencil gives the same hop sums
 // up to that rounding. Sites next to an infinity, a NaN or only components below 2^-959 (E < 64), and
-// fields whose links do not share a scale (FxField::ok = 0: a non-finite field, a link whose largest
-// component is below a quarter of the field's scale, or a scale far from 1) take the FP64 hops.
+// fields whose links do not share a scale or do not mix the colours (FxField::ok = 0: a non-finite field, a link
+// whose largest component is below a quarter of the field's scale, a scale far from 1, a link with an entry below
+// 2^-20 of its largest component, or more than half of the links with one below 2^-6) take the FP64 hops.
 #pragma once
 
 #include "wilson.cuh"
@@ -362,10 +368,11 @@ OVL_HD void fx_hop(int k, int d, bool shift, const FxHalf& h, Link link, const F
 // Field-wide scale of the fixed-point links, kept in device memory beside them (a later ovl_set_links
 // rewrites both in place, so captured graphs stay valid).
 struct FxField {
-  int ok;    // the links share a scale (see above)
+  int ok;    // the links share a scale and mix the colours (see above)
   int uexp;  // the scale is 2^uexp
   unsigned long long lo, hi;  // bits of the smallest of the links' largest components and of the largest
                               // of the links' scales (fx_link_range), over the field
+  unsigned weak;              // links that mix the colours weakly
 };
 
 // |x| rounded up to 21 bits, from x's high word. (Without the FP64 pipe: with about 130 FP64 operations a link,
@@ -382,21 +389,39 @@ OVL_HD float fx_abs_up(int hi) {
 #endif
 }
 
-// Largest component of a link, and the scale it needs: the largest of that and its row and column sums of
-// |re| + |im| over sqrt(6) (rounded up, but 1 for SU(3) to rounding).
-OVL_HD void fx_link_range(const Mat3<double>& u, double& top, double& need) {
+// Bits below the largest component of a link at which its smallest entry (its larger component) may lie: for any
+// link, and for one that is not weak. Of random SU(3) links one in 7 10^10 falls below the first and one in 250
+// below the second, so a field of 64^4 sites is refused by chance once in a thousand times; links exp(i eps H)
+// are mostly weak below eps = 0.04.
+constexpr int kFxMixAny = 20, kFxMixMost = 6;
+
+// Largest component of a link (0 if the link leaves a colour out), the scale it needs: the largest of that
+// and its row and column sums of |re| + |im| over sqrt(6) (rounded up, but 1 for SU(3) to rounding), and whether it
+// mixes the colours weakly.
+OVL_HD void fx_link_range(const Mat3<double>& u, double& top, double& need, bool& weak) {
   float row[3] = {0, 0, 0}, col[3] = {0, 0, 0};
   unsigned long long m = 0;
+  int least = 0x7fffffff;
 #pragma unroll
-  for (int i = 0; i < 18; ++i) {
-    int hi;
-    unsigned lo;
-    fx_words(i < 9 ? u.m[i / 3][i % 3].re : u.m[(i - 9) / 3][i % 3].im, hi, lo);
-    const unsigned long long w = (unsigned long long)(unsigned)(hi & 0x7fffffff) << 32 | lo;
-    m = m > w ? m : w;
-    row[i % 9 / 3] += fx_abs_up(hi);
-    col[i % 3] += fx_abs_up(hi);
+  for (int i = 0; i < 9; ++i) {
+    int hr, hi;
+    unsigned lr, li;
+    fx_words(u.m[i / 3][i % 3].re, hr, lr);
+    fx_words(u.m[i / 3][i % 3].im, hi, li);
+    hr &= 0x7fffffff;
+    hi &= 0x7fffffff;
+    const unsigned long long wr = (unsigned long long)(unsigned)hr << 32 | lr;
+    const unsigned long long wi = (unsigned long long)(unsigned)hi << 32 | li;
+    m = m > wr ? m : wr;
+    m = m > wi ? m : wi;
+    const int entry = hr > hi ? hr : hi;
+    least = least < entry ? least : entry;
+    const float a = fx_abs_up(hr) + fx_abs_up(hi);
+    row[i / 3] += a;
+    col[i % 3] += a;
   }
+  const int most = (int)(m >> 32);
+  weak = least < most - (kFxMixMost << 20);
   float sum = row[0];
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
@@ -413,7 +438,15 @@ OVL_HD void fx_link_range(const Mat3<double>& u, double& top, double& need) {
   need = sum * 0.408247f;  // 1 / 2.4495, just above sqrt(6), and 21 bits
   need = top > need ? top : need;
   if (!finite) need = 1e308 * 10;  // infinity: the field is not usable
+  if (least < most - (kFxMixAny << 20)) top = 0.0;
 }
+OVL_HD void fx_link_range(const Mat3<double>& u, double& top, double& need) {
+  bool weak;
+  fx_link_range(u, top, need, weak);
+}
+
+// Whether a field of n links, `weak` of them weakly mixing, mixes the colours.
+OVL_HD bool fx_field_mixes(unsigned weak, size_t n) { return 2 * (size_t)weak <= n; }
 
 // Scale exponent of a field with these ranges; false: the FP64 hops.
 OVL_HD bool fx_field_scale(double lo, double hi, int* uexp) {

@@ -189,13 +189,14 @@ __global__ void k_ingest_links(int vol, const double2* ucan, double2* u64, float
 __global__ void __launch_bounds__(256) k_fx_range(int vol, const double2* u64, FxField* f) {
   const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;  // over 4 V links
   unsigned long long lo = ~0ull, hi = 0ull;
+  bool weak = false;
   if (e < (size_t)4 * vol) {
     Mat3<double> u;
     const double2* p = u64 + e / vol * 9 * vol + e % vol;  // [direction][9][site]
 #pragma unroll
     for (int k = 0; k < 9; ++k) u.m[k / 3][k % 3] = ldc<double>(p, (size_t)k * vol);
     double top, need;
-    fx_link_range(u, top, need);
+    fx_link_range(u, top, need, weak);
     lo = (unsigned long long)__double_as_longlong(top);
     hi = (unsigned long long)__double_as_longlong(need);
   }
@@ -205,16 +206,19 @@ __global__ void __launch_bounds__(256) k_fx_range(int vol, const double2* u64, F
     lo = l2 < lo ? l2 : lo;
     hi = h2 > hi ? h2 : hi;
   }
+  const int nweak = __popc(__ballot_sync(0xffffffffu, weak));
   if ((threadIdx.x & 31) == 0) {
     atomicMin(&f->lo, lo);
     atomicMax(&f->hi, hi);
+    if (nweak) atomicAdd(&f->weak, (unsigned)nweak);
   }
 }
 
 __global__ void __launch_bounds__(256) k_fx_links(int vol, const double2* u64, FxField* f, FxC* ufx) {
   const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;  // over 4*9*V
   int uexp;
-  const bool ok = fx_field_scale(__longlong_as_double((long long)f->lo), __longlong_as_double((long long)f->hi), &uexp);
+  const bool ok = fx_field_scale(__longlong_as_double((long long)f->lo), __longlong_as_double((long long)f->hi), &uexp) &&
+                  fx_field_mixes(f->weak, (size_t)4 * vol);
   if (e == 0) {
     f->ok = ok ? 1 : 0;
     f->uexp = uexp;

@@ -8,6 +8,7 @@ import numpy as np
 import pytest
 
 import synth
+from oracle import gamma
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 DIMS = (4, 6, 2, 8)
@@ -57,3 +58,108 @@ def test_negative_zeros_add_nothing(lib, g5, spins):
     zero = f64 == 0
     assert 0.2 < zero.mean() < 1
     assert not fx[zero].any()
+
+
+# ------------------------------------------------------------------ colours that decouple
+@pytest.fixture(scope="module")
+def field_usable(tmp_path_factory):
+    out = str(tmp_path_factory.mktemp("fx") / "linkfield_check.so")
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    subprocess.run(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-I", os.path.join(cuda, "include"),
+                    os.path.join(HERE, "native", "linkfield_check.cpp"), "-o", out], check=True)
+    so = ctypes.CDLL(out)
+    so.field_usable.argtypes = [ctypes.c_void_p, ctypes.c_longlong]
+
+    def usable(u):
+        u = np.ascontiguousarray(u)
+        return bool(so.field_usable(u.ctypes.data, u.size // 9))
+
+    return usable
+
+
+def _blocks():
+    """SU(2) links in colours 0 and 2."""
+    rng = np.random.default_rng(5)
+    a = rng.standard_normal((4, 8, 2, 6, 4, 4))
+    a /= np.linalg.norm(a, axis=-1, keepdims=True)
+    u = synth.unit_links(DIMS)
+    p, q = a[..., 0] + 1j * a[..., 1], a[..., 2] + 1j * a[..., 3]
+    u[..., 0, 0], u[..., 0, 2], u[..., 2, 0], u[..., 2, 2] = p, q, -q.conj(), p.conj()
+    return u
+
+
+def _phases():
+    th = np.random.default_rng(6).uniform(-3, 3, (4, 8, 2, 6, 4, 3))
+    u = synth.unit_links(DIMS)
+    for c in range(3):
+        u[..., c, c] = np.exp(1j * (th[..., c] - th.mean(-1)))
+    return u
+
+
+def _monomial():
+    """Every link a permutation of the colours with phases: colours stay apart from site to site."""
+    rng = np.random.default_rng(7)
+    return np.stack([np.eye(3)[rng.permutation(3)] for _ in range(4 * VOL)]).reshape(_phases().shape) * _phases().sum(
+        -1, keepdims=True) / abs(_phases().sum(-1, keepdims=True))
+
+
+DECOUPLED = {"unit": lambda: synth.unit_links(DIMS), "phases": _phases, "su2 blocks": _blocks, "monomial": _monomial}
+
+
+def _terms(u, psi, mu):
+    """Per component, the sum of the moduli of D_W psi's terms, over re and im: [12][V]."""
+    g = gamma.GAMMA
+    a = np.abs(psi.real) + np.abs(psi.imag)
+    out, au = a.copy(), np.abs(u.real) + np.abs(u.imag)
+    for nu in range(4):
+        ax = 3 - nu
+        ef, eb = (np.exp(mu), np.exp(-mu)) if nu == 3 else (1.0, 1.0)
+        p = np.abs(np.eye(4)) + np.abs(g[nu])
+        out += KAPPA * ef * np.einsum("tzyxab,ij,tzyxjb->tzyxia", au[nu], p, np.roll(a, -1, ax))
+        out += KAPPA * eb * np.roll(np.einsum("tzyxba,ij,tzyxjb->tzyxia", au[nu], p, a), 1, ax)
+    return out.reshape(VOL, 12).T
+
+
+@pytest.mark.parametrize("field", DECOUPLED)
+@pytest.mark.parametrize("small", [1e-2, 1e-6, 1e-10, 1e-20])
+def test_decoupled_colours(lib, field, small):
+    """Fields whose links leave colours apart, a colour of the source smaller than the others: the field takes the
+    FP64 hops, or every component is off by at most the FP64 chains' bound, sixteen roundings of its own terms
+    (a projection, six multiply-adds, eight hops and the site itself)."""
+    u, psi = DECOUPLED[field](), synth.gaussian_source(DIMS, 2)
+    psi[..., 1] *= small
+    ok, _, _, efx, _, usable = _check(lib, u, psi)
+    bound = 2.0 ** -49 * _terms(u, psi, 0.3)[:, :, None]
+    assert not ok or (efx <= bound)[:, usable].all()
+
+
+@pytest.mark.parametrize("field", DECOUPLED)
+def test_decoupled_fields_are_refused(field_usable, field):
+    assert not field_usable(DECOUPLED[field]())
+
+
+@pytest.mark.parametrize("eps", [0.1, 0.3, 0.5, 2.0])
+@pytest.mark.parametrize("dims", [(2, 2, 2, 2), (4, 4, 4, 4), (8, 8, 8, 8)])
+def test_mixing_fields_are_accepted(field_usable, eps, dims):
+    for seed in range(3):
+        assert field_usable(synth.gauge_links(dims, seed, eps))
+        assert field_usable(3.0 * synth.gauge_links(dims, seed, eps))
+
+
+def test_where_the_field_rule_ends(field_usable):
+    u = synth.gauge_links(DIMS, 1, 2.0)
+    flat = u.reshape(-1, 3, 3)
+    one = flat[100].copy()
+    top = max(abs(one.real).max(), abs(one.imag).max())
+    for small, want in ((2.0 ** -19, True), (2.0 ** -21, False), (0.0, False)):
+        flat[100] = one
+        flat[100][2, 0] = top * small * 1j
+        assert field_usable(u) == want
+    flat[100] = one
+    n = len(flat)
+    weak = synth.gauge_links(DIMS, 3, 1e-3).reshape(-1, 3, 3)  # off-diagonal entries about 1e-3
+    for share, want in ((0.45, True), (0.55, False)):
+        v = flat.copy()
+        v[:int(share * n)] = weak[:int(share * n)]
+        assert field_usable(v) == want
+    assert not field_usable(synth.gauge_links(DIMS, 4, 1e-5))
