@@ -127,6 +127,9 @@ ovl_status ovl_from_native(ovl_lattice* lat, int32_t dtype, int32_t nrhs, const 
  * spinors [nrhs][n] of dtype OVL_C128 (FP64 links) or OVL_C64 (FP32 arithmetic with
  * FP32 links, or FP16 12-real links with OVL_LINKS_F16R12). in/out are device buffers,
  * must not alias, canonical layout unless OVL_NATIVE. Stream-ordered (no sync).
+ * FP64: hop sums are 59-bit integers in units of the largest neighbour component where every spin's real and
+ * imaginary parts, over the eight neighbours, are zero or reach 2^-6 of it (see also ovl_set_links), FP64
+ * elsewhere: every component is as accurate as its own terms allow, zeros are exact.
  * Section 1 defines H_W = gamma5 D_W; the stencil form is the reading above.
  * Errors: EINVAL (no links in the requested format, nrhs < 1, NULL), ECUDA. */
 ovl_status ovl_apply_DW(ovl_lattice* lat, double m_W, double mu, uint32_t flags, int32_t dtype,

@@ -397,17 +397,10 @@ static __device__ __noinline__ void hops_f64(const Geom& g, const double2* u64, 
     hops_f64_ld(g, U, s, c, k0, k1, ld, out);
 }
 
-// out += the hops k0 .. k1-1 of psi = in (or gamma5 in).
-__device__ __forceinline__ void add_hops(const Geom& g, const Links& U, int s, int k0, int k1, const FxCoef& c,
-                                         StrideLoader ld, bool g5in, bool self, Spin<double>& out) {
-  FxAcc acc;
-  fx_clear(acc);
-  int E = 0;
-  const bool fx = c.ok && U.fxf->ok && fx_hops(g, U.fx, s, k0, k1, c, ld, g5in, acc, E);
-  if (self) {
-    ld(s, out);
-    if (g5in) gamma5_inplace(out);
-  }
+// out += the accumulators' sum if they hold it (fx), else the FP64 hops k0 .. k1-1.
+__device__ __forceinline__ void finish_hops(const Geom& g, const Links& U, int s, int k0, int k1, const FxCoef& c,
+                                            StrideLoader ld, bool g5in, bool fx, const FxAcc& acc, int E,
+                                            Spin<double>& out) {
   if (fx) {
     const double f = fx_unit(E, c, U.fxf->uexp);
 #pragma unroll
@@ -423,12 +416,24 @@ __device__ __forceinline__ void add_hops(const Geom& g, const Links& U, int s, i
   }
 }
 
+// out = psi (psi = in, or gamma5 in) + its hops.
+__device__ __forceinline__ void add_hops(const Geom& g, const Links& U, int s, const FxCoef& c, StrideLoader ld, bool g5in,
+                                         Spin<double>& out) {
+  FxAcc acc;
+  fx_clear(acc);
+  int E = 0;
+  const bool fx = c.ok && U.fxf->ok && fx_hops(g, U.fx, s, 0, 8, c, ld, g5in, acc, E);
+  ld(s, out);
+  if (g5in) gamma5_inplace(out);
+  finish_hops(g, U, s, 0, 8, c, ld, g5in, fx, acc, E, out);
+}
+
 // out = D_W psi at site s, psi native.
 template <int LF, class R>
 __device__ __forceinline__ void stencil_site(const Geom& g, const Links& U, int s, const typename HopsOf<R>::T& c,
                                              const typename V2<R>::T* in, Spin<R>& out) {
   if constexpr (sizeof(R) == 8)
-    add_hops(g, U, s, 0, 8, c, StrideLoader{in, 1, g.vol}, false, true, out);
+    add_hops(g, U, s, c, StrideLoader{in, 1, g.vol}, false, out);
   else
     dslash_site<LF, R>(g, U, s, c, Loader<R, true>{in, g.vol, false}, out);
 }
@@ -461,10 +466,28 @@ __device__ __forceinline__ void pair_split(const Geom& g, const Links& U, const 
   Spin<R> acc;
 #pragma unroll
   for (int q = 0; q < 12; ++q) acc.c[q / 3][q % 3] = mk<R>(0, 0);
+  if constexpr (std::is_same_v<Coef, FxCoef>) {
+    // (a site's sums are taken or refused for its four directions together: fx_even)
+    __shared__ unsigned size[2][4][4][SITES];  // [which][spin][direction][site]
+    const StrideLoader ld{in, 1, g.vol};
+    FxAcc sum;
+    fx_clear(sum);
+    int E = 0;
+    FxSizes z;
+    bool fx = s < g.vol && c.ok && U.fxf->ok && fx_hops(g, U.fx, s, 2 * dir, 2 * dir + 2, c, ld, false, sum, E, z);
+#pragma unroll
+    for (int sp = 0; sp < 4; ++sp) size[which][sp][dir][tx] = z.m[sp];
+    __syncthreads();
+#pragma unroll
+    for (int sp = 0; sp < 4; ++sp) {
+      const unsigned(&q)[4][SITES] = size[which][sp];
+      z.m[sp] = fx_max2(fx_max2(q[0][tx], q[1][tx]), fx_max2(q[2][tx], q[3][tx]));
+    }
+    fx = fx && fx_even(z);
+    if (s < g.vol) finish_hops(g, U, s, 2 * dir, 2 * dir + 2, c, ld, false, fx, sum, E, acc);
+  }
   if (s < g.vol) {
-    if constexpr (std::is_same_v<Coef, FxCoef>) {
-      add_hops(g, U, s, 2 * dir, 2 * dir + 2, c, StrideLoader{in, 1, g.vol}, false, false, acc);
-    } else {
+    if constexpr (!std::is_same_v<Coef, FxCoef>) {
       Nbr n;
       neighbours(g, s, n);
       Loader<R, true> ld{in, g.vol, false};

@@ -26,16 +26,19 @@
 // about 1300 it takes. Against the FP64 hops D_W at 12^4 takes 22.6 us instead of 65.5, eight sources at 16^4
 // 256 instead of 801; its error against 64 bits is 1.4e-16 instead of 1.8e-16.
 //
-// That is an error relative to the largest terms around a site, so it is kept for links that carry a large
-// colour's value into every colour. Where colours decouple (unit or diagonal links, SU(2) blocks), FP64 arithmetic
-// keeps a colour's 53 bits however much smaller than the others it is: on unit links a colour 1e-10 of the others
-// came out with an error of 2e-7 from these sums.
-//
-// Integer sums do not depend on their order, so every shape of the stencil gives the same hop sums
-// up to that rounding. Sites next to an infinity, a NaN or only components below 2^-959 (E < 64), and
-// fields whose links do not share a scale or do not mix the colours (FxField::ok = 0: a non-finite field, a link
-// whose largest component is below a quarter of the field's scale, a scale far from 1, a link with an entry below
-// 2^-20 of its largest component, or more than half of the links with one below 2^-6) take the FP64 hops.
+// That is an error relative to the largest terms around a site. FP64 arithmetic keeps a component's 53 bits however
+// much smaller than the others it is, so the sums are used only where every component has terms of that size:
+//  - Fields whose links mix the colours. Where colours decouple (unit or diagonal links, SU(2) blocks), a colour
+//    1e-10 of the others came out with an error of 2e-7. FxField::ok = 0 also without a common scale: a
+//    non-finite field, a link whose largest component is below a quarter of the field's scale, a scale far
+//    from 1; a link with an entry below 2^-20 of its largest component, or more than half of the links with
+//    one below 2^-6.
+//  - Sites whose neighbours together fill the real and imaginary part of every spin to 2^-6 of the largest, or
+//    leave it zero (FxSizes): a hop joins two spins only, so a small spin beside a large one can reach the
+//    site alone. Gaussian fields fill all of them; a site beside one site of widely different spins is refused.
+//    Sites next to an infinity, a NaN or only components below 2^-959 (E < 64) are refused too.
+// Others take the FP64 hops. Integer sums do not depend on their order, so every shape of the stencil gives the
+// same hop sums up to the rounding above.
 #pragma once
 
 #include "wilson.cuh"
@@ -54,6 +57,7 @@ struct FxCoef {
   HopCoef<double> k;
   int fh, fl, fe;  // forward: (fh 2^30 + fl) 2^-57 2^fe
   int bh, bl, be;  // backward
+  int ft, bt;      // exponents of the factors (2^ft <= factor < 2^(ft+1)), for FxSizes
   int unit;        // 1: both factors are 1 (mu = 0)
   int ok;          // 0: a factor is outside the fixed-point range (FP64 path)
 };
@@ -63,16 +67,16 @@ inline FxCoef fx_coef(double m_w, double mu) {
   c.k = hop_coef<double>(m_w, mu);
   c.unit = mu == 0.0;
   c.ok = std::fabs(mu) <= 16.0;
-  auto split = [&](double f, int& h, int& l, int& e) {
-    int x;
+  auto split = [&](double f, int& h, int& l, int& e, int& x) {
     const double m = std::frexp(c.ok ? f : 1.0, &x);
     e = x > 2 ? x - 2 : 0;
     const fx64 q = std::llrint(std::ldexp(m, 57 + x - e));
     h = (int)(q >> 30);
     l = (int)(q & ((1 << 30) - 1));
+    --x;
   };
-  split(std::exp(mu), c.fh, c.fl, c.fe);
-  split(std::exp(-mu), c.bh, c.bl, c.be);
+  split(std::exp(mu), c.fh, c.fl, c.fe, c.ft);
+  split(std::exp(-mu), c.bh, c.bl, c.be, c.bt);
   return c;
 }
 
@@ -185,6 +189,54 @@ OVL_HD int fx_top_word(const Spin<double>& p) {
     m = m > (w & 0x7fffffff) ? m : (w & 0x7fffffff);
   }
   return m;
+}
+
+// Size of a complex number: the upper 15 bits (exponent and four bits of the mantissa) of |re| in the low half, of
+// |im| in the high one.
+OVL_HD unsigned fx_size(cplx<double> x) {
+  int r, i;
+  unsigned z;
+  fx_words(x.re, r, z);
+  fx_words(x.im, i, z);
+#if defined(__CUDA_ARCH__)
+  return __byte_perm(r, i, 0x7632) & 0x7fff7fffu;
+#else
+  return ((unsigned)i & 0x7fff0000u) | ((unsigned)r >> 16 & 0x7fffu);
+#endif
+}
+OVL_HD unsigned fx_max2(unsigned a, unsigned b) {  // of both halves
+#if defined(__CUDA_ARCH__)
+  unsigned r;
+  asm("max.u16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+  return r;
+#else
+  const unsigned h = a >> 16 > b >> 16 ? a : b, l = (a & 0xffffu) > (b & 0xffffu) ? a : b;
+  return (h & 0xffff0000u) | (l & 0xffffu);
+#endif
+}
+OVL_HD unsigned fx_raise(unsigned v, int e) {  // both sizes, where not zero, times 2^e
+  const int l = (int)(v & 0xffffu), h = (int)(v >> 16);
+  const int l2 = l + 16 * e > 1 ? l + 16 * e : 1, h2 = h + 16 * e > 1 ? h + 16 * e : 1;
+  return (h ? (unsigned)h2 << 16 : 0u) | (l ? (unsigned)l2 : 0u);
+}
+
+// Largest size of each spin over the neighbours of a site, times the hops' factors.
+struct FxSizes {
+  unsigned m[4] = {0, 0, 0, 0};
+};
+constexpr int kFxEven = 6;  // bits
+
+// Whether all of them are zero or within 2^-kFxEven of the largest.
+OVL_HD bool fx_even(const FxSizes& z) {
+  const unsigned t = fx_max2(fx_max2(z.m[0], z.m[1]), fx_max2(z.m[2], z.m[3]));
+  const int top = (int)(t & 0xffffu) > (int)(t >> 16) ? (int)(t & 0xffffu) : (int)(t >> 16);
+  bool even = true;
+#pragma unroll
+  for (int s = 0; s < 4; ++s) {
+    const int l = (int)(z.m[s] & 0xffffu), h = (int)(z.m[s] >> 16);
+    even = even && (l == 0 || l + (kFxEven << 4) >= top) && (h == 0 || h + (kFxEven << 4) >= top);
+  }
+  return even;
 }
 
 OVL_HD void fx_spin(const Spin<double>& p, int e, FxSpin& o) {
@@ -489,12 +541,13 @@ OVL_HD int fx_neighbour(const Geom& g, int s, unsigned long long xyzt, int k, bo
 }
 
 // Hops k0 .. k1-1 of site s, psi in FP64 loaded through `ld` and converted on the way, to limbs relative to the
-// largest exponent E met so far (+1), so that no hop is shifted afterwards. Returns whether the
-// accumulators hold the hop sum: no infinity or NaN among the neighbours, and not only components too
-// small for the common exponent (all zero, or below 2^-1042, is fine: the sum is zero).
+// largest exponent E met so far (+1), so that no hop is shifted afterwards; the neighbours' sizes in z. Returns
+// whether the accumulators hold the hop sum: no infinity or NaN among the neighbours, and not only components
+// too small for the common exponent (all zero is fine: the sum is zero). For all eight hops together fx_even(z)
+// has to hold too.
 template <class Load>
 OVL_HD bool fx_hops(const Geom& g, const FxC* U, int s, int k0, int k1, const FxCoef& c, Load ld, bool g5in, FxAcc& acc,
-                    int& E) {
+                    int& E, FxSizes& z) {
   const unsigned long long xyzt = fx_coords(g, s);
   int top = 0;
   E = 0;
@@ -506,8 +559,19 @@ OVL_HD bool fx_hops(const Geom& g, const FxC* U, int s, int k0, int k1, const Fx
     {
       Spin<double> p;
       ld(nb, p);
-      const int w = fx_top_word(p), eb = w >> 20;
+      unsigned m[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) m[i] = fx_max2(fx_max2(fx_size(p.c[i][0]), fx_size(p.c[i][1])), fx_size(p.c[i][2]));
+      const unsigned t = fx_max2(fx_max2(m[0], m[1]), fx_max2(m[2], m[3]));
+      const int w = (int)(t & 0xffffu) > (int)(t >> 16) ? (int)(t & 0xffffu) : (int)(t >> 16), eb = w >> 4;
       top = top > w ? top : w;
+      const int ft = k < 6 ? 0 : (k & 1) ? c.bt : c.ft;
+      if (ft != 0) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) m[i] = fx_raise(m[i], ft);
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) z.m[i] = fx_max2(z.m[i], m[i]);
       const int fe = fx_hop_exponent(k, 0, c), eh = (eb > 64 ? eb : 64) + fe;
       if (eh > E) {  // first hop, or a larger neighbour than any before
         if (E != 0) {
@@ -527,7 +591,32 @@ OVL_HD bool fx_hops(const Geom& g, const FxC* U, int s, int k0, int k1, const Fx
     const size_t sa = (k & 1) ? (size_t)g.vol : (size_t)3 * g.vol, sb = (k & 1) ? (size_t)3 * g.vol : (size_t)g.vol;
     fx_hop(k, 0, false, h, [&](int a, int b) { return u[a * sa + b * sb]; }, c, wraps && g.t_bc < 0, acc);
   }
-  return top < (0x7ff << 20) && E < 2000 && (top == 0 || top >= (64 << 20));
+  if (top == 0) {  // zeros, or subnormal numbers
+    unsigned any = 0;
+#pragma unroll 1
+    for (int k = k0; k < k1; ++k) {
+      bool wraps;
+      Spin<double> p;
+      ld(fx_neighbour(g, s, xyzt, k, &wraps), p);
+#pragma unroll
+      for (int i = 0; i < 12; ++i) {
+        int hr, hi;
+        unsigned lr, li;
+        fx_words(p.c[i / 3][i % 3].re, hr, lr);
+        fx_words(p.c[i / 3][i % 3].im, hi, li);
+        any |= ((unsigned)(hr | hi) & 0x7fffffffu) | lr | li;
+      }
+    }
+    return any == 0;
+  }
+  return E < 2000 && top >= 64 << 4;  // (E is above 2047 beside an infinity or a NaN)
+}
+// All eight hops.
+template <class Load>
+OVL_HD bool fx_hops(const Geom& g, const FxC* U, int s, int k0, int k1, const FxCoef& c, Load ld, bool g5in, FxAcc& acc,
+                    int& E) {
+  FxSizes z;
+  return fx_hops(g, U, s, k0, k1, c, ld, g5in, acc, E, z) && fx_even(z);
 }
 
 // FP64 value of one unit of the accumulators times the hop coefficient ks and the links' scale.

@@ -280,7 +280,7 @@ __global__ void __launch_bounds__(kBlock, 3)
   const size_t off = (size_t)blockIdx.y * 12 * g.vol;
   const int ss = native ? 1 : 12, cs = native ? g.vol : 1;
   Spin<double> o;
-  add_hops(g, U, s, 0, 8, c, StrideLoader{in + off, ss, cs}, g5_in, true, o);
+  add_hops(g, U, s, c, StrideLoader{in + off, ss, cs}, g5_in, o);
   if (g5_out) gamma5_inplace(o);
 #pragma unroll
   for (int q = 0; q < 12; ++q) stc<double>(out + off, (size_t)s * ss + (size_t)q * cs, o.c[q / 3][q % 3]);
@@ -294,6 +294,7 @@ __global__ void __launch_bounds__(128, 3)
     k_dslash_f64_split(Geom g, Links U, FxCoef c, bool native, bool g5_in, bool g5_out, const double2* in, double2* out) {
   __shared__ fx64 part[4][3][6][32];  // [receiving spin][slot of the sender][component][site]
   __shared__ int expo[4][32];
+  __shared__ unsigned size[4][4][32];  // [spin][thread][site]
   const int lane = threadIdx.x, t = threadIdx.y;
   const bool live = (int)blockIdx.x * 32 + lane < g.vol;
   const int s = live ? blockIdx.x * 32 + lane : g.vol - 1;
@@ -303,11 +304,17 @@ __global__ void __launch_bounds__(128, 3)
   FxAcc acc;
   fx_clear(acc);
   int E = 0;
-  const bool fx = c.ok && U.fxf->ok && fx_hops(g, U.fx, s, 2 * t, 2 * t + 2, c, ld, g5_in, acc, E);
+  FxSizes z;
+  const bool fx = c.ok && U.fxf->ok && fx_hops(g, U.fx, s, 2 * t, 2 * t + 2, c, ld, g5_in, acc, E, z);
   expo[t][lane] = fx ? E : 1 << 20;
+#pragma unroll
+  for (int sp = 0; sp < 4; ++sp) size[sp][t][lane] = z.m[sp];
   __syncthreads();
   const int Em = max(max(expo[0][lane], expo[1][lane]), max(expo[2][lane], expo[3][lane]));
-  const bool all = Em < 1 << 20;  // no direction needs the FP64 hops
+#pragma unroll
+  for (int sp = 0; sp < 4; ++sp)
+    z.m[sp] = fx_max2(fx_max2(size[sp][0][lane], size[sp][1][lane]), fx_max2(size[sp][2][lane], size[sp][3][lane]));
+  const bool all = Em < 1 << 20 && fx_even(z);  // no direction needs the FP64 hops
   const int d = min(Em - E, 62);
   if (__any_sync(0xffffffffu, d > 0)) {
     const fx64 half = d > 0 ? (fx64)1 << (d - 1) : 0;
