@@ -219,14 +219,16 @@ ovl_status ovl_apply_sign(ovl_lattice* lat, const ovl_sign_params* p, int32_t nr
  * site's links loaded once per group (otherwise as 3). The multishift method runs 1, 4, 5 as its eight-thread stencil and the others as its
  * one-thread stencil. variant = -1
  * clears the entry: the next direct solve for that key times every shape on its own vectors and
- * keeps the fastest. Process-wide. FP64 solves on fields with a common link scale (see
- * ovl_set_links) keep their vectors in fixed point and have two shapes: 1, 4 and 5 four threads per
- * site and stencil, the others one; results are the same bits. Otherwise all shapes compute the same
+ * keeps the fastest. Process-wide. FP64 solves on fields that fit fixed point (see
+ * ovl_set_links) keep their vectors in it and have two shapes: 1, 4 and 5 four threads per
+ * site and stencil, the others one; results are the same bits. They are timed and kept apart from the
+ * nine shapes of FP64 vectors; a pinned shape holds for both. Otherwise all shapes compute the same
  * step and results differ in the rounding of the partial sums of alpha_j only.
  * Errors: EINVAL (variant outside -1..8, volume < 1, unknown precision). */
 ovl_status ovl_set_pair_variant(int64_t volume, int32_t precision, int32_t variant);
 
-/* The shape in use for (volume, precision); -1 if no solve has tuned it yet. */
+/* The shape in use for (volume, precision); -1 if no solve has tuned it yet. FP64: the fixed-point one where a
+ * solve has tuned it, else that of FP64 vectors. */
 int32_t ovl_get_pair_variant(int64_t volume, int32_t precision);
 
 /* Allocation-free variant of ovl_apply_sign's direct method, for callers that cannot

@@ -58,13 +58,15 @@ ovl_status ovl_set_pair_variant(int64_t volume, int32_t precision, int32_t varia
                     OVL_PREC_F32_F16LINKS == ovl::LINK_F16R12,
                 "the tuner's key is the link format of the precision");
   ovl::set_pair_variant((int)volume, precision, variant);
+  if (precision == OVL_PREC_F64) ovl::set_pair_variant((int)volume, ovl::kFixedPointKey, variant);
   return OVL_OK;
 }
 
 int32_t ovl_get_pair_variant(int64_t volume, int32_t precision) {
   if (volume < 1 || volume > (int64_t(1) << 26) || precision < OVL_PREC_F64 || precision > OVL_PREC_F32_F16LINKS)
     return -1;
-  return ovl::tuned_pair_variant((int)volume, precision);
+  const int fx = precision == OVL_PREC_F64 ? ovl::tuned_pair_variant((int)volume, ovl::kFixedPointKey) : -1;
+  return fx >= 0 ? fx : ovl::tuned_pair_variant((int)volume, precision);
 }
 
 ovl_status ovl_ctx_create(int32_t device, ovl_ctx** out) {

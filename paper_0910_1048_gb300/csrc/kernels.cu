@@ -1386,8 +1386,8 @@ static cudaError_t pair_split_launch(const Geom& g, const Links& U, int lf, bool
                       (const float2*)vec.vh, (const float2*)vec.wh, (float2*)vec.av, (float2*)vec.aw);
 }
 
-int resolve_pair_variant(const Geom& g, int lf, bool f64) {
-  const int v = tuned_pair_variant(g.vol, f64 ? 0 : lf);
+int resolve_pair_variant(const Geom& g, int key) {
+  const int v = tuned_pair_variant(g.vol, key);
   return v >= 0 ? v : (use_split(g) ? 1 : 0);
 }
 
@@ -1397,7 +1397,7 @@ static bool deferred_step(bool f64, int variant) { return f64 && variant == 7 &&
 cudaError_t launch_lanczos_pair(const Geom& g, const Links& U, int lf, bool f64, double m_w, double mu,
                                 const LzDev& lz, const LzVecs& vec, cudaStream_t st, int variant, cudaEvent_t mid,
                                 cudaEvent_t first) {
-  if (variant < 0) variant = resolve_pair_variant(g, lf, f64);
+  if (variant < 0) variant = resolve_pair_variant(g, f64 ? LINK_F64 : lf);
   const HopCoef<double> dp = hop_coef<double>(m_w, mu), dm = hop_coef<double>(m_w, -mu);
   const HopCoef<float> fp = hop_coef<float>(m_w, mu), fm = hop_coef<float>(m_w, -mu);
   cudaError_t e;

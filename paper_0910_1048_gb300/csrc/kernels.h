@@ -51,6 +51,10 @@ inline cudaError_t record_timing(cudaEvent_t ev, cudaStream_t st) {
 // Thread-safe, process-wide. (A 16-thread split, one hop per thread, measured 54 us against 32 us
 // for FP64 at 8^4: more index and reduction work than the extra warps hide.)
 constexpr int kPairVariants = 9;
+// Table key of the FP64 direct method's fixed-point step, whose two shapes (1, 4, 5: four threads per site; others:
+// one) have optima of their own: a pick of the nine FP64 shapes above says nothing about them, nor the reverse. The
+// other keys are the link formats; LINK_F64 holds the shape of the steps and multishift stencils on FP64 vectors.
+constexpr int kFixedPointKey = 3;
 int tuned_pair_variant(int vol, int prec);
 // Returns the variant for the key, running `measure` (which returns the fastest variant, or -1)
 // under the table's lock the first time, so that every solve in the process uses one decision per key.
@@ -170,7 +174,7 @@ cudaError_t launch_lanczos_start(const Geom& g, bool f64, const LzDev& lz, const
 // shape 7 in FP64 the step runs deferred (the update's sums are finished by a settle kernel that
 // the next pair launch runs first, with the stencil launched early behind it; after a chunk's last
 // step launch_lanczos_settle finishes them before the host reads the scalars).
-int resolve_pair_variant(const Geom& g, int lf, bool f64);
+int resolve_pair_variant(const Geom& g, int key);
 // Kernels one Lanczos step launches.
 int lanczos_step_launches(const Geom& g, int lf, bool f64, int variant);
 // `mid`, when given, is recorded (record_timing) after the stencil or update kernel itself, before the

@@ -304,7 +304,7 @@ extern "C" ovl_status ovl_apply_sign_noalloc(ovl_lattice* lat, const ovl_sign_pa
     return OVL_OK;
   };
   int queued = 0, launches = 1 + (m > 0 ? 1 : 0) + (fxs ? 1 : 0) + 1;
-  const int pvar = resolve_pair_variant(g, lf, f64);  // one shape for every step of this call
+  const int pvar = resolve_pair_variant(g, fxs ? kFixedPointKey : lf);  // one shape for every step of this call
   while (queued < kmax) {
     int ns = std::min(chunk, kmax - queued);
     for (int i = 0; i < ns; ++i) {

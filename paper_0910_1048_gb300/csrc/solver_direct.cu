@@ -501,8 +501,9 @@ ovl_status solve_direct(ovl_lattice* lat, const ovl_sign_params* p, int nrhs, co
       if (best[var] < best[pick]) pick = var;
     return ok ? pick : -1;
   };
-  tune_pair_variant(g.vol, f64 ? 0 : lf, measure, &targ);
-  const int pvar = resolve_pair_variant(g, lf, f64);  // one shape for every step of this solve
+  const int tune_key = fxs ? kFixedPointKey : lf;
+  tune_pair_variant(g.vol, tune_key, measure, &targ);
+  const int pvar = resolve_pair_variant(g, tune_key);  // one shape for every step of this solve
   const int chunk = std::max(1, std::min(p->check_every > 0 ? p->check_every : 20, kmax));
   // one step, with timing events around its two launches when `tev` is given
   auto step = [&](cudaEvent_t* tev) -> cudaError_t {
