@@ -103,8 +103,9 @@ int64_t ovl_lattice_n(const ovl_lattice* lat);
  * (576 bytes a site) is kept for the FP64 stencils; it is used if the field has a common scale
  * (finite, every link's largest component at least a quarter of the largest of the field, and
  * that within 2^-8 .. 2^8, as for any SU(3) field) and its links mix the colours (no entry below
- * 2^-20 of its link's largest component, and at most half of the links with one below 2^-6).
- * Other fields, among them unit and diagonal links and SU(2) blocks, run FP64 arithmetic.
+ * 2^-20 of its link's largest component, and at most half of the links with one, or with their
+ * real or imaginary parts all, below 2^-6). Other fields, among them unit, diagonal and real links
+ * and SU(2) blocks, run FP64 arithmetic.
  * Errors: EINVAL, EBUSY (a solve is reading the links), ENOMEM, ECUDA. */
 ovl_status ovl_set_links(ovl_lattice* lat, const void* U, int32_t U_on_device, uint32_t formats);
 
@@ -127,9 +128,9 @@ ovl_status ovl_from_native(ovl_lattice* lat, int32_t dtype, int32_t nrhs, const 
  * spinors [nrhs][n] of dtype OVL_C128 (FP64 links) or OVL_C64 (FP32 arithmetic with
  * FP32 links, or FP16 12-real links with OVL_LINKS_F16R12). in/out are device buffers,
  * must not alias, canonical layout unless OVL_NATIVE. Stream-ordered (no sync).
- * FP64: hop sums are 59-bit integers in units of the largest neighbour component where every spin's real and
- * imaginary parts, over the eight neighbours, are zero or reach 2^-6 of it (see also ovl_set_links), FP64
- * elsewhere: every component is as accurate as its own terms allow, zeros are exact.
+ * FP64: hop sums are 59-bit integers in units of the largest neighbour component where every spin, over the
+ * eight neighbours, is zero or reaches 2^-6 of it (see also ovl_set_links), FP64 elsewhere: every component is
+ * as accurate as its own terms allow, zeros are exact.
  * Section 1 defines H_W = gamma5 D_W; the stencil form is the reading above.
  * Errors: EINVAL (no links in the requested format, nrhs < 1, NULL), ECUDA. */
 ovl_status ovl_apply_DW(ovl_lattice* lat, double m_W, double mu, uint32_t flags, int32_t dtype,

@@ -468,7 +468,7 @@ __device__ __forceinline__ void pair_split(const Geom& g, const Links& U, const 
   for (int q = 0; q < 12; ++q) acc.c[q / 3][q % 3] = mk<R>(0, 0);
   if constexpr (std::is_same_v<Coef, FxCoef>) {
     // (a site's sums are taken or refused for its four directions together: fx_even)
-    __shared__ unsigned size[2][4][4][SITES];  // [which][spin][direction][site]
+    __shared__ int size[2][4][4][SITES];  // [which][spin][direction][site]
     const StrideLoader ld{in, 1, g.vol};
     FxAcc sum;
     fx_clear(sum);
@@ -480,8 +480,8 @@ __device__ __forceinline__ void pair_split(const Geom& g, const Links& U, const 
     __syncthreads();
 #pragma unroll
     for (int sp = 0; sp < 4; ++sp) {
-      const unsigned(&q)[4][SITES] = size[which][sp];
-      z.m[sp] = fx_max2(fx_max2(q[0][tx], q[1][tx]), fx_max2(q[2][tx], q[3][tx]));
+      const int(&q)[4][SITES] = size[which][sp];
+      z.m[sp] = max(max(q[0][tx], q[1][tx]), max(q[2][tx], q[3][tx]));
     }
     fx = fx && fx_even(z);
     if (s < g.vol) finish_hops(g, U, s, 2 * dir, 2 * dir + 2, c, ld, false, fx, sum, E, acc);

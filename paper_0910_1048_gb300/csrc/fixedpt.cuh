@@ -32,11 +32,10 @@
 //    1e-10 of the others came out with an error of 2e-7. FxField::ok = 0 also without a common scale: a
 //    non-finite field, a link whose largest component is below a quarter of the field's scale, a scale far
 //    from 1; a link with an entry below 2^-20 of its largest component, or more than half of the links with
-//    one below 2^-6.
-//  - Sites whose neighbours together fill the real and imaginary part of every spin to 2^-6 of the largest, or
-//    leave it zero (FxSizes): a hop joins two spins only, so a small spin beside a large one can reach the
-//    site alone. Gaussian fields fill all of them; a site beside one site of widely different spins is refused.
-//    Sites next to an infinity, a NaN or only components below 2^-959 (E < 64) are refused too.
+//    one, or with their real or imaginary parts all, below 2^-6.
+//  - Sites whose neighbours together fill every spin to 2^-6 of the largest component, or leave it zero
+//    (FxSizes): a hop joins two spins only, so a small spin beside a large one can reach the site alone.
+//    Gaussian fields fill all of them; a site beside one site of widely different spins is refused. Sites next to an infinity, a NaN or only components below 2^-959 (E < 64) are refused too.
 // Others take the FP64 hops. Integer sums do not depend on their order, so every shape of the stencil gives the
 // same hop sums up to the rounding above.
 #pragma once
@@ -176,66 +175,49 @@ struct FxSpin {  // limbs of a site's 12 complex components relative to one expo
   int rh[4][3], rl[4][3], ih[4][3], il[4][3];
 };
 
-// High word of the site's largest component's modulus (its biased exponent is the word >> 20).
-OVL_HD int fx_top_word(const Spin<double>& p) {
+// High word of the largest modulus of spin i's components.
+OVL_HD int fx_spin_word(const Spin<double>& p, int i) {
   int m = 0;
 #pragma unroll
-  for (int i = 0; i < 12; ++i) {
+  for (int a = 0; a < 3; ++a) {
     int w;
     unsigned z;
-    fx_words(p.c[i / 3][i % 3].re, w, z);
+    fx_words(p.c[i][a].re, w, z);
     m = m > (w & 0x7fffffff) ? m : (w & 0x7fffffff);
-    fx_words(p.c[i / 3][i % 3].im, w, z);
+    fx_words(p.c[i][a].im, w, z);
     m = m > (w & 0x7fffffff) ? m : (w & 0x7fffffff);
   }
   return m;
 }
-
-// Size of a complex number: the upper 15 bits (exponent and four bits of the mantissa) of |re| in the low half, of
-// |im| in the high one.
-OVL_HD unsigned fx_size(cplx<double> x) {
-  int r, i;
-  unsigned z;
-  fx_words(x.re, r, z);
-  fx_words(x.im, i, z);
-#if defined(__CUDA_ARCH__)
-  return __byte_perm(r, i, 0x7632) & 0x7fff7fffu;
-#else
-  return ((unsigned)i & 0x7fff0000u) | ((unsigned)r >> 16 & 0x7fffu);
-#endif
-}
-OVL_HD unsigned fx_max2(unsigned a, unsigned b) {  // of both halves
-#if defined(__CUDA_ARCH__)
-  unsigned r;
-  asm("max.u16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
-  return r;
-#else
-  const unsigned h = a >> 16 > b >> 16 ? a : b, l = (a & 0xffffu) > (b & 0xffffu) ? a : b;
-  return (h & 0xffff0000u) | (l & 0xffffu);
-#endif
-}
-OVL_HD unsigned fx_raise(unsigned v, int e) {  // both sizes, where not zero, times 2^e
-  const int l = (int)(v & 0xffffu), h = (int)(v >> 16);
-  const int l2 = l + 16 * e > 1 ? l + 16 * e : 1, h2 = h + 16 * e > 1 ? h + 16 * e : 1;
-  return (h ? (unsigned)h2 << 16 : 0u) | (l ? (unsigned)l2 : 0u);
+// Of the site's (its biased exponent is the word >> 20).
+OVL_HD int fx_top_word(const Spin<double>& p) {
+  int m = 0;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int w = fx_spin_word(p, i);
+    m = m > w ? m : w;
+  }
+  return m;
 }
 
-// Largest size of each spin over the neighbours of a site, times the hops' factors.
+// Largest component of each spin over the neighbours of a site, times the hops' factors: high words of the moduli
+// (the exponent and 20 bits of the mantissa).
 struct FxSizes {
-  unsigned m[4] = {0, 0, 0, 0};
+  int m[4] = {0, 0, 0, 0};
 };
+OVL_HD int fx_raise(int w, int e) {  // times 2^e, where not zero
+  const int r = w + e * (1 << 20);
+  return w ? (r > 1 ? r : 1) : 0;
+}
 constexpr int kFxEven = 6;  // bits
 
 // Whether all of them are zero or within 2^-kFxEven of the largest.
 OVL_HD bool fx_even(const FxSizes& z) {
-  const unsigned t = fx_max2(fx_max2(z.m[0], z.m[1]), fx_max2(z.m[2], z.m[3]));
-  const int top = (int)(t & 0xffffu) > (int)(t >> 16) ? (int)(t & 0xffffu) : (int)(t >> 16);
+  const int t = z.m[0] > z.m[1] ? z.m[0] : z.m[1], u = z.m[2] > z.m[3] ? z.m[2] : z.m[3];
+  const int least = (t > u ? t : u) - (kFxEven << 20);
   bool even = true;
 #pragma unroll
-  for (int s = 0; s < 4; ++s) {
-    const int l = (int)(z.m[s] & 0xffffu), h = (int)(z.m[s] >> 16);
-    even = even && (l == 0 || l + (kFxEven << 4) >= top) && (h == 0 || h + (kFxEven << 4) >= top);
-  }
+  for (int s = 0; s < 4; ++s) even = even && (z.m[s] == 0 || z.m[s] >= least);
   return even;
 }
 
@@ -442,7 +424,7 @@ OVL_HD float fx_abs_up(int hi) {
 }
 
 // Bits below the largest component of a link at which its smallest entry (its larger component) may lie: for any
-// link, and for one that is not weak. Of random SU(3) links one in 7 10^10 falls below the first and one in 250
+// link, and for one that is not weak; there also its largest real and its largest imaginary part. Of random SU(3) links one in 7 10^10 falls below the first and one in 250
 // below the second, so a field of 64^4 sites is refused by chance once in a thousand times; links exp(i eps H)
 // are mostly weak below eps = 0.04.
 constexpr int kFxMixAny = 20, kFxMixMost = 6;
@@ -453,7 +435,7 @@ constexpr int kFxMixAny = 20, kFxMixMost = 6;
 OVL_HD void fx_link_range(const Mat3<double>& u, double& top, double& need, bool& weak) {
   float row[3] = {0, 0, 0}, col[3] = {0, 0, 0};
   unsigned long long m = 0;
-  int least = 0x7fffffff;
+  int least = 0x7fffffff, re = 0, im = 0;
 #pragma unroll
   for (int i = 0; i < 9; ++i) {
     int hr, hi;
@@ -468,12 +450,15 @@ OVL_HD void fx_link_range(const Mat3<double>& u, double& top, double& need, bool
     m = m > wi ? m : wi;
     const int entry = hr > hi ? hr : hi;
     least = least < entry ? least : entry;
+    re = re > hr ? re : hr;
+    im = im > hi ? im : hi;
     const float a = fx_abs_up(hr) + fx_abs_up(hi);
     row[i / 3] += a;
     col[i % 3] += a;
   }
   const int most = (int)(m >> 32);
-  weak = least < most - (kFxMixMost << 20);
+  const int part = re < im ? re : im;
+  weak = (least < part ? least : part) < most - (kFxMixMost << 20);
   float sum = row[0];
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
@@ -559,11 +544,10 @@ OVL_HD bool fx_hops(const Geom& g, const FxC* U, int s, int k0, int k1, const Fx
     {
       Spin<double> p;
       ld(nb, p);
-      unsigned m[4];
+      int m[4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) m[i] = fx_max2(fx_max2(fx_size(p.c[i][0]), fx_size(p.c[i][1])), fx_size(p.c[i][2]));
-      const unsigned t = fx_max2(fx_max2(m[0], m[1]), fx_max2(m[2], m[3]));
-      const int w = (int)(t & 0xffffu) > (int)(t >> 16) ? (int)(t & 0xffffu) : (int)(t >> 16), eb = w >> 4;
+      for (int i = 0; i < 4; ++i) m[i] = fx_spin_word(p, i);
+      const int t = m[0] > m[1] ? m[0] : m[1], u = m[2] > m[3] ? m[2] : m[3], w = t > u ? t : u, eb = w >> 20;
       top = top > w ? top : w;
       const int ft = k < 6 ? 0 : (k & 1) ? c.bt : c.ft;
       if (ft != 0) {
@@ -571,7 +555,7 @@ OVL_HD bool fx_hops(const Geom& g, const FxC* U, int s, int k0, int k1, const Fx
         for (int i = 0; i < 4; ++i) m[i] = fx_raise(m[i], ft);
       }
 #pragma unroll
-      for (int i = 0; i < 4; ++i) z.m[i] = fx_max2(z.m[i], m[i]);
+      for (int i = 0; i < 4; ++i) z.m[i] = z.m[i] > m[i] ? z.m[i] : m[i];
       const int fe = fx_hop_exponent(k, 0, c), eh = (eb > 64 ? eb : 64) + fe;
       if (eh > E) {  // first hop, or a larger neighbour than any before
         if (E != 0) {
@@ -609,7 +593,7 @@ OVL_HD bool fx_hops(const Geom& g, const FxC* U, int s, int k0, int k1, const Fx
     }
     return any == 0;
   }
-  return E < 2000 && top >= 64 << 4;  // (E is above 2047 beside an infinity or a NaN)
+  return E < 2000 && top >= 64 << 20;  // (E is above 2047 beside an infinity or a NaN)
 }
 // All eight hops.
 template <class Load>

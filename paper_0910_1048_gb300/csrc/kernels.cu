@@ -294,7 +294,7 @@ __global__ void __launch_bounds__(128, 3)
     k_dslash_f64_split(Geom g, Links U, FxCoef c, bool native, bool g5_in, bool g5_out, const double2* in, double2* out) {
   __shared__ fx64 part[4][3][6][32];  // [receiving spin][slot of the sender][component][site]
   __shared__ int expo[4][32];
-  __shared__ unsigned size[4][4][32];  // [spin][thread][site]
+  __shared__ int size[4][4][32];  // [spin][thread][site]
   const int lane = threadIdx.x, t = threadIdx.y;
   const bool live = (int)blockIdx.x * 32 + lane < g.vol;
   const int s = live ? blockIdx.x * 32 + lane : g.vol - 1;
@@ -313,7 +313,7 @@ __global__ void __launch_bounds__(128, 3)
   const int Em = max(max(expo[0][lane], expo[1][lane]), max(expo[2][lane], expo[3][lane]));
 #pragma unroll
   for (int sp = 0; sp < 4; ++sp)
-    z.m[sp] = fx_max2(fx_max2(size[sp][0][lane], size[sp][1][lane]), fx_max2(size[sp][2][lane], size[sp][3][lane]));
+    z.m[sp] = max(max(size[sp][0][lane], size[sp][1][lane]), max(size[sp][2][lane], size[sp][3][lane]));
   const bool all = Em < 1 << 20 && fx_even(z);  // no direction needs the FP64 hops
   const int d = min(Em - E, 62);
   if (__any_sync(0xffffffffu, d > 0)) {

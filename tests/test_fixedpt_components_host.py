@@ -165,58 +165,57 @@ def test_where_the_field_rule_ends(field_usable):
     assert not field_usable(synth.gauge_links(DIMS, 4, 1e-5))
 
 
-# ------------------------------------------------------------------ spins, and real and imaginary parts
+# ------------------------------------------------------------------ spins
 def _split_source(kind, small):
-    """Sources whose neighbourhoods hold components of very different size that a hop keeps apart."""
+    """Sources whose neighbourhoods hold spins of very different size that a hop keeps apart."""
     psi = synth.gaussian_source(DIMS, 2)
     if kind == "spin":  # gamma_3 and gamma_4 join spins 0, 2 and 1, 3; the others 0, 3 and 1, 2
         psi[..., 1:, :] *= small
         psi[:, :, 1::2] *= 0
         psi[:, :, :, 1::2] *= 0
-    if kind == "point":  # a point of one spin beside points of another
+    if kind == "point":  # points of one spin beside points of another
         one = psi.copy()
         psi = np.zeros_like(psi)
-        psi[2, 0, 1, 1, 0], psi[2, 0, 1, 3, 1], psi[2, 0, 3, 1, 2] = one[0, 0, 0, 0, 0], small * one[1, 0, 0, 0, 1], one[0, 0, 1, 0, 2]
-    if kind == "real":
-        psi = psi.real + small * 1j * psi.imag
-        psi[:, :, :, 1::2] *= 0
+        psi[2, 0, 1, 1, 0], psi[2, 0, 3, 1, 2] = one[0, 0, 0, 0, 0], one[0, 0, 1, 0, 2]
+        psi[2, 0, 1, 3, 1] = small * one[1, 0, 0, 0, 1]
     return psi
 
 
 def _spin_sizes(psi, mu):
-    """Largest of |re| and of |im| of each spin over a site's neighbours, with the time hops' factors: [V][4][2]."""
-    a = np.stack([np.abs(psi.real).max(-1), np.abs(psi.imag).max(-1)], -1)
+    """Largest component of each spin over a site's neighbours, with the time hops' factors: [V][4]."""
+    a = np.maximum(np.abs(psi.real), np.abs(psi.imag)).max(-1)
     m = np.zeros_like(a)
     for ax in range(4):
         for sh in (1, -1):
             m = np.maximum(m, np.roll(a, sh, ax) * (np.exp(-sh * mu) if ax == 0 else 1.0))
-    return m.reshape(VOL, 4, 2)
-
-
-def _real_links():
-    """SO(3) links: real and imaginary parts are joined by the gammas alone."""
-    q, r = np.linalg.qr(np.random.default_rng(8).standard_normal((4, 8, 2, 6, 4, 3, 3)))
-    return (q * np.sign(np.diagonal(r, axis1=-2, axis2=-1))[..., None, :]).astype(complex)
+    return m.reshape(VOL, 4)
 
 
 @pytest.mark.parametrize("mu", [0.0, 0.3, -5.0])
 @pytest.mark.parametrize("small", [1e-3, 1e-10, 1e-20])
-@pytest.mark.parametrize("kind", ["spin", "point", "real"])
+@pytest.mark.parametrize("kind", ["spin", "point"])
 def test_sites_with_a_small_spin_are_refused(lib, kind, small, mu):
-    """A site keeps fixed point only if the real and imaginary parts of each spin, over its neighbours, are all
-    zero or reach 2^-6 of the largest (to 2^-4 in the sizes' four mantissa bits and a factor two in the time hops'
-    factors). The other sites take the FP64 hops, so every result is as accurate as a component's terms allow."""
-    u, psi = _real_links() if kind == "real" else synth.gauge_links(DIMS, 1), _split_source(kind, small)
+    """A site keeps fixed point only if each spin, over its neighbours, is zero or reaches 2^-6 of the largest (up
+    to a factor of four: the mantissas' share of the words and the time hops' factors by their exponents). The
+    other sites take the FP64 hops."""
+    u, psi = synth.gauge_links(DIMS, 1), _split_source(kind, small)
     ok, fx, f64, efx, _, usable = _check(lib, u, psi, mu)
     assert ok
     m = _spin_sizes(psi, mu)
-    top = m.max((1, 2))[:, None, None]
-    assert ((m == 0) | (m >= 2.0 ** -7.2 * top))[usable].all()
-    zero = m.max((1, 2)) == 0
-    assert usable[zero].all()
-    even = ((m == 0) | (m >= 2.0 ** -4.8 * top)).all((1, 2))
-    assert usable[even].all()
+    top = m.max(1)[:, None]
+    assert ((m == 0) | (m >= 2.0 ** -8 * top))[usable].all()
+    assert usable[top[:, 0] == 0].all()
+    assert usable[((m == 0) | (m >= 2.0 ** -4 * top)).all(1)].all()
+    assert not usable.all()
     assert not fx[:, usable][f64[:, usable] == 0].any()
+
+
+def test_real_links_are_refused(field_usable):
+    """Real links join real and imaginary parts through the gammas alone, as single colours would be."""
+    q, r = np.linalg.qr(np.random.default_rng(8).standard_normal((4, 8, 2, 6, 4, 3, 3)))
+    u = (q * np.sign(np.diagonal(r, axis1=-2, axis2=-1))[..., None, :]).astype(complex)
+    assert not field_usable(u) and not field_usable(1j * u)
+    assert field_usable(u * np.exp(0.1j))
 
 
 def test_gaussian_sources_are_served(lib):
