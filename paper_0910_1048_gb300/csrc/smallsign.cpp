@@ -477,18 +477,20 @@ bool tri_solve(int k, const cz* al, const cz* be, const cz* de, double c, LaneVe
 // (no cancellation: the factors are applied one after the other). Returns false if a solve
 // meets a zero pivot.
 bool rational_apply(int k, const cz* al, const cz* be, const cz* de, double c, int s, const cz* v, cz* out) {
-  // the s shifted solves are independent: split them over host threads, each summing its
-  // own shifts in order, then add the per-thread sums in thread order (deterministic)
-  const int hw = std::max(1, (int)std::thread::hardware_concurrency() / std::max(1, g_sign_concurrency));
-  // (a thread takes whole groups of kLanes shifts; from about 5000 rows each it pays to start one)
+  // The s shifted solves are independent. They are split into parts by (s, k) alone, each part summing its shifts in
+  // order and the parts added in order, so that the result does not depend on how many host threads there are or
+  // how many evaluations run side by side: a source's solve is the same alone and in a batch.
+  // (a part takes whole groups of kLanes shifts; from about 5000 rows each it pays to start a thread)
   const int ngroup = (s + kLanes - 1) / kLanes;
-  const int nth = std::max(1, std::min({hw, 16, ngroup, (int)((size_t)s * k / 5000 + 1)}));
-  std::vector<std::vector<cz>> part(nth, std::vector<cz>(k, 0.0));
-  std::vector<char> ok(nth, 1);
-  auto work = [&](int tid) {
-    std::vector<cz>& acc = part[tid];
+  const int npart = std::max(1, std::min({16, ngroup, (int)((size_t)s * k / 5000 + 1)}));
+  const int hw = std::max(1, (int)std::thread::hardware_concurrency() / std::max(1, g_sign_concurrency));
+  const int nth = std::min(hw, npart);
+  std::vector<std::vector<cz>> part(npart, std::vector<cz>(k, 0.0));
+  std::vector<char> ok(npart, 1);
+  auto sum_part = [&](int p) {
+    std::vector<cz>& acc = part[p];
     std::vector<Lanes> x(k), inv(k), du(k), du2(k);
-    for (int gr = tid; gr < ngroup; gr += nth) {
+    for (int gr = p; gr < ngroup; gr += npart) {
       LaneVec om, tp;
       for (int w = 0; w < kLanes; ++w) {
         const int sh = std::min(s, gr * kLanes + w + 1);  // (lanes past the last shift repeat it, weight 0)
@@ -500,7 +502,7 @@ bool rational_apply(int k, const cz* al, const cz* be, const cz* de, double c, i
       for (int i = 0; i < k; ++i) x[i] = Lanes{zero + v[i].real(), zero + v[i].imag()};
       if (!tri_solve(k, al, be, de, c, -tp, x.data(), inv.data(), du.data(), du2.data()) ||
           !tri_solve(k, al, be, de, c, tp, x.data(), inv.data(), du.data(), du2.data())) {
-        ok[tid] = 0;
+        ok[p] = 0;
         return;
       }
       for (int i = 0; i < k; ++i) {
@@ -511,6 +513,9 @@ bool rational_apply(int k, const cz* al, const cz* be, const cz* de, double c, i
       }
     }
   };
+  auto work = [&](int tid) {
+    for (int p = tid; p < npart; p += nth) sum_part(p);
+  };
   if (nth == 1) {
     work(0);
   } else {
@@ -519,11 +524,11 @@ bool rational_apply(int k, const cz* al, const cz* be, const cz* de, double c, i
     work(0);
     for (auto& t : th) t.join();
   }
-  for (int t = 0; t < nth; ++t)
-    if (!ok[t]) return false;
+  for (int p = 0; p < npart; ++p)
+    if (!ok[p]) return false;
   std::vector<cz> acc(k, 0.0);
-  for (int t = 0; t < nth; ++t)
-    for (int i = 0; i < k; ++i) acc[i] += part[t][i];
+  for (int p = 0; p < npart; ++p)
+    for (int i = 0; i < k; ++i) acc[i] += part[p][i];
   for (int i = 0; i < k; ++i) {
     cz t = al[i] * acc[i];
     if (i > 0) t += de[i - 1] * acc[i - 1];
