@@ -58,8 +58,7 @@ def build(verbose: bool = False, extra: list[str] | None = None) -> str:
         if _stale(o, s):
             cmd = [nvcc] + ARCH + FLAGS + (extra or []) + ["-c", s, "-o", o]
             if s.endswith(".cpp"):
-                # (std::complex products and quotients without the recovery of infinities)
-                cmd = [nvcc] + FLAGS + (extra or []) + ["-Xcompiler", "-fcx-limited-range", "-x", "c++", "-c", s, "-o", o]
+                cmd = [nvcc] + FLAGS + (extra or []) + ["-x", "c++", "-c", s, "-o", o]
             jobs.append(cmd)
     probe_obj = os.path.join(BUILD, "fp64_peak.cu.o")
     if not os.path.exists(probe_obj) or os.path.getmtime(probe_obj) < os.path.getmtime(PROBE_SRC):

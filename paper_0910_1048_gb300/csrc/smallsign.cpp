@@ -56,6 +56,11 @@ inline cz csqrt_fast(cz z) {
 }
 
 
+// Product of finite numbers (std::complex's operator also looks for infinities to recover).
+inline cz cmul(cz a, cz b) {
+  return cz(a.real() * b.real() - a.imag() * b.imag(), a.real() * b.imag() + a.imag() * b.real());
+}
+
 struct Rot {
   int p;
   cz c, s;
@@ -330,24 +335,24 @@ bool cs_eigs(std::vector<cz> d, std::vector<cz> e2, std::vector<cz>& lam) {
     const cz shift = std::norm(m1 - b) < std::norm(m2 - b) ? m1 : m2;
     cz c = 1.0, s = 0.0;
     cz gam = d[lo] - shift;
-    cz p = gam * gam;
+    cz p = cmul(gam, gam);
     for (int i = lo; i < hi; ++i) {
       const cz bb = e2[i];
       const cz r = p + bb;
       const double nr = std::norm(r);
       if (!(nr > 1e-32 * (std::norm(p) + std::norm(bb)))) return false;  // cancellation, or not finite
       const cz inv_r = std::conj(r) * (1.0 / nr);
-      if (i > lo) e2[i - 1] = s * r;
+      if (i > lo) e2[i - 1] = cmul(s, r);
       const cz oldc = c, oldgam = gam;
-      c = p * inv_r;
-      s = bb * inv_r;
+      c = cmul(p, inv_r);
+      s = cmul(bb, inv_r);
       const cz alpha = d[i + 1];
-      gam = c * (alpha - shift) - s * oldgam;
+      gam = cmul(c, alpha - shift) - cmul(s, oldgam);
       d[i] = oldgam + (alpha - gam);
       const double nc = std::norm(c);
-      p = nc > 0.0 ? gam * gam * std::conj(c) * (1.0 / nc) : oldc * bb;
+      p = nc > 0.0 ? cmul(cmul(gam, gam), std::conj(c)) * (1.0 / nc) : cmul(oldc, bb);
     }
-    e2[hi - 1] = s * p;
+    e2[hi - 1] = cmul(s, p);
     d[hi] = shift + gam;
   }
   lam = d;
@@ -581,12 +586,8 @@ ovl_status small_sign_rational(int k, const cz* al, const cz* be, const cz* de, 
 // steps would dominate a solve beyond), 1 QL only, 2 Newton only, 3 rational only.
 // hint_c/hint_s (may be null) carry (c, s) between calls on growing H_k.
 constexpr int kNewtonMaxK = 200;
-ovl_status small_sign(int k, const cz* al, const cz* be, const cz* de, cz* y, int method, double* hint_c = nullptr,
-                      int* hint_s = nullptr, int* ritz_count = nullptr) {
-  if (k < 1) {
-    set_error("small_sign: k < 1");
-    return OVL_EINVAL;
-  }
+static ovl_status small_sign_routes(int k, const cz* al, const cz* be, const cz* de, cz* y, int method, double* hint_c,
+                                    int* hint_s, int* ritz_count) {
   if (k == 1) {
     if (al[0].real() == 0.0) {
       set_error("small_sign: eigenvalue on the imaginary axis");
@@ -614,6 +615,40 @@ ovl_status small_sign(int k, const cz* al, const cz* be, const cz* de, cz* y, in
     return OVL_ENOCONV;
   }
   return small_sign_newton(k, al, be, de, y);
+}
+
+// sign(c H) = sign(H): where the largest entry is far from 1, the routes (which form fourth powers of the entries)
+// get H times a power of two.
+ovl_status small_sign(int k, const cz* al, const cz* be, const cz* de, cz* y, int method, double* hint_c = nullptr,
+                      int* hint_s = nullptr, int* ritz_count = nullptr) {
+  if (k < 1) {
+    set_error("small_sign: k < 1");
+    return OVL_EINVAL;
+  }
+  double top = 0;
+  auto size = [](cz z) { return std::max(std::fabs(z.real()), std::fabs(z.imag())); };
+  for (int i = 0; i < k; ++i) top = std::max(top, size(al[i]));
+  for (int i = 0; i + 1 < k; ++i) top = std::max({top, size(be[i]), size(de[i])});
+  ovl_status s;
+  if (top > 0 && std::isfinite(top) && (top < 0x1p-60 || top > 0x1p60)) {
+    const int e = -std::ilogb(top);
+    auto scaled = [&](const cz* a, int n) {
+      std::vector<cz> v(n);
+      for (int i = 0; i < n; ++i) v[i] = cz(std::scalbn(a[i].real(), e), std::scalbn(a[i].imag(), e));
+      return v;
+    };
+    const std::vector<cz> a = scaled(al, k), b = scaled(be, k - 1), d = scaled(de, k - 1);
+    s = small_sign_routes(k, a.data(), b.data(), d.data(), y, method, nullptr, nullptr, ritz_count);
+    if (hint_s) *hint_s = 0;
+  } else {
+    s = small_sign_routes(k, al, be, de, y, method, hint_c, hint_s, ritz_count);
+  }
+  for (int i = 0; i < k && s == OVL_OK; ++i)
+    if (!std::isfinite(y[i].real()) || !std::isfinite(y[i].imag())) {
+      set_error("small_sign: the result is not finite at k = %d", k);
+      s = OVL_ENOCONV;
+    }
+  return s;
 }
 
 }  // namespace ovl
