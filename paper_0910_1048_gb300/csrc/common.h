@@ -116,6 +116,7 @@ struct Links {
   const double2* f64 = nullptr;   // [4][9][V]
   const FxC* fx = nullptr;        // [4][9][V] fixed-point copy of the FP64 links (fixedpt.cuh)
   const FxField* fxf = nullptr;   // its scale, and whether it can be used
+  bool fits = false;              // the same as the host knows it at the launch: for the choice of a kernel only
   const float2* f32 = nullptr;    // [4][9][V]
   const uint32_t* f16 = nullptr;  // [4][6][V] half2 bits, rows 0 and 1
 };
@@ -171,6 +172,7 @@ struct ovl_lattice {
     l.f64 = u64;
     l.fx = ufx;
     l.fxf = fxf;
+    l.fits = fx_ok;
     l.f32 = u32;
     l.f16 = u16;
     return l;

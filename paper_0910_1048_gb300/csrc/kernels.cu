@@ -286,6 +286,23 @@ __global__ void __launch_bounds__(kBlock, 3)
   for (int q = 0; q < 12; ++q) stc<double>(out + off, (size_t)s * ss + (size_t)q * cs, o.c[q / 3][q % 3]);
 }
 
+// In FP64 arithmetic, for fields and factors that do not fit fixed point (as the host knows them at the launch). The
+// kernels around it fall back on the FP64 hops site by site, but carry the integer hops' registers and call the others
+// out of line: unit links 4^4 37.5 us here, 54 there, 12^4 67 against 72, and 89 with four threads per site.
+template <class Ld>
+__global__ void __launch_bounds__(kBlock)
+    k_dslash_plain64(Geom g, Links U, HopCoef<double> c, bool native, bool g5_out, const double2* in, double2* out) {
+  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+  if (s >= g.vol) return;
+  const size_t off = (size_t)blockIdx.y * 12 * g.vol;
+  const int ss = native ? 1 : 12, cs = native ? g.vol : 1;
+  Spin<double> o;
+  dslash_site<LINK_F64, double>(g, U, s, c, Ld{in + off, ss, cs}, o);
+  if (g5_out) gamma5_inplace(o);
+#pragma unroll
+  for (int q = 0; q < 12; ++q) stc<double>(out + off, (size_t)s * ss + (size_t)q * cs, o.c[q / 3][q % 3]);
+}
+
 // The same with four threads per site (block (32 sites, 4)), one direction's two hops each, for fields too
 // small to fill the GPU with one thread per site: a site's eight hops in a row are about 16 K cycles of one
 // warp's latency. The directions' sums are aligned to their largest exponent and exchanged as integers;
@@ -551,12 +568,18 @@ cudaError_t launch_dslash(const Geom& g, const Links& U, int lf, bool f64, doubl
     const FxCoef c = fx_coef(m_w, mu);
     // one source at 8^4 22.8 -> 13.4 us and 12^4 29.7 -> 22.7 with four threads per site; 14^4 30.8 against
     // 33.4. By the volume alone, so that a source's result is the same alone and in a batch.
-    if (g.vol <= 28672)
+    const dim3 sites((g.vol + kBlock - 1) / kBlock, nrhs);
+    if (!(U.fits && c.ok) && g5_in)
+      k_dslash_plain64<StrideLoaderG5><<<sites, kBlock, 0, st>>>(g, U, c.k, native, g5_out, (const double2*)in,
+                                                                 (double2*)out);
+    else if (!(U.fits && c.ok))
+      k_dslash_plain64<StrideLoader><<<sites, kBlock, 0, st>>>(g, U, c.k, native, g5_out, (const double2*)in,
+                                                               (double2*)out);
+    else if (g.vol <= 28672)
       k_dslash_f64_split<<<dim3((g.vol + 31) / 32, nrhs), dim3(32, 4), 0, st>>>(g, U, c, native, g5_in, g5_out,
                                                                                (const double2*)in, (double2*)out);
     else
-      k_dslash_f64<<<dim3((g.vol + kBlock - 1) / kBlock, nrhs), kBlock, 0, st>>>(g, U, c, native, g5_in, g5_out,
-                                                                               (const double2*)in, (double2*)out);
+      k_dslash_f64<<<sites, kBlock, 0, st>>>(g, U, c, native, g5_in, g5_out, (const double2*)in, (double2*)out);
     return cudaGetLastError();
   }
   // Batches in views that start on 8 bytes: k_dslash2 by 8-byte requests where the links would come from HBM for every
