@@ -831,8 +831,9 @@ size_t direct_footprint(int vol, int nrhs, int kmax, bool f64, bool two_pass) {
   const size_t n = (size_t)12 * vol, elt = f64 ? 16 : 8;
   if (two_pass) kmax = 2;  // three basis columns in a rotating window, plus the FP64 accumulator of x
   const size_t xacc = two_pass ? n * 16 : 0;
+  const size_t fx = f64 ? kFxExponents * 4 * (size_t)vol + fx_step_bytes() : 0;  // the fixed-point step's own arrays
   const size_t slots = (n + kVecBlock - 1) / kVecBlock + kMaxFillSMs;  // partial_slots
-  return (size_t)nrhs * ((size_t)(kmax + 1) * n * elt + 4 * n * elt + 3 * n * 16 + xacc + 16 * slots * 32) +
+  return (size_t)nrhs * ((size_t)(kmax + 1) * n * elt + 4 * n * elt + 3 * n * 16 + xacc + fx + 16 * slots * 32) +
          ((size_t)1 << 20);
 }
 
