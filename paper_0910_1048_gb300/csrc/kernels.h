@@ -249,7 +249,7 @@ struct MsDev {
 struct MsVecs {
   void *r = nullptr, *rt = nullptr, *p = nullptr, *pt = nullptr;  // [nrhs][12][V]
   void *t = nullptr, *tt = nullptr;                               // [nrhs][12][V]
-  void* ps = nullptr;          // [nrhs][s][12][V] shifted directions
+  void* ps = nullptr;          // [nrhs][s][12][V] shifted directions (null: k_ms_dirs_seed, which has none)
   double2* X = nullptr;        // [nrhs][12][V] FP64 sum_i omega_i x^(i)
   double2* xp = nullptr;       // [nrhs][12][V] FP64 x_P (nullptr without deflation)
   double2* xs = nullptr;       // [nrhs][s][12][V] per-shift solutions (refinement only; else X): float-float

@@ -53,7 +53,8 @@ __global__ void __launch_bounds__(kBlock) k_ms_start(Geom g, MsDev ms, MsVecs v,
       stc<R>((T*)v.p, e, rr);
       stc<R>((T*)v.rt, e, rtt);
       stc<R>((T*)v.pt, e, rtt);
-      for (int i = 0; i < ms.s; ++i) stc<R>((T*)v.ps, ((size_t)rhs * ms.s + i) * n + (size_t)c * g.vol + s, rr);
+      if (v.ps)
+        for (int i = 0; i < ms.s; ++i) stc<R>((T*)v.ps, ((size_t)rhs * ms.s + i) * n + (size_t)c * g.vol + s, rr);
       // rho and |r| from the stored (rounded) vectors, so the recurrences start consistent
       zd rd = mk((double)rr.re, (double)rr.im), rtd = mk((double)rtt.re, (double)rtt.im);
       zd ip = cdot(rtd, rd);

@@ -123,8 +123,8 @@ static ovl_status ensure_mws(ovl_lattice* lat, int nrhs, int s, bool f64, int m,
   size_t o_ls = take((size_t)std::max(m, 1) * 8);
   const size_t rn = refine ? n : 0;
   // correction batch: at most kRefineGroup systems and about kRefineBytes of buffers
-  // (per system 9 FP32 vectors + 5 FP64 vectors)
-  const size_t per_sys = n * (9 * 8 + 5 * 16);
+  // (per system 6 FP32 vectors + 5 FP64 vectors: its only shift is the seed, so it has no shifted directions)
+  const size_t per_sys = n * (6 * 8 + 5 * 16);
   size_t ref_bytes = kRefineBytes;
   if (refine) {
     size_t free_b = 0, total_b = 0;
@@ -140,8 +140,8 @@ static ovl_status ensure_mws(ovl_lattice* lat, int nrhs, int s, bool f64, int m,
   size_t o_res = take(gq * rn * 16), o_t1 = take(gq * rn * 16), o_t2 = take(gq * rn * 16), o_ec = take(gq * rn * 16);
   size_t o_rp = take(std::max<size_t>(1, gq) * vec_blocks(lat->g) * 8), o_ro = take(std::max<size_t>(1, gq) * 8),
          o_oz = take(16), o_rc = take(std::max<size_t>(1, gq) * 4);
-  size_t o_gvec[7];
-  for (int i = 0; i < 7; ++i) o_gvec[i] = take(gq * rn * 8);
+  size_t o_gvec[6];
+  for (int i = 0; i < 6; ++i) o_gvec[i] = take(gq * rn * 8);
   size_t o_gX = take(gq * rn * 16), o_gk = take(gq * 4), o_gst = take(gq * 4), o_gseed = take(gq * 8 * 16),
          o_gz = take(gq * 3 * 16), o_ga = take(gq * 16), o_gb = take(gq * 16), o_gact = take(gq * 4),
          o_gpa = take(gq * nblk * 4 * 8), o_gcn = take(gq * 4), o_sga = take((size_t)s * 8), o_gsig = take(gq * 8),
@@ -198,8 +198,8 @@ static ovl_status ensure_mws(ovl_lattice* lat, int nrhs, int s, bool f64, int m,
     w->t1 = (double2*)(b + o_t1);
     w->t2 = (double2*)(b + o_t2);
     w->ecan = (double2*)(b + o_ec);
-    void** gp[7] = {&w->gv.r, &w->gv.rt, &w->gv.p, &w->gv.pt, &w->gv.t, &w->gv.tt, &w->gv.ps};
-    for (int i = 0; i < 7; ++i) *gp[i] = b + o_gvec[i];
+    void** gp[6] = {&w->gv.r, &w->gv.rt, &w->gv.p, &w->gv.pt, &w->gv.t, &w->gv.tt};
+    for (int i = 0; i < 6; ++i) *gp[i] = b + o_gvec[i];
     w->gv.X = (double2*)(b + o_gX);
     MsDev& gm = w->gms;
     gm.nrhs = grp;
@@ -625,7 +625,7 @@ size_t multishift_footprint(int vol, int nrhs, int s, bool f64, bool refine) {
   size_t b = nr * n * (6 * elt + (size_t)s * elt + 5 * 16) + nr * 16 * slots * 32;  // (deflation dots: m <= 16)
   if (refine) {
     const size_t gq = std::min<size_t>(nr * s, kRefineGroup);
-    b += nr * s * n * 16 + nr * n * 16 + gq * n * (4 * 16 + 7 * 8 + 16) + gq * slots * 32;
+    b += nr * s * n * 16 + nr * n * 16 + gq * n * (4 * 16 + 6 * 8 + 16) + gq * slots * 32;
   }
   return b + ((size_t)1 << 20);
 }

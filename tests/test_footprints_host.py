@@ -37,3 +37,15 @@ def test_direct(lib, vol, nrhs, f64, two_pass):
         need += 6 * 4 * vol + 256  # exponents of the six fixed-point vectors, the step's coefficients
     got = lib[0](vol, nrhs, kmax, f64, two_pass)
     assert nrhs * need <= got <= 1.001 * nrhs * need + (2 << 20)
+
+
+@pytest.mark.parametrize("vol,nrhs,s", [(256, 1, 4), (20736, 1, 20), (65536, 4, 20), (65536, 16, 80)])
+@pytest.mark.parametrize("f64,refine", [(True, False), (False, False), (False, True)])
+def test_multishift(lib, vol, nrhs, s, f64, refine):
+    elt, vec = 16 if f64 else 8, 12 * vol
+    need = nrhs * (6 * vec * elt + s * vec * elt + 5 * vec * 16 + DEFL * _slots(vol) * 32)
+    if refine:  # x^(i), r, and up to 1024 corrections: four FP64 vectors, six FP32 ones, their sum, partial sums
+        systems = min(1024, nrhs * s)
+        need += nrhs * (s + 1) * vec * 16 + systems * (vec * (4 * 16 + 6 * 8 + 16) + _slots(vol) * 32)
+    got = lib[1](vol, nrhs, s, f64, refine)
+    assert need <= got <= 1.001 * need + (2 << 20)
