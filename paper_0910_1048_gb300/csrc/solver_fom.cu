@@ -172,9 +172,6 @@ ovl_status solve_fom(ovl_lattice* lat, const ovl_sign_params* p, int nrhs, const
   OVL_CHECK_CUDA(cudaMemcpyAsync(beta.data(), f.beta, nr * 8, cudaMemcpyDeviceToHost, st));
   OVL_CHECK_CUDA(cudaStreamSynchronize(st));
   r0 = beta;
-  // the batched reduced-precision stencil picks its link-group size on its first call (it
-  // synchronises): make that call before the cycle is captured
-  OVL_CHECK_CUDA(launch_dslash(g, U, lf, f64, p->m_W, p->mu, false, true, true, nrhs, f.V, tmp, st));
   // ---- one cycle of k Arnoldi steps, captured once and replayed
   auto arnoldi_step = [&](int j, cudaEvent_t* ev) -> cudaError_t {
     cudaError_t e;
