@@ -344,15 +344,6 @@ __device__ __forceinline__ void store_spin(typename V2<R>::T* p, int vol, int s,
 
 
 // ------------------------------------------------------------------ hops of a site
-// Hop coefficients by precision: the FP64 stencils run in fixed point (fixedpt.cuh).
-template <class R> struct HopsOf { using T = HopCoef<R>; };
-template <> struct HopsOf<double> { using T = FxCoef; };
-template <class R>
-inline typename HopsOf<R>::T hops_of(double m_w, double mu) {
-  if constexpr (sizeof(R) == 8) return fx_coef(m_w, mu);
-  else return hop_coef<R>(m_w, mu);
-}
-
 // Spinor loads with the layout as run-time strides: component c of site s at s * ss + c * cs.
 struct StrideLoader {
   const double2* p;
@@ -428,11 +419,11 @@ __device__ __forceinline__ void add_hops(const Geom& g, const Links& U, int s, c
   finish_hops(g, U, s, 0, 8, c, ld, g5in, fx, acc, E, out);
 }
 
-// out = D_W psi at site s, psi native.
-template <int LF, class R>
-__device__ __forceinline__ void stencil_site(const Geom& g, const Links& U, int s, const typename HopsOf<R>::T& c,
+// out = D_W psi at site s, psi native. The type of the coefficients chooses the hops: FxCoef fixed point (FP64).
+template <int LF, class R, class Coef>
+__device__ __forceinline__ void stencil_site(const Geom& g, const Links& U, int s, const Coef& c,
                                              const typename V2<R>::T* in, Spin<R>& out) {
-  if constexpr (sizeof(R) == 8)
+  if constexpr (std::is_same_v<Coef, FxCoef>)
     add_hops(g, U, s, c, StrideLoader{in, 1, g.vol}, false, out);
   else
     dslash_site<LF, R>(g, U, s, c, Loader<R, true>{in, g.vol, false}, out);

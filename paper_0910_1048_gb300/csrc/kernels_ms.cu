@@ -270,10 +270,9 @@ struct MsPairSum {
   }
 };
 
-template <class R, int LF, int MODE>
-__global__ void __launch_bounds__(2 * kPairSites, sizeof(R) == 8 ? 3 : 5) k_ms_pair(Geom g, Links U, typename HopsOf<R>::T cp,
-                                                            typename HopsOf<R>::T cm, MsDev ms,
-                                                            MsVecs v) {
+template <class R, int LF, int MODE, class Coef>
+__global__ void __launch_bounds__(2 * kPairSites, std::is_same_v<Coef, FxCoef> ? 3 : sizeof(R) == 8 ? 1 : 5)
+    k_ms_pair(Geom g, Links U, Coef cp, Coef cm, MsDev ms, MsVecs v) {
   using T = typename V2<R>::T;
   __shared__ cplx<R> xch[12][kPairSites];
   const int rhs = blockIdx.y;
@@ -359,10 +358,8 @@ __global__ void __launch_bounds__(2 * kPairSites, sizeof(R) == 8 ? 3 : 5) k_ms_p
 }
 
 // The same with eight threads per site (pair_split): each thread finishes one spin of its site.
-template <class R, int LF, int MODE>
-__global__ void __launch_bounds__(8 * kSplitSites) k_ms_pair_split(Geom g, Links U, typename HopsOf<R>::T cp,
-                                                                   typename HopsOf<R>::T cm,
-                                                                   MsDev ms, MsVecs v) {
+template <class R, int LF, int MODE, class Coef>
+__global__ void __launch_bounds__(8 * kSplitSites) k_ms_pair_split(Geom g, Links U, Coef cp, Coef cm, MsDev ms, MsVecs v) {
   using T = typename V2<R>::T;
   __shared__ SplitSmem<R> sm;
   __shared__ cplx<R> xch[12][kSplitSites];
@@ -381,7 +378,7 @@ __global__ void __launch_bounds__(8 * kSplitSites) k_ms_pair_split(Geom g, Links
   const R s1 = s1v[0];
   MsPairSum<R, MODE> sum;
   cplx<R> x[3];
-  pair_split<R, LF, typename HopsOf<R>::T>(g, U, cp, cm, in0, in1, sm, [&](int which, int s, int sp, cplx<R> (&o)[3]) {
+  pair_split<R, LF, Coef>(g, U, cp, cm, in0, in1, sm, [&](int which, int s, int sp, cplx<R> (&o)[3]) {
     const R g5 = sp >= 2 ? (R)-1 : (R)1;
     if constexpr (MODE == 0) {
       T* out = (T*)(which ? v.tt : v.t) + voff<R>(rhs, n);
@@ -597,22 +594,21 @@ bool ms_pair_split(const Geom& g, int key) {
   return tv < 0 ? use_split(g) : (tv == 1 || tv == 4 || tv == 5);  // 0, 2, 3, 6, 7, 8: one thread per site
 }
 
-template <class R, int LF>
-static cudaError_t ms_step_t(const Geom& g, const Links& U, double m_w, double mu, const MsDev& ms, const MsVecs& v,
-                             cudaStream_t st, cudaEvent_t* ev) {
+template <class R, int LF, class Coef>
+static cudaError_t ms_step_t(const Geom& g, const Links& U, const Coef& cp, const Coef& cm, const MsDev& ms,
+                             const MsVecs& v, cudaStream_t st, cudaEvent_t* ev) {
   dim3 grid(vec_blocks(g), ms.nrhs);
   dim3 pgrid((g.vol + kPairSites - 1) / kPairSites, ms.nrhs), pblock(kPairSites, 2);
-  const typename HopsOf<R>::T cp = hops_of<R>(m_w, mu), cm = hops_of<R>(m_w, -mu);
   dim3 sgrid((g.vol + kSplitSites - 1) / kSplitSites, ms.nrhs), sblock(kSplitSites, 8);
   const bool split = ms_pair_split(g, sizeof(R) == 8 ? 0 : LF);
   cudaError_t e;
   if (ev && (e = record_timing(ev[0], st))) return e;
-  e = split ? launch_plain(k_ms_pair_split<R, LF, 0>, sgrid, sblock, st, g, U, cp, cm, ms, v)
-            : launch_plain(k_ms_pair<R, LF, 0>, pgrid, pblock, st, g, U, cp, cm, ms, v);
+  e = split ? launch_plain(k_ms_pair_split<R, LF, 0, Coef>, sgrid, sblock, st, g, U, cp, cm, ms, v)
+            : launch_plain(k_ms_pair<R, LF, 0, Coef>, pgrid, pblock, st, g, U, cp, cm, ms, v);
   if (e) return e;
   if (ev && (e = record_timing(ev[1], st))) return e;
-  e = split ? launch_plain(k_ms_pair_split<R, LF, 1>, sgrid, sblock, st, g, U, cp, cm, ms, v)
-            : launch_plain(k_ms_pair<R, LF, 1>, pgrid, pblock, st, g, U, cp, cm, ms, v);
+  e = split ? launch_plain(k_ms_pair_split<R, LF, 1, Coef>, sgrid, sblock, st, g, U, cp, cm, ms, v)
+            : launch_plain(k_ms_pair<R, LF, 1, Coef>, pgrid, pblock, st, g, U, cp, cm, ms, v);
   if (e) return e;
   if (ev && (e = record_timing(ev[2], st))) return e;
   if (sizeof(R) == 4 && ms.s == 1 && ms.sig1v) {  // a correction batch (each system its own shift as the seed)
@@ -630,9 +626,16 @@ static cudaError_t ms_step_t(const Geom& g, const Links& U, double m_w, double m
 
 cudaError_t launch_ms_step(const Geom& g, const Links& U, int lf, bool f64, double m_w, double mu, const MsDev& ms,
                            const MsVecs& v, cudaStream_t st, cudaEvent_t* ev) {
-  if (f64) return ms_step_t<double, LINK_F64>(g, U, m_w, mu, ms, v, st, ev);
-  if (lf == LINK_F16R12) return ms_step_t<float, LINK_F16R12>(g, U, m_w, mu, ms, v, st, ev);
-  return ms_step_t<float, LINK_F32>(g, U, m_w, mu, ms, v, st, ev);
+  if (f64) {
+    // fixed-point hops where the field and the factors fit them; FP64 ones inlined otherwise (their fallback inside
+    // the fixed-point kernels: unit links, 12^4 pair1 + pair2 129 us against 107 here)
+    const FxCoef cp = fx_coef(m_w, mu), cm = fx_coef(m_w, -mu);
+    if (U.fits && cp.ok && cm.ok) return ms_step_t<double, LINK_F64>(g, U, cp, cm, ms, v, st, ev);
+    return ms_step_t<double, LINK_F64>(g, U, cp.k, cm.k, ms, v, st, ev);
+  }
+  const HopCoef<float> cp = hop_coef<float>(m_w, mu), cm = hop_coef<float>(m_w, -mu);
+  if (lf == LINK_F16R12) return ms_step_t<float, LINK_F16R12>(g, U, cp, cm, ms, v, st, ev);
+  return ms_step_t<float, LINK_F32>(g, U, cp, cm, ms, v, st, ev);
 }
 
 __global__ void __launch_bounds__(kVecBlock) k_ms_residual_batch(int vol, int j0, int s, const double2* r64,

@@ -49,7 +49,7 @@ struct MultiWS {
   int* h_status = nullptr;  // pinned [2][nrhs] status + [2][nrhs] k
   cudaGraphExec_t graph[2] = {nullptr, nullptr};  // alternating chunks, each with its events
   cudaEvent_t tev[2][4] = {};
-  int gchunk = 0, g_lf = -1;
+  int gchunk = 0, g_lf = -1, g_fits = -1;  // (g_fits: whether the field fitted fixed point)
   int g_var = -1, rg_var = -1;  // the pair-stencil shape the graphs were captured with
   double g_mw = 0, g_mu = 0, g_s1 = 0, g_tol = 0;
   cudaStream_t stream = nullptr;
@@ -343,7 +343,8 @@ ovl_status solve_multishift(ovl_lattice* lat, const ovl_sign_params* p, int nrhs
   // middle iteration, so the sampled launches are steady-state ones inside a busy stream
   const int gvar = ms_pair_split(g, f64 ? 0 : lf) ? 1 : 0;  // the stencil shape the graphs launch
   if (use_graph && !(w->graph[0] && w->graph[1] && w->gchunk == chunk && w->g_lf == lf && w->g_mw == p->m_W &&
-                     w->g_mu == p->mu && w->g_s1 == s1 && w->g_tol == ms.tol && w->g_var == gvar)) {
+                     w->g_mu == p->mu && w->g_s1 == s1 && w->g_tol == ms.tol && w->g_var == gvar &&
+                     w->g_fits == (int)U.fits)) {
     const int mid = std::max(1, chunk / 2);
     for (int q = 0; q < 2; ++q) {
       if (w->graph[q]) cudaGraphExecDestroy(w->graph[q]);
@@ -363,6 +364,7 @@ ovl_status solve_multishift(ovl_lattice* lat, const ovl_sign_params* p, int nrhs
     w->gchunk = chunk;
     w->g_lf = lf;
     w->g_var = gvar;
+    w->g_fits = U.fits;
     w->g_mw = p->m_W;
     w->g_mu = p->mu;
     w->g_s1 = s1;

@@ -5,7 +5,7 @@ import numpy as np
 import pytest
 
 import synth
-from oracle import krylov, matsign, wilson
+from oracle import krylov, lanczos, matsign, rational, wilson
 
 pytestmark = pytest.mark.gpu
 
@@ -122,3 +122,29 @@ def test_without_allocation(ovl, ctx, var):
         ovl.ovl_set_pair_variant(256, ovl.OVL_PREC_F64, -1)
         ovl.ovl_destroy_lattice(lat)
     assert float(torch.linalg.vector_norm(x - x_ref) / torch.linalg.vector_norm(x_ref)) < 1e-10
+
+
+@pytest.mark.parametrize("var", [0, 1])
+def test_multishift(ovl, ctx, var):
+    """FP64 multishift (one and eight threads per site) against the dense g(A) b of the same rational function, with a
+    field that does fit in between (the cached graphs follow the field)."""
+    dims, eps = (2, 2, 2, 4), 1e-10
+    u, b = _links(dims, 35, 0.1), synth.gaussian_source(dims, 36, nrhs=2)
+    fit = synth.gauge_links(dims, 37, 0.3)
+    lat = ovl.ovl_create_lattice(ctx, dims, -1)
+    ovl.ovl_set_pair_variant(32, ovl.OVL_PREC_F64, var)
+    try:
+        for links in (u, fit, u):
+            h = wilson.dense_hw(links, dims, -2.0, 0.3)
+            ev = np.linalg.eigvals(h)
+            lo, hi = 0.9 * float(np.abs(ev).min()), 1.1 * float(np.abs(ev).max())
+            s, c, w, sg = rational.neuberger_for_spectrum(lo, hi, eps)
+            ovl.ovl_set_links(lat, links, ovl.OVL_F64)
+            st, info, x = _solve(ovl, lat, b, method=ovl.OVL_MULTISHIFT_BICG, mu=0.3, tol=eps, k_max=2000, spec_lo=lo,
+                                 spec_hi=hi, check_every=10)
+            assert st == ovl.OVL_OK and info[0]["poles"] == s
+            for r in range(2):
+                assert _rel(x[r].ravel(), lanczos.rational_sign_dense(h, b[r].ravel(), w, sg)) < 2e-9, r
+    finally:
+        ovl.ovl_set_pair_variant(32, ovl.OVL_PREC_F64, -1)
+        ovl.ovl_destroy_lattice(lat)
