@@ -5,7 +5,7 @@
 
 using namespace ovl;
 
-// Whether n links u[n][3][3] (complex) may be kept in fixed point: what k_fx_range and k_fx_links decide.
+// Whether n links u[n][3][3] (complex) may be kept in fixed point: what k_fx_links and k_fx_field decide.
 extern "C" int field_usable(const double* u, long long n) {
   double lo = 1e308, hi = 0;
   unsigned weak = 0;
@@ -21,4 +21,12 @@ extern "C" int field_usable(const double* u, long long n) {
   }
   int uexp;
   return fx_field_scale(lo, hi, &uexp) && fx_field_mixes(weak, (size_t)n);
+}
+
+// Fixed-point copies of n components and what the library's conversion is to equal: x 2^(58 - uexp), ties to even.
+extern "C" void convert(const double* x, long long n, int uexp, long long* got, long long* want) {
+  for (long long i = 0; i < n; ++i) {
+    got[i] = fx_link_fixed(x[i], uexp);
+    want[i] = std::llrint(std::ldexp(x[i], 58 - uexp));
+  }
 }

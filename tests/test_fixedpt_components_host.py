@@ -69,11 +69,13 @@ def field_usable(tmp_path_factory):
                     os.path.join(HERE, "native", "linkfield_check.cpp"), "-o", out], check=True)
     so = ctypes.CDLL(out)
     so.field_usable.argtypes = [ctypes.c_void_p, ctypes.c_longlong]
+    so.convert.argtypes = [ctypes.c_void_p, ctypes.c_longlong, ctypes.c_int, ctypes.c_void_p, ctypes.c_void_p]
 
     def usable(u):
         u = np.ascontiguousarray(u)
         return bool(so.field_usable(u.ctypes.data, u.size // 9))
 
+    usable.lib = so
     return usable
 
 
@@ -228,3 +230,16 @@ def test_subnormal_neighbours(lib):
     """A neighbourhood of subnormal components only is not zero."""
     psi = 1e-312 * synth.gaussian_source(DIMS, 2)
     assert not _check(lib, synth.gauge_links(DIMS, 1), psi)[5].any()
+
+
+@pytest.mark.parametrize("uexp", [-8, -1, 0, 3, 8])
+def test_link_components_round_to_nearest(field_usable, uexp):
+    """The links' copy by shifts: x 2^(58 - uexp) to nearest, ties to even, over sizes from the scale to nothing."""
+    rng = np.random.default_rng(9)
+    x = rng.uniform(-1, 1, 20000) * 2.0 ** rng.integers(-70, 1, 20000)
+    ties = (rng.integers(-2 ** 20, 2 ** 20, 4000) + 0.5) * 2.0 ** -58  # halfway between two units
+    x = np.concatenate([x, ties, [0.0, -0.0, 1.0, -1.0, 1 - 2.0 ** -53, 2.0 ** -59, -2.0 ** -59, 2.0 ** -60, 3 * 2.0 ** -60]])
+    x = np.ascontiguousarray(np.concatenate([x * 2.0 ** uexp, [5e-324, -5e-324, 1e-310]]))
+    got, want = np.zeros(len(x), np.int64), np.zeros(len(x), np.int64)
+    field_usable.lib.convert(x.ctypes.data, len(x), uexp, got.ctypes.data, want.ctypes.data)
+    assert (got == want).all()
