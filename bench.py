@@ -148,6 +148,16 @@ def pair_bytes(prec, vol, nrhs):
     """Algorithmic bytes of one pair-stencil launch over `nrhs` right-hand sides."""
     return vol * (PAIR_LINK_BYTES_PER_SITE[prec] + nrhs * PAIR_SPINOR_BYTES_PER_SITE[prec])
 
+
+def fx_pair_work(vol, nrhs, time_factors=True):
+    """(bytes, multiply-adds) of one launch of the fixed-point pair stencil k_fx_pair: the links and, per right-hand
+    side, four vectors of 12 limb quadruples (16 B, as a complex double) with one exponent each a site; 216 integer
+    multiply-adds a hop, three per component for the time hops' factors and for the diagonal, twelve per
+    component for what^H A v."""
+    per_rhs = 2 * 8 * 216 + (2 * 2 * 12 * 3 if time_factors else 0) + 2 * 24 * 3 + 12 * 12
+    return pair_bytes("f64", vol, nrhs) + vol * nrhs * 16, vol * nrhs * per_rhs
+
+
 # FP64 FMA throughput of a GB300 in TFLOP/s (the FMA-chain probe fp64_peak.cu; the
 # bench runs the probe itself and uses this value only when the probe library is missing)
 FP64_PEAK_TFLOPS = 1.256
@@ -331,6 +341,20 @@ def _fp64_peak():
     return FP64_PEAK_TFLOPS, "FP64 FMA-chain probe, earlier measurement on a GB300"
 
 
+def _madwide_peak():
+    """32 x 32 + 64 bit integer multiply-adds of this GPU (10^12 a second) from the same probe library, or None."""
+    import ctypes
+
+    try:
+        lib = ctypes.CDLL(os.path.join(ROOT, "libfp64_peak.so"))
+        out = ctypes.c_double(0.0)
+        if lib.ovl_probe_madwide_tops(ctypes.byref(out)) == 0 and out.value > 0:
+            return out.value
+    except (OSError, AttributeError):
+        pass
+    return None
+
+
 def _sources(wl):
     import synth
 
@@ -464,8 +488,8 @@ def _dslash_gbs(ovl, ctx, u_fn, L=32, reps=20):
 
 def _dslash_batch_gbs(ovl, ctx, u_fn, L=24, nrhs=16, reps=5):
     """FP32 stencil on a batch of `nrhs` sources on an L^4 lattice (native layout): one launch over
-    the batch (links loaded once per site for each group of sources) against `nrhs` single-source
-    launches. Algorithmic bytes per launch: the links once (288 B per site) plus 192 B per site and
+    the batch (two sites per thread, the links from HBM once and from L2 for the other sources) against `nrhs`
+    single-source launches. Algorithmic bytes per launch: the links once (288 B per site) plus 192 B per site and
     source (spinor in and out)."""
     import torch
 
@@ -504,7 +528,10 @@ def _prec_code(ovl, prec):
     return {"f64": ovl.OVL_PREC_F64, "f32": ovl.OVL_PREC_F32, "f16": ovl.OVL_PREC_F32_F16LINKS}[prec]
 
 
-def _roofline(wl, infos, fp64_peak, fp64_src):
+def _roofline(wl, infos, fp64_peak, fp64_src, madwide_peak=None):
+    """The dominant kernel against its bound. FP64 direct solves run k_fx_pair (the workloads' SU(3) fields fit fixed
+    point): integer multiply-adds against the probe's rate; without that rate, and for the other FP64 methods,
+    algorithmic flops against the FP64 peak."""
     peaks, src = _peaks()
     vol = int(np.prod(wl["dims"]))
     kt = [i["t_kernel_ms"] for step in infos for _, inf in step for i in inf[:1] if i["kernel_samples"] > 0]
@@ -515,6 +542,20 @@ def _roofline(wl, infos, fp64_peak, fp64_src):
     import paper_0910_1048_gb300 as ovl
     shape = ovl.ovl_get_pair_variant(vol, _prec_code(ovl, prec))  # the autotuner's pick (ovl_set_pair_variant)
     traffic = TRAFFIC.get((kernel, prec, tuple(wl["dims"]), nr, shape))
+    if prec == "f64" and wl["method"] == "direct" and madwide_peak:
+        kernel = "k_fx_pair"
+        byts, mads = fx_pair_work(vol, nr, any(m != 0 for m in wl["mus"]))
+        ach = mads / (t_pair * 1e-3) / 1e12 if t_pair else None
+        return {"kernel": kernel, "bound": "alu", "achieved": ach, "peak": madwide_peak,
+                "unit": "10^12 integer multiply-adds/s (mad.wide.s32)", "frac": ach / madwide_peak if ach else None,
+                "traffic": TRAFFIC.get((kernel, prec, tuple(wl["dims"]), nr, shape)),
+                "peak_source": "mad.wide.s32 chain probe (fp64_peak.cu) run by bench.py on this GPU",
+                "algorithmic_multiply_adds_per_launch": mads, "algorithmic_bytes_per_launch": byts,
+                "hbm_frac": byts / (t_pair * 1e-3) / 1e9 / peaks["hbm_gbs"] if t_pair else None,
+                "fp64_equivalent_tflops": PAIR_FLOPS_PER_SITE * vol * nr / (t_pair * 1e-3) / 1e12 if t_pair else None,
+                "pair_variant": shape,
+                "note": "at 12^4 the kernel is bound by instruction and load latency at two warps per scheduler "
+                        "(profiles/k_fx_step_f64_lattice12.md)"}
     if prec == "f64":
         flops = PAIR_FLOPS_PER_SITE * vol * nr
         ach = flops / (t_pair * 1e-3) / 1e12 if t_pair else None
@@ -522,9 +563,8 @@ def _roofline(wl, infos, fp64_peak, fp64_src):
                 "frac": (ach / fp64_peak) if ach else None, "traffic": traffic, "peak_source": fp64_src,
                 "algorithmic_flops_per_launch": flops,
                 "algorithmic_bytes_per_launch": pair_bytes("f64", vol, nr), "pair_variant": shape,
-                "note": "the direct method's FP64 stencils run in fixed point on the integer pipe (FP64-accurate), "
-                        "so frac can exceed 1 of the FP64 pipe's peak; at 12^4 the pair stencil is bound by "
-                        "integer issue and load latency at two warps per scheduler"}
+                "note": "FP64 stencils of SU(3) fields run in fixed point on the integer pipe, so frac can exceed 1 "
+                        "of the FP64 pipe's peak"}
     byts = pair_bytes(prec, vol, nr)
     ach = byts / (t_pair * 1e-3) / 1e9 if t_pair else None
     return {"kernel": kernel, "bound": "hbm", "achieved": ach, "peak": peaks["hbm_gbs"], "unit": "GB/s",
@@ -553,7 +593,7 @@ def _summary(wl, per_mu, infos, acc):
     return its, per_mu_stats, statuses, launches
 
 
-def _companion(ovl, ctx, args, cname, flush, world, local, fp64_peak, fp64_src, ref_value):
+def _companion(ovl, ctx, args, cname, flush, world, local, fp64_peak, fp64_src, madwide_peak, ref_value):
     """One companion workload, timed like the headline with at most 3 warm-up and 3 timed steps."""
     wm = WORKLOADS[cname]
     lat_m, u_m, _, pm = _setup(ovl, ctx, wm, cache=args.setup_cache)
@@ -570,7 +610,7 @@ def _companion(ovl, ctx, args, cname, flush, world, local, fp64_peak, fp64_src, 
             "tol": wm["tol"], "nrhs": wm.get("nrhs", 1), "value": vm, "unit": UNIT, "steps": steps, "warmup": warm,
             "ms_per_step": tm / steps, "speedup_vs_line_value": vm / ref_value,
             "e2e_value": steps * sps * world / em, "statuses": stm, "accuracy_half_sign2b_minus_b": am,
-            "per_mu": pms, "gpu_launches": int(lm), "roofline": _roofline(wm, im, fp64_peak, fp64_src),
+            "per_mu": pms, "gpu_launches": int(lm), "roofline": _roofline(wm, im, fp64_peak, fp64_src, madwide_peak),
             "clocks": clk.summary()}
 
 
@@ -624,6 +664,7 @@ def run_ours(args, wl):
     n = b.size // nrhs
     flush = torch.empty(64 * 1024 * 1024, dtype=torch.float32, device="cuda")  # 256 MB > L2
     fp64_peak, fp64_src = _fp64_peak()
+    madwide_peak = _madwide_peak()
 
     with ClockSampler(local) as clk:
         total_ms, e2e_s, infos, acc = _time_workload(ovl, ctx, args, wl, u, per_mu, b, flush, world)
@@ -652,14 +693,14 @@ def run_ours(args, wl):
                    "setup_inverse_solves": [d.get("setup_inverse_solves", 0) for d in per_mu],
                    "parallelism": "replicas" if world > 1 else "single",
                    "pair_variant_pinned": args.pair_variant if args.pair_variant >= 0 else None},
-        "roofline": _roofline(wl, infos, fp64_peak, fp64_src), "e2e": e2e, "clocks": clocks,
+        "roofline": _roofline(wl, infos, fp64_peak, fp64_src, madwide_peak), "e2e": e2e, "clocks": clocks,
         "gpu_launches": int(launches),
     }
     # companion lines: the same problem in mixed precision (speedup over this line's value), the
     # 16-source batch; each timed with at most 3 warm-up and 3 timed steps
     if not args.no_extras:
         for key, cname in COMPANIONS.get(args.workload, []):
-            res[key] = _companion(ovl, ctx, args, cname, flush, world, local, fp64_peak, fp64_src, value)
+            res[key] = _companion(ovl, ctx, args, cname, flush, world, local, fp64_peak, fp64_src, madwide_peak, value)
         if args.workload == DEFAULT_WORKLOAD:
             res["lattice8_defl16"] = _c2_line(ovl, ctx, args)
     k_table = K_TABLE.get(args.workload)

@@ -5,6 +5,8 @@
 // (no data dependence between chains, so the pipe, not latency, limits the rate); the grid is
 // 8 blocks of 256 threads per SM. Rate = 2 flops x 8 chains x iterations x threads / best time
 // of 5 launches (CUDA events). The loop count is fixed: the kernel always ends.
+// The same for 32 x 32 + 64 bit integer multiply-adds, x <- (low word of x) * b + x, the instruction that the
+// fixed-point kernels are made of.
 #include <cuda_runtime.h>
 
 namespace {
@@ -24,8 +26,32 @@ __global__ void k_fma_chains(T* out, int iters, T a, T b) {
   out[(size_t)blockIdx.x * blockDim.x + threadIdx.x] = s;  // keeps the chains live
 }
 
+__global__ void k_madwide_chains(long long* out, int iters, int b) {
+  long long x[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) x[k] = threadIdx.x * 77 + k;
+  for (int i = 0; i < iters; ++i) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) asm volatile("mad.wide.s32 %0, %1, %2, %0;" : "+l"(x[k]) : "r"((int)x[k]), "r"(b));
+  }
+  long long s = 0;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) s += x[k];
+  out[(size_t)blockIdx.x * blockDim.x + threadIdx.x] = s;
+}
+
 template <class T>
-int measure(int iters, double* tflops) {
+void run(T* out, int iters, int blocks, int threads) {
+  k_fma_chains<T><<<blocks, threads>>>(out, iters, (T)0.999, (T)0.001);
+}
+template <>
+void run<long long>(long long* out, int iters, int blocks, int threads) {
+  k_madwide_chains<<<blocks, threads>>>(out, iters, 7);
+}
+
+// Chain steps per second, in 10^12.
+template <class T>
+int measure(int iters, double* tops) {
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return -3;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return -3;
@@ -35,11 +61,11 @@ int measure(int iters, double* tflops) {
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
-  k_fma_chains<T><<<blocks, threads>>>(out, 100, (T)0.999, (T)0.001);  // warm-up
+  run<T>(out, 100, blocks, threads);  // warm-up
   float best = 1e30f;
   for (int r = 0; r < 5; ++r) {
     cudaEventRecord(e0);
-    k_fma_chains<T><<<blocks, threads>>>(out, iters, (T)0.999, (T)0.001);
+    run<T>(out, iters, blocks, threads);
     cudaEventRecord(e1);
     cudaEventSynchronize(e1);
     float ms = 0;
@@ -51,7 +77,7 @@ int measure(int iters, double* tflops) {
   cudaEventDestroy(e1);
   cudaFree(out);
   if (err != cudaSuccess) return -3;
-  *tflops = 2.0 * 8 * (double)iters * blocks * threads / (best * 1e-3) / 1e12;
+  *tops = 8 * (double)iters * blocks * threads / (best * 1e-3) / 1e12;
   return 0;
 }
 
@@ -61,5 +87,10 @@ int measure(int iters, double* tflops) {
 // Returns 0, or -2 (allocation failed) / -3 (CUDA error).
 extern "C" int ovl_probe_fma_tflops(int fp64, double* tflops) {
   if (!tflops) return -1;
-  return fp64 ? measure<double>(4000, tflops) : measure<float>(40000, tflops);
+  const int e = fp64 ? measure<double>(4000, tflops) : measure<float>(40000, tflops);
+  *tflops *= 2;
+  return e;
 }
+
+// Integer multiply-adds (mad.wide.s32) of the current device in 10^12 a second; the same return values.
+extern "C" int ovl_probe_madwide_tops(double* tops) { return tops ? measure<long long>(20000, tops) : -1; }
