@@ -100,7 +100,9 @@ int64_t ovl_lattice_n(const ovl_lattice* lat);
  * always kept). Every format the lattice already holds from an earlier call is rewritten
  * from U as well, so no copy keeps the previous field. The caller's buffer may be freed on
  * return (the call synchronises). Beside the FP64 links a fixed-point copy of the same size
- * (576 bytes a site) is kept for the FP64 stencils; it is used if the field has a common scale
+ * (576 bytes a site) is kept for the FP64 stencils: from this call if `formats` names OVL_F64, else
+ * from the first FP64 operator or solve that needs it (and may allocate: not ovl_apply_sign_noalloc, not
+ * a call under stream capture; those run FP64 arithmetic). It is used if the field has a common scale
  * (finite, every link's largest component at least a quarter of the largest of the field, and
  * that within 2^-8 .. 2^8, as for any SU(3) field) and its links mix the colours (no entry below
  * 2^-20 of its link's largest component, and at most half of the links with one, or with their

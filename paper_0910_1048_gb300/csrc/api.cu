@@ -25,6 +25,50 @@ ovl_status solve_multishift(ovl_lattice* lat, const ovl_sign_params* p, int nrhs
 ovl_status solve_fom(ovl_lattice* lat, const ovl_sign_params* p, int nrhs, const double2* b, double2* x,
                      ovl_sign_info* info, cudaStream_t st);
 
+// Links to their fixed-point copy and scale, and whether the field fits it (synchronises st).
+static cudaError_t make_fixed_point(const Geom& g, const double2* u64, FxC* ufx, FxField* fxf, cudaStream_t st, bool* ok) {
+  char field[64];
+  cudaError_t e = launch_fixed_point_links(g, u64, ufx, fxf, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(field, fxf, fx_field_bytes(), cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (e == cudaSuccess) *ok = fx_field_ok(field);
+  return e;
+}
+
+// The fixed-point copy of a lattice whose ovl_set_links did not name FP64, at its first FP64 operator or solve (callers that
+// stay with the reduced formats neither wait for it nor hold its 576 bytes a site). Without it, in a capture or
+// where memory is short, FP64 arithmetic serves. The caller holds the lattice's lock shared.
+static void ensure_fixed_point(ovl_lattice* l, cudaStream_t user) {
+  if (!l->u64 || l->ufx.load(std::memory_order_acquire)) return;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(user, &cs) != cudaSuccess) {
+    cudaGetLastError();
+    return;
+  }
+  if (cs != cudaStreamCaptureStatusNone) return;
+  std::lock_guard<std::mutex> lk(l->fx_mu);
+  if (l->ufx.load(std::memory_order_acquire) || l->fx_tried) return;
+  l->fx_tried = true;
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;  // (another thread may be capturing)
+  if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) {
+    cudaGetLastError();
+    return;
+  }
+  FxC* p = nullptr;
+  bool ok = false;
+  if (cudaMalloc(&p, (size_t)36 * l->g.vol * 16) != cudaSuccess ||
+      make_fixed_point(l->g, l->u64, p, l->fxf, l->ctx->stream, &ok) != cudaSuccess) {
+    cudaGetLastError();
+    cudaFree(p);
+    p = nullptr;
+  }
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  if (!p) return;
+  l->ufx_own = p;
+  l->fx_ok.store(ok, std::memory_order_relaxed);
+  l->ufx.store(p, std::memory_order_release);
+}
+
 // A lattice with its own workspaces that reads `parent`'s links and deflation set at every solve
 // (so it sees later ovl_set_links / ovl_set_deflation on the parent).
 ovl_lattice* lattice_view(ovl_lattice* parent) {
@@ -136,6 +180,7 @@ ovl_status ovl_destroy_lattice(ovl_lattice* lat) {
   free_multi_ws(lat->mws);
   if (lat->owns_links) {
     cudaFree(lat->u64);
+    cudaFree(lat->ufx_own);
     cudaFree(lat->u32);
     cudaFree(lat->u16);
     cudaFree(lat->defl.R);
@@ -158,14 +203,21 @@ ovl_status ovl_set_links(ovl_lattice* lat, const void* U, int32_t U_on_device, u
   }
   OVL_DEVICE_SCOPE(lat->ctx->device);
   const size_t nl = (size_t)36 * lat->g.vol;  // complex entries
+  // the fixed-point copy serves FP64 operators and solves: made here for callers that name the format or have it already
+  const bool fx = (formats & OVL_F64) || lat->ufx;
   formats |= OVL_F64;
   // a copy held from an earlier call is refreshed too: no format may keep the previous field
   if (lat->u32) formats |= OVL_F32;
   if (lat->u16) formats |= OVL_F16R12;
-  if (!lat->u64) {  // one allocation: links, fixed-point copy, scale
-    OVL_CHECK_CUDA(cudaMalloc(&lat->u64, 2 * nl * 16 + fx_field_bytes()));
-    lat->ufx = (FxC*)((char*)lat->u64 + nl * 16);
-    lat->fxf = (FxField*)((char*)lat->u64 + 2 * nl * 16);
+  FxC* ufx = lat->ufx;
+  if (!lat->u64) {  // one allocation: links, scale, fixed-point copy
+    const size_t field = (fx_field_bytes() + 255) & ~(size_t)255;
+    OVL_CHECK_CUDA(cudaMalloc(&lat->u64, (fx ? 2 : 1) * nl * 16 + field));
+    lat->fxf = (FxField*)((char*)lat->u64 + nl * 16);
+    if (fx) ufx = (FxC*)((char*)lat->u64 + nl * 16 + field);
+  } else if (fx && !ufx) {
+    if (!lat->ufx_own) OVL_CHECK_CUDA(cudaMalloc(&lat->ufx_own, nl * 16));
+    ufx = lat->ufx_own;
   }
   if ((formats & OVL_F32) && !lat->u32) OVL_CHECK_CUDA(cudaMalloc(&lat->u32, nl * 8));
   if ((formats & OVL_F16R12) && !lat->u16) OVL_CHECK_CUDA(cudaMalloc(&lat->u16, (size_t)24 * lat->g.vol * 4));
@@ -177,14 +229,17 @@ ovl_status ovl_set_links(ovl_lattice* lat, const void* U, int32_t U_on_device, u
     OVL_CHECK_CUDA(cudaMemcpyAsync(tmp, U, nl * 16, cudaMemcpyHostToDevice, st));
     src = tmp;
   }
-  cudaError_t e = launch_ingest_links(lat->g, src, lat->u64, lat->ufx, lat->fxf, (formats & OVL_F32) ? lat->u32 : nullptr,
+  cudaError_t e = launch_ingest_links(lat->g, src, lat->u64, (formats & OVL_F32) ? lat->u32 : nullptr,
                                       (formats & OVL_F16R12) ? lat->u16 : nullptr, st);
-  char field[64];
-  if (e == cudaSuccess) e = cudaMemcpyAsync(field, lat->fxf, fx_field_bytes(), cudaMemcpyDeviceToHost, st);
+  bool ok = false;
+  if (e == cudaSuccess) e = fx ? make_fixed_point(lat->g, lat->u64, ufx, lat->fxf, st, &ok)
+                               : cudaMemsetAsync(lat->fxf, 0, fx_field_bytes(), st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (tmp) cudaFree(tmp);
   OVL_CHECK_CUDA(e);
-  lat->fx_ok = fx_field_ok(field);
+  lat->fx_ok = ok;
+  lat->ufx = ufx;
+  lat->fx_tried = false;
   lat->formats |= formats;
   return OVL_OK;
 }
@@ -283,6 +338,7 @@ ovl_status ovl_apply_DW(ovl_lattice* lat, double m_W, double mu, uint32_t flags,
   if (f64) {
     OVL_REQUIRE(!(flags & (OVL_LINKS_F32 | OVL_LINKS_F16R12)), "ovl_apply_DW: FP64 uses FP64 links");
     OVL_REQUIRE(lat->src()->u64, "ovl_apply_DW: links not set");
+    ensure_fixed_point(lat->src(), (cudaStream_t)stream);
   } else {
     lf = (flags & OVL_LINKS_F16R12) ? LINK_F16R12 : LINK_F32;
     OVL_REQUIRE(lf == LINK_F32 ? lat->src()->u32 != nullptr : lat->src()->u16 != nullptr,
@@ -320,6 +376,8 @@ ovl_status ovl_apply_sign(ovl_lattice* lat, const ovl_sign_params* p, int32_t nr
   OVL_REQUIRE(2.0 * p->m_W + 8.0 != 0.0, "ovl_apply_sign: m_W = -4 has no kappa");
   std::shared_lock<std::shared_mutex> shared(lat->src()->guard);  // links / deflation set stay as they are
   OVL_DEVICE_SCOPE(lat->ctx->device);
+  if (p->precision == OVL_PREC_F64 || p->method != OVL_DIRECT_2SL)  // (A^2 solves end with an FP64 stencil)
+    ensure_fixed_point(lat->src(), (cudaStream_t)stream);
   if (p->method == OVL_DIRECT_2SL)
     return solve_direct(lat, p, nrhs, (const double2*)b, (double2*)x, info, (cudaStream_t)stream);
   if (p->method == OVL_MULTISHIFT_BICG)

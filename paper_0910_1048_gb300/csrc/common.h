@@ -8,6 +8,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <shared_mutex>
 #include <string>
 #include <vector>
@@ -114,7 +115,7 @@ struct FxC;
 struct FxField;
 struct Links {
   const double2* f64 = nullptr;   // [4][9][V]
-  const FxC* fx = nullptr;        // [4][9][V] fixed-point copy of the FP64 links (fixedpt.cuh)
+  const FxC* fx = nullptr;        // [4][9][V] fixed-point copy of the FP64 links (fixedpt.cuh), or nullptr
   const FxField* fxf = nullptr;   // its scale, and whether it can be used
   bool fits = false;              // the same as the host knows it at the launch: for the choice of a kernel only
   const float2* f32 = nullptr;    // [4][9][V]
@@ -159,9 +160,14 @@ struct ovl_lattice {
   ovl::Geom g{};
   uint32_t formats = 0;
   double2* u64 = nullptr;
-  ovl::FxC* ufx = nullptr;        // fixed-point copy of u64 and its scale (in u64's allocation)
+  // Fixed-point copy of u64 (nullptr: none yet; see ensure_fixed_point) and its scale, the latter and a copy made with
+  // the links in u64's allocation. Published by ufx, under fx_mu where solves may be running.
+  std::atomic<ovl::FxC*> ufx{nullptr};
+  ovl::FxC* ufx_own = nullptr;    // the copy's own allocation, if it came later
   ovl::FxField* fxf = nullptr;
-  bool fx_ok = false;             // the fixed-point copy is usable (FxField::ok)
+  std::atomic<bool> fx_ok{false}; // the copy is usable (FxField::ok)
+  std::mutex fx_mu;
+  bool fx_tried = false;          // (no second attempt for these links)
   float2* u32 = nullptr;
   uint32_t* u16 = nullptr;
   ovl_deflation defl;
@@ -170,9 +176,9 @@ struct ovl_lattice {
   ovl::Links links() const {
     ovl::Links l;
     l.f64 = u64;
-    l.fx = ufx;
+    l.fx = ufx.load(std::memory_order_acquire);
     l.fxf = fxf;
-    l.fits = fx_ok;
+    l.fits = l.fx && fx_ok.load(std::memory_order_relaxed);
     l.f32 = u32;
     l.f16 = u16;
     return l;

@@ -413,7 +413,7 @@ __device__ __forceinline__ void add_hops(const Geom& g, const Links& U, int s, c
   FxAcc acc;
   fx_clear(acc);
   int E = 0;
-  const bool fx = c.ok && U.fxf->ok && fx_hops(g, U.fx, s, 0, 8, c, ld, g5in, acc, E);
+  const bool fx = c.ok && U.fx && U.fxf->ok && fx_hops(g, U.fx, s, 0, 8, c, ld, g5in, acc, E);
   ld(s, out);
   if (g5in) gamma5_inplace(out);
   finish_hops(g, U, s, 0, 8, c, ld, g5in, fx, acc, E, out);
@@ -465,7 +465,7 @@ __device__ __forceinline__ void pair_split(const Geom& g, const Links& U, const 
     fx_clear(sum);
     int E = 0;
     FxSizes z;
-    bool fx = s < g.vol && c.ok && U.fxf->ok && fx_hops(g, U.fx, s, 2 * dir, 2 * dir + 2, c, ld, false, sum, E, z);
+    bool fx = s < g.vol && c.ok && U.fx && U.fxf->ok && fx_hops(g, U.fx, s, 2 * dir, 2 * dir + 2, c, ld, false, sum, E, z);
 #pragma unroll
     for (int sp = 0; sp < 4; ++sp) size[which][sp][dir][tx] = z.m[sp];
     __syncthreads();

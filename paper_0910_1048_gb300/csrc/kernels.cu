@@ -237,12 +237,16 @@ __global__ void __launch_bounds__(256) k_fx_field(int vol, const double2* u64, F
 size_t fx_field_bytes() { return sizeof(FxField); }
 bool fx_field_ok(const void* host_copy) { return ((const FxField*)host_copy)->ok != 0; }
 
-cudaError_t launch_ingest_links(const Geom& g, const double* ucan, double2* u64, FxC* ufx, FxField* fxf, float2* u32,
-                                uint32_t* u16, cudaStream_t st) {
+cudaError_t launch_ingest_links(const Geom& g, const double* ucan, double2* u64, float2* u32, uint32_t* u16, cudaStream_t st) {
   size_t n = (size_t)36 * g.vol;
   k_ingest_links<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(g.vol, (const double2*)ucan, u64, u32, u16);
-  cudaError_t e;
-  if ((e = cudaMemsetAsync(fxf, 0, sizeof(FxField), st))) return e;
+  return cudaGetLastError();
+}
+
+cudaError_t launch_fixed_point_links(const Geom& g, const double2* u64, FxC* ufx, FxField* fxf, cudaStream_t st) {
+  const size_t n = (size_t)36 * g.vol;
+  cudaError_t e = cudaMemsetAsync(fxf, 0, sizeof(FxField), st);
+  if (e != cudaSuccess) return e;
   k_fx_links<<<(unsigned)(((size_t)4 * g.vol + 255) / 256), 256, 0, st>>>(g.vol, u64, fxf, ufx);
   k_fx_field<<<(unsigned)std::min<size_t>((n + 255) / 256, 1216), 256, 0, st>>>(g.vol, u64, fxf, ufx);
   return cudaGetLastError();
@@ -329,7 +333,7 @@ __global__ void __launch_bounds__(128, 3)
   fx_clear(acc);
   int E = 0;
   FxSizes z;
-  const bool fx = c.ok && U.fxf->ok && fx_hops(g, U.fx, s, 2 * t, 2 * t + 2, c, ld, g5_in, acc, E, z);
+  const bool fx = c.ok && U.fx && U.fxf->ok && fx_hops(g, U.fx, s, 2 * t, 2 * t + 2, c, ld, g5_in, acc, E, z);
   expo[t][lane] = fx ? E : 1 << 20;
 #pragma unroll
   for (int sp = 0; sp < 4; ++sp) size[sp][t][lane] = z.m[sp];

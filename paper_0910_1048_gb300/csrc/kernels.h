@@ -112,10 +112,10 @@ struct LzDev {
 cudaError_t launch_to_native(const Geom& g, int nrhs, bool in_f64, const void* in, bool out_f64, void* out, cudaStream_t st);
 cudaError_t launch_from_native(const Geom& g, int nrhs, bool in_f64, const void* in, bool out_f64, void* out, cudaStream_t st);
 
-// Links: canonical complex128 [4][V][3][3] (device) -> [4][9][V] f64 / f32, [4][6][V] f16 rows 0-1, and
-// the fixed-point copy of the FP64 links with its scale (fixedpt.cuh).
-cudaError_t launch_ingest_links(const Geom& g, const double* ucan, double2* u64, FxC* ufx, FxField* fxf, float2* u32,
-                                uint32_t* u16, cudaStream_t st);
+// Links: canonical complex128 [4][V][3][3] (device) -> [4][9][V] f64 / f32, [4][6][V] f16 rows 0-1.
+cudaError_t launch_ingest_links(const Geom& g, const double* ucan, double2* u64, float2* u32, uint32_t* u16, cudaStream_t st);
+// FP64 links -> their fixed-point copy and its scale (fixedpt.cuh).
+cudaError_t launch_fixed_point_links(const Geom& g, const double2* u64, FxC* ufx, FxField* fxf, cudaStream_t st);
 size_t fx_field_bytes();  // sizeof(FxField)
 bool fx_field_ok(const void* host_copy);  // FxField::ok of a copy of it in host memory
 
@@ -144,7 +144,7 @@ struct FxVecs {
 };
 constexpr size_t kFxExponents = 6;   // int arrays of FxVecs per site and rhs
 size_t fx_step_bytes();
-// Whether (m_W, mu) fit (the field: ovl_lattice::fx_ok).
+// Whether (m_W, mu) fit (the field: Links::fits).
 bool fx_step_usable(double m_w, double mu);
 // After launch_lanczos_start: slot 1 from vhat_1 (basis column 1) and what_1 (FP64 in w1).
 cudaError_t launch_fx_begin(const Geom& g, const Links& U, double m_w, const LzDev& lz, const FxVecs& fx, const void* vh,

@@ -201,7 +201,7 @@ extern "C" ovl_status ovl_apply_sign_noalloc(ovl_lattice* lat, const ovl_sign_pa
   if (m > 0) OVL_CHECK_CUDA(cudaMemcpyAsync(lam_sign, ls.data(), m * 8, cudaMemcpyHostToDevice, st));
   const Links U = lat->src()->links();
   // the FP64 step in fixed point as in ovl_apply_sign
-  const bool fxs = f64 && lat->src()->fx_ok && fx_step_usable(p->m_W, p->mu);
+  const bool fxs = f64 && U.fits && fx_step_usable(p->m_W, p->mu);
   FxVecs fx;
   if (fxs) {
     OVL_REQUIRE(fx_step_bytes() <= 256, "apply_sign_noalloc: step coefficients");

@@ -437,7 +437,7 @@ ovl_status solve_direct(ovl_lattice* lat, const ovl_sign_params* p, int nrhs, co
   if (m == 0) vec.xp = nullptr;
   const Links U = lat->src()->links();
   // the FP64 step in fixed point where the field and the coefficients fit it (kernels_fx.cu)
-  const bool fxs = f64 && lat->src()->fx_ok && fx_step_usable(p->m_W, p->mu);
+  const bool fxs = f64 && U.fits && fx_step_usable(p->m_W, p->mu);
   auto start = [&](const LzDev& lz) -> cudaError_t {
     LzVecs v = vec;
     if (fxs) v.wh = (char*)vec.aw - (size_t)nrhs * n * 16;  // what_1 (slot 1 of wh) goes to aw, in FP64
