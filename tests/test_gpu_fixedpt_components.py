@@ -126,3 +126,23 @@ def test_stencil_of_small_spins(ovl, ctx, dims, small):
     got, ref = _dw(ovl, lat, half), wilson.apply_dw(u, half, -2.0, 0.3, -1)
     assert np.abs(got - ref).max() <= 1e-13 * np.abs(ref).max()
     ovl.ovl_destroy_lattice(lat)
+
+
+@pytest.mark.parametrize("small", [1e-6, 1e-14])
+def test_direct_solve_of_a_source_with_small_spins(ovl, ctx, small):
+    """On links that mix the colours the solve fills the small spins from the large one: each spin of x as Algorithm 4
+    gives it at equal k, to 1e-10."""
+    dims, k = (4, 2, 6, 4), 20
+    u, b = synth.gauge_links(dims, 47), synth.gaussian_source(dims, 48)
+    b[..., 1:, :] *= small
+    lat = _lat(ovl, ctx, dims, u)
+    bt = torch.from_numpy(b).cuda()
+    xt = torch.empty_like(bt)
+    assert ovl.ovl_apply_sign(lat, ovl.ovl_sign_params_default(mu=0.3, fixed_k=k, check_every=6), bt, xt)[0] == ovl.OVL_OK
+    x = xt.cpu().numpy()
+    ovl.ovl_destroy_lattice(lat)
+    a, ah = deflation.sparse_hw(u, dims, -2.0, 0.3), deflation.sparse_hw(u, dims, -2.0, -0.3)
+    xo, _ = lanczos.direct_lanczos_lr(lambda v: (a @ v.ravel()).reshape(v.shape),
+                                      lambda w: (ah @ w.ravel()).reshape(w.shape), b, k)
+    for s in range(4):
+        assert np.linalg.norm(x[..., s, :] - xo[..., s, :]) < 1e-10 * np.linalg.norm(xo[..., s, :])
