@@ -207,7 +207,8 @@ void ovl_sign_params_default(ovl_sign_params* p);
  * Algorithm 4 (direct), Algorithm 3 (multishift BiCG) or Algorithm 1 (restarted FOM: k_max
  * bounds the Arnoldi steps over all cycles, tol the shifted residuals |rho_i| |r| / |r_0|, the
  * rational function as for the multishift method); LR split x = x_P + f(A)(I-P)b (Eq. action)
- * when use_deflation. Errors: EINVAL, ENOMEM, ECUDA. */
+ * when use_deflation. Accuracy is in the norm of x: FP64 direct solves on fields that fit fixed point keep
+ * their recurrence vectors to 56 to 59 bits of each site's largest component. Errors: EINVAL, ENOMEM, ECUDA. */
 ovl_status ovl_apply_sign(ovl_lattice* lat, const ovl_sign_params* p, int32_t nrhs,
                           const void* b, void* x, ovl_sign_info* info, void* stream);
 

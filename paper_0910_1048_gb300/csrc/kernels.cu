@@ -11,7 +11,6 @@
 #include <map>
 #include <mutex>
 #include <set>
-#include <tuple>
 #include <type_traits>
 
 #include "devutil.cuh"

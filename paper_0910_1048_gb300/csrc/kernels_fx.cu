@@ -3,11 +3,12 @@
 // GB300's FP64 pipe (about two lanes per SM and clock) bound every kernel of the FP64 step: the pair
 // stencil at 12^4 took 84 us and the update 24.5 us against 4.2 and 4.8 us of HBM time. Here the
 // recurrence vectors vhat_j, vhat_{j-1}, what_j, what_{j-1} are kept as limbs with one exponent per site
-// (59 bits of the site's largest component, so at least as much as FP64 holds of it), and both the
-// stencil and the update are integer arithmetic: products of limbs by mad.wide.s32, sums in 64 bits.
-// FP64 is left for the basis columns (one conversion per component), the step's scalars and the sums
-// over blocks. Every sum inside a block is an integer sum with one rounding per term, so the
-// results do not depend on the shape or the order of the launch.
+// (59 bits of the site's largest component, 56 where sites share an exponent: in the norm more than FP64
+// holds, of a component 2^-m of the largest m bits less), and both the stencil and the update are
+// integer arithmetic: products of limbs by mad.wide.s32, sums in 64 bits. FP64 is left for the basis
+// columns (one conversion per component), the step's scalars and the sums over blocks. Every sum inside a
+// block is an integer sum with one rounding per term, so the results do not depend on the shape or the
+// order of the launch.
 //
 // Step j:
 //   k_fx_pair:   A v = H(mu) vhat_j / k, A w = H(-mu) what_j / k (k = the hop coefficient ks times the links'
