@@ -251,9 +251,11 @@ __global__ void __launch_bounds__(64) k_fx_begin(Geom g, LzDev lz, FxVecs fx, co
 // Block (32 sites, 2 T): warp y computes the hops of role y / T (0: H(mu) vhat_j, 1: H(-mu) what_j) whose
 // index is in [8 t / T, 8 (t+1) / T), t = y % T. T = 1: one thread per site and role; T = 4: one direction
 // per thread, for lattices too small to fill the GPU with one (each thread finishes one spin). Block 0
-// settles the previous step, block b > 0 takes chunk b - 1. A source that has ended costs its blocks' launch:
-// a status above 1 (retired, or no Krylov part) is written by stream work before the step alone, so every thread
-// sees it; a breakdown (1) also by block 0.
+// settles the previous step, block b > 0 takes chunk b - 1. A source that has ended (status above 1:
+// retired by the host, or without a Krylov part) costs its blocks' launch: seven beside one at 12^4 take a step from
+// 44.9 to 45.7 us, where running their hops took it to 231. Every thread of a block sees such a status alike, since
+// only stream work before the step writes it; a breakdown (1) is also written by block 0, and the host retires it.
+// (A barrier that caught it at once cost 0.4 us a step; the test before the wait cost 0.7.)
 // With 8.5 warps per SM (12^4) the latency of the loads is not hidden by other warps, so a hop's inputs are
 // copied to shared memory while the previous one is computed: the neighbour's 12 components per thread,
 // and the link's nine once for the two roles; what_j for the dot during the last hop (12^4 step 45.7 -> 44.2 us;
@@ -323,7 +325,7 @@ __global__ void __launch_bounds__(64 * T, T == 1 ? 5 : 1)
   grid_wait();
   grid_launch();
   const int status = lz.status[rhs], j = lz.j[rhs];
-  if (status > 1) {  // ended before this launch
+  if (status > 1 || j == 0) {  // ended before this launch, or broke down at the start (no column 1)
     copy_wait();
     return;
   }
@@ -346,18 +348,12 @@ __global__ void __launch_bounds__(64 * T, T == 1 ? 5 : 1)
     E = max(E, fx_hop_exponent(k, ex[fx_neighbour(g, s, xyzt, k, &w)], c));
   }
   const FxC* w = args.q[1][j & 1] + (size_t)rhs * n + s;
-  copy_wait();
-  // The first hop's inputs are there. Nothing is left to do after a breakdown (block 0 may be storing it in this
-  // very launch, so the threads of a block decide together).
-  if (__syncthreads_or(status)) return;
 #pragma unroll 1
   for (int i = 0; i < NH; ++i) {
     const int k = t * NH + i, eh = fx_hop_exponent(k, ex[nb], c);
     const bool flip = wraps && g.t_bc < 0;
-    if (i > 0) {
-      copy_wait();
-      __syncthreads();  // hop k's inputs are there, and the other stage has been read
-    }
+    copy_wait();
+    __syncthreads();  // hop k's inputs are there, and the other stage has been read
     if (i + 1 < NH) {
       nb = fx_neighbour(g, s, xyzt, k + 1, &wraps);
       fetch_spinor((i + 1) & 1, q + nb);
@@ -571,7 +567,7 @@ __global__ void __launch_bounds__(128 * kFxGroups, 1)
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nt = blockDim.x;
   const int ended = lz.status[rhs];
   const int j = lz.j[rhs];  // (the settle block may take it back, with a status: see below)
-  if (ended > 1) {  // before this launch: see k_fx_pair
+  if (ended > 1 || j == 0) {  // see k_fx_pair
     grid_wait();
     return;
   }

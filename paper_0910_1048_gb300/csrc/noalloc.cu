@@ -358,7 +358,7 @@ extern "C" ovl_status ovl_apply_sign_noalloc(ovl_lattice* lat, const ovl_sign_pa
       } else if (final_snapshot) {
         s.status = OVL_ENOCONV, s.done = true;
       }
-      if (s.done && h_st[r] == 0) OVL_CHECK_CUDA(cudaMemsetAsync(lz.status + r, 2, sizeof(int), st));
+      if (s.done && h_st[r] < 2) OVL_CHECK_CUDA(cudaMemsetAsync(lz.status + r, 2, sizeof(int), st));
     }
     bool all = true;
     for (int r = 0; r < nrhs; ++r) all = all && rs[r].done;

@@ -704,8 +704,8 @@ ovl_status solve_direct(ovl_lattice* lat, const ovl_sign_params* p, int nrhs, co
           s.status = OVL_ENOCONV;
           s.done = true;
         }
-        if (s.done && w->h[q].status[r] == 0) {
-          // retire this right-hand side: later steps skip it (any nonzero status)
+        if (s.done && w->h[q].status[r] < 2) {
+          // retire this right-hand side, after a breakdown too: later steps skip it (status 2)
           ce = cudaMemsetAsync(w->lz.status + r, 2, sizeof(int), st);
           if (ce) break;
         }
