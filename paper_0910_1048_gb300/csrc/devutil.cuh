@@ -459,7 +459,7 @@ __device__ __forceinline__ void pair_split(const Geom& g, const Links& U, const 
   for (int q = 0; q < 12; ++q) acc.c[q / 3][q % 3] = mk<R>(0, 0);
   if constexpr (std::is_same_v<Coef, FxCoef>) {
     // (a site's sums are taken or refused for its four directions together: fx_even)
-    __shared__ int size[2][4][4][SITES];  // [which][spin][direction][site]
+    __shared__ unsigned size[2][2][4][SITES];  // [which][pair of spins][direction][site]
     const StrideLoader ld{in, 1, g.vol};
     FxAcc sum;
     fx_clear(sum);
@@ -467,12 +467,12 @@ __device__ __forceinline__ void pair_split(const Geom& g, const Links& U, const 
     FxSizes z;
     bool fx = s < g.vol && c.ok && U.fx && U.fxf->ok && fx_hops(g, U.fx, s, 2 * dir, 2 * dir + 2, c, ld, false, sum, E, z);
 #pragma unroll
-    for (int sp = 0; sp < 4; ++sp) size[which][sp][dir][tx] = z.m[sp];
+    for (int i = 0; i < 2; ++i) size[which][i][dir][tx] = z.m[i];
     __syncthreads();
 #pragma unroll
-    for (int sp = 0; sp < 4; ++sp) {
-      const int(&q)[4][SITES] = size[which][sp];
-      z.m[sp] = max(max(q[0][tx], q[1][tx]), max(q[2][tx], q[3][tx]));
+    for (int i = 0; i < 2; ++i) {
+      const unsigned(&q)[4][SITES] = size[which][i];
+      z.m[i] = fx_max2(fx_max2(q[0][tx], q[1][tx]), fx_max2(q[2][tx], q[3][tx]));
     }
     fx = fx && fx_even(z);
     if (s < g.vol) finish_hops(g, U, s, 2 * dir, 2 * dir + 2, c, ld, false, fx, sum, E, acc);

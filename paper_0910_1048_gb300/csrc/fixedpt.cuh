@@ -200,25 +200,39 @@ OVL_HD int fx_top_word(const Spin<double>& p) {
   return m;
 }
 
-// Largest component of each spin over the neighbours of a site, times the hops' factors: high words of the moduli
-// (the exponent and 20 bits of the mantissa).
+// Largest component of each spin over the neighbours of a site, times the hops' factors: the upper halves of the
+// moduli's high words (exponent and four bits of the mantissa), two spins to a word.
 struct FxSizes {
-  int m[4] = {0, 0, 0, 0};
+  unsigned m[2] = {0, 0};
 };
-OVL_HD int fx_raise(int w, int e) {  // times 2^e, where not zero
+OVL_HD unsigned fx_max2(unsigned a, unsigned b) {  // of both halves
+#if defined(__CUDA_ARCH__)
+  unsigned r;
+  asm("max.u16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+  return r;
+#else
+  const unsigned h = a >> 16 > b >> 16 ? a : b, l = (a & 0xffffu) > (b & 0xffffu) ? a : b;
+  return (h & 0xffff0000u) | (l & 0xffffu);
+#endif
+}
+OVL_HD unsigned fx_sizes2(int a, int b) {  // from two high words of moduli
+#if defined(__CUDA_ARCH__)
+  return __byte_perm((unsigned)a, (unsigned)b, 0x7632);
+#else
+  return ((unsigned)b & 0xffff0000u) | (unsigned)a >> 16;
+#endif
+}
+OVL_HD int fx_raise(int w, int e) {  // a high word times 2^e, where not zero
   const int r = w + e * (1 << 20);
-  return w ? (r > 1 ? r : 1) : 0;
+  return w ? (r > 1 << 16 ? r : 1 << 16) : 0;
 }
 constexpr int kFxEven = 6;  // bits
 
 // Whether all of them are zero or within 2^-kFxEven of the largest.
 OVL_HD bool fx_even(const FxSizes& z) {
-  const int t = z.m[0] > z.m[1] ? z.m[0] : z.m[1], u = z.m[2] > z.m[3] ? z.m[2] : z.m[3];
-  const int least = (t > u ? t : u) - (kFxEven << 20);
-  bool even = true;
-#pragma unroll
-  for (int s = 0; s < 4; ++s) even = even && (z.m[s] == 0 || z.m[s] >= least);
-  return even;
+  const int a = (int)(z.m[0] & 0xffffu), b = (int)(z.m[0] >> 16), c = (int)(z.m[1] & 0xffffu), d = (int)(z.m[1] >> 16);
+  const int t = a > b ? a : b, u = c > d ? c : d, least = (t > u ? t : u) - (kFxEven << 4);
+  return (a == 0 || a >= least) && (b == 0 || b >= least) && (c == 0 || c >= least) && (d == 0 || d >= least);
 }
 
 OVL_HD void fx_spin(const Spin<double>& p, int e, FxSpin& o) {
@@ -573,8 +587,8 @@ OVL_HD bool fx_hops(const Geom& g, const FxC* U, int s, int k0, int k1, const Fx
 #pragma unroll
         for (int i = 0; i < 4; ++i) m[i] = fx_raise(m[i], ft);
       }
-#pragma unroll
-      for (int i = 0; i < 4; ++i) z.m[i] = z.m[i] > m[i] ? z.m[i] : m[i];
+      z.m[0] = fx_max2(z.m[0], fx_sizes2(m[0], m[1]));
+      z.m[1] = fx_max2(z.m[1], fx_sizes2(m[2], m[3]));
       const int fe = fx_hop_exponent(k, 0, c), eh = (eb > 64 ? eb : 64) + fe;
       if (eh > E) {  // first hop, or a larger neighbour than any before
         if (E != 0) {

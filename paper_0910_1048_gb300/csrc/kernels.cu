@@ -321,7 +321,7 @@ __global__ void __launch_bounds__(128, 3)
     k_dslash_f64_split(Geom g, Links U, FxCoef c, bool native, bool g5_in, bool g5_out, const double2* in, double2* out) {
   __shared__ fx64 part[4][3][6][32];  // [receiving spin][slot of the sender][component][site]
   __shared__ int expo[4][32];
-  __shared__ int size[4][4][32];  // [spin][thread][site]
+  __shared__ unsigned size[2][4][32];  // [pair of spins][thread][site]
   const int lane = threadIdx.x, t = threadIdx.y;
   const bool live = (int)blockIdx.x * 32 + lane < g.vol;
   const int s = live ? blockIdx.x * 32 + lane : g.vol - 1;
@@ -335,12 +335,12 @@ __global__ void __launch_bounds__(128, 3)
   const bool fx = c.ok && U.fx && U.fxf->ok && fx_hops(g, U.fx, s, 2 * t, 2 * t + 2, c, ld, g5_in, acc, E, z);
   expo[t][lane] = fx ? E : 1 << 20;
 #pragma unroll
-  for (int sp = 0; sp < 4; ++sp) size[sp][t][lane] = z.m[sp];
+  for (int i = 0; i < 2; ++i) size[i][t][lane] = z.m[i];
   __syncthreads();
   const int Em = max(max(expo[0][lane], expo[1][lane]), max(expo[2][lane], expo[3][lane]));
 #pragma unroll
-  for (int sp = 0; sp < 4; ++sp)
-    z.m[sp] = max(max(size[sp][0][lane], size[sp][1][lane]), max(size[sp][2][lane], size[sp][3][lane]));
+  for (int i = 0; i < 2; ++i)
+    z.m[i] = fx_max2(fx_max2(size[i][0][lane], size[i][1][lane]), fx_max2(size[i][2][lane], size[i][3][lane]));
   const bool all = Em < 1 << 20 && fx_even(z);  // no direction needs the FP64 hops
   const int d = min(Em - E, 62);
   if (__any_sync(0xffffffffu, d > 0)) {
@@ -577,7 +577,8 @@ cudaError_t launch_dslash(const Geom& g, const Links& U, int lf, bool f64, doubl
   if (f64) {
     const FxCoef c = fx_coef(m_w, mu);
     // one source at 8^4 22.8 -> 13.4 us and 12^4 29.7 -> 22.7 with four threads per site; 14^4 30.8 against
-    // 33.4. By the volume alone, so that a source's result is the same alone and in a batch.
+    // 33.4. By the volume alone, so that a source's result is the same alone and in a batch (the shapes
+    // round at different scales; eight sources at 12^4 110 us, one thread per site 91).
     const dim3 sites((g.vol + kBlock - 1) / kBlock, nrhs);
     if (!(U.fits && c.ok) && g5_in)
       k_dslash_plain64<StrideLoaderG5><<<sites, kBlock, 0, st>>>(g, U, c.k, native, g5_out, (const double2*)in,
