@@ -165,7 +165,7 @@ FP64_PEAK_TFLOPS = 1.256
 # DRAM bytes (read + write) per launch of the dominant kernel from one ncu capture (cold L2, every
 # pass flushed), keyed (kernel, precision, lattice, nrhs, pair-stencil shape); the captures and their
 # commands are in profiles/. An entry is removed when its kernel changes.
-TRAFFIC = {}
+TRAFFIC = {("k_fx_pair", "f64", (12, 12, 12, 12), 1, 0): 20.17e6}  # profiles/k_fx_step_f64_lattice12.md
 
 
 def _peaks():
@@ -538,6 +538,8 @@ def _roofline(wl, infos, fp64_peak, fp64_src, madwide_peak=None):
     t_pair = float(np.mean(kt)) if kt else None
     prec = wl["precision"]
     kernel = {"direct": "k_lz_pair", "multishift": "k_ms_pair", "fom": "k_dslash (two per Arnoldi step)"}[wl["method"]]
+    if wl["method"] == "fom" and prec == "f64":
+        kernel = "k_dslash_f64 (two per Arnoldi step)"
     nr = wl.get("nrhs", 1)
     import paper_0910_1048_gb300 as ovl
     shape = ovl.ovl_get_pair_variant(vol, _prec_code(ovl, prec))  # the autotuner's pick (ovl_set_pair_variant)
