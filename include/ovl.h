@@ -101,7 +101,7 @@ int64_t ovl_lattice_n(const ovl_lattice* lat);
  * from U as well, so no copy keeps the previous field. The caller's buffer may be freed on
  * return (the call synchronises). Beside the FP64 links a fixed-point copy of the same size
  * (576 bytes a site) is kept for the FP64 stencils: from this call if `formats` names OVL_F64, else
- * from the first FP64 operator or solve that needs it (and may allocate: not ovl_apply_sign_noalloc, not
+ * from the first FP64 operator or solve that needs it (and may allocate and wait: not ovl_apply_sign_noalloc, not
  * a call under stream capture; those run FP64 arithmetic). It is used if the field has a common scale
  * (finite, every link's largest component at least a quarter of the largest of the field, and
  * that within 2^-8 .. 2^8, as for any SU(3) field) and its links mix the colours (no entry below
@@ -220,10 +220,10 @@ ovl_status ovl_apply_sign(ovl_lattice* lat, const ovl_sign_params* p, int32_t nr
  * sites per one-warp block computing one of the two stencils; 7 one thread per site, the warps of
  * a grid that fills the GPU claiming 32-site tasks (one of the two stencils each) from a counter;
  * 8 (FP32 batches) one thread per site and stencil for a group of four right-hand sides, each
- * site's links loaded once per group (otherwise as 3). The multishift method runs 1, 4, 5 as its eight-thread stencil and the others as its
- * one-thread stencil. variant = -1
- * clears the entry: the next direct solve for that key times every shape on its own vectors and
- * keeps the fastest. Process-wide. FP64 solves on fields that fit fixed point (see
+ * site's links loaded once per group (otherwise as 3). The multishift method runs 1, 4, 5 as its
+ * eight-thread stencil and the others as its one-thread stencil. variant = -1 clears the entry: the
+ * next direct solve for that key times every shape on its own vectors and keeps the fastest.
+ * Process-wide. FP64 solves on fields that fit fixed point (see
  * ovl_set_links) keep their vectors in it and have two shapes: 1, 4 and 5 four threads per
  * site and stencil, the others one; results are the same bits. They are timed and kept apart from the
  * nine shapes of FP64 vectors; a pinned shape holds for both. Otherwise all shapes compute the same

@@ -23,8 +23,9 @@
 // dropped products), against about 2^-52 of their largest component for the FP64 chains it replaces.
 // Measured on GB300 (independent chains, operands that change): mad.wide.s32 3.7 to 4.6 clocks per warp and
 // scheduler, logic operations and shifts 2, mul.hi 3.6. So a hop's 216 products are 800 to 1000 clocks a warp of the
-// about 1300 it takes. Against the FP64 hops D_W at 12^4 takes 22.6 us instead of 65.5, eight sources at 16^4
-// 256 instead of 801; its error against 64 bits is 1.4e-16 instead of 1.8e-16.
+// about 1300 it takes. Against the FP64 hops D_W at 12^4 takes 23.8 us instead of 65.5, eight sources at 16^4
+// 262 instead of 801 (22.6 and 257 without the zeros' signs and the neighbours' sizes, see below); its error against
+// 64 bits is 1.4e-16 instead of 1.8e-16.
 //
 // That is an error relative to the largest terms around a site. FP64 arithmetic keeps a component's 53 bits however
 // much smaller than the others it is, so the sums are used only where every component has terms of that size:
@@ -35,7 +36,8 @@
 //    one, or with their real or imaginary parts all, below 2^-6.
 //  - Sites whose neighbours together fill every spin to 2^-6 of the largest component, or leave it zero
 //    (FxSizes): a hop joins two spins only, so a small spin beside a large one can reach the site alone.
-//    Gaussian fields fill all of them; a site beside one site of widely different spins is refused. Sites next to an infinity, a NaN or only components below 2^-959 (E < 64) are refused too.
+//    Gaussian fields fill all of them; a site beside one site of widely different spins is refused, and so are
+//    sites next to an infinity, a NaN or only components below 2^-959 (E < 64).
 // Others take the FP64 hops. Integer sums do not depend on their order, so every shape of the stencil gives the
 // same hop sums up to the rounding above.
 #pragma once
@@ -438,9 +440,9 @@ OVL_HD float fx_abs_up(int hi) {
 }
 
 // Bits below the largest component of a link at which its smallest entry (its larger component) may lie: for any
-// link, and for one that is not weak; there also its largest real and its largest imaginary part. Of random SU(3) links one in 7 10^10 falls below the first and one in 250
-// below the second, so a field of 64^4 sites is refused by chance once in a thousand times; links exp(i eps H)
-// are mostly weak below eps = 0.04.
+// link, and for one that is not weak; there also its largest real and its largest imaginary part. Of random SU(3)
+// links one in 7 10^10 falls below the first and one in 250 below the second, so a field of 64^4 sites is refused by
+// chance once in a thousand times; links exp(i eps H) are mostly weak below eps = 0.04.
 constexpr int kFxMixAny = 20, kFxMixMost = 6;
 
 // Largest component of a link (0 if the link leaves a colour out), the scale it needs: the largest of that

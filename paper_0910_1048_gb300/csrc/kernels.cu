@@ -281,8 +281,8 @@ __global__ void __launch_bounds__(kBlock, (LF == LINK_F16R12 ? 6 : 7) - (LAYOUT 
     store_spin<float, LAYOUT == kNative>(out + off, g.vol, s, o);
 }
 
-// FP64 (fixed-point hops, see fixedpt.cuh): the layout and gamma5 are run-time values. Three blocks per SM (168 registers): 16^4 x 8 sources 271 us; two (198 registers) 328, four (128,
-// spilled) 277.
+// FP64 (fixed-point hops, see fixedpt.cuh): the layout and gamma5 are run-time values. Three blocks per SM (168
+// registers): 16^4 x 8 sources 261 us; when that took 271, two blocks (198 registers) took 328, four (128, spilled) 277.
 __global__ void __launch_bounds__(kBlock, 3)
     k_dslash_f64(Geom g, Links U, FxCoef c, bool native, bool g5_in, bool g5_out, const double2* in, double2* out) {
   const int s = blockIdx.x * blockDim.x + threadIdx.x;

@@ -20,8 +20,8 @@ namespace ovl {
 // of an element are shared by 2 / E threads (added in column-group order); in the dots every warp takes
 // whole columns of the tile, so a column costs one butterfly per block. (With the block reducing every
 // column together, two barriers and twenty FP64 instructions each, the three passes of a step took 83,
-// 120 and 52 us on average at 2304 sites and k = 40, bound by those; now 12, 17 and 11.) FP64: the pipe's 16 (j + 1) operations per
-// element and step, 16 us on average there.
+// 120 and 52 us on average at 2304 sites and k = 40, bound by those; now 12, 17 and 11.) FP64: the pipe's 16 (j + 1)
+// operations per element and step, 16 us on average there.
 constexpr int kGsThreads = 256;
 
 // Sum of (re, im) over a warp: lanes below 16 keep re, the others im; result in lanes 0 and 16.
