@@ -23,9 +23,9 @@
 // dropped products), against about 2^-52 of their largest component for the FP64 chains it replaces.
 // Measured on GB300 (independent chains, operands that change): mad.wide.s32 3.7 to 4.6 clocks per warp and
 // scheduler, logic operations and shifts 2, mul.hi 3.6. So a hop's 216 products are 800 to 1000 clocks a warp of the
-// about 1300 it takes. Against the FP64 hops D_W at 12^4 takes 23.8 us instead of 65.5, eight sources at 16^4
-// 262 instead of 801 (22.6 and 257 without the zeros' signs and the neighbours' sizes, see below); its error against
-// 64 bits is 1.4e-16 instead of 1.8e-16.
+// about 1300 it takes. Against the FP64 hops D_W at 12^4 takes 22.9 us instead of 65.5, eight sources at 16^4
+// 261 instead of 801 (255 without the zeros' signs and the neighbours' sizes, see below); its error against 64 bits
+// is 1.4e-16 instead of 1.8e-16.
 //
 // That is an error relative to the largest terms around a site. FP64 arithmetic keeps a component's 53 bits however
 // much smaller than the others it is, so the sums are used only where every component has terms of that size:
@@ -35,7 +35,8 @@
 //    from 1; a link with an entry below 2^-20 of its largest component, or more than half of the links with
 //    one, or with their real or imaginary parts all, below 2^-6.
 //  - Sites whose neighbours together fill every spin to 2^-6 of the largest component, or leave it zero
-//    (FxSizes): a hop joins two spins only, so a small spin beside a large one can reach the site alone.
+//    (FxSizes), or where a spin's sums come out large (fx_large, the split shape): a hop joins two spins only, so a
+//    small spin beside a large one can reach the site alone.
 //    Gaussian fields fill all of them; a site beside one site of widely different spins is refused, and so are
 //    sites next to an infinity, a NaN or only components below 2^-959 (E < 64).
 // Others take the FP64 hops. Integer sums do not depend on their order, so every shape of the stencil gives the
@@ -630,6 +631,19 @@ OVL_HD bool fx_hops(const Geom& g, const FxC* U, int s, int k0, int k1, const Fx
   }
   return E < 2000 && top >= 64 << 20;  // (E is above 2047 beside an infinity or a NaN)
 }
+// Whether a spin's sums over all eight hops are at least 2^53 units, 2^-3 of the neighbours' largest component or more: some
+// of its terms are then of that component's size, whatever the neighbours' spins are.
+OVL_HD bool fx_large(const fx64 (&re)[3], const fx64 (&im)[3]) {
+  int m = 0;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const int r = (int)(re[a] >> 32), i = (int)(im[a] >> 32);
+    m = m > (r ^ (r >> 31)) ? m : (r ^ (r >> 31));
+    m = m > (i ^ (i >> 31)) ? m : (i ^ (i >> 31));
+  }
+  return m >= 1 << 21;
+}
+
 // All eight hops.
 template <class Load>
 OVL_HD bool fx_hops(const Geom& g, const FxC* U, int s, int k0, int k1, const FxCoef& c, Load ld, bool g5in, FxAcc& acc,

@@ -316,7 +316,8 @@ __global__ void __launch_bounds__(kBlock)
 // The same with four threads per site (block (32 sites, 4)), one direction's two hops each, for fields too
 // small to fill the GPU with one thread per site: a site's eight hops in a row are about 16 K cycles of one
 // warp's latency. The directions' sums are aligned to their largest exponent and exchanged as integers;
-// thread t finishes spin t.
+// thread t finishes spin t, and looks at the neighbours' sizes only where its sums are small (always: 23.7 us at 12^4
+// instead of 22.9).
 __global__ void __launch_bounds__(128, 3)
     k_dslash_f64_split(Geom g, Links U, FxCoef c, bool native, bool g5_in, bool g5_out, const double2* in, double2* out) {
   __shared__ fx64 part[4][3][6][32];  // [receiving spin][slot of the sender][component][site]
@@ -338,10 +339,7 @@ __global__ void __launch_bounds__(128, 3)
   for (int i = 0; i < 2; ++i) size[i][t][lane] = z.m[i];
   __syncthreads();
   const int Em = max(max(expo[0][lane], expo[1][lane]), max(expo[2][lane], expo[3][lane]));
-#pragma unroll
-  for (int i = 0; i < 2; ++i)
-    z.m[i] = fx_max2(fx_max2(size[i][0][lane], size[i][1][lane]), fx_max2(size[i][2][lane], size[i][3][lane]));
-  const bool all = Em < 1 << 20 && fx_even(z);  // no direction needs the FP64 hops
+  const bool all = Em < 1 << 20;  // no direction needs the FP64 hops
   const int d = min(Em - E, 62);
   if (__any_sync(0xffffffffu, d > 0)) {
     const fx64 half = d > 0 ? (fx64)1 << (d - 1) : 0;
@@ -387,6 +385,25 @@ __global__ void __launch_bounds__(128, 3)
       ar[a] += part[t][p][2 * a][lane];
       ai[a] += part[t][p][2 * a + 1][lane];
     }
+  }
+  if (!fx_large(ar, ai)) {  // (zeros and small spins, and one Gaussian site in 10^6)
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+      z.m[i] = fx_max2(fx_max2(size[i][0][lane], size[i][1][lane]), fx_max2(size[i][2][lane], size[i][3][lane]));
+    if (!fx_even(z)) {  // this spin alone in FP64
+      Spin<double> o;
+      ld(s, o);
+      if (g5_in) gamma5_inplace(o);
+      hops_f64(g, U.f64, s, c.k, 0, 8, ld, g5_in, o);
+      if (g5_out) gamma5_inplace(o);
+#pragma unroll
+      for (int q = 0; q < 12; ++q)
+        if (q / 3 == t) stc<double>(out + off, (size_t)s * ss + (size_t)q * cs, o.c[q / 3][q % 3]);
+      return;
+    }
+  }
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
     const size_t i = (size_t)s * ss + (size_t)(t * 3 + a) * cs;
     const zd x = ldc<double>(in + off, i);
     zd o = mk(fma(f, (double)ar[a], gi * x.re), fma(f, (double)ai[a], gi * x.im));

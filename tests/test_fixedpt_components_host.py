@@ -75,6 +75,7 @@ def field_usable(tmp_path_factory):
         u = np.ascontiguousarray(u)
         return bool(so.field_usable(u.ctypes.data, u.size // 9))
 
+    so.large_spins.argtypes = [ctypes.c_void_p, ctypes.c_double] + [ctypes.c_void_p] * 3
     usable.lib = so
     return usable
 
@@ -243,3 +244,48 @@ def test_link_components_round_to_nearest(field_usable, uexp):
     got, want = np.zeros(len(x), np.int64), np.zeros(len(x), np.int64)
     field_usable.lib.convert(x.ctypes.data, len(x), uexp, got.ctypes.data, want.ctypes.data)
     assert (got == want).all()
+
+
+@pytest.mark.parametrize("mu", [0.0, 0.3, 1.3])
+@pytest.mark.parametrize("spins", [(0,), (1,), (0, 1), (2, 3), (0, 2), (0, 1, 2)])
+@pytest.mark.parametrize("small", [1e-2, 1e-5, 1e-9, 1e-20])
+def test_small_components_where_fixed_point_is_kept(lib, spins, small, mu):
+    """Whatever spins are small on whatever sites: where fixed point is kept, each spin's sum has terms of at least
+    2^-9 of the largest neighbour component (fx_even: 2^-6 and a factor of four), and the sums meet their own bound,
+    2^-49 of four times that component."""
+    u, psi = synth.gauge_links(DIMS, 11), synth.gaussian_source(DIMS, 12)
+    some = np.random.default_rng(13).random((8, 2, 6, 4)) < 0.7
+    for s in spins:
+        psi[..., s, :] *= np.where(some, small, 1.0)[..., None]
+    ok, fx, f64, efx, _, usable = _check(lib, u, psi, mu)
+    assert ok and usable.any()
+    own = (np.abs(psi.real) + np.abs(psi.imag)).reshape(VOL, 12).T
+    terms = (_terms(u, psi, mu) - own).reshape(4, 3, VOL).max(1)
+    top = _spin_sizes(psi, mu).max(1)
+    assert (terms >= 2.0 ** -9 * KAPPA * top)[:, usable].all()
+    hop = 2.0 ** -49 * 4 * top * KAPPA * max(1.0, np.exp(abs(mu)))
+    bound = hop[None, :, None] + 2.0 ** -53 * (3 * np.abs(fx) + 2 * own[:, :, None])
+    assert (efx <= bound)[:, usable].all()
+
+
+@pytest.mark.parametrize("mu", [0.0, 0.3, 1.3])
+@pytest.mark.parametrize("spins", [(), (0,), (1,), (0, 1), (2, 3), (0, 2), (0, 1, 2)])
+@pytest.mark.parametrize("small", [1e-2, 1e-20])
+def test_large_sums_have_large_terms(field_usable, spins, small, mu):
+    """fx_large: sums of at least 2^-3 of the largest neighbour component (2^-5 with the time hops' factors) have terms
+    of 2^-9 of it, over at most three colours and both parts; nearly every sum of a Gaussian field is large, none of a
+    spin without large terms."""
+    u, psi = synth.gauge_links(DIMS, 11), synth.gaussian_source(DIMS, 12)
+    psi[..., list(spins), :] *= small
+    un = np.ascontiguousarray(u.reshape(4, VOL, 9).transpose(0, 2, 1))
+    pn = np.ascontiguousarray(psi.reshape(VOL, 12).T)
+    d, large = np.array(DIMS, np.int32), np.zeros((4, VOL), np.int32)
+    field_usable.lib.large_spins(d.ctypes.data, mu, un.ctypes.data, pn.ctypes.data, large.ctypes.data)
+    large = large.astype(bool)
+    own = (np.abs(psi.real) + np.abs(psi.imag)).reshape(VOL, 12).T
+    terms = (_terms(u, psi, mu) - own).reshape(4, 3, VOL).max(1)
+    top = _spin_sizes(psi, mu).max(1)
+    assert (terms >= 2.0 ** -9 * KAPPA * top)[large].all()
+    assert not large[terms < 2.0 ** -9 * KAPPA * top].any()
+    if not spins:
+        assert large.mean() > 0.999
